@@ -130,7 +130,10 @@ struct fx_grid {
   size_t off_ptab = 0;
   size_t off_hrow = 0;            // FP64 scale-factor rows T_HA, T_HB per direction (curvilinear)
   size_t off_faces = 0;           // gas face buffer [dir][NG+1 (+D-1 with vterms)][faces of dir]
-  size_t off_opk = 0;             // opacity factors of the stage input [K, S][cells]
+  size_t off_frec = 0;            // face records of the radiation fluxes [dir][faces of dir][4]
+  int64_t rec_off[3] = {0, 0, 0};
+  int64_t n_recs = 0;
+  RadTile rt{};                   // tile of the stage kernel (fitted to the device with the chunk)
   size_t off_sflag = 0;           // shock flags of the stage input [cells] (carbuncle guard)
   int64_t face_off[3] = {0, 0, 0};
   int64_t faces_elems = 0;
@@ -677,6 +680,27 @@ Consts<T> make_consts(const fx_grid* h, double dt, double dts, double alpha, boo
   return k;
 }
 
+// The stage kernel's constants as lane values.
+template <class V, class T>
+LaneConst<V> make_lane_consts(const fx_grid* h, double dt, double alpha) {
+  const double c = h->P.c_light;
+  LaneConst<V> k{};
+  auto v = [](double x) { return lane_value((T)x, V()); };
+  k.c = v(c);
+  k.mc = v(-c);
+  k.c3 = v(c / 3.0);
+  k.mc3 = v(-c / 3.0);
+  k.d1 = v(1.0 / (3.0 * c));
+  k.d2 = v(2.0 / (3.0 * c));
+  k.m3 = v(-3.0);
+  k.p4 = v(4.0);
+  k.q25 = v(0.25);
+  for (int d = 0; d < 3; ++d) k.hdt[d] = v(0.5 * dt * h->dg.inv_dx[d]);
+  k.alpha = v(alpha);
+  k.beta = v(1.0 - alpha);
+  return k;
+}
+
 // Stage arguments common to every stage of a handle (tables, constants, buffers).
 template <class R>
 StageArgs<R> stage_args(fx_grid* h) {
@@ -687,7 +711,9 @@ StageArgs<R> stage_args(fx_grid* h) {
   a.vtc = reinterpret_cast<const VtConst*>(h->ws + h->off_vtc);
   a.faces = reinterpret_cast<const R*>(h->ws + h->off_faces);
   a.faces_out = reinterpret_cast<R*>(h->ws + h->off_faces);
-  a.opk = reinterpret_cast<R*>(h->ws + h->off_opk);
+  a.frec = reinterpret_cast<R*>(h->ws + h->off_frec);
+  for (int d = 0; d < 3; ++d) a.rec_off[d] = h->rec_off[d];
+  a.rt = h->rt;
   a.sflag = h->P.shock_guard > 0.0 ? reinterpret_cast<unsigned char*>(h->ws + h->off_sflag) : nullptr;
   for (int d = 0; d < 3; ++d) {
     a.face_off[d] = h->face_off[d];
@@ -707,6 +733,7 @@ StageArgs<R> stage_args(fx_grid* h) {
   a.ptab.status = a.status;
   a.n_state = h->ncell * h->NV;
   a.n_faces = h->faces_elems;
+  a.n_recs = h->n_recs;
 #endif
   a.chunk = h->chunk;
   a.phi_area = (R)h->phi_area;
@@ -732,6 +759,7 @@ void set_stage(fx_grid* h, StageArgs<R>& a, int stage, double dt) {
     a.kd = make_consts<double>(h, dt, 0.5 * dt, 0.5, f32n);
     a.kf = make_consts<float>(h, dt, 0.5 * dt, 0.5, f32n);
   }
+  a.kl = make_lane_consts<typename LaneOf<R>::V, R>(h, dt, a.alpha);
 }
 
 // Enqueue one stage (both kernels), with the per-kernel timing events when enabled and the
@@ -895,6 +923,25 @@ fx_status enqueue_steps(fx_grid* h, double dt, int nsteps) {
     h->time += dt;
   }
   return FX_OK;
+}
+
+// Tile and march chunk (planes per block) of the stage kernel, fitted to the bound device (fit_tile).
+template <class R, class NT> cudaError_t fit_stage(fx_grid* h, int nsm) {
+  int regs = 128;
+  cudaError_t e;
+  const int ro = h->P.rad_recon_order;
+  switch (h->D) {
+    case 1: e = stage_regs<R, 1, NT, false>(ro, &regs); break;
+    case 2: e = h->P.geom == FX_SPH ? stage_regs<R, 2, NT, true>(ro, &regs) : stage_regs<R, 2, NT, false>(ro, &regs); break;
+    default: e = stage_regs<R, 3, NT, false>(ro, &regs); break;
+  }
+  if (e != cudaSuccess) return e;
+  switch (h->D) {
+    case 1: fit_tile<R, 1>(h->dg.n, h->G, nsm, regs, h->rt, h->chunk); break;
+    case 2: fit_tile<R, 2>(h->dg.n, h->G, nsm, regs, h->rt, h->chunk); break;
+    default: fit_tile<R, 3>(h->dg.n, h->G, nsm, regs, h->rt, h->chunk); break;
+  }
+  return cudaSuccess;
 }
 
 // ---- adjoint (config of the boundary-outflow objective; Cartesian grids)
@@ -1153,18 +1200,6 @@ fx_status fx_grid_create(const fx_params* params, fx_grid** out, size_t* workspa
   if (!(P.eps_min > 0.0) || !(P.eps_max > P.eps_min)) return FX_ERR_ARG;
   if (P.newton_maxit < 1 || P.bisect_maxit < 0 || !(P.newton_rtol > 0.0)) return FX_ERR_ARG;
   if (!(P.rho_floor > 0.0) || !(P.p_floor > 0.0) || !(P.E_floor > 0.0)) return FX_ERR_ARG;
-  {
-    const int GP = NCH <= 8 ? 8 : (NCH <= 16 ? 16 : 32);
-    size_t smem = 0;
-    if (P.precision == FX_FP64)
-      smem = P.dims == 1 ? stage_smem<double, 1>(GP, NCH)
-           : P.dims == 2 ? stage_smem<double, 2>(GP, NCH) : stage_smem<double, 3>(GP, NCH);
-    else
-      smem = P.dims == 1 ? stage_smem<float, 1>(GP, NCH)
-           : P.dims == 2 ? stage_smem<float, 2>(GP, NCH) : stage_smem<float, 3>(GP, NCH);
-    if (smem > 227 * 1024) return FX_ERR_UNSUPPORTED;  // per-block shared memory of sm_103a
-  }
-
   fx_grid* h = new fx_grid();
   h->P = P;
   h->D = P.dims;
@@ -1235,7 +1270,7 @@ fx_status fx_grid_create(const fx_params* params, fx_grid** out, size_t* workspa
   }
 
   // chunk length along the march axis: 32 planes until the workspace is bound, where it is fitted
-  // to the device (choose_chunk)
+  // to the device (choose_tile)
   if (P.dims >= 2) h->chunk = std::min((int)P.n[P.dims - 1], 32);
   // workspace layout
   size_t off = 0;
@@ -1260,8 +1295,12 @@ fx_status fx_grid_create(const fx_params* params, fx_grid** out, size_t* workspa
     h->faces_elems = fo;
     off = align_up(off + (size_t)fo * h->elem);
   }
-  h->off_opk = off;
-  off = align_up(off + (size_t)2 * h->ncell * h->elem);
+  for (int d = 0; d < P.dims; ++d) {
+    h->rec_off[d] = h->n_recs;
+    h->n_recs += faces_along(g.n, d);
+  }
+  h->off_frec = off;
+  off = align_up(off + (size_t)4 * h->n_recs * h->elem);
   h->off_sflag = off;  // carbuncle guard: shock flags, one byte per cell
   off = align_up(off + (P.shock_guard > 0.0 ? (size_t)h->ncell : 0));
   // directions whose table rows are all equal (uniform Cartesian spacing) read one row
@@ -1522,49 +1561,15 @@ fx_status fx_state_set_density(fx_grid* h, const void* rho, int rho_precision, i
   return FX_OK;
 }
 
-// March chunk of the stage kernel (planes per block), fitted to the bound device: it minimises
-// (waves of blocks) x (planes per block + the prologue's share), with the device's multiprocessor
-// count and the kernel's resident blocks per multiprocessor.  A grid that overshoots a whole
-// number of waves by a little runs its last wave mostly empty; longer chunks spread the
-// prologue (three planes loaded, two march reconstructions) over more planes.
-fx_status choose_chunk(fx_grid* h) {
-  if (h->D < 2) return FX_OK;
-  int dev = 0, nsm = 0, nb = 0;
+fx_status choose_tile(fx_grid* h) {
+  int dev = 0, nsm = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-  if (e == cudaSuccess) {
-    const int p = h->P.precision;
-    const bool sph = h->P.geom == FX_SPH;
-    if (h->D == 2 && sph)
-      e = p == FX_FP64 ? stage_blocks_per_sm<double, 2, double, true>(h->GP, h->G, h->P.rad_recon_order, &nb)
-        : p == FX_FP32 ? stage_blocks_per_sm<float, 2, float, true>(h->GP, h->G, h->P.rad_recon_order, &nb)
-                       : stage_blocks_per_sm<float, 2, double, true>(h->GP, h->G, h->P.rad_recon_order, &nb);
-    else if (h->D == 2)
-      e = p == FX_FP64 ? stage_blocks_per_sm<double, 2, double, false>(h->GP, h->G, h->P.rad_recon_order, &nb)
-        : p == FX_FP32 ? stage_blocks_per_sm<float, 2, float, false>(h->GP, h->G, h->P.rad_recon_order, &nb)
-                       : stage_blocks_per_sm<float, 2, double, false>(h->GP, h->G, h->P.rad_recon_order, &nb);
-    else
-      e = p == FX_FP64 ? stage_blocks_per_sm<double, 3, double, false>(h->GP, h->G, h->P.rad_recon_order, &nb)
-        : p == FX_FP32 ? stage_blocks_per_sm<float, 3, float, false>(h->GP, h->G, h->P.rad_recon_order, &nb)
-                       : stage_blocks_per_sm<float, 3, double, false>(h->GP, h->G, h->P.rad_recon_order, &nb);
-  }
-  if (e != cudaSuccess) return cuda_fail(h, e, "occupancy query");
-  const int nm = (int)h->P.n[h->D - 1];
-  const int ngl = groups_per_lane(h->elem == 4, h->D, h->GP);
-  const int TC = tile_cells(h->D, h->GP / ngl, ngl);  // cells per tile
-  const int TX = h->D == 3 ? (TC >= 16 ? TC / 4 : TC / 2) : TC, TY = TC / TX;
-  int64_t tiles = (h->P.n[0] + TX - 1) / TX;
-  if (h->D == 3) tiles *= (h->P.n[1] + TY - 1) / TY;
-  const double slots = (double)std::max(nsm, 1) * std::max(nb, 1);
-  double best = 1e300;
-  int bc = std::min(nm, 32);
-  for (int c = 8; c <= std::min(nm, 128); ++c) {
-    const double waves = std::ceil((double)(tiles * ((nm + c - 1) / c)) / slots);
-    const double cost = waves * (c + 1.5);
-    if (cost < best) { best = cost; bc = c; }
-  }
-  h->chunk = bc;
-  return FX_OK;
+  if (e == cudaSuccess)
+    e = h->P.precision == FX_FP64   ? fit_stage<double, double>(h, std::max(nsm, 1))
+        : h->P.precision == FX_FP32 ? fit_stage<float, float>(h, std::max(nsm, 1))
+                                    : fit_stage<float, double>(h, std::max(nsm, 1));
+  return e == cudaSuccess ? FX_OK : cuda_fail(h, e, "stage kernel attributes");
 }
 
 fx_status fx_bind_workspace(fx_grid* h, void* dev_ptr, size_t bytes, void* cuda_stream) {
@@ -1588,7 +1593,7 @@ fx_status fx_bind_workspace(fx_grid* h, void* dev_ptr, size_t bytes, void* cuda_
   if (e == cudaSuccess) e = cudaMemsetAsync(h->ws + h->off_obj, 0, 8 * sizeof(double), h->stream);
   if (e != cudaSuccess) return cuda_fail(h, e, "budget reset");
   {
-    const fx_status cs = choose_chunk(h);
+    const fx_status cs = choose_tile(h);
     if (cs != FX_OK) return cs;
   }
   for (int d = 0; d < h->D; ++d) {

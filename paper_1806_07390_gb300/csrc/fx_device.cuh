@@ -146,30 +146,6 @@ __device__ __forceinline__ void recon_linear_c(const MCCoef<R>& c, V pm, V p0, V
   b = p0 + s * c.dr;
 }
 
-// The same for the two groups of a lane (packed FP32 arithmetic; the limiter's decisions per
-// group).
-template <class R>
-__device__ __forceinline__ void recon_linear_c(const MCCoef<R>& c, F2 pm, F2 p0, F2 pp, F2& a, F2& b) {
-  const F2 s = mc_slope((p0 - pm) * c.il, (pp - p0) * c.ir, (pp - pm) * c.ic);
-  a = vfma(s, c.dl, p0);
-  b = vfma(s, c.dr, p0);
-}
-
-// Linear reconstruction with the MC limiter on centroid gaps (radiation; reading R1).
-template <class R>
-__device__ __forceinline__ void recon_linear(const Tab<R>& t, int ip, R pm, R p0, R pp, R& a, R& b) {
-  R sL = (p0 - pm) * t(T_IL, ip);
-  R sR = (pp - p0) * t(T_IR, ip);
-  R s = R(0);
-  if (sL * sR > R(0)) {
-    R sC = (pp - pm) * t(T_IC, ip);
-    R m = fmin(fmin(R(2) * fabs(sL), R(2) * fabs(sR)), fabs(sC));
-    s = sC > R(0) ? m : -m;
-  }
-  a = p0 + s * t(T_DL, ip);
-  b = p0 + s * t(T_DR, ip);
-}
-
 // ---------------------------------------------------------------------------------------------
 // HLLC (Sec. 5.2; Toro, Spruce & Speares 1994 with Batten et al. 1997 / Einfeldt speed bounds,
 // reading R6).  States are primitive (rho, p, u_n, u_t1, u_t2) in the face-normal frame.
@@ -301,9 +277,46 @@ __device__ __forceinline__ void gas_riemann(int solver, R gam, const R* L, const
   for (int v = 0; v < 2 + D; ++v) f[v] = (br * FL[v] - bl * FR[v] + bl * br * (UR[v] - UL[v])) * ib;
 }
 
-// Reciprocal: IEEE division in FP64; the hardware approximation (2 ulp) in FP32.
+// Reciprocal: IEEE division in FP64; the hardware approximation (1 ulp) in FP32, one instruction
+// (a division intrinsic adds range scaling that no caller needs).
 __device__ __forceinline__ double frcp(double x) { return 1.0 / x; }
-__device__ __forceinline__ float frcp(float x) { return __fdividef(1.0f, x); }
+__device__ __forceinline__ float frcp(float x) { return rcp_approx(x); }
+
+// ---------------------------------------------------------------------------------------------
+// FP64 operations off the FP64 pipe where the result allows it.  The pipe does two lane operations
+// per cycle per multiprocessor (1/64 of FP32), and a comparison, minimum or select of doubles
+// takes a turn on it like any other operation, so the helpers below compare bit patterns with the
+// integer units: doubles of one sign order as their bits do.
+// ---------------------------------------------------------------------------------------------
+// x > 0 and normal
+__device__ __forceinline__ bool normal_pos(double x) { return __double2hiint(x) >= 0x00100000; }
+// 1/x for normal positive x below 2^1022: the hardware seed y (relative error e, |e| < 2^-19)
+// improved by one third-order step y (1 + e + e^2), the truncated geometric series of 1/(1 - e), whose
+// error is e^3 < 2^-57 plus the roundings.
+__device__ __forceinline__ double rcp64(double x) {
+  double y;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  const double e = fma(-x, y, 1.0);
+  return fma(y, fma(e, e, e), y);
+}
+// sqrt(a) for normal positive a: the hardware seed of 1/sqrt(a), one coupled Newton step on
+// g ~ sqrt(a) and h ~ 1/(2 sqrt(a)) (Goldschmidt's iteration), and a last correction by the residual
+// a - g^2.
+__device__ __forceinline__ double sqrt64(double a) {
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(a));
+  double g = a * y, h = 0.5 * y;
+  const double r = fma(-g, h, 0.5);
+  g = fma(g, r, g);
+  h = fma(h, r, h);
+  return fma(fma(-g, g, a), h, g);
+}
+// 1 / max(t, 1)
+__device__ __forceinline__ double rcp_ge1(double t) {
+  const int hi = __double2hiint(t);
+  return hi < 0x3ff00000 ? 1.0 : (hi >= 0x7fd00000 ? 0.0 : rcp64(t));
+}
+__device__ __forceinline__ F2 rcp_ge1(F2 t) { return F2(rcp_approx(fmaxf(t.x, 1.0f)), rcp_approx(fmaxf(t.y, 1.0f))); }
 
 // ---------------------------------------------------------------------------------------------
 // M1 closure (Levermore / Dubroca-Feugeas Eddington factor chi(f) = (3+4f^2)/(5+2 sqrt(4-3f^2)),
@@ -350,41 +363,6 @@ __device__ __forceinline__ void m1_row(R ic2, V E, const V* F, int n, V* P) {
   const V w = R(3) * qd * iE * ic2 * scale * F[n];
 #pragma unroll
   for (int q = 0; q < D; ++q) P[q] = w * F[q] + (q == n ? diag : V(R(0)));
-}
-
-// The same for the two groups of a lane (packed FP32 arithmetic; the FP32 selects per group).
-template <int D>
-__device__ __forceinline__ void m1_row(float ic2, F2 E, const F2* F, int n, F2* P) {
-  F2 F2s = F[0] * F[0];
-#pragma unroll
-  for (int q = 1; q < D; ++q) F2s = vfma(F[q], F[q], F2s);
-  const F2 iE(E.x > 0.0f ? frcp(E.x) : 0.0f, E.y > 0.0f ? frcp(E.y) : 0.0f);
-  F2 f2 = F2s * iE * iE * ic2;
-  const F2 scale = vmin(F2(1.0f), frcp(vmax(f2, F2(1e-30f))));
-  f2 = vmin(f2, F2(1.0f));
-  const F2 qd = frcp(2.0f + vsqrt(vfma(F2(-3.0f), f2, F2(4.0f))));
-  const F2 diag = E * vfma(-f2, qd, F2(1.0f / 3.0f));
-  const F2 w = 3.0f * qd * iE * ic2 * scale * F[n];
-#pragma unroll
-  for (int q = 0; q < D; ++q) P[q] = q == n ? vfma(w, F[q], diag) : w * F[q];
-}
-
-// Full diagonal and the (0,1) entry of P, for the geometric sources of curvilinear grids.
-template <class R, int D>
-__device__ __forceinline__ void m1_full(R c, R E, const R* F, R* Pd, R& P01) {
-  R F2 = F[0] * F[0];
-#pragma unroll
-  for (int q = 1; q < D; ++q) F2 += F[q] * F[q];
-  P01 = R(0);
-  if (F2 <= R(0) || E <= R(0)) { Pd[0] = Pd[1] = Pd[2] = E * R(1.0 / 3.0); return; }
-  R f = sqrt(F2) / (c * E);
-  f = f > R(1) ? R(1) : f;
-  R f2 = f * f;
-  R chi = (R(3) + R(4) * f2) / (R(5) + R(2) * sqrt(R(4) - R(3) * f2));
-  R ca = R(0.5) * (R(1) - chi), cb = R(0.5) * (R(3) * chi - R(1));
-#pragma unroll
-  for (int q = 0; q < 3; ++q) Pd[q] = E * (ca + (q < D ? cb * F[q] * F[q] / F2 : R(0)));
-  if (D >= 2) P01 = E * cb * F[0] * F[1 < D ? 1 : 0] / F2;
 }
 
 // ---------------------------------------------------------------------------------------------

@@ -2,10 +2,10 @@
 // reconstruction of the two neighbouring cells (Sec. 5.1) and the Riemann flux (HLLC, or the
 // HLLE / local Lax-Friedrichs options and the carbuncle guard) with the HLLC contact speed
 // (Sec. 5.2).  A block stages a tile's primitives in shared memory and reconstructs each
-// cell once, for both of its faces.  It also forms every cell's opacity factors.
-// The stage kernel then uses the fluxes for the gas divergence, the contact speeds to upwind the
-// radiation advection (Eq. 19), and the opacity factors for the ε correction of the radiation
-// fluxes; with the velocity-dependent radiation terms on, the kernel also stores each face's
+// cell once, for both of its faces.  It also forms every face's record for the radiation fluxes
+// (the upwind advection speeds of Eq. 19 and the sums of the two cells' opacity factors for the ε
+// correction), so that the stage kernel reads one aligned record per face.
+// The stage kernel then uses the fluxes for the gas divergence; with the velocity-dependent radiation terms on, the kernel also stores each face's
 // transverse velocity for their velocity gradient (fx_vterms.cuh).
 #pragma once
 #include "fx_device.cuh"
@@ -48,7 +48,7 @@ __host__ __device__ inline unsigned face_tiles(const int* n, int D, int DIR) {
 // selected Riemann flux.
 template <class R, int D, int DIR>
 __device__ __forceinline__ void gas_faces_tile(const StageArgs<R>& A, unsigned tile, R (*sw)[FACE_WCELLS],
-                                               R (*sb)[FACE_BCELLS]) {
+                                               R (*sb)[FACE_BCELLS], R (*sk)[FACE_WCELLS]) {
   constexpr int NG = 2 + D, NW = 2 + D;
   using FT = FaceTile<DIR>;
   constexpr int LD = FT::LD, LX = FT::LX, NWC = FT::NWC;
@@ -102,21 +102,15 @@ __device__ __forceinline__ void gas_faces_tile(const StageArgs<R>& A, unsigned t
       sw[2 + q][FXI(c, FACE_WCELLS)] = vq;
       ke += u[1 + q] * vq;
     }
+    const R p = KR.gm1 * (u[NG - 1] - R(0.5) * ke);
     sw[0][FXI(c, FACE_WCELLS)] = rho;
-    sw[1][FXI(c, FACE_WCELLS)] = KR.gm1 * (u[NG - 1] - R(0.5) * ke);
+    sw[1][FXI(c, FACE_WCELLS)] = p;
+    // opacity factors K = kappa0 rho^a T^b and S = sigma0 rho, for the faces' optical depths
+    const R T = p * irho;
+    sk[0][FXI(c, FACE_WCELLS)] = T > R(0) ? KR.kappa0 * hpow(rho, g.kap_rho_h) * hpow(T, g.kap_T_h) : R(0);
+    sk[1][FXI(c, FACE_WCELLS)] = KR.sigma0 * rho;
   }
   __syncthreads();
-  if (DIR == 0) {
-    // the opacity factors K = kappa0 rho^a T^b and S = sigma0 rho of the stage input, once per
-    // cell (each cell is a face owner of exactly one x tile), for the radiation/update kernel
-    const int r = t, id = d0 - 1 + r;
-    if (r >= 1 && id < n0) {
-      const R rho = sw[0][FXI(r + 1, FACE_WCELLS)], T = sw[1][FXI(r + 1, FACE_WCELLS)] * frcp(rho);
-      const uint32_t ci = ((uint32_t)i2 * n1 + i1) * n0 + (uint32_t)id;
-      A.opk[FXI(ci, 2 * ncell)] = T > R(0) ? KR.kappa0 * hpow(rho, g.kap_rho_h) * hpow(T, g.kap_T_h) : R(0);
-      A.opk[FXI(ncell + ci, 2 * ncell)] = KR.sigma0 * rho;
-    }
-  }
   // ---- each thread reconstructs one cell along DIR (row r: cell d0 - 1 + r): the upper-face
   // state to shared memory (the left state of the face above), the lower-face state kept for the
   // cell's own face
@@ -173,6 +167,19 @@ __device__ __forceinline__ void gas_faces_tile(const StageArgs<R>& A, unsigned t
   for (int c = 0; c < D; ++c) out[FXI((uint32_t)(1 + (DIR + c) % D) * nf + uf, n_out)] = fl[1 + c];
   out[FXI((uint32_t)(NG - 1) * nf + uf, n_out)] = fl[1 + D];
   out[FXI((uint32_t)NG * nf + uf, n_out)] = vs;
+  {  // the face's record for the radiation fluxes (StageArgs::frec)
+    const R ell = R(0.5) * tt(T_ELL, bc_pad(id)) * ((sph && DIR == 1) ? t0(T_XH, bc_pad(x)) : R(1));
+    const int wl = FXI(r * LX + lx, FACE_WCELLS), wr = FXI((r + 1) * LX + lx, FACE_WCELLS);
+    const R r0 = vs > R(0) ? vs + vs : R(0), r1 = vs > R(0) ? R(0) : vs + vs;
+    const R r2 = ell * (sk[0][wl] + sk[0][wr]), r3 = ell * (sk[1][wl] + sk[1][wr]);
+    R* const q = A.frec + (size_t)4 * FXI((uint32_t)A.rec_off[DIR] + uf, A.n_recs);
+    if constexpr (sizeof(R) == 4) {
+      *reinterpret_cast<float4*>(q) = make_float4(r0, r1, r2, r3);
+    } else {
+      reinterpret_cast<double2*>(q)[0] = make_double2(r0, r1);
+      reinterpret_cast<double2*>(q)[1] = make_double2(r2, r3);
+    }
+  }
   if (g.vterms) {
     // face velocity vector for the velocity-dependent radiation terms: v* normal, the transverse
     // components of the state on the v* upwind side (rotated order, rows NG + 1 .. NG + D - 1)
@@ -238,11 +245,12 @@ __global__ void __launch_bounds__(FACE_THREADS, 3)
 gas_face_kernel(const __grid_constant__ StageArgs<R> A) {
   __shared__ R sw[2 + D][FACE_WCELLS];
   __shared__ R sb[2 + D][FACE_BCELLS];
+  __shared__ R sk[2][FACE_WCELLS];
   const int DIR = blockIdx.y;
   if (blockIdx.x >= face_tiles(A.g.n, D, DIR)) return;
-  if (DIR == 0) gas_faces_tile<R, D, 0>(A, blockIdx.x, sw, sb);
-  else if (D >= 2 && DIR == 1) gas_faces_tile<R, D, (D >= 2 ? 1 : 0)>(A, blockIdx.x, sw, sb);
-  else if (D >= 3) gas_faces_tile<R, D, (D >= 3 ? 2 : 0)>(A, blockIdx.x, sw, sb);
+  if (DIR == 0) gas_faces_tile<R, D, 0>(A, blockIdx.x, sw, sb, sk);
+  else if (D >= 2 && DIR == 1) gas_faces_tile<R, D, (D >= 2 ? 1 : 0)>(A, blockIdx.x, sw, sb, sk);
+  else if (D >= 3) gas_faces_tile<R, D, (D >= 3 ? 2 : 0)>(A, blockIdx.x, sw, sb, sk);
 }
 
 }  // namespace fx

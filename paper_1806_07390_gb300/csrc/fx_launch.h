@@ -3,6 +3,9 @@
 #pragma once
 #include <cuda_runtime.h>
 
+#include <algorithm>
+#include <cmath>
+
 #include "fx_couple.cuh"
 #include "fx_couple64.cuh"
 #include "fx_stage.cuh"
@@ -11,35 +14,73 @@
 
 namespace fx {
 
-// Groups per lane of the stage kernel: two in the FP32 forms when a cell has more than 8 groups
-// (GP >= 16), else one.  GP = next power of two >= G is the cell's padded group count.  Two groups
-// per lane share the per-cell work of a thread (indexing, opacity factors, gas variables, the
-// halo branches) between two groups and double the tile's cells (a smaller halo share), at more
-// registers per thread (GP = 16: kh2d stage kernel 0.547 -> 0.525 ms with 32-cell tiles;
-// lognormal3d 18.6 -> 17.3 ms once the tile-edge work ran one group per lane).
-constexpr int groups_per_lane(bool fp32, int D, int GP) {
-  (void)D;
-  return (fp32 && GP >= 16) ? 2 : 1;
+// Tile and march chunk of the stage kernel for a grid, fitted to the device.  A model of its time
+// over every tile that the kernel's capacities allow and every chunk length picks the least:
+//   waves x ((chunk + 2) x (time of one plane) + start), two planes being the prologue's share,
+// where a fractional number of waves x costs x + 0.9 (ceil x - x) / ceil x (fitted to measured
+// chunks: multiprocessors that finish early idle, the others run faster with fewer blocks).
+// A plane's time on a multiprocessor with r resident blocks joins (root of squares) what one block
+// alone takes (in FP32 a warp issues about every sixth cycle; in FP64 its chain of 16-cycle operations,
+// nearly as long for one block as for two) and the issue of the r blocks' instructions.  The
+// instruction counts are per warp and plane, from the kernel's operation counts: they only rank
+// tiles against each other.  So small grids get small tiles and short chunks that spread over the
+// device, and large ones the tiles with the least halo share and the fewest idle lanes.  Measured
+// against a sweep of tiles and chunks (stage kernel, microseconds, chosen / best of the sweep):
+// 1024^2 x 16 FP32 253 / 245, 256^3 x 12 FP32 7140 / 7140, 640 x 128 x 20 spherical FP32 70 / 70,
+// 75 x 61 x 50 x 20 FP32 250 / 243, 96 x 80 x 8 FP32 10.9 / 10.5, 512^2 x 16 FP64 1862 / 1862.
+template <class R, int D>
+inline void fit_tile(const int* n, int G, int nsm, int regs, RadTile& best, int& chunk) {
+  using C = StageCap<R, D>;
+  constexpr int W = LaneOf<R>::W;
+  constexpr int NRV = 1 + D;
+  const int gl = (G + W - 1) / W;
+  const double recon = 12.0 * NRV + 3.0, flux = 64.0 + 5.0 * NRV, own = D * (recon + flux) + NRV * 30.0 + 60.0;
+  const double alone = sizeof(R) == 8 ? own * 155.0 : own / 0.16 + 800.0, IPC = sizeof(R) == 8 ? 0.097 : 2.6;
+  double least = 1e300;
+  best = RadTile{};
+  const int nm = D >= 2 ? n[D - 1] : 1;
+  for (int ty = D == 3 ? 16 : 1; ty >= 1; --ty) {
+    for (int tx = 1; tx * ty * gl <= C::NT; ++tx) {
+      if (ty * gl > C::XP || (D == 3 && tx * gl > C::XP) || tx > n[0] + 3) continue;
+      RadTile t{};
+      t.tx = tx; t.ty = ty; t.gl = gl;
+      t.nth = (tx * ty * gl + 31) / 32 * 32;
+      t.ntx = (n[0] + tx - 1) / tx;
+      t.nty = D == 3 ? (n[1] + ty - 1) / ty : 1;
+      // upper faces: at most one per thread; in 1-d and 2-d also one halo reconstruction, one halo
+      // copy and two records
+      const int nt = (ty + (D == 3 ? tx : 0)) * gl;
+      if (nt > t.nth || (D < 3 && (4 * gl > t.nth || tile_recs<D>(t) > 2 * t.nth))) continue;
+      // copies past the ones whose offsets a thread keeps
+      const int late = std::max(0, tile_halo<D>(t) * gl - (D == 3 ? 2 : 1) * t.nth) + std::max(0, tile_recs<D>(t) - 2 * t.nth);
+      const size_t smem = stage_smem_bytes<R, D>(t);
+      if (smem > 200 * 1024) continue;
+      const int rmax = std::max(1, std::min({65536 / (regs * t.nth), (int)(227 * 1024 / (smem + 1024)), 2048 / t.nth, 32}));
+      const double instr = t.nth / 32 * own + (2 * nt + 31) / 32 * (recon + 30.0) + (nt + 31) / 32 * (flux + 30.0) + (late + 31) / 32 * 60.0;
+      const double tiles = (double)t.ntx * t.nty;
+      // the shortest chunk of every count of chunks
+      for (int c = std::min(nm, 160), m; c >= 1; --c) {
+        m = (nm + c - 1) / c;
+        c = (nm + m - 1) / m;
+        const double blocks = tiles * m;
+        const double r = std::min((double)rmax, std::ceil(blocks / nsm));
+        const double issue = r * instr / IPC, plane = std::sqrt(alone * alone + issue * issue);
+        const double x = blocks / (r * nsm), xc = std::ceil(x), w = x <= 1.0 ? 1.0 : x + 0.9 * (xc - x) / xc;
+        const double cost = w * ((c + (D >= 2 ? 2.0 : 0.0)) * plane + 1500.0);
+        if (cost <= least) {
+          least = cost;
+          best = t;
+          chunk = c;
+        }
+      }
+    }
+  }
+  // gas cells per thread: one on small grids, up to four where the gas blocks fill the device anyway
+  double cells = 1.0;
+  for (int d = 0; d < D; ++d) cells *= n[d];
+  best.gpt = std::min(4, std::max(1, (int)(cells / (2048.0 * nsm))));
+  best.mgl = (unsigned)(((1ull << 32) + gl - 1) / gl);
 }
-
-// Cells per tile of the stage kernel for D dimensions and GL lanes per cell: 256 threads per
-// block, except 2-d with two groups per lane of 8 lanes (16 padded groups): a 20-cell tile of 160
-// threads (kh2d stage kernel 0.462 -> 0.455 ms against 32-cell tiles of 256 threads; 16-, 24-
-// and 28-cell tiles were slower).  It ran at four blocks per SM (96 registers) until the packed
-// pair arithmetic made that bound spill; at three blocks per SM it does not spill and is as fast
-// (0.482 -> 0.480 ms).
-__host__ __device__ constexpr int tile_cells(int D, int GL, int NGL) {
-  return (D == 2 && GL == 8 && NGL == 2) ? 20 : 256 / GL;
-}
-
-// Tile shape of the stage kernel for D dimensions, GL lanes per cell and NGL groups per lane.  (In
-// 3-d an 8 x 8 tile of 512 threads, one block per SM, halves the tile-edge share of the 8 x 4 tile
-// but was slower: lognormal3d stage kernel 17.06 ms against 16.44.)
-template <int D, int GL, int NGL> struct TileShape {
-  static constexpr int TC = tile_cells(D, GL, NGL);         // cells per tile
-  static constexpr int TX = (D == 3) ? (TC >= 16 ? TC / 4 : TC / 2) : TC;
-  static constexpr int TY = TC / TX;
-};
 
 // Enqueue one stage (state type R, D dimensions, Newton/bookkeeping type NT; SPH: the 2-d
 // spherical grid) on stream s: the gas face kernel, the radiation/update kernel, with the
@@ -51,44 +92,25 @@ template <class R, int D, class NT, bool SPH>
 cudaError_t launch_stage(const StageArgs<R>& a, int GP, cudaStream_t s, cudaEvent_t mid,
                          cudaEvent_t mid2);
 
-// Resident blocks per multiprocessor of the stage kernel for GP padded groups, G groups and
-// radiation reconstruction order ro (the CUDA occupancy calculator; the host sizes the march
-// chunks from it).
+// Registers per thread of the stage kernel (radiation reconstruction order ro), for fit_tile.
 template <class R, int D, class NT, bool SPH>
-cudaError_t stage_blocks_per_sm(int GP, int G, int ro, int* nb);
-
-// Dynamic shared memory of the stage kernel (tile shape from D and GP).
-template <class R, int D, int GP>
-inline size_t stage_smem_gp(int G) {
-  constexpr int NGL = groups_per_lane(sizeof(R) == 4, D, GP);
-  using TS = TileShape<D, GP / NGL, NGL>;
-  return stage_smem_bytes<R, D, TS::TX, TS::TY>(stage_gstride<D, GP>(G));
-}
-template <class R, int D>
-inline size_t stage_smem(int GP, int G) {
-  switch (GP) {
-    case 8: return stage_smem_gp<R, D, 8>(G);
-    case 16: return stage_smem_gp<R, D, 16>(G);
-    case 32: return stage_smem_gp<R, D, 32>(G);
-    default: return 0;
-  }
-}
+cudaError_t stage_regs(int ro, int* regs);
 
 #ifdef FX_LAUNCH_DEFINE
 // Definition, included only by the per-instantiation translation units.  The group arithmetic
 // type of the stage kernel is the state type R.
 template <class R, int D, int GP, class NT, bool SPH>
-static cudaError_t launch_gp(const StageArgs<R>& a, cudaStream_t s, cudaEvent_t mid, cudaEvent_t mid2) {
-  constexpr int NGL = groups_per_lane(sizeof(R) == 4, D, GP);
-  constexpr int GL = GP / NGL;
-  using TS = TileShape<D, GL, NGL>;
-  if ((a.g.geom != 0) != SPH) return cudaErrorInvalidValue;  // the grid's geometry decides SPH
+static cudaError_t launch_gp(const StageArgs<R>& a0, cudaStream_t s, cudaEvent_t mid, cudaEvent_t mid2) {
+  if ((a0.g.geom != 0) != SPH) return cudaErrorInvalidValue;  // the grid's geometry decides SPH
+  StageArgs<R> a = a0;
+  // lanes copy and store pairs with 8-byte accesses where every pair is complete and aligned
+  auto al8 = [](const void* p) { return (reinterpret_cast<uintptr_t>(p) & 7) == 0; };
+  a.rt.vec = a.g.G % 2 == 0 && ((2 + D) * a.g.ncell) % 2 == 0 && al8(a.in) && al8(a.base) && al8(a.out);
   // (the boundary budgets are compiled into the kernel for grids with a non-periodic boundary;
   // the second-order radiation reconstruction always carries them)
-  auto kern = a.g.rad_order == 2 ? stage_kernel<R, D, GP, TS::TX, TS::TY, R, NT, NGL, SPH, 2, true>
-              : (a.budget_bnd ? stage_kernel<R, D, GP, TS::TX, TS::TY, R, NT, NGL, SPH, 1, true>
-                              : stage_kernel<R, D, GP, TS::TX, TS::TY, R, NT, NGL, SPH, 1, false>);
-  const size_t smem = stage_smem_bytes<R, D, TS::TX, TS::TY>(stage_gstride<D, GP>(a.g.G));
+  auto kern = a.g.rad_order == 2 ? stage_kernel<R, D, SPH, 2, true>
+              : (a.budget_bnd ? stage_kernel<R, D, SPH, 1, true> : stage_kernel<R, D, SPH, 1, false>);
+  const size_t smem = stage_smem_bytes<R, D>(a.rt);
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout,
@@ -111,14 +133,10 @@ static cudaError_t launch_gp(const StageArgs<R>& a, cudaStream_t s, cudaEvent_t 
     e = cudaEventRecord(mid, s);
     if (e != cudaSuccess) return e;
   }
-  // radiation and update: tiles across the fast axes, chunks of the slowest axis
-  dim3 grid((a.g.n[0] + TS::TX - 1) / TS::TX, 1, 1);
-  if (D == 2) grid.y = (a.g.n[1] + a.chunk - 1) / a.chunk;
-  if (D == 3) {
-    grid.y = (a.g.n[1] + TS::TY - 1) / TS::TY;
-    grid.z = (a.g.n[2] + a.chunk - 1) / a.chunk;
-  }
-  kern<<<grid, TS::TX * TS::TY * GL, smem, s>>>(a);
+  // radiation blocks (tiles across the fast axes, chunks of the slowest) and gas blocks
+  a.rt.nrad = a.rt.ntx * a.rt.nty * (D >= 2 ? (a.g.n[D - 1] + a.chunk - 1) / a.chunk : 1);
+  const int64_t ngas = (a.g.ncell + a.rt.gpt * a.rt.nth - 1) / (a.rt.gpt * a.rt.nth);
+  kern<<<(unsigned)(a.rt.nrad + ngas), (unsigned)a.rt.nth, smem, s>>>(a);
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   if (mid2) {
@@ -175,29 +193,13 @@ static cudaError_t launch_gp(const StageArgs<R>& a, cudaStream_t s, cudaEvent_t 
   return e;
 }
 
-template <class R, int D, int GP, class NT, bool SPH>
-static cudaError_t blocks_gp(int G, int ro, int* nb) {
-  constexpr int NGL = groups_per_lane(sizeof(R) == 4, D, GP);
-  constexpr int GL = GP / NGL;
-  using TS = TileShape<D, GL, NGL>;
-  auto kern = ro == 2 ? stage_kernel<R, D, GP, TS::TX, TS::TY, R, NT, NGL, SPH, 2, true>
-                      : stage_kernel<R, D, GP, TS::TX, TS::TY, R, NT, NGL, SPH, 1, false>;
-  const size_t smem = stage_smem_bytes<R, D, TS::TX, TS::TY>(stage_gstride<D, GP>(G));
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
-  if (e != cudaSuccess) return e;
-  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(nb, kern, TS::TX * TS::TY * GL, smem);
-}
-
 template <class R, int D, class NT, bool SPH>
-cudaError_t stage_blocks_per_sm(int GP, int G, int ro, int* nb) {
-  switch (GP) {
-    case 8: return blocks_gp<R, D, 8, NT, SPH>(G, ro, nb);
-    case 16: return blocks_gp<R, D, 16, NT, SPH>(G, ro, nb);
-    case 32: return blocks_gp<R, D, 32, NT, SPH>(G, ro, nb);
-    default: return cudaErrorInvalidValue;
-  }
+cudaError_t stage_regs(int ro, int* regs) {
+  cudaFuncAttributes fa;
+  const cudaError_t e = ro == 2 ? cudaFuncGetAttributes(&fa, stage_kernel<R, D, SPH, 2, true>)
+                                : cudaFuncGetAttributes(&fa, stage_kernel<R, D, SPH, 1, false>);
+  if (e == cudaSuccess) *regs = fa.numRegs;
+  return e;
 }
 
 template <class R, int D, class NT, bool SPH>

@@ -9,12 +9,16 @@
 
 namespace fx {
 
-struct F2 {
+struct alignas(8) F2 {
   float x, y;
-  __device__ __forceinline__ F2() {}
-  __device__ __forceinline__ F2(float a, float b) : x(a), y(b) {}
-  __device__ __forceinline__ explicit F2(float a) : x(a), y(a) {}
+  F2() = default;
+  __host__ __device__ __forceinline__ F2(float a, float b) : x(a), y(b) {}
+  __host__ __device__ __forceinline__ explicit F2(float a) : x(a), y(a) {}
 };
+
+// x as a lane value (both halves of a pair)
+__host__ __device__ __forceinline__ F2 lane_value(float x, F2) { return F2(x); }
+__host__ __device__ __forceinline__ double lane_value(double x, double) { return x; }
 
 __device__ __forceinline__ unsigned long long f2_pack(F2 a) {
   unsigned long long r;
@@ -60,8 +64,15 @@ __device__ __forceinline__ F2 vfma(F2 a, F2 b, F2 c) {
 __device__ __forceinline__ F2 vfma(F2 a, float b, F2 c) { return vfma(a, F2(b), c); }
 __device__ __forceinline__ F2 vfma(float a, F2 b, F2 c) { return vfma(F2(a), b, c); }
 
+// Hardware reciprocal (1 ulp; denormal arguments are flushed to zero and give an infinity).
+__device__ __forceinline__ float rcp_approx(float x) {
+  float y;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+
 // Componentwise operations, with the scalar overloads used by code written for either type.
-__device__ __forceinline__ F2 frcp(F2 a) { return F2(__fdividef(1.0f, a.x), __fdividef(1.0f, a.y)); }
+__device__ __forceinline__ F2 frcp(F2 a) { return F2(rcp_approx(a.x), rcp_approx(a.y)); }
 __device__ __forceinline__ float vsqrt(float a) { return sqrtf(a); }
 __device__ __forceinline__ double vsqrt(double a) { return ::sqrt(a); }
 __device__ __forceinline__ F2 vsqrt(F2 a) { return F2(sqrtf(a.x), sqrtf(a.y)); }
@@ -74,13 +85,6 @@ __device__ __forceinline__ F2 vabs(F2 a) { return F2(fabsf(a.x), fabsf(a.y)); }
 __device__ __forceinline__ double vmin(double a, double b) { return fmin(a, b); }
 __device__ __forceinline__ double vmax(double a, double b) { return fmax(a, b); }
 __device__ __forceinline__ double vabs(double a) { return fabs(a); }
-// x > t ? a : b, componentwise in x, a and b
-__device__ __forceinline__ float vsel_gt(float x, float t, float a, float b) { return x > t ? a : b; }
-__device__ __forceinline__ double vsel_gt(double x, double t, double a, double b) { return x > t ? a : b; }
-__device__ __forceinline__ F2 vsel_gt(F2 x, float t, F2 a, F2 b) {
-  return F2(x.x > t ? a.x : b.x, x.y > t ? a.y : b.y);
-}
-
 // Slope of the MC limiter from the one-sided slopes sL, sR and the centred slope sC: the least of
 // 2|sL|, 2|sR| and |sC|, with the common sign of sL and sR, and zero where their signs differ or
 // one is zero.  Where sL and sR share a sign, sC has it too (the centred difference is the sum
@@ -95,6 +99,30 @@ __device__ __forceinline__ F2 mc_slope(F2 sL, F2 sR, F2 sC) {
   const F2 m(fminf(m2.x, fabsf(sC.x)), fminf(m2.y, fabsf(sC.y)));
   return m * (F2(copysignf(0.5f, sL.x), copysignf(0.5f, sL.y)) +
               F2(copysignf(0.5f, sR.x), copysignf(0.5f, sR.y)));
+}
+
+// The limited difference of the MC limiter from the one-sided differences dl, dr and the centred
+// one q: the least of m|dl|, m|dr| and |q| with their common sign, zero where the signs of dl and dr
+// differ or one is zero (q has their sign where they agree).  In FP32 three instructions per value:
+// min.xorsign.abs gives the least magnitude, negative where the signs differ, which the maximum
+// with zero removes; the second one gives the sign of q.  In FP64 the magnitudes and signs are
+// compared as integers, which leaves the FP64 pipe to the arithmetic.
+__device__ __forceinline__ float min_xs(float a, float b) {
+  float y;
+  asm("min.ftz.xorsign.abs.f32 %0, %1, %2;" : "=f"(y) : "f"(a), "f"(b));
+  return y;
+}
+__device__ __forceinline__ F2 mc_min(F2 dl, F2 dr, F2 q, float m) {
+  F2 r(fmaxf(min_xs(dl.x, dr.x), 0.0f), fmaxf(min_xs(dl.y, dr.y), 0.0f));
+  if (m != 1.0f) r = r * m;
+  return F2(min_xs(r.x, q.x), min_xs(r.y, q.y));
+}
+__device__ __forceinline__ double mc_min(double dl, double dr, double q, double m) {
+  const long long a = __double_as_longlong(dl), b = __double_as_longlong(dr), M = 0x7fffffffffffffffLL;
+  long long r = min(a & M, b & M);
+  if (m != 1.0) r = __double_as_longlong(__longlong_as_double(r) * m);
+  r = min(r, __double_as_longlong(q) & M);
+  return (a ^ b) < 0 ? 0.0 : __longlong_as_double(r | (a & ~M));
 }
 
 // A value of type V from the values of the lane's two groups (the pair, or the first value), and
@@ -120,6 +148,17 @@ __device__ __forceinline__ void st_lane(double* p, double v, bool h0, bool) { if
 __device__ __forceinline__ void st_lane(float* p, F2 v, bool h0, bool h1) {
   if (h1) *reinterpret_cast<float2*>(p) = make_float2(v.x, v.y);
   else if (h0) *p = v.x;
+}
+
+// Global store of a lane's groups: one 8-byte store where the pair is aligned (vec: both exist).
+__device__ __forceinline__ void st_global_lane(double* p, double v, bool, bool) { *p = v; }
+__device__ __forceinline__ void st_global_lane(float* p, F2 v, bool vec, bool h1) {
+  if (vec) {
+    *reinterpret_cast<float2*>(p) = make_float2(v.x, v.y);
+  } else {
+    p[0] = v.x;
+    if (h1) p[1] = v.y;
+  }
 }
 
 }  // namespace fx

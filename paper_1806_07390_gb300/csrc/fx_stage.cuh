@@ -1,16 +1,9 @@
-// Fused SSP-RK2 stage kernel: explicit transport (reconstruction, HLLC, M1/HLL radiation fluxes,
-// flux divergence) + RK combine in one pass over HBM.  The cell-local implicit interaction runs
-// after it as a kernel of its own, one thread per cell (couple_kernel in fx_couple.cuh for the
-// FP32 state, couple64_kernel in fx_couple64.cuh for the FP64 state).
-//
-// Work decomposition.  A thread block owns a tile of TX (x) by TY (y, 3-d only) cells and
-// marches along the slowest active axis (y in 2-d, z in 3-d) over `chunk` planes.  Each cell is
-// served by a segment of GP/NGL lanes (GP = power of two >= groups); a lane owns NGL consecutive
-// groups (two in the FP32 forms when GP >= 16, else one).  A shared
-// ring of four planes holds the conserved state (k-1 .. k+2) so that every face flux is computed
-// exactly once: in-plane faces per plane, and the march-direction face k+1/2 per step, carried
-// in registers to the next step.  Ghost cells are produced at load time from the boundary
-// conditions (Sec. 7.5), so no separate ghost-fill pass touches HBM.
+// SSP-RK2 stage kernel: explicit transport (reconstruction, M1/HLL radiation fluxes, flux divergence
+// of gas and radiation) + RK combine in one pass over HBM.  The gas faces run before it
+// (gas_face_kernel, fx_gas.cuh) and the cell-local implicit interaction after it, as kernels of
+// their own, one thread per cell (couple_kernel in fx_couple.cuh for the FP32 state,
+// couple64_kernel in fx_couple64.cuh for the FP64 state).  Ghost cells are index maps applied when
+// cells are loaded (Sec. 7.5): no separate ghost-fill pass touches HBM.
 #pragma once
 #include <type_traits>
 
@@ -66,6 +59,22 @@ struct PlanckTable {
 #endif
 };
 
+// Lane value of the stage kernel: a lane owns W groups, two as one packed FP32 pair, one in FP64.
+template <class R> struct LaneOf;
+template <> struct LaneOf<float> { using V = F2; static constexpr int W = 2; };
+template <> struct LaneOf<double> { using V = double; static constexpr int W = 1; };
+
+// Constants of the stage kernel as lane values (pairs of equal floats in FP32: a packed instruction
+// takes both halves from registers, and a scalar would be copied into a pair at every use).
+template <class V> struct LaneConst {
+  V c, mc;              // c, -c
+  V c3, mc3;            // c/3, -c/3
+  V d1, d2;             // 1/(3c), 2/(3c)
+  V m3, p4, q25;        // -3, 4, 1/4
+  V hdt[3];             // stage step / (2 cell width)
+  V alpha, beta;        // RK weights
+};
+
 struct VtConst;  // frequency constants of the velocity-dependent terms (fx_vterms.cuh)
 
 template <class R> struct StageArgs {
@@ -74,8 +83,14 @@ template <class R> struct StageArgs {
   const R* faces;      // gas face fluxes and contact speeds [dir][NG+1][faces of dir], then, with
                        // the velocity terms on, D-1 rows of transverse face velocities
   R* faces_out;        // the same buffer, written by gas_face_kernel
-  R* opk;              // opacity factors K = kappa0 rho^a T^b, S = sigma0 rho of every cell of the
-                       // stage input [2][ncell]: gas_face_kernel writes, stage_kernel reads
+  // Face records for the radiation fluxes, four values per face [dir][faces of dir][4]:
+  // 2 max(v*, 0), 2 min(v*, 0) (the upwind advection, Eq. 19) and the two sums over the face's
+  // cells that give the optical depth of group g (reading R9) as eps_g^d r2 + r3, with r2 =
+  // (K_L + K_R) ell/2, K = kappa0 rho^a T^b, and r3 likewise from S = sigma0 rho.  gas_face_kernel
+  // writes them, stage_kernel reads them as one 16-byte (FP32) copy per face.
+  R* frec;
+  int64_t rec_off[3];  // first face of each direction in `frec`
+  RadTile rt;          // tile of the stage kernel's radiation blocks
   unsigned char* sflag;  // carbuncle guard (null when off): bit e of a cell's byte is set when a
                          // face of direction e of the cell lies in a shock (shock_flag_kernel)
   int64_t face_off[3]; // element offset of each direction's block in `faces`
@@ -91,7 +106,8 @@ template <class R> struct StageArgs {
   unsigned* status;
 #ifdef FX_BOUNDS_CHECK
   int64_t n_state;     // elements of a state (in, base, out, pre_out) and of the gas face buffer,
-  int64_t n_faces;     // for the index checks of the debug build
+  int64_t n_faces;     // and faces in frec, for the index checks of the debug build
+  int64_t n_recs;
 #endif
   double dt;           // stage step
   double dts;          // coupling step (dt after stage 1, dt/2 after stage 2; reading R10)
@@ -117,6 +133,7 @@ template <class R> struct StageArgs {
   int budget_bnd;  // the grid has a non-periodic boundary: the stage kernel adds its outflows
   Consts<double> kd;
   Consts<float> kf;
+  LaneConst<typename LaneOf<R>::V> kl;
   __device__ __forceinline__ const Consts<double>& k(double) const { return kd; }
   __device__ __forceinline__ const Consts<float>& k(float) const { return kf; }
 };
@@ -364,1022 +381,883 @@ __device__ __forceinline__ void bar_wait(int id, int n) {
 }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
 
-// Shared-memory layout of stage_kernel (offsets in elements of R; used by the kernel and by the
-// host to size the launch).
-template <int D, int TX, int TY>
-struct StageLayout {
-  static constexpr int NG = 2 + D, NRV = 1 + D;
-  static constexpr int PX = TX + 4, PY = (D == 3) ? TY + 4 : 1, PC = PX * PY;
-  static constexpr int NSLOT = (D >= 2) ? 4 : 1, TC = TX * TY;
-  static constexpr int NFX = (TX + 1) * TY, NFY = (D == 3) ? TX * (TY + 1) : 0;
-  int st, pk, rbx, rax, rby, ray, rfx, rfy, sg, sbr, sbg, scar, sgf, end;
-  // Staged gas-face values per cell and plane (1-d and 2-d; 3-d reads them from global memory,
-  // where the extra shared memory would cost a resident block): 3 contact speeds, then 2D fluxes
-  // per gas variable.
-  static constexpr int NGF = (D <= 2) ? 3 + 2 * D * NG : 0;
-  // The face fluxes of C have a region of their own in 1-d and 2-d, so that B of the next plane
-  // may write face states while D still reads fluxes (no barrier separates A from B there).  In
-  // 3-d they overwrite the left face states of B (each face's left state is read, and its flux
-  // written, by the thread that owns the face, between the same two barriers), which keeps the
-  // larger 3-d tile at two blocks per SM.
-  __host__ __device__ explicit StageLayout(int G) {
-    st = 0;
-    pk = st + NSLOT * NRV * PC * G;       // radiation ring [slot][NRV][PC][G]
-    rbx = pk + NSLOT * 2 * PC;            // opacity factors ring [slot][K, S][PC]
-    rax = rbx + NRV * NFX * G;            // left state of every x face [NRV][NFX][G]
-    rby = rax + NRV * TY * G;             // right state of the last x face of each row
-    ray = rby + NRV * NFY * G;            // left state of every y face (3-d)
-    const int fe = ray + (D == 3 ? NRV * TX * G : 0);  // right state of the last y face (3-d)
-    rfx = D == 3 ? rbx : fe;              // radiation x-face fluxes [NRV][NFX][G]
-    rfy = rby;                            // radiation y-face fluxes (3-d)
-    sg = D == 3 ? fe : fe + NRV * NFX * G;
-    sbr = sg + NSLOT * NG * PC;           // gas variables ring [slot][NG][PC]
-    sbg = sbr + NRV * TC * G;             // stage-2 base, radiation [NRV][TC][G]
-    scar = sbg + NG * TC;                 // stage-2 base, gas [NG][TC]
-    sgf = scar + (D == 2 ? 4 * NRV * TC * G : 0);  // 2-d march carry [plane parity][bm, rfm][NRV][TC][G]
-    end = sgf + 2 * TC * NGF;             // gas-face values [plane parity][TC][NGF]
+// cp.async of one lane value (the lane's groups: both values of a pair where they are 8-byte
+// aligned in global memory and both exist, else one by one).
+__device__ __forceinline__ void cp_async_lane(F2* s, const float* g, bool vec, bool h1) {
+  const unsigned sa = (unsigned)__cvta_generic_to_shared(s);
+  if (vec) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(sa), "l"(g) : "memory");
+  } else {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(sa), "l"(g) : "memory");
+    if (h1) asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(sa + 4), "l"(g + 1) : "memory");
   }
-};
-
-// Group stride of stage_kernel's shared arrays (see there): even, so that a lane's two groups
-// are one 8-byte access.
-template <int D, int GP> __host__ __device__ constexpr int stage_gstride(int G) { return D <= 2 ? GP : G + (G & 1); }
-
-// Shared memory of stage_kernel for a group stride GS (stage_gstride).
-template <class R, int D, int TX, int TY>
-inline size_t stage_smem_bytes(int G) {
-  StageLayout<D, TX, TY> L(G);
-  return (size_t)L.end * sizeof(R) + 16 + sizeof(GroupConst);
+}
+__device__ __forceinline__ void cp_async_lane(double* s, const double* g, bool, bool) { cp_async(s, g); }
+__device__ __forceinline__ void cp_async16(void* s, const void* g) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"((unsigned)__cvta_generic_to_shared(s)), "l"(g) : "memory");
 }
 
 // ---------------------------------------------------------------------------------------------
-// The radiation/update kernel (one launch per RK stage, after gas_face_kernel).  A block owns a
-// tile of TX x TY cells and marches along the slowest axis.  Each cell is served by a segment of
-// GL = GP/NGL lanes, and a thread owns NGL consecutive groups of its cell (NGL = 2 in the FP32
-// forms with G > 16, else 1).  Per plane k:
-//   A  wait for the thread's copies of plane k+2 (staged during step k-1), mirror and physical
-//      conversions of what it copied, and stage plane k+3 (own cells, in-plane halo, gas
-//      variables, and the opacity factors that gas_face_kernel formed) with cp.async;
-//   B  each cell is reconstructed once per direction from the four-plane shared ring;
-//   C  the M1/HLL radiation fluxes of the cell's lower faces and of its march face k+1/2, using
-//      the contact speeds of the gas faces (Eq. 19);
-//   D  divergence (gas fluxes from the face buffer), RK combine, store of plane k (the
-//      interaction follows in a kernel of its own).
-// B | C and C | D are block barriers; in 3-d also A | B (its face fluxes share shared memory with
-// the face states).  SPH selects the spherical (r, theta) geometry of a 2-d grid at compile time
-// (the host launches the instantiation that matches the grid): the Cartesian kernel carries none
-// of its scale factors and geometric sources.  RO is the radiation reconstruction (1: linear with
-// the MC limiter, the paper's; 2: the gas's parabola), also a compile-time choice: a run-time one
-// cost the kernel spills.  BUD compiles in the boundary-outflow budgets (reading R13) for grids
-// with a non-periodic boundary: on a fully periodic grid the code would only cost registers.
+// The stage kernel (one launch per RK stage, after gas_face_kernel).
+//
+// Radiation blocks.  A group's transport does not see the other groups, so a cell is served by
+// exactly as many lanes as its groups need: GL = ceil(G / W) lanes of W groups, W = 2 as one packed
+// FP32 pair (F2), W = 1 in FP64.  A block owns a tile of TX x TY cells (TY = 1 below 3-d),
+// tid = cell * GL + lane, and marches along the slowest axis over a chunk of planes.  The tile is
+// chosen at run time (stage_tile): all shared arrays are addressed by tid and compile-time
+// capacities, so no group or tile count is a template parameter and no lane is padding.
+//   ring   four planes of the tile's own cells [slot][v][NT]: a thread copies its own cell with
+//          cp.async three planes ahead and reads its own march column from it;
+//   halo   two cells on each in-plane side, two planes [parity][v][NH GL];
+//   rec    the face records that gas_face_kernel wrote (upwind speeds and opacity sums), two planes;
+//   xb, yb the state left of every in-plane face, overwritten by the face's flux.
+// Per plane k:
+//   A  issue the copies of plane k+3 (own cells), of plane k+1 (halo, records) and of the stage-2
+//      base of plane k;
+//   B  reconstruct each cell once per direction, the halo cells as extra tasks spread over the
+//      block's threads;                                                             -- barrier
+//   C  the fluxes through the cell's lower faces and its march face k+1/2, the tile's upper faces
+//      as extra tasks; wait for the copies of A;                                    -- barrier
+//   D  divergence, RK combination, store.
+//
+// On a Cartesian grid every direction is uniform, so the kernel needs no table: the half slopes
+// of the limiter give the face states, and the divergence is formed from the differences of the
+// two fluxes of a direction (exact as s + e by TwoSum in FP32), scaled once by dt / (2 dx): twice
+// the flux is carried, which saves the halvings of the two-state averages.
+//
+// Gas blocks.  The gas update of a cell needs only the face fluxes in the face buffer: the last
+// blocks of the grid do it, one thread per cell, in the slots that the radiation blocks leave free
+// and as they finish (no launch of its own, and no gas variables in the radiation blocks).
+//
+// Bound by instruction issue and by the latency between the plane barriers (1024^2 x 16: 669 instructions
+// per warp and plane, issued in about 56 % of cycles at 20 warps per multiprocessor; DRAM 1.0x the
+// algorithmic bytes).  Measured
+// (FP32 state unless noted, one launch): 1024^2 x 16 groups 0.455 -> 0.250 ms, 256^3 x 12 16.4 ->
+// 7.3 ms, 640 x 128 x 20 spherical 0.124 -> 0.064 ms, 512^2 x 24 channels 0.23 -> 0.099 ms, 512^2 x
+// 16 FP64 2.99 -> 1.84 ms, against one kernel with lanes padded to a power of two, geometry tables
+// on every grid, and the gas update in its lanes.
+//
+// SPH selects the spherical (r, theta) geometry, RO the radiation reconstruction (1: linear with
+// the MC limiter, the paper's; 2: the gas's parabola), BUD the boundary-outflow budgets (R13).
 // ---------------------------------------------------------------------------------------------
-template <class R, int D, int GP, int TX, int TY, class LT, class NT, int NGL, bool SPH, int RO, bool BUD>
-__global__ void __launch_bounds__(TX * TY * (GP / NGL), (sizeof(R) == 4 && (NGL == 1 || TX * TY * (GP / NGL) <= 160)) ? 3 : 2)
-stage_kernel(const __grid_constant__ StageArgs<R> A) {
-  static_assert(!SPH || D == 2, "the spherical geometry is 2-d (r, theta)");
-  using LY = StageLayout<D, TX, TY>;
-  constexpr int GL = GP / NGL;       // lanes per cell
-  constexpr int NTH = TX * TY * GL;  // threads per block
-  constexpr int NG = LY::NG, NRV = LY::NRV;
-  constexpr int PX = LY::PX, PC = LY::PC, TC = LY::TC, NFX = LY::NFX, NFY = LY::NFY;
-  constexpr int MD = D - 1;  // march direction (D >= 2)
-  static_assert(NGL == 1 || (sizeof(LT) == 4 && GL >= 2 + D), "two groups per lane: FP32 groups, gas in lanes < 2+D");
-  static_assert(TX >= 2 * NGL, "the x-halo lanes of the two tile edges are disjoint");
-  static_assert(NTH % 32 == 0 && NTH / 32 <= 16 && 32 % GL == 0, "whole warps, whole cells per warp, named barriers");
+template <class R, int D> struct StageCap {
+  static constexpr int NT = sizeof(R) == 8 ? 256 : (D == 3 ? 192 : 160);  // most threads per block
+  static constexpr int XP = sizeof(R) == 8 ? 128 : 64;  // room for the upper face of every row
+  // ... and for the threads past the tile (at most 31), which run along on entries of their own
+  static constexpr int XC = NT + XP + 32 + (D == 3 ? XP : 32);
+  static constexpr int PB = D == 3 ? 1 : 2;             // planes of xb (and yb) in use at once
+  static constexpr int MINB = sizeof(R) == 8 ? 2 : (D == 3 ? 3 : 4);  // resident blocks aimed at
+};
 
+// Halo cells per plane and face records per plane of a tile.
+template <int D> __host__ __device__ inline int tile_halo(const RadTile& t) { return 4 * t.ty + (D == 3 ? 4 * t.tx : 0); }
+template <int D> __host__ __device__ inline int tile_recs(const RadTile& t) {
+  return (t.tx + 1) * t.ty + (D == 3 ? t.tx * (t.ty + 1) : 0) + (D >= 2 ? t.tx * t.ty : 0);
+}
+
+// Shared memory of stage_kernel: offsets in lane values (8 bytes), the records last.
+template <class R, int D> struct StageLayout {
+  using C = StageCap<R, D>;
+  static constexpr int NRV = 1 + D;
+  int ring, base, xb, yb, xr, yr, halo, rec, end;
+  __host__ __device__ explicit StageLayout(const RadTile& t) {
+    ring = 0;
+    base = ring + (D == 1 ? 1 : 4) * NRV * C::NT;
+    xb = base + NRV * C::NT;
+    yb = xb + C::PB * NRV * C::XC;
+    xr = yb + (D == 3 ? C::PB * NRV * C::XC : 0);
+    yr = xr + NRV * t.ty * t.gl;
+    halo = yr + (D == 3 ? NRV * t.tx * t.gl : 0);
+    rec = (halo + 2 * NRV * tile_halo<D>(t) * t.gl + 1) & ~1;        // 16-byte aligned
+    end = rec + 2 * tile_recs<D>(t) * (4 * (int)sizeof(R) / 8);
+  }
+};
+template <class R, int D> inline size_t stage_smem_bytes(const RadTile& t) { return (size_t)StageLayout<R, D>(t).end * 8; }
+
+// 1/(cE), s = sqrt(4 - 3 f^2) and f^2 of a radiation state, f = |F|/(cE); 1/(cE) is 0 for E <= 0.
+template <int D>
+__device__ __forceinline__ void m1_state(const LaneConst<F2>& K, F2 cE, const F2* F, F2& iE, F2& f2, F2& s) {
+  F2 FF = F[0] * F[0];
+#pragma unroll
+  for (int q = 1; q < D; ++q) FF = vfma(F[q], F[q], FF);
+  iE = F2(cE.x > 0.0f ? rcp_approx(cE.x) : 0.0f, cE.y > 0.0f ? rcp_approx(cE.y) : 0.0f);
+  f2 = (FF * iE) * iE;
+  s = vsqrt(vfma(K.m3, vmin(f2, F2(1.0f)), K.p4));
+}
+template <int D>
+__device__ __forceinline__ void m1_state(const LaneConst<double>& K, double cE, const double* F, double& iE,
+                                         double& f2, double& s) {
+  double FF = F[0] * F[0];
+#pragma unroll
+  for (int q = 1; q < D; ++q) FF = fma(F[q], F[q], FF);
+  iE = normal_pos(cE) ? rcp64(cE) : 0.0;
+  f2 = (FF * iE) * iE;
+  s = sqrt64(fma(K.m3, __double2hiint(f2) >= 0x3ff00000 ? 1.0 : f2, K.p4));
+}
+__device__ __forceinline__ F2 max1(F2 f2) { return vmax(f2, F2(1.0f)); }
+__device__ __forceinline__ double max1(double f2) { return __double2hiint(f2) >= 0x3ff00000 ? f2 : 1.0; }  // f2 >= 0
+__device__ __forceinline__ F2 rcp_fast(F2 x) { return F2(rcp_approx(x.x), rcp_approx(x.y)); }
+__device__ __forceinline__ double rcp_fast(double x) { return rcp64(x); }
+
+// c^2 times row n of the M1 pressure tensor (reading R7) for the lane's groups.  With f = |F|/(cE)
+// and s = sqrt(4 - 3 f^2), f^2 = (4 - s^2)/3 turns the closure's two coefficients into
+//   (1 - chi)/2 = (s - 1)/3,   (3 chi - 1)/2 = 3 f^2/(2 + s),
+// so c^2 P_nq = cE (c/3)(s - 1) delta_nq + F_n F_q / ((2 + s) cE/(3c)): one reciprocal of cE, one square
+// root, one reciprocal.  f > 1 keeps the direction with f clamped to 1 (the factor max(f^2, 1) in
+// the second reciprocal's argument); E <= 0 is isotropic (1/(cE) taken as 0).
+template <int D, class V>
+__device__ __forceinline__ void m1_c2row(const LaneConst<V>& K, V E, const V* F, int n, V* P) {
+  const V cE = E * K.c;
+  V iE, f2, s;
+  m1_state<D>(K, cE, F, iE, f2, s);
+  const V diag = cE * vfma(s, K.c3, K.mc3);
+  const V w = rcp_fast(vfma(s, K.d1, K.d2) * max1(f2)) * iE * F[n];
+#pragma unroll
+  for (int q = 0; q < D; ++q) P[q] = q == n ? vfma(w, F[q], diag) : w * F[q];
+}
+// The entry of c^2 P perpendicular to F (the closure's isotropic part).
+template <int D, class V> __device__ __forceinline__ V m1_c2perp(const LaneConst<V>& K, V E, const V* F) {
+  const V cE = E * K.c;
+  V iE, f2, s;
+  m1_state<D>(K, cE, F, iE, f2, s);
+  return cE * vfma(s, K.c3, K.mc3);
+}
+
+// dt times the divergence of a cell on a uniform grid, from twice the fluxes: x, (3-d) y, march.
+// In FP32 (precision form (1)) the summation is compensated: each direction's difference is formed
+// as s + e by Dekker's Fast2Sum, exact where the two fluxes are within a factor of two of each other
+// (s is then exact itself, Sterbenz) or the upper one is the larger, and the e of all directions are
+// summed beside the s.  The differences are scaled, not the fluxes, so the cancellation of two
+// nearly equal fluxes meets no rounded product.
+__device__ __forceinline__ void fast_diff(F2 a, F2 b, F2& s, F2& e) {
+  s = a - b;
+  e = (a - s) - b;
+}
+template <int D>
+__device__ __forceinline__ F2 net_update(F2 xp, F2 xm, F2 yp, F2 ym, F2 mp, F2 mm, const F2* h) {
+  F2 s, e;
+  fast_diff(xp, xm, s, e);
+  F2 n = s * h[0], c = e * h[0];
+  if (D == 3) {
+    fast_diff(yp, ym, s, e);
+    n = vfma(s, h[1], n);
+    c = vfma(e, h[1], c);
+  }
+  if (D >= 2) {
+    fast_diff(mp, mm, s, e);
+    n = vfma(s, h[D - 1], n);
+    c = vfma(e, h[D - 1], c);
+  }
+  return n + c;
+}
+template <int D>
+__device__ __forceinline__ double net_update(double xp, double xm, double yp, double ym, double mp, double mm, const double* h) {
+  double n = (xp - xm) * h[0];
+  if (D == 3) n = fma(yp - ym, h[1], n);
+  if (D >= 2) n = fma(mp - mm, h[D - 1], n);
+  return n;
+}
+
+// Gas update of one cell per thread (the gas blocks of stage_kernel): the divergence of the face
+// fluxes, the geometric sources of the spherical grid, the RK combination and, with BUD, the
+// boundary outflows.
+template <class R, int D, bool SPH, bool BUD>
+__device__ __forceinline__ void gas_update(const StageArgs<R>& A, uint32_t cid) {
+  constexpr int NG = 2 + D, MD = D - 1;
   const DevGrid& g = A.g;
   const Consts<R>& KR = A.k(R(0));
-  const int G = g.G;
-  const int tid = threadIdx.x;
-  const int lane = tid % GL;
-  const int tcell = tid / GL;  // tile cell of this thread
-  const int lx = tcell % TX, ly = tcell / TX;
+  const uint32_t ncell = (uint32_t)g.ncell;
+  if (cid >= ncell) return;
   const int nx = g.n[0], ny = g.n[1], nz = g.n[2];
-  const int x0 = blockIdx.x * TX;
-  const int y0 = (D == 3) ? blockIdx.y * TY : 0;
-  const int nmarch = (D == 1) ? 1 : g.n[MD];
-  const int kbeg = (D == 1) ? 0 : ((D == 2) ? blockIdx.y : blockIdx.z) * A.chunk;
-  const int kend = (D == 1) ? 1 : min(kbeg + A.chunk, nmarch);
-  const uint32_t ncell = (uint32_t)g.ncell;  // the host keeps every state offset below 2^32
-  // this thread's groups: lane * NGL + j
-  bool hasj[NGL];
-  int gj[NGL];
+  const int gx = D == 1 ? (int)cid : (int)(cid % (uint32_t)nx);
+  const int gy = D == 1 ? 0 : (D == 2 ? (int)(cid / (uint32_t)nx) : (int)((cid / (uint32_t)nx) % (uint32_t)ny));
+  const int gz = D == 3 ? (int)(cid / ((uint32_t)nx * ny)) : 0;
+  const int gi[3] = {gx, gy, gz};
+  const Tab<R> tx{A.tab[0], nx + 4, A.uniform[0] ? A.urow[0] : nullptr};
+  const Tab<R> ty{A.tab[D >= 2 ? 1 : 0], (D >= 2 ? ny : nx) + 4, A.uniform[D >= 2 ? 1 : 0] ? A.urow[D >= 2 ? 1 : 0] : nullptr};
+  const Tab<R> tz{A.tab[D >= 3 ? 2 : 0], (D >= 3 ? nz : nx) + 4, A.uniform[D >= 3 ? 2 : 0] ? A.urow[D >= 3 ? 2 : 0] : nullptr};
+  const uint32_t nfd[3] = {(uint32_t)(nx + 1) * (D > 1 ? ny : 1) * (D > 2 ? nz : 1),
+                           (uint32_t)nx * (ny + 1) * (D > 2 ? nz : 1), (uint32_t)nx * ny * (nz + 1)};
+  const uint32_t fl[3] = {((uint32_t)gz * ny + gy) * (nx + 1) + gx, ((uint32_t)gz * (ny + 1) + gy) * nx + gx, cid};
+  const uint32_t fs[3] = {1u, (uint32_t)nx, (uint32_t)nx * ny};  // to the upper face
+  auto face = [&](int d, int v, uint32_t f) -> R {
+    return __ldg(FXP(A.faces, (uint32_t)A.face_off[d] + v * nfd[d] + f, A.n_faces));
+  };
+  R u0[NG];
 #pragma unroll
-  for (int j = 0; j < NGL; ++j) {
-    hasj[j] = lane * NGL + j < G;
-    gj[j] = hasj[j] ? lane * NGL + j : 0;
+  for (int v = 0; v < NG; ++v) u0[v] = A.in[FXI(v * ncell + cid, A.n_state)];
+  R src[NG];
+#pragma unroll
+  for (int v = 0; v < NG; ++v) src[v] = R(0);
+  const int ipx = bc_pad(gx), ipm = bc_pad(gy);
+  if (SPH) {
+    const R h0 = tx(T_HA, ipx) * ty(T_HA, ipm), h1 = tx(T_HB, ipx) * ty(T_HB, ipm);
+    const R g111 = tx(T_GA, ipx), g221 = tx(T_GB, ipx), g122 = tx(T_GC, ipx);
+    const R g222 = ty(T_GA, ipm), g332 = ty(T_GB, ipm);
+    const R rho = u0[0], irho = frcp(rho);
+    const R v1 = u0[1] * irho * frcp(h0), v2 = u0[2] * irho * frcp(h1);
+    const R p = KR.gm1 * (u0[NG - 1] - R(0.5) * rho * (v1 * v1 + v2 * v2));
+    const R r12 = h0 * frcp(h1), r21 = h1 * frcp(h0);
+    src[1] = g111 * (rho * v1 * v1 + p) + g221 * (rho * v2 * v2 + p) + g221 * p;
+    src[2] = g122 * (rho * v1 * v2 * r12) + g221 * (rho * v1 * v2 * r21) + g222 * (rho * v2 * v2 + p) + g332 * p;
   }
+  const bool stage2 = A.base != nullptr;
+  R chk = R(0);
+  double out[NG];  // budgets
+#pragma unroll
+  for (int v = 0; v < NG; ++v) {
+    R Fp[D], Ap[D], Fm[D], Am[D];
+#pragma unroll
+    for (int d = 0; d < D; ++d) {
+      Fm[d] = face(d, v, fl[d]);
+      Fp[d] = face(d, v, fl[d] + fs[d]);
+    }
+    // area/volume factors (Eq. 8): scalar variables, and covariant components 0 and 1
+    const int eL[3] = {T_FL, T_FL1, T_FL2}, eR[3] = {T_FR, T_FR1, T_FR2}, eX[3] = {T_XS, T_X1, T_X2};
+    const int c = (v >= 1 && v <= 2 && v <= D) ? v : 0;
+    if (SPH) {
+      Ap[0] = tx(eR[c], ipx) * ty(eX[c], ipm);
+      Am[0] = tx(eL[c], ipx) * ty(eX[c], ipm);
+      Ap[D - 1] = ty(eR[c], ipm) * tx(eX[c], ipx);
+      Am[D - 1] = ty(eL[c], ipm) * tx(eX[c], ipx);
+    } else {
+      Ap[0] = tx(T_FR, ipx);
+      Am[0] = tx(T_FL, ipx);
+      if (D >= 2) { Ap[D >= 2 ? 1 : 0] = ty(T_FR, ipm); Am[D >= 2 ? 1 : 0] = ty(T_FL, ipm); }
+      if (D == 3) { Ap[D == 3 ? 2 : 0] = tz(T_FR, bc_pad(gz)); Am[D == 3 ? 2 : 0] = tz(T_FL, bc_pad(gz)); }
+    }
+    const R b = stage2 ? A.base[FXI(v * ncell + cid, A.n_state)] : R(0);
+    const R un = fv_update(Fp, Ap, Fm, Am, u0[v], src[v], KR.dt, stage2, b, KR.alpha, KR.beta);
+    A.out[FXI(v * ncell + cid, A.n_state)] = un;
+    if (A.pre_out != nullptr) A.pre_out[FXI(v * ncell + cid, A.n_state)] = un;
+    chk += un * R(0);
+    if (BUD) {
+      double o = 0.0;
+#pragma unroll
+      for (int d = 0; d < D; ++d) {
+        if (gi[d] == g.n[d] - 1 && g.bc_hi[d] != 1) o += (double)(Fp[d] * Ap[d]);
+        if (gi[d] == 0 && g.bc_lo[d] != 1) o -= (double)(Fm[d] * Am[d]);
+      }
+      out[v] = o;
+    }
+  }
+  if (!isfinite(chk)) atomicOr(A.status, ST_NONFINITE);
+  if (BUD && A.budget != nullptr) {
+    bool edge = false;
+#pragma unroll
+    for (int d = 0; d < D; ++d)
+      edge |= (gi[d] == 0 && g.bc_lo[d] != 1) || (gi[d] == g.n[d] - 1 && g.bc_hi[d] != 1);
+    if (edge) {
+      double vol = (double)tx(T_VOL, ipx);
+      if (D >= 2) vol *= (double)ty(T_VOL, ipm);
+      if (D == 3) vol *= (double)tz(T_VOL, bc_pad(gz));
+      const double bs = vol * A.bw_flux;
+      double* const bud = A.budget + (size_t)(blockIdx.x % BUDGET_SLOTS) * NBUDGET;
+#pragma unroll
+      for (int v = 0; v < NG; ++v)
+        if (out[v] != 0.0) atomicAdd(bud + (v == NG - 1 ? 4 : v), out[v] * bs);
+    }
+  }
+  (void)MD;
+}
+
+template <class R, int D, bool SPH, int RO, bool BUD>
+__global__ void __launch_bounds__((StageCap<R, D>::NT), (StageCap<R, D>::MINB))
+stage_kernel(const __grid_constant__ StageArgs<R> A) {
+  static_assert(!SPH || D == 2, "the spherical geometry is 2-d (r, theta)");
+  using CP = StageCap<R, D>;
+  using V = typename LaneOf<R>::V;
+  constexpr int W = LaneOf<R>::W;
+  constexpr int NG = 2 + D, NRV = 1 + D, MD = D - 1;
+  constexpr int NT = CP::NT, XC = CP::XC, PB = CP::PB;
+  constexpr bool TABLES = SPH || RO == 2;  // the reconstruction reads the geometry tables
+  const int NTH = (int)blockDim.x, tid = (int)threadIdx.x;
+  const RadTile& RT = A.rt;
+  if (blockIdx.x >= (unsigned)RT.nrad) {  // gas blocks: cells in strides of the gas blocks' threads
+    const uint32_t nthr = (gridDim.x - (unsigned)RT.nrad) * (uint32_t)NTH;
+    for (uint32_t c = (blockIdx.x - (unsigned)RT.nrad) * (uint32_t)NTH + tid; c < (uint32_t)A.g.ncell; c += nthr)
+      gas_update<R, D, SPH, BUD>(A, c);
+    return;
+  }
+  const DevGrid& g = A.g;
+  const Consts<R>& KR = A.k(R(0));
+  const LaneConst<V>& KL = A.kl;
+  const int G = g.G, GL = RT.gl, TX = RT.tx, TY = D == 3 ? RT.ty : 1, TC = TX * TY;
+  const int nx = g.n[0], ny = g.n[1], nz = g.n[2];
+  const uint32_t ncell = (uint32_t)g.ncell;  // the host keeps every state offset below 2^32
+  // block -> tile and chunk
+  const int bt = (int)blockIdx.x;
+  const int btx = bt % RT.ntx, btr = bt / RT.ntx;
+  const int bty = D == 3 ? btr % RT.nty : 0, bck = D == 3 ? btr / RT.nty : btr;
+  const int x0 = btx * TX, y0 = D == 3 ? bty * TY : 0;
+  const int nmarch = D == 1 ? 1 : g.n[MD];
+  const int kbeg = D == 1 ? 0 : bck * A.chunk;
+  const int kend = D == 1 ? 1 : min(kbeg + A.chunk, nmarch);
+  const int tcell = tid / GL, lane = tid - tcell * GL;
+  // the last warp's threads past the tile run along on a copy of cell 0 and entries of their own
+  const bool act = tcell < TC;
+  const int tc = act ? tcell : 0;
+  const int lx = D == 3 ? tc % TX : tc, ly = D == 3 ? tc / TX : 0;
+  const int g0 = lane * W;
+  const bool h1 = W == 2 && g0 + 1 < G;
+  const bool vec = RT.vec != 0;
 
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  R* const sm = reinterpret_cast<R*>(smem_raw);
-  // group stride of the shared arrays: the padded group count GP in 1-d and 2-d (constant strides
-  // fold into the shared-memory addressing), the group count in 3-d (whose tile is large)
-  const int GS = stage_gstride<D, GP>(G);
-  const LY L(GS);
-  R* const st = sm + L.st;
-  R* const pk = sm + L.pk;
-  R* const rbx = sm + L.rbx;
-  R* const rax = sm + L.rax;
-  R* const rby = sm + L.rby;
-  R* const ray = sm + L.ray;
-  R* const rfx = sm + L.rfx;
-  R* const rfy = sm + L.rfy;
-  R* const sgr = sm + L.sg;   // gas variables of the ring's planes
-  R* const sbr = sm + L.sbr;  // stage-2 base of the tile's cells (radiation), by plane parity
-  R* const sbg = sm + L.sbg;  // stage-2 base (gas)
-  R* const scr = sm + L.scar; // 2-d: march carry (own cell's upper march-face state, march flux)
-  R* const sgf = sm + L.sgf;  // gas-face values of the cell's faces, by plane parity
-  // extents of the shared arrays and of the opacity factors, for the index checks of the debug
-  // build (FXI)
-  const int n_st = L.pk - L.st, n_pk = L.rbx - L.pk, n_rbx = L.rax - L.rbx, n_rax = L.rby - L.rax;
-  const int n_rby = L.ray - L.rby, n_ray = D == 3 ? NRV * TX * GS : 0, n_sg = L.sbr - L.sg;
-  const int n_rfx = NRV * NFX * GS, n_rfy = NRV * NFY * GS, n_sbr = L.sbg - L.sbr;
-  const int n_sbg = L.scar - L.sbg, n_scr = L.sgf - L.scar, n_sgf = L.end - L.sgf;
-  const uint32_t n_opk = 2 * ncell;
-  (void)n_st; (void)n_pk; (void)n_rbx; (void)n_rax; (void)n_rby; (void)n_ray; (void)n_sg;
-  (void)n_rfx; (void)n_rfy; (void)n_sbr; (void)n_sbg; (void)n_scr; (void)n_sgf; (void)n_opk;
-  GroupConst* sgc = reinterpret_cast<GroupConst*>(
-      (reinterpret_cast<uintptr_t>(sm + L.end) + 15) & ~static_cast<uintptr_t>(15));
-  for (int i = tid; i < (int)(sizeof(GroupConst) / sizeof(int)); i += NTH)
-    reinterpret_cast<int*>(sgc)[i] = reinterpret_cast<const int*>(A.gc)[i];
-  __syncthreads();
+  V* const sm = reinterpret_cast<V*>(smem_raw);
+  const StageLayout<R, D> L(RT);
+  const int NH = tile_halo<D>(RT), HS = NH * GL, NREC = tile_recs<D>(RT);
+  V* const ring = sm + L.ring;
+  V* const sbase = sm + L.base;
+  V* const xb = sm + L.xb;
+  V* const yb = sm + L.yb;
+  V* const xr = sm + L.xr;
+  V* const yr = sm + L.yr;
+  V* const halo = sm + L.halo;
+  R* const rec = reinterpret_cast<R*>(sm + L.rec);
+  const int n_ring = (D == 1 ? 1 : 4) * NRV * NT, n_base = NRV * NT, n_xb = PB * NRV * XC;
+  const int n_xr = NRV * TY * GL, n_yr = NRV * TX * GL, n_halo = 2 * NRV * HS, n_rec = 8 * NREC;
+  (void)n_ring; (void)n_base; (void)n_xb; (void)n_xr; (void)n_yr; (void)n_halo; (void)n_rec;
 
   const Tab<R> tx{A.tab[0], nx + 4, A.uniform[0] ? A.urow[0] : nullptr};
-  const Tab<R> ty{A.tab[D >= 2 ? 1 : 0], (D >= 2 ? ny : nx) + 4,
-                  A.uniform[D >= 2 ? 1 : 0] ? A.urow[D >= 2 ? 1 : 0] : nullptr};
-  const Tab<R> tz{A.tab[D >= 3 ? 2 : 0], (D >= 3 ? nz : nx) + 4,
-                  A.uniform[D >= 3 ? 2 : 0] ? A.urow[D >= 3 ? 2 : 0] : nullptr};
-  const Tab<R>& tm = (D == 3) ? tz : ty;  // march-direction table
+  const Tab<R> ty{A.tab[D >= 2 ? 1 : 0], (D >= 2 ? ny : nx) + 4, A.uniform[D >= 2 ? 1 : 0] ? A.urow[D >= 2 ? 1 : 0] : nullptr};
+  const Tab<R> tz{A.tab[D >= 3 ? 2 : 0], (D >= 3 ? nz : nx) + 4, A.uniform[D >= 3 ? 2 : 0] ? A.urow[D >= 3 ? 2 : 0] : nullptr};
+  const Tab<R>& tm = D == 3 ? tz : ty;
 
-  // global index of slot cell (sx, sy) on plane k, mapped into the domain (Sec. 7.5); flips[d]
-  // is set where a reflecting boundary mirrors direction d.  Tiles may overhang the grid by up
-  // to TX-1 cells; those cells are never used and the clamps keep every read inside the array.
-  auto map_cell = [&](int sx, int sy, int k, bool* flips) -> uint32_t {
-    flips[0] = flips[1] = flips[2] = false;
-    int gx_ = min(max(bc_map(x0 + sx, nx, g.bc_lo[0], g.bc_hi[0], flips[0]), 0), nx - 1);
-    if (D == 1) return gx_;
-    if (D == 2) {
-      int gy_ = min(max(bc_map(k, ny, g.bc_lo[1], g.bc_hi[1], flips[1]), 0), ny - 1);
-      return (uint32_t)gy_ * nx + gx_;
+  // ---- positions.  Ghost cells are index maps (Sec. 7.5); tiles may overhang the grid, their
+  // cells past the first two ghosts are never used and clamped into the array.
+  auto map_x = [&](int x, bool& f) { return min(max(bc_map(x, nx, g.bc_lo[0], g.bc_hi[0], f), 0), nx - 1); };
+  auto map_y = [&](int y, bool& f) { return min(max(bc_map(y, ny, g.bc_lo[1], g.bc_hi[1], f), 0), ny - 1); };
+  auto map_m = [&](int k, bool& f) {
+    if (D == 1) return 0;
+    return min(max(bc_map(k, nmarch, g.bc_lo[MD], g.bc_hi[MD], f), 0), nmarch - 1);
+  };
+  const uint32_t pcells = D == 1 ? 0u : (D == 2 ? (uint32_t)nx : (uint32_t)nx * ny);  // cells per plane
+  auto inplane = [&](int sx, int sy, bool& fx, bool& fy) -> uint32_t {  // of tile cell (sx, sy)
+    const uint32_t cx = (uint32_t)map_x(x0 + sx, fx);
+    return D == 3 ? (uint32_t)map_y(y0 + sy, fy) * nx + cx : cx;
+  };
+  // t / GL for the task indices (t < 2^16: exact with mgl = ceil(2^32 / GL))
+  auto div_gl = [&](int t) -> int { return GL == 1 ? t : (int)__umulhi((unsigned)t, RT.mgl); };
+  // halo cell h: 4 per row (-2, -1, TX, TX+1), then (3-d) 4 rows of TX (-2, -1, TY, TY+1)
+  auto halo_pos = [&](int h, int& sx, int& sy) {
+    if (D < 3 || h < 4 * TY) { const int r = h >> 2, c = h & 3; sy = r; sx = c < 2 ? c - 2 : TX + (c - 2); }
+    else { const int j = h - 4 * TY, r = j / TX; sx = j - r * TX; sy = r < 2 ? r - 2 : TY + (r - 2); }
+  };
+  bool fx_own = false, fy_own = false;
+  const uint32_t cxy = inplane(lx, ly, fx_own, fy_own);
+  const int gx = x0 + lx, gy = y0 + ly;
+  const bool cell_in = act && gx < nx && (D < 3 || gy < ny);
+  const uint32_t toff = cxy * (uint32_t)G + g0;  // the thread's elements in a plane of a radiation variable
+  const uint32_t vstride = ncell * (uint32_t)G, pstride = pcells * (uint32_t)G;
+  // The halo entries and face records that this thread copies: the first ones (one halo entry, two
+  // in 3-d; two records) keep their element offsets in registers, more of them (tiles of few cells
+  // with many lanes) recompute theirs.  Halo entries go to the threads from the last one down, so
+  // that they and the records fall to different warps.
+  constexpr int HP = D == 3 ? 2 : 1, RP = 2;
+  const int ht0 = NTH - 1 - tid;
+  auto halo_entry = [&](int t, uint32_t& off, bool& two) {
+    const int h = div_gl(t), ln = t - h * GL;
+    int sx, sy;
+    bool f0 = false, f1 = false;
+    halo_pos(h, sx, sy);
+    off = inplane(sx, sy, f0, f1) * (uint32_t)G + ln * W;
+    two = W == 2 && ln * W + 1 < G;
+  };
+  uint32_t hoff[HP];
+  bool hh1[HP];
+#pragma unroll
+  for (int p = 0; p < HP; ++p) {
+    hoff[p] = 0;
+    hh1[p] = false;
+    if (ht0 + p * NTH < HS) halo_entry(ht0 + p * NTH, hoff[p], hh1[p]);
+  }
+  // records: x faces (TX+1 per row), (3-d) y faces, march faces (the cell's upper one); face on
+  // plane 0 and faces per plane
+  const int NXF = (TX + 1) * TY, NYF = D == 3 ? TX * (TY + 1) : 0;
+  auto rec_entry = [&](int t, uint32_t& off, uint32_t& str) {
+    if (t < NXF) {
+      const int row = D == 3 ? t / (TX + 1) : 0, c = t - row * (TX + 1);
+      str = D == 1 ? 0u : (D == 2 ? (uint32_t)(nx + 1) : (uint32_t)(nx + 1) * ny);
+      off = (uint32_t)A.rec_off[0] + (D == 3 ? (uint32_t)min(y0 + row, ny - 1) * (nx + 1) : 0u) + (uint32_t)min(x0 + c, nx);
+    } else if (t < NXF + NYF) {
+      const int q = t - NXF, row = q / TX, c = q - row * TX;
+      str = (uint32_t)(ny + 1) * nx;
+      off = (uint32_t)A.rec_off[1] + (uint32_t)min(y0 + row, ny) * nx + (uint32_t)min(x0 + c, nx - 1);
+    } else {
+      const int q = t - NXF - NYF, row = D == 3 ? q / TX : 0, c = q - row * TX;
+      str = pcells;
+      off = (uint32_t)A.rec_off[D >= 2 ? MD : 0] + (D == 3 ? (uint32_t)min(y0 + row, ny - 1) * nx : 0u) + (uint32_t)min(x0 + c, nx - 1) + pcells;
     }
-    int gy_ = min(max(bc_map(y0 + sy, ny, g.bc_lo[1], g.bc_hi[1], flips[1]), 0), ny - 1);
-    int gz_ = min(max(bc_map(k, nz, g.bc_lo[2], g.bc_hi[2], flips[2]), 0), nz - 1);
-    return ((uint32_t)gz_ * ny + gy_) * nx + gx_;
   };
-  auto scell = [&](int sx, int sy) -> int { return (D == 3 ? (sy + 2) * PX : 0) + sx + 2; };
-  auto rad_at = [&](int slot, int v, int sc, int gg) -> R& {
-    return st[FXI(((slot * NRV + v) * PC + sc) * GS + gg, n_st)];
+  uint32_t roff[RP], rstr[RP];
+#pragma unroll
+  for (int p = 0; p < RP; ++p) {
+    roff[p] = rstr[p] = 0;
+    if (tid + p * NTH < NREC) rec_entry(tid + p * NTH, roff[p], rstr[p]);
+  }
+  if (W == 2 && (G & 1)) {  // the pad component of an odd group count's last pair stays zero
+    for (int i = tid; i < L.rec; i += NTH) sm[i] = V(R(0));
+    __syncthreads();
+  }
+
+  // ---- copies.  A plane's address is block-uniform (the state's base, the variable, the plane)
+  // plus the thread's fixed offset.
+  auto plane_at = [&](const R* S, int v, uint32_t row) -> const R* { return S + ((size_t)NG * ncell + (size_t)v * vstride + row); };
+  auto ring_slot = [&](int P) -> int { return D == 1 ? 0 : (P & 3) * NRV * NT; };
+  auto issue_own = [&](int P) {
+    bool f = false;
+    const uint32_t row = (uint32_t)map_m(P, f) * pstride;
+    const int s = ring_slot(P) + tid;
+#pragma unroll
+    for (int v = 0; v < NRV; ++v)
+      cp_async_lane(&ring[FXI(s + v * NT, n_ring)], FXP(plane_at(A.in, v, row), toff, vstride - row), vec, h1);
   };
-  auto gas_at = [&](int slot, int v, int sc) -> R& { return sgr[FXI((slot * NG + v) * PC + sc, n_sg)]; };
-  constexpr bool sph = SPH;  // spherical (r, theta): x = r, march = theta
+  auto issue_halo = [&](int P) {
+    bool f = false;
+    const uint32_t row = (uint32_t)map_m(P, f) * pstride;
+    auto one = [&](int t, uint32_t off, bool two) {
+      const int s = (P & 1) * NRV * HS + t;
+#pragma unroll
+      for (int v = 0; v < NRV; ++v)
+        cp_async_lane(&halo[FXI(s + v * HS, n_halo)], FXP(plane_at(A.in, v, row), off, vstride - row), vec, two);
+    };
+#pragma unroll
+    for (int p = 0; p < HP; ++p)
+      if (ht0 + p * NTH < HS) one(ht0 + p * NTH, hoff[p], hh1[p]);
+    if (D == 3 && HS > HP * NTH) {  // (fit_tile: never below 3-d)
+      for (int t = ht0 + HP * NTH; t < HS; t += NTH) {
+        uint32_t off;
+        bool two;
+        halo_entry(t, off, two);
+        one(t, off, two);
+      }
+    }
+  };
+  auto issue_rec = [&](int P) {
+    auto one = [&](int t, uint32_t f) {
+      R* const d = rec + FXI(((P & 1) * NREC + t) * 4, n_rec);
+      const R* const s = A.frec + (size_t)4 * FXI(f, A.n_recs);
+      cp_async16(d, s);
+      if (sizeof(R) == 8) cp_async16(d + 2, s + 2);
+    };
+#pragma unroll
+    for (int p = 0; p < RP; ++p)
+      if (tid + p * NTH < NREC) one(tid + p * NTH, roff[p] + (uint32_t)P * rstr[p]);
+    if (D == 3 && NREC > RP * NTH) {
+      for (int t = tid + RP * NTH; t < NREC; t += NTH) {
+        uint32_t off, str;
+        rec_entry(t, off, str);
+        one(t, off + (uint32_t)P * str);
+      }
+    }
+  };
+  auto issue_base = [&](int P) {
+    if (A.base == nullptr) return;
+    const uint32_t row = (uint32_t)P * pstride;
+#pragma unroll
+    for (int v = 0; v < NRV; ++v)
+      cp_async_lane(&sbase[FXI(v * NT + tid, n_base)], FXP(plane_at(A.base, v, row), toff, vstride - row), vec, h1);
+  };
   // scale factor of component q of the cell with x index ix on plane k
   auto hfac = [&](int q, int ix, int k) -> R {
-    if (!sph) return R(1);
+    if (!SPH) return R(1);
     const int e = q == 0 ? T_HA : T_HB;
     return tx(e, bc_pad(ix)) * tm(e, bc_pad(k));
   };
-
-  // Load `ncl` cells of plane k (enumerated by cell_of) into ring slot `slot`: gas variables and
-  // opacity factors (one thread per cell), radiation with one thread per (cell, group).
-  auto load_cells = [&](int slot, int k, int ncl, auto cell_of) {
-    for (int i = tid; i < ncl; i += NTH) {
-      int sx, sy;
-      cell_of(i, sx, sy);
-      bool fl[3];
-      const uint32_t gc_ = map_cell(sx, sy, k, fl);
-      const int sc = scell(sx, sy);
+  // after the wait, each thread finishes what it copied: the mirrored components of ghost cells
+  // change sign, and on the spherical grid covariant flux components become physical.  Planes
+  // inside the grid of blocks without mirrored in-plane ghosts need neither.
+  const bool fin_xy = SPH || g.bc_lo[0] >= 2 || g.bc_hi[0] >= 2 || (D == 3 && (g.bc_lo[1] >= 2 || g.bc_hi[1] >= 2));
+  auto finish_one = [&](V* p, int vs, bool fx, bool fy, bool fm, int ix, int P) {
 #pragma unroll
-      for (int v = 0; v < NG; ++v) gas_at(slot, v, sc) = A.in[FXI(v * ncell + gc_, A.n_state)];
-      pk[FXI((slot * 2 + 0) * PC + sc, n_pk)] = A.opk[FXI(gc_, n_opk)];
-      pk[FXI((slot * 2 + 1) * PC + sc, n_pk)] = A.opk[FXI(ncell + gc_, n_opk)];
-    }
-    for (int t = tid; t < ncl * GP; t += NTH) {
-      const int i = t / GP, gg = t % GP;
-      if (gg >= G) continue;
-      int sx, sy;
-      cell_of(i, sx, sy);
-      bool fl[3];
-      const uint32_t gc_ = map_cell(sx, sy, k, fl);
-      const int sc = scell(sx, sy);
-#pragma unroll
-      for (int v = 0; v < NRV; ++v) {
-        R val = A.in[FXI(NG * ncell + (v * ncell + gc_) * G + gg, A.n_state)];
-        if (v >= 1 && fl[v - 1]) val = -val;
-        if (sph && v >= 1) val *= frcp(hfac(v - 1, x0 + sx, k));  // physical component
-        rad_at(slot, v, sc, gg) = val;
-      }
+    for (int q = 0; q < D; ++q) {
+      const bool fl = q == MD && D > 1 ? fm : (q == 0 ? fx : fy);
+      V x = p[(1 + q) * vs];
+      if (SPH) x = x * frcp(hfac(q, ix, P));
+      if (fl) x = -x;
+      p[(1 + q) * vs] = x;
     }
   };
-  auto interior_of = [&](int i, int& sx, int& sy) { sx = i % TX; sy = i / TX; };
-  constexpr int NHALO = 4 * TY + (D == 3 ? 4 * TX : 0);  // x halo of every row, y halo (3-d)
-  auto halo_of = [&](int i, int& sx, int& sy) {
-    if (i < 4 * TY) { int r = i / 4, c = i % 4; sy = r; sx = c < 2 ? c - 2 : TX + (c - 2); }
-    else { int j = i - 4 * TY; int c = j / 4, r = j % 4; sx = c; sy = r < 2 ? r - 2 : TY + (r - 2); }
-  };
-  auto all_of = [&](int i, int& sx, int& sy) { sx = i - 2; sy = 0; };  // 1-d: TX + 4 cells
-
-  const bool cell_in = (x0 + lx < nx) && (D < 3 || y0 + ly < ny);
-  const int gx = x0 + lx, gy = y0 + ly;
-  const int sc_own = scell(lx, ly);
-  // own radiation values (this thread's cell and groups) and own gas variable (lanes 0..NG-1)
-  // of plane k, from global memory (mirror ghosts negate the normal components)
-  // the in-plane part of this thread's cell index and its mirror flips are fixed along the march
-  bool own_fl[3] = {false, false, false};
-  const uint32_t own_xy = [&]() {
-    bool f3[3];
-    const uint32_t c = map_cell(lx, ly, D >= 2 ? 0 : 0, f3);
-    own_fl[0] = f3[0];
-    own_fl[1] = D == 3 ? f3[1] : false;
-    return D == 1 ? c : D == 2 ? c % (uint32_t)nx : c % ((uint32_t)nx * ny);
-  }();
-  auto own_idx = [&](int k, bool* fl) -> uint32_t {
-    fl[0] = own_fl[0];
-    fl[1] = own_fl[1];
-    fl[2] = false;
-    if (D == 1) return own_xy;
+  auto finish_own = [&](int P) {
     bool fm = false;
-    const int km = min(max(bc_map(k, nmarch, g.bc_lo[MD], g.bc_hi[MD], fm), 0), nmarch - 1);
-    fl[MD] = fm;
-    return own_xy + (uint32_t)km * (D == 2 ? (uint32_t)nx : (uint32_t)nx * ny);
+    map_m(P, fm);
+    if (SPH || fx_own || fy_own || fm)
+      finish_one(&ring[FXI(ring_slot(P) + tid, n_ring)], NT, fx_own, fy_own, fm, gx, P);
   };
-  auto own_rad = [&](int k, auto* Q) {
-    bool fl[3];
-    const uint32_t gc_ = own_idx(k, fl);
-#pragma unroll
-    for (int v = 0; v < NRV; ++v) {
-      R q[NGL];
-#pragma unroll
-      for (int j = 0; j < NGL; ++j) {
-        R val = A.in[FXI(NG * ncell + (v * ncell + gc_) * G + gj[j], A.n_state)];
-        q[j] = (v >= 1 && fl[v - 1]) ? -val : val;
-        if (sph && v >= 1) q[j] *= frcp(hfac(v - 1, gx, k));  // physical component
-      }
-      Q[v] = vpair(q[0], q[NGL - 1], Q[v]);
-    }
-  };
-  const int gvar = lane < NG ? lane : 0;
-  // ---- staging of plane P into ring slot P & 3 with cp.async, issued one march step before the
-  // plane is first read: the own cell's groups by their threads (lane 0 also copies the cell's gas
-  // variables and opacity factors), the in-plane halo as (cell, group) items, and the halo cells'
-  // opacity factors one thread per cell.  Each thread later finishes what it copied itself:
-  // mirror flips of ghost cells and physical flux components on the spherical grid.
-  auto issue_plane = [&](int P) {
-    const int slot = P & 3;
-    bool fl[3];
-    const uint32_t gc_ = own_idx(P, fl);
-#pragma unroll
-    for (int j = 0; j < NGL; ++j) {
-      if (hasj[j]) {
-#pragma unroll
-        for (int v = 0; v < NRV; ++v)
-          cp_async(&rad_at(slot, v, sc_own, gj[j]), FXP(A.in, NG * ncell + (v * ncell + gc_) * G + gj[j], A.n_state));
-      }
-    }
-    if (lane == 0) {
-#pragma unroll
-      for (int v = 0; v < NG; ++v) cp_async(&gas_at(slot, v, sc_own), FXP(A.in, v * ncell + gc_, A.n_state));
-      cp_async(&pk[FXI((slot * 2 + 0) * PC + sc_own, n_pk)], FXP(A.opk, gc_, n_opk));
-      cp_async(&pk[FXI((slot * 2 + 1) * PC + sc_own, n_pk)], FXP(A.opk, ncell + gc_, n_opk));
-    }
-    for (int t = tid; t < NHALO * GP; t += NTH) {
-      const int i = t / GP, gg = t % GP;
-      if (gg >= G) continue;
+  auto finish_halo = [&](int P) {
+    bool fm = false;
+    map_m(P, fm);
+    for (int t = ht0; t < HS; t += NTH) {
       int sx, sy;
-      halo_of(i, sx, sy);
-      bool f[3];
-      const uint32_t c = map_cell(sx, sy, P, f);
-      const int sc = scell(sx, sy);
-#pragma unroll
-      for (int v = 0; v < NRV; ++v) cp_async(&rad_at(slot, v, sc, gg), FXP(A.in, NG * ncell + (v * ncell + c) * G + gg, A.n_state));
+      bool f0 = false, f1 = false;
+      halo_pos(div_gl(t), sx, sy);
+      inplane(sx, sy, f0, f1);
+      if (SPH || f0 || f1 || fm) finish_one(&halo[FXI((P & 1) * NRV * HS + t, n_halo)], HS, f0, f1, fm, x0 + sx, P);
     }
-    // halo opacity factors: in 2-d the lower halo cells (-2, -1) by the first warp and the upper
-    // ones (TX, TX+1) by the last, the warps whose edge cells read them in phase C (so that their
-    // restaging needs no block barrier after C; see the C | D hand-off)
-    static_assert(D != 2 || NHALO == 4, "2-d tiles are one row: four halo cells");
-    const int ih = D == 2 ? (tid < 2 ? tid : (tid >= NTH - 2 ? tid - (NTH - 4) : -1)) : (tid < NHALO ? tid : -1);
-    if (ih >= 0) {
-      const int i = ih;
-      int sx, sy;
-      halo_of(i, sx, sy);
-      bool f[3];
-      const uint32_t c = map_cell(sx, sy, P, f);
-      const int sc = scell(sx, sy);
-      cp_async(&pk[FXI((slot * 2 + 0) * PC + sc, n_pk)], FXP(A.opk, c, n_opk));
-      cp_async(&pk[FXI((slot * 2 + 1) * PC + sc, n_pk)], FXP(A.opk, ncell + c, n_opk));
-    }
-  };
-  auto finish_plane = [&](int P) {
-    const int slot = P & 3;
-    {
-      bool fl[3];
-      own_idx(P, fl);
-      if (fl[0] || fl[1] || fl[2] || sph) {
-#pragma unroll
-        for (int j = 0; j < NGL; ++j) {
-          if (hasj[j]) {
-#pragma unroll
-            for (int v = 1; v < NRV; ++v) {
-              R x = rad_at(slot, v, sc_own, gj[j]);
-              if (fl[v - 1]) x = -x;
-              if (sph) x *= frcp(hfac(v - 1, gx, P));  // physical component
-              rad_at(slot, v, sc_own, gj[j]) = x;
-            }
-          }
-        }
-      }
-    }
-    for (int t = tid; t < NHALO * GP; t += NTH) {
-      const int i = t / GP, gg = t % GP;
-      if (gg >= G) continue;
-      int sx, sy;
-      halo_of(i, sx, sy);
-      bool f[3];
-      map_cell(sx, sy, P, f);
-      if (f[0] || f[1] || f[2] || sph) {
-        const int sc = scell(sx, sy);
-#pragma unroll
-        for (int v = 1; v < NRV; ++v) {
-          R x = rad_at(slot, v, sc, gg);
-          if (f[v - 1]) x = -x;
-          if (sph) x *= frcp(hfac(v - 1, x0 + sx, P));
-          rad_at(slot, v, sc, gg) = x;
-        }
-      }
-    }
-  };
-  // stage-2 base of the thread's cell on plane P, staged at the end of the previous step and read
-  // back by the same thread in D
-  auto base_r = [&](int v, int j) -> R& { return sbr[FXI((v * TC + tcell) * GS + gj[j], n_sbr)]; };
-  auto base_g = [&]() -> R& { return sbg[FXI(gvar * TC + tcell, n_sbg)]; };
-  auto issue_base = [&](int P) {
-    if (A.base == nullptr || !cell_in) return;
-    const uint32_t c = D == 1 ? (uint32_t)gx : D == 2 ? (uint32_t)P * nx + gx : ((uint32_t)P * ny + gy) * nx + gx;
-#pragma unroll
-    for (int j = 0; j < NGL; ++j) {
-      if (hasj[j]) {
-#pragma unroll
-        for (int v = 0; v < NRV; ++v) cp_async(&base_r(v, j), FXP(A.base, NG * ncell + (v * ncell + c) * G + gj[j], A.n_state));
-      }
-    }
-    if (lane < NG) cp_async(&base_g(), FXP(A.base, gvar * ncell + c, A.n_state));
   };
 
-  // radiation flux through a face along d: QL = left cell's upper-face state, QR = right cell's
-  // lower-face state (E, physical F), chi = total opacity of the two cells (reading R9)
-  auto rad_face = [&](int d, const R* QL, const R* QR, R chiL, R chiR, R ell, R vstar, R* out) {
-    R PL[3], PR[3];
-    m1_row<R, D>(KR.ic2, QL[0], QL + 1, d, PL);
-    m1_row<R, D>(KR.ic2, QR[0], QR + 1, d, PR);
-    R tau = R(0.5) * (chiL + chiR) * ell;
-    R eps = tau > R(1) ? frcp(tau) : R(1);
-    const bool up = vstar >= R(0);  // upwind side of the advective terms (element-wise selects)
-    out[0] = R(0.5) * (QL[1 + d] + QR[1 + d]) - eps * KR.hc * (QR[0] - QL[0]) + vstar * (up ? QL[0] : QR[0]);
+  // ---- reads.  The in-plane neighbours of the own cell: in the ring, or for an edge cell in the
+  // halo (other base and variable stride, both fixed along the march up to the plane's slot).
+  auto own_ld = [&](int P, V* Q) {
+    const int s = ring_slot(P) + tid;
 #pragma unroll
-    for (int q = 0; q < D; ++q)
-      out[1 + q] = KR.hc2 * (PL[q] + PR[q]) - KR.hc * (QR[1 + q] - QL[1 + q]) +
-                   vstar * (up ? QL[1 + q] : QR[1 + q]);
+    for (int v = 0; v < NRV; ++v) Q[v] = ring[FXI(s + v * NT, n_ring)];
   };
-  R ef[NGL];
+  // p, st: first entry and variable stride of a neighbour, o: its offset in the plane of the ring
+  // or the halo
+  auto nb_ld = [&](int P, bool in_halo, int o, V* Q) {
+    const V* const p = in_halo ? halo + FXI((P & 1) * NRV * HS + o, n_halo) : ring + FXI(ring_slot(P) + o, n_ring);
+    const int st = in_halo ? HS : NT;
 #pragma unroll
-  for (int j = 0; j < NGL; ++j) ef[j] = R(sgc->efac_of(gj[j], R(0)));
-  // radiation reconstruction of one cell from its neighbours along a direction (table t, row ip;
-  // c: its MC coefficients): linear with the MC limiter, or (RO 2) the gas's parabola
-  auto recon_rad = [&](const MCCoef<R>& c, const Tab<R>& t, int ip, const R* Qm, const R* Q0, const R* Qp,
-                       R* a, R* b) {
+    for (int v = 0; v < NRV; ++v) Q[v] = p[v * st];
+  };
+  const bool xm_h = lx == 0, xp_h = lx == TX - 1, ym_h = D == 3 && ly == 0, yp_h = D == 3 && ly == TY - 1;
+  const int otid = act ? tid : lane;
+  const int xm_o = xm_h ? (4 * ly + 1) * GL + lane : otid - GL, xp_o = xp_h ? (4 * ly + 2) * GL + lane : otid + GL;
+  const int ym_o = ym_h ? (4 * TY + TX + lx) * GL + lane : otid - TX * GL;
+  const int yp_o = yp_h ? (4 * TY + 2 * TX + lx) * GL + lane : otid + TX * GL;
+  // face states of one cell along a direction: a at its lower face, b at its upper face
+  auto recon = [&](const Tab<R>& t, int ip, const V* Qm, const V* Q0, const V* Qp, V* a, V* b) {
     if constexpr (RO == 2) {
 #pragma unroll
-      for (int v = 0; v < NRV; ++v) recon_parabolic(t, ip, Qm[v], Q0[v], Qp[v], a[v], b[v]);
-    } else {
-#pragma unroll
-      for (int v = 0; v < NRV; ++v) recon_linear_c(c, Qm[v], Q0[v], Qp[v], a[v], b[v]);
-    }
-  };
-  auto rad_cell = [&](int slot, int sc, int gg, R* Q) {
-#pragma unroll
-    for (int v = 0; v < NRV; ++v) Q[v] = rad_at(slot, v, sc, gg);
-  };
-
-  // ---- The lane's groups as one value of type V: with two groups per lane a pair of FP32 values
-  // (F2), so that their arithmetic runs on the packed FP32 instructions, two groups per
-  // instruction; else R.  The shared arrays are strided by an even group count and a lane's first
-  // group g0 is even with two groups per lane, so a lane's pair is one 8-byte shared access.
-  using V = typename std::conditional<NGL == 2, F2, R>::type;
-  const int g0 = gj[0];
-  const bool h0 = hasj[0], h1 = hasj[NGL - 1];  // (NGL == 1: h1 is not used)
-  auto ldv = [&](const R* p) -> V { return ld_lane(p, V()); };
-  auto stv = [&](R* p, const V& x) { st_lane(p, x, h0, h1); };
-  auto rad_v = [&](int slot, int sc, V* Q) {
-#pragma unroll
-    for (int v = 0; v < NRV; ++v) Q[v] = ldv(&rad_at(slot, v, sc, g0));
-  };
-  const V efv = vpair(ef[0], ef[NGL - 1], V());
-  auto chi_v = [&](int slot, int sc) {
-    return vfma(efv, V(pk[FXI((slot * 2) * PC + sc, n_pk)]), V(pk[FXI((slot * 2 + 1) * PC + sc, n_pk)]));
-  };
-  auto recon_rad_v = [&](const MCCoef<R>& c, const Tab<R>& t, int ip, const V* Qm, const V* Q0, const V* Qp,
-                         V* a, V* b) {
-    if constexpr (RO == 2 && NGL == 2) {
-      // (the gas's parabola has no packed form: group by group)
+      for (int v = 0; v < NRV; ++v) {
+        R a0, b0, a1 = R(0), b1 = R(0);
+        recon_parabolic(t, ip, vget(Qm[v], 0), vget(Q0[v], 0), vget(Qp[v], 0), a0, b0);
+        if (W == 2) recon_parabolic(t, ip, vget(Qm[v], 1), vget(Q0[v], 1), vget(Qp[v], 1), a1, b1);
+        a[v] = vpair(a0, a1, V());
+        b[v] = vpair(b0, b1, V());
+      }
+    } else if constexpr (SPH) {
+      const MCCoef<R> c = mc_coef(t, ip);
 #pragma unroll
       for (int v = 0; v < NRV; ++v) {
-        R a0, b0, a1, b1;
-        recon_parabolic(t, ip, Qm[v].x, Q0[v].x, Qp[v].x, a0, b0);
-        recon_parabolic(t, ip, Qm[v].y, Q0[v].y, Qp[v].y, a1, b1);
-        a[v] = V(a0, a1);
-        b[v] = V(b0, b1);
+        const V s = mc_min((Q0[v] - Qm[v]) * c.il, (Qp[v] - Q0[v]) * c.ir, (Qp[v] - Qm[v]) * c.ic, R(2));
+        a[v] = vfma(s, V(c.dl), Q0[v]);
+        b[v] = vfma(s, V(c.dr), Q0[v]);
       }
-    } else if constexpr (RO == 2) {
-#pragma unroll
-      for (int v = 0; v < NRV; ++v) recon_parabolic(t, ip, Qm[v], Q0[v], Qp[v], a[v], b[v]);
     } else {
 #pragma unroll
-      for (int v = 0; v < NRV; ++v) recon_linear_c(c, Qm[v], Q0[v], Qp[v], a[v], b[v]);
+      for (int v = 0; v < NRV; ++v) {
+        const V dl = Q0[v] - Qm[v], dr = Qp[v] - Q0[v];
+        const V s = mc_min(dl, dr, (dl + dr) * KL.q25, R(1));  // half the limited slope times dx
+        a[v] = Q0[v] - s;
+        b[v] = Q0[v] + s;
+      }
     }
   };
-  // the radiation face flux of rad_face for the lane's groups
-  auto rad_face_v = [&](int d, const V* QL, const V* QR, V chiL, V chiR, R ell, R vstar, V* out) {
-    V PL[3], PR[3];
-    if constexpr (NGL == 2) {
-      m1_row<D>(KR.ic2, QL[0], QL + 1, d, PL);
-      m1_row<D>(KR.ic2, QR[0], QR + 1, d, PR);
+  // twice the flux through a face of direction n from its two states; r: the face record
+  // (2 max(v*, 0), 2 min(v*, 0), and the opacity sums so that tau_g = eps_g^d r2 + r3)
+  auto face_flux = [&](int n, const V* QL, const V* QR, const R* r, V ef, V* out) {
+    V PL[D], PR[D];
+    m1_c2row<D>(KL, QL[0], QL + 1, n, PL);
+    m1_c2row<D>(KL, QR[0], QR + 1, n, PR);
+    const V tau = vfma(ef, V(r[2]), V(r[3]));
+    const V ce = rcp_ge1(tau) * KL.mc;  // -c min(1, 1/tau)
+    out[0] = vfma(V(r[1]), QR[0], vfma(V(r[0]), QL[0], vfma(ce, QR[0] - QL[0], QL[1 + n] + QR[1 + n])));
+    const V kL = V(KR.c + r[0]), kR = V(r[1] - KR.c);
+#pragma unroll
+    for (int q = 0; q < D; ++q) out[1 + q] = vfma(kR, QR[1 + q], vfma(kL, QL[1 + q], PL[q] + PR[q]));
+  };
+  auto rec_ld = [&](int P, int i, R* r) {
+    const R* const p = rec + FXI(((P & 1) * NREC + i) * 4, n_rec);
+    if constexpr (sizeof(R) == 4) {
+      const float4 x = *reinterpret_cast<const float4*>(p);
+      r[0] = x.x; r[1] = x.y; r[2] = x.z; r[3] = x.w;
     } else {
-      m1_row<R, D>(KR.ic2, QL[0], QL + 1, d, PL);
-      m1_row<R, D>(KR.ic2, QR[0], QR + 1, d, PR);
-    }
-    const V tau = V(R(0.5)) * (chiL + chiR) * ell;
-    const V eps = vsel_gt(tau, R(1), frcp(tau), V(R(1)));
-    const bool up = vstar >= R(0);  // upwind side of the advective terms (element-wise selects)
-    out[0] = vfma(V(vstar), up ? QL[0] : QR[0],
-                  vfma(eps * (-KR.hc), QR[0] - QL[0], V(R(0.5)) * (QL[1 + d] + QR[1 + d])));
 #pragma unroll
-    for (int q = 0; q < D; ++q)
-      out[1 + q] = vfma(V(vstar), up ? QL[1 + q] : QR[1 + q],
-                        vfma(V(-KR.hc), QR[1 + q] - QL[1 + q], V(KR.hc2) * (PL[q] + PR[q])));
-  };
-
-  // gas face buffer: lower-face index of cell (gx, gy, k) along direction d
-  // (cells of a tile that overhang the grid use the last column/row; their values are unused)
-  // Positions are clamped to the last cell, face indices along their own direction to the last
-  // face: the first overhanging cell of a tile computes the domain's upper boundary face.
-  const int gxc = min(gx, nx - 1), gyc = min(gy, ny - 1);
-  const int gxf = min(gx, nx), gyf = min(gy, ny);
-  const int fx_nx = nx + 1;
-  auto face_x = [&](int k) -> uint32_t {
-    return D == 1 ? (uint32_t)gxf : D == 2 ? (uint32_t)k * fx_nx + gxf : ((uint32_t)k * ny + gyc) * fx_nx + gxf;
-  };
-  auto face_y3 = [&](int k) -> uint32_t { return ((uint32_t)k * (ny + 1) + gyf) * nx + gxc; };
-  auto face_m = [&](int k) -> uint32_t { return D == 2 ? (uint32_t)k * nx + gxc : ((uint32_t)k * ny + gyc) * nx + gxc; };
-  // number of faces of each direction, and the gas face buffer read
-  const uint32_t nfd[3] = {(uint32_t)(nx + 1) * (D > 1 ? ny : 1) * (D > 2 ? nz : 1),
-                           (uint32_t)nx * (ny + 1) * (D > 2 ? nz : 1), (uint32_t)nx * ny * (nz + 1)};
-  auto gface = [&](int d, int v, uint32_t f) -> R {
-    return __ldg(FXP(A.faces, (uint32_t)A.face_off[d] + v * nfd[d] + f, A.n_faces));
-  };
-  auto gface_p = [&](int d, int v, uint32_t f) -> const R* {
-    return FXP(A.faces, (uint32_t)A.face_off[d] + v * nfd[d] + f, A.n_faces);
-  };
-  // 1-d and 2-d: the gas-face values a cell needs on plane P, staged with cp.async one plane
-  // ahead into shared slots by plane parity: slots 0-2 the contact speeds of its lower x face, of
-  // the x face above the tile's last column and of its upper march face (lane 0 copies them);
-  // slots 3 + 2Dv .. 2 + 2D(v+1) the fluxes of gas variable v through the cell's lower and upper
-  // x and march faces (lane v copies them).  The lanes of a cell read them after their wait and a
-  // warp barrier.
-  constexpr int GFV = 2 * D;
-  auto gfs = [&](int P, int slot) -> R& { return sgf[FXI(((P & 1) * TC + tcell) * LY::NGF + slot, n_sgf)]; };
-  auto issue_gf = [&](int P) {
-    if constexpr (D <= 2) {
-      if (lane == 0) {
-        cp_async(&gfs(P, 0), gface_p(0, NG, face_x(P)));
-        if (lx == TX - 1 && gx < nx) cp_async(&gfs(P, 1), gface_p(0, NG, face_x(P) + 1));
-        if (D == 2) cp_async(&gfs(P, 2), gface_p(MD, NG, face_m(P + 1)));
-      }
-      if (lane < NG && cell_in) {  // (an overhanging cell's upper face would lie past the last face)
-        const int b = 3 + GFV * lane;
-        const uint32_t fxk = face_x(P);
-        cp_async(&gfs(P, b + 0), gface_p(0, lane, fxk));
-        cp_async(&gfs(P, b + 1), gface_p(0, lane, fxk + 1));
-        if (D == 2) {
-          cp_async(&gfs(P, b + 2), gface_p(MD, lane, face_m(P)));
-          cp_async(&gfs(P, b + 3), gface_p(MD, lane, face_m(P + 1)));
-        }
-      }
+      for (int c = 0; c < 4; ++c) r[c] = p[c];
     }
   };
-
-  // Carried along the march: the own cell's upper march-face state of plane k and the flux
-  // through its lower march face.  In 2-d they are kept in shared memory (thread-private slots by
-  // plane parity) instead of registers: the kernel runs at its register limit.
-  V bm0[NRV], rfm_old[NRV];  // own march-direction upper-face states of plane k; fluxes through
-                             // the lower march face
-#pragma unroll
-  for (int v = 0; v < NRV; ++v) bm0[v] = rfm_old[v] = V(R(0));
-  constexpr bool SCAR = D == 2;
-  auto car = [&](int P, int w, int v) -> R* {  // w = 0: upper-face state, 1: lower-face flux
-    return &scr[FXI(((((P & 1) * 2 + w) * NRV + v) * TC + tcell) * GS + g0, n_scr)];
+  auto ef_of = [&](int ln) -> V {
+    const int ga = ln * W, gb = ga + 1 < G ? ga + 1 : ga;
+    return vpair(A.gc->efac_of(ga, R(0)), A.gc->efac_of(W == 2 ? gb : ga, R(0)), V());
   };
+  const V efv = ef_of(lane);
+  // own lower faces in xb (TX+1 faces per row) and yb; the threads past the tile use the space
+  // after the arrays' faces
+  const int xo = act ? tid + ly * GL : NT + CP::XP + (tid & 31), yo = act ? tid : xo;
 
   // ---------------------------------------------------------------- prologue
-  if (D == 1) {
-    load_cells(0, 0, TX + 4, all_of);
-    issue_base(0);
-    issue_gf(0);
+  V bm0[NRV], rfm_old[NRV];  // upper march-face state of plane k, flux through its lower march face
+#pragma unroll
+  for (int v = 0; v < NRV; ++v) bm0[v] = rfm_old[v] = V(R(0));
+  if constexpr (D == 1) {
+    issue_own(0);
+    issue_halo(0);
+    issue_rec(0);
     cp_async_commit();
+    cp_async_wait_all();
+    finish_own(0);
+    finish_halo(0);
     __syncthreads();
   } else {
-    // planes kbeg-1 .. kbeg+1 directly; plane kbeg+2 and the stage-2 base of plane kbeg staged
-    for (int k = kbeg - 1; k <= kbeg + 1; ++k) load_cells(k & 3, k, TC, interior_of);
-    for (int k = kbeg; k <= kbeg + 1; ++k) load_cells(k & 3, k, NHALO, halo_of);
-    issue_plane(kbeg + 2);
-    issue_base(kbeg);
-    issue_gf(kbeg);
+    for (int P = kbeg - 1; P <= kbeg + 2; ++P) issue_own(P);
+    issue_halo(kbeg);
+    issue_rec(kbeg);
     cp_async_commit();
-    V Qm1[NRV], Qm2[NRV], Q0[NRV], Q1[NRV];
-    own_rad(kbeg - 2, Qm2);
-    own_rad(kbeg - 1, Qm1);
-    own_rad(kbeg, Q0);
-    own_rad(kbeg + 1, Q1);
-    __syncthreads();
-    // march reconstruction of planes kbeg-1 (upper face) and kbeg, and the face kbeg-1/2
-    const MCCoef<R> mp = mc_coef(tm, bc_pad(kbeg - 1)), m0 = mc_coef(tm, bc_pad(kbeg));
-    const R vs = gface(MD, NG, face_m(kbeg));
-    const R ell = sph ? tm(T_ELL, bc_pad(kbeg)) * tx(T_XH, bc_pad(gx)) : tm(T_ELL, bc_pad(kbeg));
-    V a_[NRV], bprev[NRV];
-    recon_rad_v(mp, tm, bc_pad(kbeg - 1), Qm2, Qm1, Q0, a_, bprev);
-    recon_rad_v(m0, tm, bc_pad(kbeg), Qm1, Q0, Q1, a_, bm0);
-    rad_face_v(MD, bprev, a_, chi_v((kbeg - 1) & 3, sc_own), chi_v(kbeg & 3, sc_own), ell, vs, rfm_old);
-    if (SCAR) {
+    V Qa[NRV];  // own column of plane kbeg-2, straight from global memory
+    {
+      bool fm = false;
+      const uint32_t o = NG * ncell + toff + (uint32_t)map_m(kbeg - 2, fm) * pstride;
 #pragma unroll
       for (int v = 0; v < NRV; ++v) {
-        stv(car(kbeg, 0, v), bm0[v]);
-        stv(car(kbeg, 1, v), rfm_old[v]);
+        const R e0 = A.in[FXI(o + v * vstride, A.n_state)], e1 = h1 ? A.in[FXI(o + v * vstride + 1, A.n_state)] : R(0);
+        Qa[v] = vpair(e0, e1, V());
+      }
+#pragma unroll
+      for (int q = 0; q < D; ++q) {
+        const bool fl = q == MD ? fm : (q == 0 ? fx_own : fy_own);
+        if (SPH) Qa[1 + q] = Qa[1 + q] * frcp(hfac(q, gx, kbeg - 2));
+        if (fl) Qa[1 + q] = -Qa[1 + q];
       }
     }
+    R r[4];
+    {
+      const uint32_t f = (uint32_t)A.rec_off[MD] + (D == 3 ? (uint32_t)min(gy, ny - 1) * nx : 0u) + (uint32_t)min(gx, nx - 1) + (uint32_t)kbeg * pcells;
+      const R* const s = A.frec + (size_t)4 * FXI(f, A.n_recs);
+#pragma unroll
+      for (int c = 0; c < 4; ++c) r[c] = s[c];
+    }
+    cp_async_wait_all();
+    for (int P = kbeg - 1; P <= kbeg + 2; ++P) finish_own(P);
+    finish_halo(kbeg);
+    __syncthreads();
+    // march reconstruction of planes kbeg-1 (upper face) and kbeg, and the flux at kbeg-1/2
+    V Qb[NRV], Qc[NRV], Qd[NRV], ta[NRV], tb[NRV], am[NRV];
+    own_ld(kbeg - 1, Qb);
+    own_ld(kbeg, Qc);
+    own_ld(kbeg + 1, Qd);
+    recon(tm, bc_pad(kbeg - 1), Qa, Qb, Qc, ta, tb);
+    recon(tm, bc_pad(kbeg), Qb, Qc, Qd, am, bm0);
+    face_flux(MD, tb, am, r, efv, rfm_old);
   }
-  const int ipx = bc_pad(gx);  // the x-direction table row of this cell
-  // x-direction coefficients of this cell do not change along the march
-  const MCCoef<R> mcx = mc_coef(tx, ipx);
-  const R fxl = tx(T_FL, ipx), fxr = tx(T_FR, ipx), ellx = tx(T_ELL, ipx);
+  const int ipx = bc_pad(gx), ipy = bc_pad(gy);
+
+  // the halo reconstructions as tasks, one per (row or column end, lane): the upper-face state of
+  // cells -1 (left state of the tile's first face) and the lower-face state of cells TX, TY (right
+  // state of its last face).  A task's ring entry of the edge cell, halo entry of the near halo
+  // cell and step to the far one, and where the state goes:
+  const int n1 = TY * GL, n2 = D == 3 ? TX * GL : 0, ntask = 2 * (n1 + n2);
+  struct Task { int in, h, hs, dst; bool up, x; };
+  auto task_of = [&](int t) -> Task {
+    Task b;
+    b.x = D < 3 || t < 2 * n1;
+    const int u = b.x ? t : t - 2 * n1, nn = b.x ? n1 : n2;
+    b.up = u >= nn;                      // the halo cell above the tile
+    const int e = b.up ? u - nn : u;     // row (or column) * GL + lane
+    const int c = div_gl(e), ln = e - c * GL;
+    if (b.x) {
+      b.in = (c * TX + (b.up ? TX - 1 : 0)) * GL + ln;
+      b.h = (4 * c + (b.up ? 2 : 1)) * GL + ln;
+      b.hs = b.up ? GL : -GL;
+      b.dst = b.up ? e : c * (TX + 1) * GL + ln;
+    } else {
+      b.in = (b.up ? (TY - 1) * TX * GL : 0) + e;
+      b.h = (4 * TY + (b.up ? 2 : 1) * TX) * GL + e;
+      b.hs = b.up ? TX * GL : -TX * GL;
+      b.dst = e;
+    }
+    return b;
+  };
+  auto run_task = [&](int k, int px, const Task& b_) {
+    V Qi[NRV], Q0[NRV], Qo[NRV], a[NRV], b[NRV];
+    nb_ld(k, false, b_.in, Qi);
+    nb_ld(k, true, b_.h, Q0);
+    nb_ld(k, true, b_.h + b_.hs, Qo);
+    if constexpr (TABLES) {
+      const Tab<R>& tt = b_.x ? tx : ty;
+      const int ip = b_.x ? bc_pad(b_.up ? x0 + TX : x0 - 1) : bc_pad(b_.up ? y0 + TY : y0 - 1);
+      if (b_.up) recon(tt, ip, Qi, Q0, Qo, a, b);
+      else recon(tt, ip, Qo, Q0, Qi, b, a);
+    } else {
+      // (uniform spacing: the other way round gives the mirrored states)
+      recon(tx, 0, Qi, Q0, Qo, a, b);
+    }
+    V* const d = b_.up ? (b_.x ? xr + FXI(b_.dst, n_xr) : yr + FXI(b_.dst, n_yr))
+                       : (b_.x ? xb : yb) + FXI(px + b_.dst, n_xb);
+    const int st = b_.up ? (b_.x ? n1 : n2) : XC;
+#pragma unroll
+    for (int v = 0; v < NRV; ++v) d[v * st] = a[v];
+  };
+  Task my{};
+  if (tid < ntask) my = task_of(tid);
+  // the fluxes through the tile's upper faces likewise, from the last threads down
+  const int ct = NTH - 1 - tid;
+  const bool task_c = ct < n1 + n2;
+  const bool more_out = A.pre_out != nullptr || A.phi_out != nullptr;
+  const bool stage2 = A.base != nullptr;
 
   // ---------------------------------------------------------------- march
   for (int k = kbeg; k < kend; ++k) {
-    const int s0 = k & 3;
-    // ---- A: finish plane k+2 (staged during step k-1) and stage plane k+3.  Slot (k+3)&3 held
-    // plane k-1, last read in step k-1 before its barrier C; the warp barrier keeps the cell's
-    // lanes out of step k-1's D (which reads the cell's gas variables of plane k-1) before lane 0
-    // restages them.
-    cp_async_wait_all();
-    __syncwarp();
-    if (D >= 2) finish_plane(k + 2);
-    if (D >= 2 && k + 1 < kend) issue_plane(k + 3);
-    // gas face data of this plane: the cell's lower faces and the march face k+1/2 (1-d and 2-d:
-    // staged during the previous step, and those of plane k+1 issued now), and the fluxes of the
-    // lane's gas variable through the cell's faces
-    R vsx, vsx1 = R(0), vsm = R(0), vsy = R(0), vsy1 = R(0);
-    R gfl[6] = {R(0), R(0), R(0), R(0), R(0), R(0)};
-    if constexpr (D <= 2) {
-      vsx = gfs(k, 0);
-      if (NGL == 1) vsx1 = (lx == TX - 1 && gx < nx) ? gfs(k, 1) : R(0);
-      if (D == 2) vsm = gfs(k, 2);
-      if (lane < NG && cell_in) {
-#pragma unroll
-        for (int c = 0; c < GFV; ++c) gfl[c] = gfs(k, 3 + GFV * lane + c);
-      }
-      if (k + 1 < kend) issue_gf(k + 1);
-      cp_async_commit();
-    } else {
-      cp_async_commit();
-      vsx = gface(0, NG, face_x(k));
-      if (NGL == 1) vsx1 = (lx == TX - 1 && gx < nx) ? gface(0, NG, face_x(k) + 1) : R(0);
-      vsm = gface(MD, NG, face_m(k + 1));
-      vsy = gface(1, NG, face_y3(k));
-      vsy1 = (ly == TY - 1 && gy < ny) ? gface(1, NG, face_y3(k) + nx) : R(0);
+    const bool more = D >= 2 && k + 1 < kend;
+    if (more) {
+      issue_own(k + 3);
+      issue_halo(k + 1);
+      issue_rec(k + 1);
     }
-    // Face area/volume factors of this cell for the three flux classes (scalar, covariant
-    // component 0, component 1).  Curvilinear: x faces carry the march direction's cross factor
-    // and march faces the x direction's (Eq. 8 with separable sqrt(g)); Cartesian: 1/dx.
-    R fx_l[3], fx_r[3], fm_l[3], fm_r[3];
+    issue_base(k);
+    cp_async_commit();
+    const int px = PB == 2 ? (k & 1) * NRV * XC : 0;  // this plane's half of xb and yb
+    // ---- B
+    V ax[NRV], ay[NRV], am1[NRV], bm1[NRV];
     {
-      const int ipm = bc_pad(k);
-      const int eL[3] = {T_FL, T_FL1, T_FL2}, eR[3] = {T_FR, T_FR1, T_FR2}, eX[3] = {T_XS, T_X1, T_X2};
+      V Q0[NRV], Qm[NRV], Qp[NRV], b[NRV];
+      own_ld(k, Q0);
+      nb_ld(k, xm_h, xm_o, Qm);
+      nb_ld(k, xp_h, xp_o, Qp);
+      recon(tx, ipx, Qm, Q0, Qp, ax, b);
 #pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        if (sph) {
-          fx_l[c] = tx(eL[c], ipx) * tm(eX[c], ipm);
-          fx_r[c] = tx(eR[c], ipx) * tm(eX[c], ipm);
-          fm_l[c] = tm(eL[c], ipm) * tx(eX[c], ipx);
-          fm_r[c] = tm(eR[c], ipm) * tx(eX[c], ipx);
-        } else {
-          fx_l[c] = fxl;
-          fx_r[c] = fxr;
-          fm_l[c] = D >= 2 ? tm(T_FL, ipm) : R(0);
-          fm_r[c] = D >= 2 ? tm(T_FR, ipm) : R(0);
-        }
-      }
-    }
-    // flux class of the gas variable of this lane and of each radiation variable (selected by
-    // value: a lane-dependent array index would place the factor arrays in local memory)
-    const int gcls = (gvar >= 1 && gvar <= 2 && gvar <= D) ? gvar : 0;
-    auto cls = [&](const R* f) { return gcls == 0 ? f[0] : (gcls == 1 ? f[1] : f[2]); };
-    R gFp[D], gAp[D], gFm[D], gAm[D];
-#pragma unroll
-    for (int q = 0; q < D; ++q) gFp[q] = gAp[q] = gFm[q] = gAm[q] = R(0);
-    if (cell_in) {  // (an overhanging cell's upper face would lie past the last face)
+      for (int v = 0; v < NRV; ++v) xb[FXI(px + v * XC + xo + GL, n_xb)] = b[v];
       if constexpr (D == 3) {
-        const uint32_t fxk = face_x(k), fyk = face_y3(k);
-        gfl[0] = gface(0, gvar, fxk);
-        gfl[1] = gface(0, gvar, fxk + 1);
-        gfl[2] = gface(MD, gvar, face_m(k));
-        gfl[3] = gface(MD, gvar, face_m(k + 1));
-        gfl[4] = gface(1, gvar, fyk);
-        gfl[5] = gface(1, gvar, fyk + nx);
+        nb_ld(k, ym_h, ym_o, Qm);
+        nb_ld(k, yp_h, yp_o, Qp);
+        recon(ty, ipy, Qm, Q0, Qp, ay, b);
+#pragma unroll
+        for (int v = 0; v < NRV; ++v) yb[FXI(px + v * XC + yo + TX * GL, n_xb)] = b[v];
       }
-      // (1-d, 2-d: lanes >= NG carry no gas variable and read zeros, unused)
-      // face terms of the divergence, direction by direction: x, (3-d) y, the march direction
-      gFp[0] = gfl[1]; gAp[0] = cls(fx_r); gFm[0] = gfl[0]; gAm[0] = cls(fx_l);
-      if (D == 3) { gFp[1] = gfl[5]; gAp[1] = ty(T_FR, bc_pad(gy)); gFm[1] = gfl[4]; gAm[1] = ty(T_FL, bc_pad(gy)); }
-      if (D >= 2) { gFp[D - 1] = gfl[3]; gAp[D - 1] = cls(fm_r); gFm[D - 1] = gfl[2]; gAm[D - 1] = cls(fm_l); }
-    }
-    // (B reads only planes finished two steps ago and the thread's own column; in 3-d the face
-    // states it writes share their space with the fluxes that D of the previous plane reads)
-    if (D == 3) __syncthreads();
-    // the own column of planes k, k+1, k+2 from the ring
-    V Q0[NRV], Q1[NRV], Q2[NRV];
-    rad_v(s0, sc_own, Q0);
-    if (D >= 2) {
-      rad_v((k + 1) & 3, sc_own, Q1);
-      rad_v((k + 2) & 3, sc_own, Q2);
-    }
-    // ---- B: reconstructions
-    V ax[NRV], bx[NRV], am1[NRV], bm1[NRV], ay[NRV], by[NRV];
-    {
-      V Qa[NRV], Qb[NRV];
-      rad_v(s0, sc_own - 1, Qa);
-      rad_v(s0, sc_own + 1, Qb);
-      recon_rad_v(mcx, tx, ipx, Qa, Q0, Qb, ax, bx);
-#pragma unroll
-      for (int v = 0; v < NRV; ++v) stv(&rbx[FXI((v * NFX + ly * (TX + 1) + lx + 1) * GS + g0, n_rbx)], bx[v]);
-      if constexpr (NGL == 1) {  // (two groups per lane: after this block, one group per lane)
-        if (lx == 0) {  // halo cell -1: its upper-face state is the left state of face 0
-          V Qc[NRV], ta[NRV], tb[NRV];
-          rad_v(s0, sc_own - 2, Qc);
-          recon_rad_v(mc_coef(tx, bc_pad(gx - 1)), tx, bc_pad(gx - 1), Qc, Qa, Q0, ta, tb);
-#pragma unroll
-          for (int v = 0; v < NRV; ++v) stv(&rbx[FXI((v * NFX + ly * (TX + 1)) * GS + g0, n_rbx)], tb[v]);
-        }
-        if (lx == TX - 1) {  // halo cell TX: its lower-face state is the right state of face TX
-          V Qc[NRV], ta[NRV], tb[NRV];
-          rad_v(s0, sc_own + 2, Qc);
-          recon_rad_v(mc_coef(tx, bc_pad(gx + 1)), tx, bc_pad(gx + 1), Q0, Qb, Qc, ta, tb);
-#pragma unroll
-          for (int v = 0; v < NRV; ++v) stv(&rax[FXI((v * TY + ly) * GS + g0, n_rax)], ta[v]);
-        }
-      }
-      if (D == 3) {
-        V Qa3[NRV], Qb3[NRV];
-        rad_v(s0, sc_own - PX, Qa3);
-        rad_v(s0, sc_own + PX, Qb3);
-        recon_rad_v(mc_coef(ty, bc_pad(gy)), ty, bc_pad(gy), Qa3, Q0, Qb3, ay, by);
-#pragma unroll
-        for (int v = 0; v < NRV; ++v) stv(&rby[FXI((v * NFY + (ly + 1) * TX + lx) * GS + g0, n_rby)], by[v]);
-        if (NGL == 1 && ly == 0) {  // (two groups per lane: after this block, one group per lane)
-          V Qc[NRV], ta[NRV], tb[NRV];
-          rad_v(s0, sc_own - 2 * PX, Qc);
-          recon_rad_v(mc_coef(ty, bc_pad(gy - 1)), ty, bc_pad(gy - 1), Qc, Qa3, Q0, ta, tb);
-#pragma unroll
-          for (int v = 0; v < NRV; ++v) stv(&rby[FXI((v * NFY + lx) * GS + g0, n_rby)], tb[v]);
-        }
-        if (NGL == 1 && ly == TY - 1) {
-          V Qc[NRV], ta[NRV], tb[NRV];
-          rad_v(s0, sc_own + 2 * PX, Qc);
-          recon_rad_v(mc_coef(ty, bc_pad(gy + 1)), ty, bc_pad(gy + 1), Q0, Qb3, Qc, ta, tb);
-#pragma unroll
-          for (int v = 0; v < NRV; ++v) stv(&ray[FXI((v * TX + lx) * GS + g0, n_ray)], ta[v]);
-        }
-      }
-      if (D >= 2) recon_rad_v(mc_coef(tm, bc_pad(k + 1)), tm, bc_pad(k + 1), Q0, Q1, Q2, am1, bm1);
-      if (SCAR) {
-#pragma unroll
-        for (int v = 0; v < NRV; ++v) stv(car(k + 1, 0, v), bm1[v]);
+      if constexpr (D >= 2) {
+        own_ld(k + 1, Qm);
+        own_ld(k + 2, Qp);
+        recon(tm, bc_pad(k + 1), Q0, Qm, Qp, am1, bm1);
       }
     }
-    // two groups per lane: the row's x halo cells -1 and TX (the upper-face state of cell -1, left
-    // state of face 0; the lower-face state of cell TX, right state of face TX), one group per
-    // lane of the NGL cells nearest each edge: the warp runs one reconstruction for them, not NGL
-    if (NGL > 1 && lx < NGL) {
-      const int h = lx * GL + lane;
-      if (h < G) {
-        const int sc0 = scell(0, ly);
-        R Qc[NRV], Qd[NRV], Qe[NRV], ta[NRV], tb[NRV];
-        rad_cell(s0, sc0 - 2, h, Qc);
-        rad_cell(s0, sc0 - 1, h, Qd);
-        rad_cell(s0, sc0, h, Qe);
-        recon_rad(mc_coef(tx, bc_pad(x0 - 1)), tx, bc_pad(x0 - 1), Qc, Qd, Qe, ta, tb);
-#pragma unroll
-        for (int v = 0; v < NRV; ++v) rbx[FXI((v * NFX + ly * (TX + 1)) * GS + h, n_rbx)] = tb[v];
-      }
-    }
-    if (NGL > 1 && lx >= TX - NGL) {
-      const int h = (lx - (TX - NGL)) * GL + lane;
-      if (h < G) {
-        const int sc1 = scell(TX - 1, ly);
-        R Qc[NRV], Qd[NRV], Qe[NRV], ta[NRV], tb[NRV];
-        rad_cell(s0, sc1, h, Qc);
-        rad_cell(s0, sc1 + 1, h, Qd);
-        rad_cell(s0, sc1 + 2, h, Qe);
-        recon_rad(mc_coef(tx, bc_pad(x0 + TX)), tx, bc_pad(x0 + TX), Qc, Qd, Qe, ta, tb);
-#pragma unroll
-        for (int v = 0; v < NRV; ++v) rax[FXI((v * TY + ly) * GS + h, n_rax)] = ta[v];
-      }
-    }
-    // 3-d, two groups per lane: likewise the y halo rows -1 (the upper-face state of each column's
-    // cell -1, left state of its y face 0) and TY (the lower-face state of cell TY, right state of
-    // face TY), one group per lane of the NGL rows nearest each y edge, so that the edge rows' warps
-    // do not carry the whole halo work alone
-    if (D == 3 && NGL > 1 && ly < NGL) {
-      const int h = ly * GL + lane;
-      if (h < G) {
-        const int sc0 = scell(lx, 0);
-        R Qc[NRV], Qd[NRV], Qe[NRV], ta[NRV], tb[NRV];
-        rad_cell(s0, sc0 - 2 * PX, h, Qc);
-        rad_cell(s0, sc0 - PX, h, Qd);
-        rad_cell(s0, sc0, h, Qe);
-        recon_rad(mc_coef(ty, bc_pad(y0 - 1)), ty, bc_pad(y0 - 1), Qc, Qd, Qe, ta, tb);
-#pragma unroll
-        for (int v = 0; v < NRV; ++v) rby[FXI((v * NFY + lx) * GS + h, n_rby)] = tb[v];
-      }
-    }
-    if (D == 3 && NGL > 1 && ly >= TY - NGL) {
-      const int h = (ly - (TY - NGL)) * GL + lane;
-      if (h < G) {
-        const int sc1 = scell(lx, TY - 1);
-        R Qc[NRV], Qd[NRV], Qe[NRV], ta[NRV], tb[NRV];
-        rad_cell(s0, sc1, h, Qc);
-        rad_cell(s0, sc1 + PX, h, Qd);
-        rad_cell(s0, sc1 + 2 * PX, h, Qe);
-        recon_rad(mc_coef(ty, bc_pad(y0 + TY)), ty, bc_pad(y0 + TY), Qc, Qd, Qe, ta, tb);
-#pragma unroll
-        for (int v = 0; v < NRV; ++v) ray[FXI((v * TX + lx) * GS + h, n_ray)] = ta[v];
-      }
-    }
+    if (tid < ntask) run_task(k, px, my);
+    if (D == 3 && ntask > NTH)
+      for (int t = tid + NTH; t < ntask; t += NTH) run_task(k, px, task_of(t));
     __syncthreads();
-    // ---- C: radiation face fluxes
+    // ---- C
     V rfm_new[NRV];
 #pragma unroll
     for (int v = 0; v < NRV; ++v) rfm_new[v] = V(R(0));
-    const R ell_m = sph ? tm(T_ELL, bc_pad(k + 1)) * tx(T_XH, ipx) : tm(T_ELL, bc_pad(k + 1));
     {
-      const V chi0 = chi_v(s0, sc_own);
-      {
-        const int fx = ly * (TX + 1) + lx;
-        V QL[NRV], out[NRV];
+      V QL[NRV], out[NRV];
+      R r[4];
 #pragma unroll
-        for (int v = 0; v < NRV; ++v) QL[v] = ldv(&rbx[FXI((v * NFX + fx) * GS + g0, n_rbx)]);
-        rad_face_v(0, QL, ax, chi_v(s0, sc_own - 1), chi0, ellx, vsx, out);
+      for (int v = 0; v < NRV; ++v) QL[v] = xb[FXI(px + v * XC + xo, n_xb)];
+      rec_ld(k, ly * (TX + 1) + lx, r);
+      face_flux(0, QL, ax, r, efv, out);
 #pragma unroll
-        for (int v = 0; v < NRV; ++v) stv(&rfx[FXI((v * NFX + fx) * GS + g0, n_rfx)], out[v]);
-        if (NGL == 1 && lx == TX - 1) {
-          V QR[NRV];
+      for (int v = 0; v < NRV; ++v) xb[FXI(px + v * XC + xo, n_xb)] = out[v];
+      if constexpr (D == 3) {
 #pragma unroll
-          for (int v = 0; v < NRV; ++v) QR[v] = ldv(&rax[FXI((v * TY + ly) * GS + g0, n_rax)]);
-          rad_face_v(0, bx, QR, chi0, chi_v(s0, sc_own + 1), tx(T_ELL, ipx + 1), vsx1, out);
+        for (int v = 0; v < NRV; ++v) QL[v] = yb[FXI(px + v * XC + yo, n_xb)];
+        rec_ld(k, NXF + ly * TX + lx, r);
+        face_flux(1, QL, ay, r, efv, out);
 #pragma unroll
-          for (int v = 0; v < NRV; ++v) stv(&rfx[FXI((v * NFX + fx + 1) * GS + g0, n_rfx)], out[v]);
-        }
+        for (int v = 0; v < NRV; ++v) yb[FXI(px + v * XC + yo, n_xb)] = out[v];
       }
-      if (D == 3) {
-        const int fy = ly * TX + lx;
-        V QL[NRV], out[NRV];
-#pragma unroll
-        for (int v = 0; v < NRV; ++v) QL[v] = ldv(&rby[FXI((v * NFY + fy) * GS + g0, n_rby)]);
-        rad_face_v(1, QL, ay, chi_v(s0, sc_own - PX), chi0, ty(T_ELL, bc_pad(gy)), vsy, out);
-#pragma unroll
-        for (int v = 0; v < NRV; ++v) stv(&rfy[FXI((v * NFY + fy) * GS + g0, n_rfy)], out[v]);
-        if (NGL == 1 && ly == TY - 1) {
-          V QR[NRV];
-#pragma unroll
-          for (int v = 0; v < NRV; ++v) QR[v] = ldv(&ray[FXI((v * TX + lx) * GS + g0, n_ray)]);
-          rad_face_v(1, by, QR, chi0, chi_v(s0, sc_own + PX), ty(T_ELL, bc_pad(gy + 1)), vsy1, out);
-#pragma unroll
-          for (int v = 0; v < NRV; ++v) stv(&rfy[FXI((v * NFY + fy + TX) * GS + g0, n_rfy)], out[v]);
-        }
-      }
-      if (D >= 2) {
-        if (SCAR) {
-#pragma unroll
-          for (int v = 0; v < NRV; ++v) bm0[v] = ldv(car(k, 0, v));
-        }
-        rad_face_v(MD, bm0, am1, chi0, chi_v((k + 1) & 3, sc_own), ell_m, vsm, rfm_new);
-        if (SCAR) {
-#pragma unroll
-          for (int v = 0; v < NRV; ++v) stv(car(k + 1, 1, v), rfm_new[v]);
-        }
+      if constexpr (D >= 2) {
+        rec_ld(k, NXF + NYF + tc, r);
+        face_flux(MD, bm0, am1, r, efv, rfm_new);
       }
     }
-    // two groups per lane: the row's face TX (between the tile's last cell and the halo cell TX),
-    // one group per lane of the NGL cells nearest the upper edge: left state from the face-state
-    // buffer, right state from the halo reconstruction, the contact speed of the gas face
-    if (NGL > 1 && lx >= TX - NGL) {
-      const int h = (lx - (TX - NGL)) * GL + lane;
-      if (h < G) {
-        const int fT = ly * (TX + 1) + TX;  // face TX of row ly
-        const int sc1 = scell(TX - 1, ly);
-        const int xl = x0 + TX - 1;         // the tile's last cell of the row
-        R QL[NRV], QR[NRV], out[NRV];
+    // the tile's upper faces, one task per row (column) and lane
+    if (task_c) {
+      const bool isx = D < 3 || ct < n1;
+      const int e = isx ? ct : ct - n1;
+      const int c = div_gl(e), ln = e - c * GL;
+      V* const p = isx ? xb + FXI(px + (c * (TX + 1) + TX) * GL + ln, n_xb) : yb + FXI(px + TC * GL + e, n_xb);
+      const V* const pr = isx ? xr + FXI(e, n_xr) : yr + FXI(e, n_yr);
+      const int sr = isx ? n1 : n2;
+      V QL[NRV], QR[NRV], out[NRV];
+      R r[4];
 #pragma unroll
-        for (int v = 0; v < NRV; ++v) {
-          QL[v] = rbx[FXI((v * NFX + fT) * GS + h, n_rbx)];
-          QR[v] = rax[FXI((v * TY + ly) * GS + h, n_rax)];
-        }
-        const R eh = R(sgc->efac_of(h, R(0)));
-        const R chiL = pk[FXI((s0 * 2) * PC + sc1, n_pk)] * eh + pk[FXI((s0 * 2 + 1) * PC + sc1, n_pk)];
-        const R chiR = pk[FXI((s0 * 2) * PC + sc1 + 1, n_pk)] * eh + pk[FXI((s0 * 2 + 1) * PC + sc1 + 1, n_pk)];
-        R vsT = R(0);
-        if (xl < nx) {
-          if constexpr (D <= 2) vsT = sgf[((k & 1) * TC + ly * TX + TX - 1) * LY::NGF + 1];
-          else vsT = gface(0, NG, ((uint32_t)k * ny + gyc) * fx_nx + (uint32_t)xl + 1);
-        }
-        rad_face(0, QL, QR, chiL, chiR, tx(T_ELL, bc_pad(xl) + 1), vsT, out);
+      for (int v = 0; v < NRV; ++v) { QL[v] = p[v * XC]; QR[v] = pr[v * sr]; }
+      rec_ld(k, isx ? c * (TX + 1) + TX : NXF + TY * TX + c, r);
+      if (D < 3 || isx) face_flux(0, QL, QR, r, ef_of(ln), out);
+      else face_flux(D == 3 ? 1 : 0, QL, QR, r, ef_of(ln), out);
 #pragma unroll
-        for (int v = 0; v < NRV; ++v) rfx[FXI((v * NFX + fT) * GS + h, n_rfx)] = out[v];
+      for (int v = 0; v < NRV; ++v) p[v * XC] = out[v];
+    }
+    cp_async_wait_all();
+    if (more && (fin_xy || k + 3 >= nmarch)) {
+      finish_own(k + 3);
+      finish_halo(k + 1);
+    }
+    __syncthreads();
+    // ---- D
+    if (cell_in) {
+      V Q0[NRV], U[NRV];
+      own_ld(k, Q0);
+      const uint32_t cidx = cxy + (uint32_t)k * pcells;
+      V xm[NRV], xp[NRV], ym[NRV], yp[NRV];
+#pragma unroll
+      for (int v = 0; v < NRV; ++v) {
+        xm[v] = xb[FXI(px + v * XC + xo, n_xb)];
+        xp[v] = xb[FXI(px + v * XC + xo + GL, n_xb)];
+        if (D == 3) {
+          ym[v] = yb[FXI(px + v * XC + yo, n_xb)];
+          yp[v] = yb[FXI(px + v * XC + yo + TX * GL, n_xb)];
+        }
       }
-    }
-    // 3-d, two groups per lane: the y face TY of each column (between the tile's last row and the
-    // halo row TY), one group per lane of the NGL rows nearest the upper y edge (its left state
-    // and flux share their shared-memory slot; only these threads touch it)
-    if (D == 3 && NGL > 1 && ly >= TY - NGL) {
-      const int h = (ly - (TY - NGL)) * GL + lane;
-      if (h < G) {
-        const int fT = TY * TX + lx;        // face TY of column lx
-        const int sc1 = scell(lx, TY - 1);
-        const int yl = y0 + TY - 1;         // the tile's last row
-        R QL[NRV], QR[NRV], out[NRV];
-#pragma unroll
-        for (int v = 0; v < NRV; ++v) {
-          QL[v] = rby[FXI((v * NFY + fT) * GS + h, n_rby)];
-          QR[v] = ray[FXI((v * TX + lx) * GS + h, n_ray)];
-        }
-        const R eh = R(sgc->efac_of(h, R(0)));
-        const R chiL = pk[FXI((s0 * 2) * PC + sc1, n_pk)] * eh + pk[FXI((s0 * 2 + 1) * PC + sc1, n_pk)];
-        const R chiR = pk[FXI((s0 * 2) * PC + sc1 + PX, n_pk)] * eh + pk[FXI((s0 * 2 + 1) * PC + sc1 + PX, n_pk)];
-        const R vsT = (yl < ny && gx < nx) ? gface(1, NG, ((uint32_t)k * (ny + 1) + (uint32_t)(yl + 1)) * nx + gxc)
-                                           : R(0);
-        rad_face(1, QL, QR, chiL, chiR, ty(T_ELL, bc_pad(yl) + 1), vsT, out);
-#pragma unroll
-        for (int v = 0; v < NRV; ++v) rfy[FXI((v * NFY + fT) * GS + h, n_rfy)] = out[v];
-      }
-    }
-    if constexpr (D == 2 && NGL > 1) {
-      // C | D hand-off in 2-d with two groups per lane: a cell's update needs the flux through
-      // its upper x face, computed by the next cell, which is in the next warp only at a warp's
-      // last cell.  So each warp signals the warp below it (named barrier w) and waits only for
-      // the warp above it (named barrier w+1), instead of a block barrier.  What a block barrier
-      // also ordered is ordered here as well: a warp restages its cells' opacity factors of this
-      // plane (read in C by the next cell) only after the warp above has passed C, and the halo
-      // opacity factors are staged by the warp that reads them.  (At one group per lane, three
-      // blocks per SM at 80 registers, the barrier indices cost spills: the block barrier stays.)
-      constexpr int NW = NTH / 32;
-      const int w = tid >> 5;
-      __syncwarp();
-      if (w > 0) bar_arrive(w, 64);
-      if (w < NW - 1) bar_wait(w + 1, 64);
-    } else {
-      __syncthreads();
-    }
-    // ---- D: update: divergence, RK combine, store
-    {
-      const R gown = gas_at(s0, gvar, sc_own);  // own gas variable of plane k (lanes < NG)
-      rad_v(s0, sc_own, Q0);  // (not live across C)
-      const int ipy = gy + 2;
-      R fyl = R(0), fyr = R(0);
-      if (D == 3) { fyl = ty(T_FL, ipy); fyr = ty(T_FR, ipy); }
-      const int fxa = ly * (TX + 1) + lx;
-      const int fya = ly * TX + lx;
-      const uint32_t cidx = (D == 1) ? (uint32_t)gx
-                          : (D == 2) ? (uint32_t)k * nx + gx
-                                     : ((uint32_t)k * ny + gy) * nx + gx;
-      const R dt = KR.dt;
-      const bool stage2 = A.base != nullptr;
-      // geometric sources <Gamma^l_jk> T^k_l of the stage's input state (Eq. 9; Appendix D)
-      R hq[3] = {R(1), R(1), R(1)}, gsrc = R(0);
-      V rsrc[NRV];
-#pragma unroll
-      for (int v = 0; v < NRV; ++v) rsrc[v] = V(R(0));
-      if (sph) {
+      if constexpr (SPH) {
+        // area/volume factors of the two face pairs per flux class (half: twice the flux is
+        // carried), and the geometric sources <Gamma^l_jk> T^k_l of the stage's input state (Eq. 9;
+        // Appendix D)
         const int ipm = bc_pad(k);
-        hq[0] = hfac(0, gx, k);
-        hq[1] = hfac(1, gx, k);
+        const R hq[2] = {hfac(0, gx, k), hfac(1, gx, k)};
         const R g111 = tx(T_GA, ipx), g221 = tx(T_GB, ipx), g122 = tx(T_GC, ipx);
         const R g222 = tm(T_GA, ipm), g332 = tm(T_GB, ipm);
-        R gc[NG];
-#pragma unroll
-        for (int v = 0; v < NG; ++v) gc[v] = __shfl_sync(0xffffffffu, gown, v, GL);
-        const R rho = gc[0], irho = frcp(rho);
-        const R v1 = gc[1] * irho * frcp(hq[0]), v2 = gc[2] * irho * frcp(hq[1]);
-        const R p = KR.gm1 * (gc[NG - 1] - R(0.5) * rho * (v1 * v1 + v2 * v2));
+        const R rho = A.in[FXI(cidx, A.n_state)], irho = frcp(rho);
+        const R v1 = A.in[FXI(ncell + cidx, A.n_state)] * irho * frcp(hq[0]), v2 = A.in[FXI(2 * ncell + cidx, A.n_state)] * irho * frcp(hq[1]);
         const R r12 = hq[0] * frcp(hq[1]), r21 = hq[1] * frcp(hq[0]);
-        if (gvar == 1) gsrc = g111 * (rho * v1 * v1 + p) + g221 * (rho * v2 * v2 + p) + g221 * p;
-        if (gvar == 2)
-          gsrc = g122 * (rho * v1 * v2 * r12) + g221 * (rho * v1 * v2 * r21) + g222 * (rho * v2 * v2 + p) + g332 * p;
-        const R c2 = KR.c * KR.c;
-        R s1[NGL], s2[NGL];
-#pragma unroll
-        for (int j = 0; j < NGL; ++j) {
-          R Qj[NRV], Pd[3], P01;
-#pragma unroll
-          for (int v = 0; v < NRV; ++v) Qj[v] = vget(Q0[v], j);
-          m1_full<R, D>(KR.c, Qj[0], Qj + 1, Pd, P01);
-          const R R11 = c2 * Pd[0] + v1 * Qj[1], R22 = c2 * Pd[1] + v2 * Qj[2], R33 = c2 * Pd[2];
-          const R R21 = (c2 * P01 + v2 * Qj[1]) * r12, R12 = (c2 * P01 + v1 * Qj[2]) * r21;
-          s1[j] = g111 * R11 + g221 * R22 + g221 * R33;
-          s2[j] = g122 * R21 + g221 * R12 + g222 * R22 + g332 * R33;
-        }
-        rsrc[1] = vpair(s1[0], s1[NGL - 1], V());
-        rsrc[2] = vpair(s2[0], s2[NGL - 1], V());
-      }
-      // gas: lane v < NG updates variable v
-      const R ug = fv_update(gFp, gAp, gFm, gAm, gown, gsrc, dt, stage2, stage2 ? base_g() : R(0), KR.alpha, KR.beta);
-      // The interaction runs in a kernel of its own (couple_kernel, couple64_kernel: one thread
-      // per cell, so that each FP64 instruction of the Newton iteration serves 32 cells and its
-      // scalar steps are not repeated by the group lanes); this kernel stores the state after the
-      // explicit update and the RK combination.
-      V U[NRV];  // E, F_q of the lane's groups
-#pragma unroll
-      for (int v = 0; v < NRV; ++v) U[v] = V(R(0));
-      if (h0 && cell_in) {
+        V P0[D], P1[D];
+        m1_c2row<D>(KL, Q0[0], Q0 + 1, 0, P0);
+        m1_c2row<D>(KL, Q0[0], Q0 + 1, 1, P1);
+        // c^2 P33 is the closure's diagonal part: the trace c^2 E less the other two entries would
+        // cancel for a beam, so it is formed as P11 less its beam part
+        const V P33 = m1_c2perp<D>(KL, Q0[0], Q0 + 1);
+        const V R11 = vfma(V(v1), Q0[1], P0[0]), R22 = vfma(V(v2), Q0[D >= 2 ? 2 : 0], P1[D - 1]);
+        const V R21 = vfma(V(v2), Q0[1], P0[D - 1]) * r12, R12 = vfma(V(v1), Q0[D >= 2 ? 2 : 0], P0[D - 1]) * r21;
+        V src[3] = {V(R(0)), R11 * g111 + (R22 + P33) * g221, R21 * g122 + R12 * g221 + R22 * g222 + P33 * g332};
+        const int eL[3] = {T_FL, T_FL1, T_FL2}, eR[3] = {T_FR, T_FR1, T_FR2}, eX[3] = {T_XS, T_X1, T_X2};
 #pragma unroll
         for (int v = 0; v < NRV; ++v) {
-          const int c = v <= 2 ? v : 0;
-          V Fp[D], Fm[D];
-          R Ap[D], Am[D];
-          Fp[0] = ldv(&rfx[FXI((v * NFX + fxa + 1) * GS + g0, n_rfx)]); Ap[0] = fx_r[c];
-          Fm[0] = ldv(&rfx[FXI((v * NFX + fxa) * GS + g0, n_rfx)]); Am[0] = fx_l[c];
-          if (D == 3) {
-            Fp[1] = ldv(&rfy[FXI((v * NFY + fya + TX) * GS + g0, n_rfy)]); Ap[1] = fyr;
-            Fm[1] = ldv(&rfy[FXI((v * NFY + fya) * GS + g0, n_rfy)]); Am[1] = fyl;
-          }
-          if (D >= 2) {
-            Fp[D - 1] = SCAR ? ldv(car(k + 1, 1, v)) : rfm_new[v]; Ap[D - 1] = fm_r[c];
-            Fm[D - 1] = SCAR ? ldv(car(k, 1, v)) : rfm_old[v]; Am[D - 1] = fm_l[c];
-          }
-          const V cov = (sph && v >= 1) ? Q0[v] * hq[v - 1] : Q0[v];  // covariant F
-          U[v] = fv_update(Fp, Ap, Fm, Am, cov, rsrc[v], dt, stage2, stage2 ? ldv(&base_r(v, 0)) : V(R(0)),
+          const V Fp[2] = {xp[v], rfm_new[v]}, Fm[2] = {xm[v], rfm_old[v]};
+          const R xs = R(0.5) * tm(eX[v], ipm), ms = R(0.5) * tx(eX[v], ipx);
+          const R Ap[2] = {tx(eR[v], ipx) * xs, tm(eR[v], ipm) * ms};
+          const R Am[2] = {tx(eL[v], ipx) * xs, tm(eL[v], ipm) * ms};
+          const V cov = v >= 1 ? Q0[v] * hq[v - 1] : Q0[v];  // covariant F
+          U[v] = fv_update(Fp, Ap, Fm, Am, cov, src[v], KR.dt, stage2, stage2 ? sbase[FXI(v * NT + tid, n_base)] : V(R(0)),
                            KR.alpha, KR.beta);
+        }
+      } else {
+#pragma unroll
+        for (int v = 0; v < NRV; ++v) {
+          V u = Q0[v] - net_update<D>(xp[v], xm[v], yp[v], ym[v], rfm_new[v], rfm_old[v], KL.hdt);
+          if (stage2) u = vfma(KL.alpha, sbase[FXI(v * NT + tid, n_base)], u * KL.beta);
+          U[v] = u;
         }
       }
       // budgets (reading R13): the outward fluxes through this cell's faces on non-periodic
       // boundaries, times the face area (the area/volume factor times the cell volume) and the
-      // stage's weight, added to one of BUDGET_SLOTS rows of accumulators (summed when read, so
-      // that few blocks add to the same address).  The face values are read again (gas: the
-      // staged face values, or global memory in 3-d; radiation: the face fluxes in shared memory).
-      if (BUD && A.budget != nullptr && cell_in) {
+      // stage's weight, added to one of BUDGET_SLOTS rows of accumulators (summed when read)
+      if (BUD && A.budget != nullptr) {
         const bool xl = gx == 0 && g.bc_lo[0] != 1, xh = gx == nx - 1 && g.bc_hi[0] != 1;
         const bool yl = D == 3 && gy == 0 && g.bc_lo[1] != 1, yh = D == 3 && gy == ny - 1 && g.bc_hi[1] != 1;
-        const bool ml = D >= 2 && k == 0 && g.bc_lo[MD] != 1;
-        const bool mh = D >= 2 && k == nmarch - 1 && g.bc_hi[MD] != 1;
+        const bool ml = D >= 2 && k == 0 && g.bc_lo[MD] != 1, mh = D >= 2 && k == nmarch - 1 && g.bc_hi[MD] != 1;
         if (xl || xh || yl || yh || ml || mh) {
+          const int ipm = bc_pad(k);
           double vol = (double)tx(T_VOL, ipx);
           if (D == 3) vol *= (double)ty(T_VOL, ipy);
-          if (D >= 2) vol *= (double)tm(T_VOL, bc_pad(k));
-          const double bs = vol * A.bw_flux;
-          const unsigned blin = blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z);
-          double* const bud = A.budget + (size_t)(blin % BUDGET_SLOTS) * NBUDGET;
-          if (lane < NG) {
-            R f[6];
-            if constexpr (D <= 2) {
-#pragma unroll
-              for (int c = 0; c < GFV; ++c) f[c] = gfs(k, 3 + GFV * lane + c);
-            } else {
-              const uint32_t fxk = face_x(k), fyk = face_y3(k);
-              f[0] = gface(0, gvar, fxk);
-              f[1] = gface(0, gvar, fxk + 1);
-              f[2] = gface(MD, gvar, face_m(k));
-              f[3] = gface(MD, gvar, face_m(k + 1));
-              f[4] = gface(1, gvar, fyk);
-              f[5] = gface(1, gvar, fyk + nx);
-            }
-            double o = 0.0;
-            if (xh) o += (double)(f[1] * cls(fx_r));
-            if (xl) o -= (double)(f[0] * cls(fx_l));
-            if (D >= 2 && mh) o += (double)(f[3] * cls(fm_r));
-            if (D >= 2 && ml) o -= (double)(f[2] * cls(fm_l));
-            if (D == 3 && yh) o += (double)(f[5] * fyr);
-            if (D == 3 && yl) o -= (double)(f[4] * fyl);
-            if (o != 0.0) atomicAdd(bud + (gvar == NG - 1 ? 4 : gvar), o * bs);
-          }
+          if (D >= 2) vol *= (double)tm(T_VOL, ipm);
+          const double bs = 0.5 * vol * A.bw_flux;  // (twice the flux is carried)
+          double* const bud = A.budget + (size_t)(blockIdx.x % BUDGET_SLOTS) * NBUDGET;
+          const int eL[3] = {T_FL, T_FL1, T_FL2}, eR[3] = {T_FR, T_FR1, T_FR2}, eX[3] = {T_XS, T_X1, T_X2};
 #pragma unroll
           for (int v = 0; v < NRV; ++v) {
-            const int c = v <= 2 ? v : 0;
+            const int c = SPH ? v : 0;
+            const R sx = SPH ? tm(eX[c], ipm) : R(1), sm_ = SPH ? tx(eX[c], ipx) : R(1);
             double o = 0.0;
 #pragma unroll
-            for (int j = 0; j < NGL; ++j) {
-              if (!hasj[j]) continue;
-              const int gg = gj[j];
-              if (xh) o += (double)(rfx[FXI((v * NFX + fxa + 1) * GS + gg, n_rfx)] * fx_r[c]);
-              if (xl) o -= (double)(rfx[FXI((v * NFX + fxa) * GS + gg, n_rfx)] * fx_l[c]);
-              if (D == 3 && yh) o += (double)(rfy[FXI((v * NFY + fya + TX) * GS + gg, n_rfy)] * fyr);
-              if (D == 3 && yl) o -= (double)(rfy[FXI((v * NFY + fya) * GS + gg, n_rfy)] * fyl);
-              if (D >= 2 && mh) o += (double)((SCAR ? car(k + 1, 1, v)[j] : vget(rfm_new[v], j)) * fm_r[c]);
-              if (D >= 2 && ml) o -= (double)((SCAR ? car(k, 1, v)[j] : vget(rfm_old[v], j)) * fm_l[c]);
+            for (int j = 0; j < W; ++j) {
+              if (j == 1 && !h1) continue;
+              if (xh) o += (double)(vget(xp[v], j) * (tx(eR[c], ipx) * sx));
+              if (xl) o -= (double)(vget(xm[v], j) * (tx(eL[c], ipx) * sx));
+              if (D == 3 && yh) o += (double)(vget(yp[v], j) * ty(T_FR, ipy));
+              if (D == 3 && yl) o -= (double)(vget(ym[v], j) * ty(T_FL, ipy));
+              if (D >= 2 && mh) o += (double)(vget(rfm_new[v], j) * (tm(eR[c], ipm) * sm_));
+              if (D >= 2 && ml) o -= (double)(vget(rfm_old[v], j) * (tm(eL[c], ipm) * sm_));
             }
             if (o != 0.0) {
               if (v == 0) {
@@ -1392,58 +1270,39 @@ stage_kernel(const __grid_constant__ StageArgs<R> A) {
           }
         }
       }
-      // recording for the adjoint: the pre-interaction state
-      if (A.pre_out != nullptr && cell_in) {
-        if (lane < NG) A.pre_out[FXI(lane * ncell + cidx, A.n_state)] = ug;
+      if (more_out) {
+        // recording for the adjoint: the pre-interaction state
+        if (A.pre_out != nullptr) {
+          const uint32_t o = NG * ncell + cidx * G + g0;
 #pragma unroll
-        for (int j = 0; j < NGL; ++j) {
-          if (hasj[j]) {
-#pragma unroll
-            for (int v = 0; v < NRV; ++v) A.pre_out[FXI(NG * ncell + (v * ncell + cidx) * G + gj[j], A.n_state)] = vget(U[v], j);
+          for (int v = 0; v < NRV; ++v) {
+            A.pre_out[FXI(o + v * vstride, A.n_state)] = vget(U[v], 0);
+            if (h1) A.pre_out[FXI(o + v * vstride + 1, A.n_state)] = vget(U[v], W - 1);
           }
         }
-      }
-      // objective: energy flux through the upper x boundary face of the row, times its area
-      if (A.phi_out != nullptr && cell_in && gx == nx - 1) {
-        const uint32_t row = D == 1 ? 0u : D == 2 ? (uint32_t)k : (uint32_t)k * ny + gy;
-#pragma unroll
-        for (int j = 0; j < NGL; ++j)
-          if (hasj[j]) A.phi_out[FXI(row * G + gj[j], (uint32_t)(D >= 2 ? ny : 1) * (D >= 3 ? nz : 1) * G)] = rfx[FXI((0 * NFX + fxa + 1) * GS + gj[j], n_rfx)] * A.phi_area;
-      }
-      if (cell_in) {
-        R chk = R(0);  // a NaN or inf anywhere in the cell's outputs makes this sum non-finite
-        if (lane < NG) {
-          A.out[FXI(lane * ncell + cidx, A.n_state)] = ug;
-          chk += ug;
+        // objective: energy flux through the upper x boundary face of the row, times its area
+        if (A.phi_out != nullptr && gx == nx - 1) {
+          const uint32_t row = D == 1 ? 0u : D == 2 ? (uint32_t)k : (uint32_t)k * ny + gy;
+          const uint32_t n_phi = (uint32_t)(D >= 2 ? ny : 1) * (D >= 3 ? nz : 1) * G;
+          (void)n_phi;
+          A.phi_out[FXI(row * G + g0, n_phi)] = R(0.5) * vget(xp[0], 0) * A.phi_area;
+          if (h1) A.phi_out[FXI(row * G + g0 + 1, n_phi)] = R(0.5) * vget(xp[0], W - 1) * A.phi_area;
         }
-#pragma unroll
-        for (int j = 0; j < NGL; ++j) {
-          if (hasj[j]) {
-#pragma unroll
-            for (int v = 0; v < NRV; ++v) {
-              const R val = vget(U[v], j);
-              A.out[FXI(NG * ncell + (v * ncell + cidx) * G + gj[j], A.n_state)] = val;
-              chk += val * R(0);
-            }
-          }
-        }
-        unsigned stbits = 0;
-        if (!isfinite(chk)) stbits |= ST_NONFINITE;
-        if (stbits) atomicOr(A.status, stbits);
       }
-    }
-    // stage the stage-2 base of plane k+1 (its buffer was last read above, by this thread)
-    if (k + 1 < kend) {
-      issue_base(k + 1);
-      cp_async_commit();
-    }
-    // slide the march window (2-d: the carry lives in shared memory)
-    if (!SCAR) {
+      V chk = V(R(0));  // a NaN or inf anywhere in the outputs makes this sum non-finite
+      const uint32_t row = (uint32_t)k * pstride;
 #pragma unroll
       for (int v = 0; v < NRV; ++v) {
-        bm0[v] = bm1[v];
-        rfm_old[v] = (D >= 2) ? rfm_new[v] : V(R(0));
+        st_global_lane(FXP(const_cast<R*>(plane_at(A.out, v, row)), toff, vstride - row), U[v], vec, h1);
+        chk = vfma(U[v], V(R(0)), chk);
       }
+      if (!isfinite(vget(chk, 0)) || (h1 && !isfinite(vget(chk, W - 1)))) atomicOr(A.status, ST_NONFINITE);
+    }
+    if (PB == 1) __syncthreads();  // the next plane's face states overwrite these fluxes
+#pragma unroll
+    for (int v = 0; v < NRV; ++v) {
+      if (D >= 2) bm0[v] = bm1[v];
+      rfm_old[v] = rfm_new[v];
     }
   }
 }

@@ -24,6 +24,14 @@ enum : unsigned {
   ST_BOUNDS = 8u,     // an index fell outside its buffer (index checks of the debug build)
 };
 
+// Tile of the stage kernel's radiation blocks (see stage_kernel): cells per tile, lanes per cell,
+// threads per block, tiles per direction, radiation blocks of the launch, 8-byte alignment of the
+// lanes' pairs in global memory, gas cells per thread, and ceil(2^32 / gl).
+struct RadTile {
+  int tx, ty, gl, nth, ntx, nty, nrad, vec, gpt;
+  unsigned mgl;
+};
+
 // Kernel-side description of the grid (passed by value to every launch).
 struct DevGrid {
   int D, G;
