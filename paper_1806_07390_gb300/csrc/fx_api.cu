@@ -19,6 +19,7 @@
 #include "fx_vterms.cuh"
 #include "fx_layers.cuh"
 #include "fx_launch.h"
+#include "fx_planck.h"
 
 using namespace fx;
 
@@ -128,6 +129,7 @@ struct fx_grid {
   int ptab_nu = 0;
   float ptab_u0 = 0.0f;
   size_t off_ptab = 0;
+  size_t off_petab = 0;           // FP64 Planck edge table (FP64 form only)
   size_t off_hrow = 0;            // FP64 scale-factor rows T_HA, T_HB per direction (curvilinear)
   size_t off_faces = 0;           // gas face buffer [dir][NG+1 (+D-1 with vterms)][faces of dir]
   size_t off_frec = 0;            // face records of the radiation fluxes [dir][faces of dir][4]
@@ -727,6 +729,7 @@ StageArgs<R> stage_args(fx_grid* h) {
   a.ptab.si = ptab_node_major(h) ? h->P.ngroups : 1;
   a.ptab.sg = ptab_node_major(h) ? 1 : h->ptab_nu;
   a.pk = h->pk;
+  a.pk.petab = h->elem == 8 ? reinterpret_cast<const double*>(h->ws + h->off_petab) : nullptr;
   a.status = reinterpret_cast<unsigned*>(h->ws + h->off_status);
 #ifdef FX_BOUNDS_CHECK
   a.ptab.n = (int)h->ptab.size();
@@ -1284,6 +1287,8 @@ fx_status fx_grid_create(const fx_params* params, fx_grid** out, size_t* workspa
   }
   h->off_vtc = off; off = align_up(off + sizeof(VtConst));
   h->off_ptab = off; off = align_up(off + h->ptab.size() * sizeof(float4));
+  h->off_petab = off;
+  if (h->elem == 8) off = align_up(off + planck_edge_table().size() * sizeof(double));
   {
     int64_t fo = 0;
     for (int d = 0; d < P.dims; ++d) {
@@ -1630,6 +1635,11 @@ fx_status fx_bind_workspace(fx_grid* h, void* dev_ptr, size_t bytes, void* cuda_
     if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
   }
   if (e != cudaSuccess) return cuda_fail(h, e, "Planck table upload");
+  if (h->elem == 8) {
+    const std::vector<double>& pt = planck_edge_table();
+    e = cudaMemcpyAsync(h->ws + h->off_petab, pt.data(), pt.size() * sizeof(double), cudaMemcpyHostToDevice, h->stream);
+    if (e != cudaSuccess) return cuda_fail(h, e, "Planck edge table upload");
+  }
   e = cudaMemcpyAsync(h->ws + h->off_gc, &h->gc, sizeof(GroupConst), cudaMemcpyHostToDevice, h->stream);
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(h->ws + h->off_vtc, &h->vtc, sizeof(VtConst), cudaMemcpyHostToDevice, h->stream);

@@ -1,5 +1,5 @@
 // Cell-local implicit matter-radiation interaction of the FP64 state as a kernel of its own, one
-// thread per cell (Sec. 5.3: the backward-Euler group update of Eq. 25 inside the Newton iteration
+// thread per cell on all but the smallest grids (Sec. 5.3: the backward-Euler group update of Eq. 25 inside the Newton iteration
 // on T of Eqs. 26-27, the gas energy by conservation, then the flux absorption of Eq. 28 and its
 // momentum and energy feedback, Eqs. 31-32; readings R10-R12).
 //
@@ -13,10 +13,16 @@
 // instruction serves 32 cells, group sums are sequential additions, and the scalar steps run
 // once per cell.
 //
+// Bound by the FP64 pipe (87 % busy), so the band edges come from a table of polynomials instead of
+// the power and exponential series (planck_edge_tab: 20 operations an edge), reciprocals are a
+// hardware seed with one third-order step instead of divisions, and a group takes 36 operations an
+// evaluation: 512^2 x 16 groups 1.90 -> 0.97 ms per launch, 217 -> 120 FP64 operations per group.
+//
 // The stage kernel leaves the state after the explicit update and RK combination in its output;
 // this kernel updates that state in place.  The decisions (Newton step and its tests, the
 // backtracking line search, the bisection fallback and its bracket) are those of the oracle's
-// cell interaction, in the same order; the group energies of the accepted temperature are the
+// cell interaction, in the same order (with several lanes per cell, group sums are formed per lane
+// and then over the lanes); the group energies of the accepted temperature are the
 // last evaluation's, linearised to T + dT at convergence as the FP32 forms do (exact to O(dT^2)).
 #pragma once
 #include <cuda_runtime.h>
@@ -25,7 +31,15 @@
 
 namespace fx {
 
-constexpr int CPL64_THREADS = 128;  // cells (threads) per block of couple64_kernel
+constexpr int CPL64_THREADS = 128;  // threads per block of couple64_kernel
+
+// Lanes per cell of couple64_kernel.  One lane per cell does the least FP64 work: every operation
+// serves 32 cells, and neighbouring groups share their edge.  A grid whose cells at one lane each
+// would leave a multiprocessor with fewer than four warps is bound by the latency of a cell's group
+// loop instead: eight lanes share it (512 cells x 12 groups: 0.117 -> 0.031 ms
+// per launch, with the edge table).
+constexpr int64_t CPL64_SPLIT_CELLS = 152 * 128;
+constexpr int CPL64_SPLIT_LANES = 8;
 
 // Rows of couple64_kernel's shared memory per cell: E^- (then the new E), the last evaluation's
 // E_g and dE_g/dT (then the F_q).
@@ -33,8 +47,8 @@ constexpr int couple64_rows(int D) { return 1 + D > 3 ? 1 + D : 3; }
 
 // Dynamic shared memory of couple64_kernel: couple64_rows(D) rows per cell of G + 1 doubles (the
 // pad spreads the threads' row reads over the banks).
-template <int D> inline size_t couple64_smem_bytes(int G) {
-  return (size_t)couple64_rows(D) * CPL64_THREADS * (size_t)(G + 1) * sizeof(double);
+template <int D> inline size_t couple64_smem_bytes(int G, int cells) {
+  return (size_t)couple64_rows(D) * cells * (size_t)(G + 1) * sizeof(double);
 }
 
 // Copy between a contiguous run of nc*G doubles in global memory (nc cells of G groups) and the
@@ -42,11 +56,11 @@ template <int D> inline size_t couple64_smem_bytes(int G) {
 // aligned and G is even (a double2 then never straddles two rows).
 template <bool TO_SHARED>
 __device__ __forceinline__ void stage_rows64(double* gmem, double* rows, int nc, int G, int RS) {
-  const int t = threadIdx.x;
+  const int t = threadIdx.x, nt = (int)blockDim.x;
   if (G % 2 == 0 && (reinterpret_cast<uintptr_t>(gmem) & 15) == 0) {
     const int G2 = G / 2, tot = nc * G2;
     double2* g2 = reinterpret_cast<double2*>(gmem);
-    for (int e = t; e < tot; e += CPL64_THREADS) {
+    for (int e = t; e < tot; e += nt) {
       const int row = e / G2, c2 = e - row * G2;
       double* r = rows + row * RS + 2 * c2;
       if (TO_SHARED) {
@@ -59,7 +73,7 @@ __device__ __forceinline__ void stage_rows64(double* gmem, double* rows, int nc,
     }
   } else {
     const int tot = nc * G;
-    for (int e = t; e < tot; e += CPL64_THREADS) {
+    for (int e = t; e < tot; e += nt) {
       const int row = e / G, gg = e - row * G;
       if (TO_SHARED) rows[row * RS + gg] = gmem[e];
       else gmem[e] = rows[row * RS + gg];
@@ -67,8 +81,18 @@ __device__ __forceinline__ void stage_rows64(double* gmem, double* rows, int nc,
   }
 }
 
-template <int D>
-__global__ void __launch_bounds__(CPL64_THREADS) couple64_kernel(StageArgs<double> A) {
+// Sum over the L lanes of a cell (every lane gets the same bits: the butterfly adds the same pairs).
+template <int L> __device__ __forceinline__ double cell_sum(double v) {
+  if (L > 1) {
+    const unsigned m = (L == 32 ? 0xffffffffu : ((1u << L) - 1u)) << ((threadIdx.x & 31) & ~(L - 1));
+#pragma unroll
+    for (int o = L / 2; o >= 1; o >>= 1) v += __shfl_xor_sync(m, v, o);
+  }
+  return v;
+}
+
+template <int D, int L>
+__global__ void __launch_bounds__(CPL64_THREADS, 4) couple64_kernel(const __grid_constant__ StageArgs<double> A) {
   constexpr int NG = 2 + D, NRV = 1 + D;
   const DevGrid& g = A.g;
   const int G = g.G;
@@ -78,15 +102,16 @@ __global__ void __launch_bounds__(CPL64_THREADS) couple64_kernel(StageArgs<doubl
   double* const srow = reinterpret_cast<double*>(smem_raw);  // [rows][CPL64_THREADS][G + 1]
   __shared__ double s_ef[MAXG], s_ed[MAXG + 1];
   const int RS = G + 1;
-  const int t = threadIdx.x;
-  const uint32_t c0 = blockIdx.x * (uint32_t)CPL64_THREADS;
-  const int nc = (int)min((uint32_t)CPL64_THREADS, ncell - c0);
+  const int CPB = (int)blockDim.x / L;  // cells per block
+  const int t = (int)threadIdx.x / L, ln = (int)threadIdx.x % L;  // cell of the block, lane of the cell
+  const uint32_t c0 = blockIdx.x * (uint32_t)CPB;
+  const int nc = (int)min((uint32_t)CPB, ncell - c0);
   const bool act = t < nc;
   const uint32_t cid = c0 + (uint32_t)t;
 
-  for (int j = t; j <= G; j += CPL64_THREADS) {
+  for (int j = threadIdx.x; j <= G; j += (int)blockDim.x) {
     if (j < G) s_ef[j] = A.gc->efac[j];
-    s_ed[j] = A.gc->edge[j];
+    s_ed[j] = 16.0 * A.gc->edge[j];  // 16 eps: the edge table's argument is 16 eps / T
   }
   stage_rows64<true>(FXPR(A.out, (size_t)NG * ncell + (size_t)c0 * G, nc * G, A.n_state), srow, nc, G, RS);
   double rho = 1.0, m[3] = {0.0, 0.0, 0.0}, rhoe = 1.0;
@@ -110,8 +135,8 @@ __global__ void __launch_bounds__(CPL64_THREADS) couple64_kernel(StageArgs<doubl
   __syncthreads();
 
   double* const rE = srow + t * RS;                         // E^-, then the new E
-  double* const rEt = srow + (CPL64_THREADS + t) * RS;      // last evaluation: E_g
-  double* const rDt = srow + (2 * CPL64_THREADS + t) * RS;  // last evaluation: dE_g/dT
+  double* const rEt = srow + (CPB + t) * RS;      // last evaluation: E_g
+  double* const rDt = srow + (2 * CPB + t) * RS;  // last evaluation: dE_g/dT
   const bool work = act && g.couple;
   unsigned st = 0;
   double irho = 1.0, ke = 0.0, Tst = 0.0, K = 0.0, Sg = 0.0;
@@ -131,7 +156,7 @@ __global__ void __launch_bounds__(CPL64_THREADS) couple64_kernel(StageArgs<doubl
     double um = rhoe - ke;
     if (um < kn.u_floor) { um = kn.u_floor; rhoe = ke + um; st |= ST_FLOOR; }
     double Esum = 0.0, fadd = 0.0;
-    for (int j = 0; j < G; ++j) {
+    for (int j = ln; j < G; j += L) {
       double e = rE[j];
       if (e < kn.E_floor) {  // silent positivity floor (Wien tails)
         fadd += kn.E_floor - e;
@@ -140,7 +165,11 @@ __global__ void __launch_bounds__(CPL64_THREADS) couple64_kernel(StageArgs<doubl
       }
       Esum += e;
     }
-    if (A.budget != nullptr) s_floor[t] = fadd;
+    Esum = cell_sum<L>(Esum);
+    if (A.budget != nullptr) {
+      fadd = cell_sum<L>(fadd);
+      if (ln == 0) s_floor[t] = fadd;
+    }
     const double rcv = rho * kn.cv;
     const double Tm = um * frcp(rcv);
     K = kn.kappa0 * hpow(rho, g.kap_rho_h);
@@ -151,28 +180,30 @@ __global__ void __launch_bounds__(CPL64_THREADS) couple64_kernel(StageArgs<doubl
     auto eval = [&](double dl, double& r, double& dr) {
       const double T = Tm + dl, invT = frcp(T), T3 = T * T * T;
       const double kT = K * hpow(T, g.kap_T_h);
+      const double aT3 = aN * T3, aT4 = aT3 * T, ck = cdts * kT, hT = hh * invT;
       double s1 = 0.0, s2 = 0.0;
-      PlanckEdge<double> lo = planck_edge64(s_ed[0] * invT, A.pk.c64);
-#pragma unroll 1
-      for (int j = 0; j < G; ++j) {
-        const PlanckEdge<double> hi = planck_edge64(s_ed[j + 1] * invT, A.pk.c64);
+      PlanckEdge<double> lo;
+      if (L == 1) lo = planck_edge_tab(s_ed[0] * invT, A.pk.petab, A.pk.c64);
+#pragma unroll 2
+      for (int j = ln; j < G; j += L) {
+        if (L > 1) lo = planck_edge_tab(s_ed[j] * invT, A.pk.petab, A.pk.c64);
+        const PlanckEdge<double> hi = planck_edge_tab(s_ed[j + 1] * invT, A.pk.petab, A.pk.c64);
         const double I = planck_band(lo, hi);
-        const double B = aN * T3 * T * I;
-        const double dB = aN * T3 * (4.0 * I + (lo.w - hi.w));
-        const double tau = cdts * (kT * s_ef[j]);
-        const double dtau = tau * hh * invT;
-        const double inv = frcp(1.0 + tau);
+        const double B = aT4 * I;
+        const double dB = aT3 * fma(4.0, I, lo.w - hi.w);
+        const double tau = ck * s_ef[j];
+        const double inv = rcp_pos(1.0 + tau);
         const double Em = rE[j];
-        const double Eg = (Em + tau * B) * inv;
-        const double dEg = (tau * dB + dtau * (B - Eg)) * inv;
+        const double Eg = fma(tau, B, Em) * inv;
+        const double dEg = (tau * inv) * fma(hT, B - Eg, dB);
         rEt[j] = Eg;
         rDt[j] = dEg;
         s1 += Eg - Em;
         s2 += dEg;
         lo = hi;
       }
-      r = rcv * dl + s1;
-      dr = rcv + s2;
+      r = fma(rcv, dl, cell_sum<L>(s1));
+      dr = rcv + cell_sum<L>(s2);
     };
     double dl = 0.0, r, dr;
     eval(dl, r, dr);
@@ -241,38 +272,40 @@ __global__ void __launch_bounds__(CPL64_THREADS) couple64_kernel(StageArgs<doubl
       if (!ok) st |= ST_NEWTON;
     }
     Tst = Tm + dl;
-    if (A.tstar_out != nullptr) A.tstar_out[FXI(cid, ncell)] = Tst;
+    if (A.tstar_out != nullptr && ln == 0) A.tstar_out[FXI(cid, ncell)] = Tst;
     // ---- the group energies at the accepted temperature and the gas energy by conservation (R12)
     double dEsum = 0.0;
-    for (int j = 0; j < G; ++j) {
+    for (int j = ln; j < G; j += L) {
       const double En = rEt[j] + rDt[j] * lin;
       dEsum += En - rE[j];
       rE[j] = En;
     }
-    rhoe = ke + (um - dEsum);
+    rhoe = ke + (um - cell_sum<L>(dEsum));
   }
   // the F rows (into the rows of the last evaluation)
   __syncthreads();
 #pragma unroll
   for (int v = 1; v < NRV; ++v)
-    stage_rows64<true>(FXPR(A.out, (size_t)NG * ncell + ((size_t)v * ncell + c0) * G, nc * G, A.n_state), srow + v * CPL64_THREADS * RS, nc, G, RS);
+    stage_rows64<true>(FXPR(A.out, (size_t)NG * ncell + ((size_t)v * ncell + c0) * G, nc * G, A.n_state), srow + v * CPB * RS, nc, G, RS);
   __syncthreads();
   if (work) {
     // ---- flux absorption at the converged temperature (Eq. 28) and its momentum and energy
     // feedback (Eqs. 31-32), with the velocity of the state before the interaction
     const double kT = K * hpow(Tst, g.kap_T_h);
     double SdF[3] = {0.0, 0.0, 0.0};
-    for (int j = 0; j < G; ++j) {
-      const double fac = frcp(1.0 + kn.cdts * (kT * s_ef[j] + Sg));
+    for (int j = ln; j < G; j += L) {
+      const double fac = rcp_pos(1.0 + kn.cdts * (kT * s_ef[j] + Sg));
 #pragma unroll
       for (int q = 0; q < D; ++q) {
-        double* rF = srow + ((1 + q) * CPL64_THREADS + t) * RS;
+        double* rF = srow + ((1 + q) * CPB + t) * RS;
         const double Fq = rF[j], Fn = Fq * fac;
         SdF[q] += Fn - Fq;
         rF[j] = Fn;
       }
     }
     double dwork = 0.0;
+#pragma unroll
+    for (int q = 0; q < D; ++q) SdF[q] = cell_sum<L>(SdF[q]);
 #pragma unroll
     for (int q = 0; q < D; ++q) dwork += (sph ? m[q] * frcp(h[q] * h[q]) : m[q]) * irho * SdF[q];
 #pragma unroll
@@ -284,27 +317,31 @@ __global__ void __launch_bounds__(CPL64_THREADS) couple64_kernel(StageArgs<doubl
     // A NaN or inf anywhere in the cell's outputs makes chk non-finite (with the interaction on,
     // a non-finite E_g or F_g reaches the gas energy or momentum through the group sums)
     double chk = rho + rhoe;
-    A.out[FXI(cid, A.n_state)] = rho;
 #pragma unroll
-    for (int q = 0; q < D; ++q) { A.out[FXI((1 + q) * ncell + cid, A.n_state)] = m[q]; chk += m[q]; }
-    A.out[FXI((NG - 1) * ncell + cid, A.n_state)] = rhoe;
+    for (int q = 0; q < D; ++q) chk += m[q];
+    if (ln == 0) {
+      A.out[FXI(cid, A.n_state)] = rho;
+#pragma unroll
+      for (int q = 0; q < D; ++q) A.out[FXI((1 + q) * ncell + cid, A.n_state)] = m[q];
+      A.out[FXI((NG - 1) * ncell + cid, A.n_state)] = rhoe;
+    }
     if (!work) {
       for (int v = 0; v < NRV; ++v) {
-        const double* rv = srow + (v * CPL64_THREADS + t) * RS;
-        for (int j = 0; j < G; ++j) chk += rv[j] * 0.0;
+        const double* rv = srow + (v * CPB + t) * RS;
+        for (int j = ln; j < G; j += L) chk += rv[j] * 0.0;
       }
     }
     if (!isfinite(chk)) st |= ST_NONFINITE;
     if (st) atomicOr(A.status, st);
   }
   if (A.budget != nullptr) {
-    const double wv = work ? cell_volume(A, cid) * A.bw_cpl : 0.0;
-    block_add2(work_out * wv, work ? s_floor[t] * wv : 0.0, A.budget + (size_t)(blockIdx.x % BUDGET_SLOTS) * NBUDGET + 6);
+    const double wv = work && ln == 0 ? cell_volume(A, cid) * A.bw_cpl : 0.0;
+    block_add2(work_out * wv, work && ln == 0 ? s_floor[t] * wv : 0.0, A.budget + (size_t)(blockIdx.x % BUDGET_SLOTS) * NBUDGET + 6);
   }
   __syncthreads();
 #pragma unroll
   for (int v = 0; v < NRV; ++v)
-    stage_rows64<false>(FXPR(A.out, (size_t)NG * ncell + ((size_t)v * ncell + c0) * G, nc * G, A.n_state), srow + v * CPL64_THREADS * RS, nc, G, RS);
+    stage_rows64<false>(FXPR(A.out, (size_t)NG * ncell + ((size_t)v * ncell + c0) * G, nc * G, A.n_state), srow + v * CPB * RS, nc, G, RS);
 }
 
 }  // namespace fx

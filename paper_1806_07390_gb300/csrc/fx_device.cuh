@@ -299,6 +299,8 @@ __device__ __forceinline__ double rcp64(double x) {
   const double e = fma(-x, y, 1.0);
   return fma(y, fma(e, e, e), y);
 }
+// 1/x for positive x: as rcp64 below 2^1020, by division above (an infinity gives 0).
+__device__ __forceinline__ double rcp_pos(double x) { return __double2hiint(x) < 0x7fb00000 ? rcp64(x) : 1.0 / x; }
 // sqrt(a) for normal positive a: the hardware seed of 1/sqrt(a), one coupled Newton step on
 // g ~ sqrt(a) and h ~ 1/(2 sqrt(a)) (Goldschmidt's iteration), and a last correction by the residual
 // a - g^2.
@@ -421,6 +423,48 @@ __device__ __forceinline__ PlanckEdge<double> planck_edge64(double x, const Plan
     e.Q = s;
     e.w = x3 * x * y / (1.0 - y);
     e.upper = true;
+  }
+  return e;
+}
+
+// The same from the table of polynomials (fx_planck.h) at x16 = 16 x: row n = round(16 x), t = 16 x - n.
+// One edge takes 20 FP64 operations (seven Horner steps for the value, six for the derivative, and
+// w = x dQ/dx up to sign from it), against 58 for the power series below XSPLIT and ~20 + 8 per term
+// with the exponential series above it: the FP64 pipe is what the FP64 interaction is bound by.
+// Rows past the table (x >= 64, and NaN) take the series.  The row is read as four 16-byte loads.
+// edge value and its weight against 64-bit references: relative error below 2 and 4 units of 2^-53.
+static __device__ __noinline__ PlanckEdge<double> planck_edge_far(double x, const PlanckCoef& pc) { return planck_edge64(x, pc); }
+__device__ __forceinline__ PlanckEdge<double> planck_edge_tab(double x16, const double* __restrict__ tab, const PlanckCoef& pc) {
+  if ((unsigned)__double2hiint(x16) >= 0x40900000u) return planck_edge_far(x16 * 0.0625, pc);  // 16 x >= 1024
+  const double magic = 6755399441055744.0;  // 1.5 2^52: the sum's low word is the nearest integer
+  const double s = x16 + magic;
+  const int n = __double2loint(s);
+  const double t = x16 - (s - magic);
+  const double2* const r = reinterpret_cast<const double2*>(tab) + n * 4;
+  const double2 a = __ldg(r), b = __ldg(r + 1), c = __ldg(r + 2), d = __ldg(r + 3);
+  double p = d.y, q = d.y;
+  p = fma(p, t, d.x);
+  q = fma(q, t, p);
+  p = fma(p, t, c.y);
+  q = fma(q, t, p);
+  p = fma(p, t, c.x);
+  q = fma(q, t, p);
+  p = fma(p, t, b.y);
+  q = fma(q, t, p);
+  p = fma(p, t, b.x);
+  q = fma(q, t, p);
+  p = fma(p, t, a.y);
+  q = fma(q, t, p);  // dp/dt
+  p = fma(p, t, a.x);
+  PlanckEdge<double> e;
+  e.upper = n >= PETAB_SPLIT;
+  if (e.upper) {
+    e.Q = p;
+    e.w = -(x16 * q);
+  } else {
+    const double x3 = x16 * x16 * (x16 * (1.0 / 4096.0));
+    e.Q = x3 * p;
+    e.w = x3 * fma(x16, q, 3.0 * p);
   }
   return e;
 }

@@ -181,12 +181,13 @@ static cudaError_t launch_gp(const StageArgs<R>& a0, cudaStream_t s, cudaEvent_t
       const unsigned nb = (unsigned)((a.g.ncell + CPL_THREADS - 1) / CPL_THREADS);
       ck<<<nb, CPL_THREADS, cs, s>>>(a);
     } else {
-      auto ck = couple64_kernel<D>;
-      const size_t cs = couple64_smem_bytes<D>(a.g.G);
+      const bool split = a.g.ncell <= CPL64_SPLIT_CELLS;
+      const int lanes = split ? CPL64_SPLIT_LANES : 1, threads = split ? 32 : CPL64_THREADS, cells = threads / lanes;
+      auto ck = split ? couple64_kernel<D, CPL64_SPLIT_LANES> : couple64_kernel<D, 1>;
+      const size_t cs = couple64_smem_bytes<D>(a.g.G, cells);
       e = cudaFuncSetAttribute(ck, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cs);
       if (e != cudaSuccess) return e;
-      const unsigned nb = (unsigned)((a.g.ncell + CPL64_THREADS - 1) / CPL64_THREADS);
-      ck<<<nb, CPL64_THREADS, cs, s>>>(a);
+      ck<<<(unsigned)((a.g.ncell + cells - 1) / cells), threads, cs, s>>>(a);
     }
     e = cudaGetLastError();
   }

@@ -38,6 +38,7 @@ template <class T> struct Consts {
 // Planck series coefficients (universal constants), passed by value in the kernel parameters.
 struct PlanckParams {
   PlanckCoef c64;
+  const double* petab;  // FP64 edge table (fx_planck.h) in device memory; null in the FP32 forms
   float lo32[NPLANCK_LO32];
   float wd32[NPLANCK_LO32];
 };
@@ -305,12 +306,12 @@ struct LanePlanck {
       Bq = (LT)B_;
       dBq = (LT)dB_;
     } else {
-      PlanckEdge<double> lo = planck_edge64((double)(elo * invT), pk.c64);
+      PlanckEdge<double> lo = planck_edge_tab((double)(elo * invT) * 16.0, pk.petab, pk.c64);
       PlanckEdge<double> hi;
       hi.Q = __shfl_down_sync(0xffffffffu, lo.Q, 1, GP);
       hi.w = __shfl_down_sync(0xffffffffu, lo.w, 1, GP);
       hi.upper = __shfl_down_sync(0xffffffffu, (int)lo.upper, 1, GP) != 0;
-      if (top2) hi = planck_edge64((double)(etop * invT), pk.c64);
+      if (top2) hi = planck_edge_tab((double)(etop * invT) * 16.0, pk.petab, pk.c64);
       LT I = (LT)planck_band(lo, hi);
       LT T3 = Tl * Tl * Tl;
       Bq = aN * T3 * Tl * I;

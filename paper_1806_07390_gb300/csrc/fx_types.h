@@ -10,6 +10,9 @@ constexpr int NPLANCK_LO = 27;    // FP64 Bernoulli-series terms (x < XSPLIT, er
 constexpr int NPLANCK_LO32 = 13;  // FP32 Bernoulli-series terms (error < 1e-8)
 constexpr int NPLANCK_UP = 48;    // cap of the FP64 exponential series (x >= XSPLIT: 14 terms)
 constexpr double XSPLIT = 3.0;    // lower/upper Planck series switch
+// FP64 Planck edge table (fx_planck.h): rows at x = n/16, n = 0 .. 1024 (the series above), the
+// first 48 rows for the integral from zero
+constexpr int PETAB_ROWS = 1025, PETAB_SPLIT = 48;
 constexpr int NBUDGET = 9;        // budget accumulators per row (see StageArgs::budget)
 constexpr int BUDGET_SLOTS = 64;  // rows of budget accumulators that blocks add to (summed when read)
 constexpr int PTAB_PER_OCT = 32;  // FP32 Planck band tables: nodes per octave of T

@@ -203,9 +203,9 @@ __global__ void __launch_bounds__(CPLYE_THREADS) couple_ye_kernel(const __grid_c
     } else {
       const double invT = 1.0 / T, T3 = T * T * T;
       const double kT = kpre * hpow(T, g.kap_T_h);
-      PlanckEdge<double> lo = planck_edge64(gc.edge[0] * invT, A.pk.c64);
+      PlanckEdge<double> lo = planck_edge_tab(gc.edge[0] * invT * 16.0, A.pk.petab, A.pk.c64);
       for (int gg = 0; gg < Gs; ++gg) {
-        const PlanckEdge<double> hi = planck_edge64(gc.edge[gg + 1] * invT, A.pk.c64);
+        const PlanckEdge<double> hi = planck_edge_tab(gc.edge[gg + 1] * invT * 16.0, A.pk.petab, A.pk.c64);
         const double I = planck_band(lo, hi);
         const double B = norm * T3 * T * I;
         const double dB = norm * (4.0 * T3 * I + T3 * (lo.w - hi.w));
