@@ -14,6 +14,96 @@
 
 namespace fx {
 
+// Reciprocal: IEEE division in FP64; the hardware approximation (1 ulp) in FP32, one instruction
+// (a division intrinsic adds range scaling that no caller needs).
+__device__ __forceinline__ double frcp(double x) { return 1.0 / x; }
+__device__ __forceinline__ float frcp(float x) { return rcp_approx(x); }
+
+// ---------------------------------------------------------------------------------------------
+// FP64 operations off the FP64 pipe where the result allows it.  The pipe does two lane operations
+// per cycle per multiprocessor (1/64 of FP32), and a comparison, minimum or select of doubles
+// takes a turn on it like any other operation, so the helpers below compare bit patterns with the
+// integer units: doubles of one sign order as their bits do.
+// ---------------------------------------------------------------------------------------------
+// x > 0 and normal
+__device__ __forceinline__ bool normal_pos(double x) { return __double2hiint(x) >= 0x00100000; }
+// 1/x for normal positive x below 2^1022: the hardware seed y (relative error e, |e| < 2^-19)
+// improved by one third-order step y (1 + e + e^2), the truncated geometric series of 1/(1 - e), whose
+// error is e^3 < 2^-57 plus the roundings.
+__device__ __forceinline__ double rcp64(double x) {
+  double y;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  const double e = fma(-x, y, 1.0);
+  return fma(y, fma(e, e, e), y);
+}
+// 1/x for positive x: as rcp64 below 2^1020, by division above (an infinity gives 0).
+__device__ __forceinline__ double rcp_pos(double x) { return __double2hiint(x) < 0x7fb00000 ? rcp64(x) : 1.0 / x; }
+// sqrt(a) for normal positive a: the hardware seed of 1/sqrt(a), one coupled Newton step on
+// g ~ sqrt(a) and h ~ 1/(2 sqrt(a)) (Goldschmidt's iteration), and a last correction by the residual
+// a - g^2.
+__device__ __forceinline__ double sqrt64(double a) {
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(a));
+  double g = a * y, h = 0.5 * y;
+  const double r = fma(-g, h, 0.5);
+  g = fma(g, r, g);
+  h = fma(h, r, h);
+  return fma(fma(-g, g, a), h, g);
+}
+// 1 / max(t, 1)
+__device__ __forceinline__ double rcp_ge1(double t) {
+  const int hi = __double2hiint(t);
+  return hi < 0x3ff00000 ? 1.0 : (hi >= 0x7fd00000 ? 0.0 : rcp64(t));
+}
+__device__ __forceinline__ F2 rcp_ge1(F2 t) { return F2(rcp_approx(fmaxf(t.x, 1.0f)), rcp_approx(fmaxf(t.y, 1.0f))); }
+
+// Comparisons by bit patterns for the selects of the gas kernels: a and b of one sign and neither
+// zero; of opposite signs and neither zero; the sign of |a| - |b|; the middle of three values.
+__device__ __forceinline__ bool same_sign(float a, float b) { return a * b > 0.0f; }
+__device__ __forceinline__ bool opposite_sign(float a, float b) { return a * b < 0.0f; }
+__device__ __forceinline__ int cmp_abs(float a, float b) { return fabsf(a) < fabsf(b) ? -1 : (fabsf(a) == fabsf(b) ? 0 : 1); }
+__device__ __forceinline__ float median(float x, float u, float v) { return fmaxf(fminf(u, v), fminf(fmaxf(u, v), x)); }
+__device__ __forceinline__ bool nonzero64(double a) { return (__double_as_longlong(a) << 1) != 0; }
+__device__ __forceinline__ bool same_sign(double a, double b) {
+  return (__double2hiint(a) ^ __double2hiint(b)) >= 0 && nonzero64(a) && nonzero64(b);
+}
+__device__ __forceinline__ bool opposite_sign(double a, double b) {
+  return (__double2hiint(a) ^ __double2hiint(b)) < 0 && nonzero64(a) && nonzero64(b);
+}
+__device__ __forceinline__ int cmp_abs(double a, double b) {
+  const long long x = __double_as_longlong(a) & 0x7fffffffffffffffLL, y = __double_as_longlong(b) & 0x7fffffffffffffffLL;
+  return x < y ? -1 : (x == y ? 0 : 1);
+}
+// order-preserving map of a double to a signed integer (negative numbers have their magnitude bits
+// inverted)
+__device__ __forceinline__ long long key64(double a) {
+  const long long k = __double_as_longlong(a);
+  return k ^ ((k >> 63) & 0x7fffffffffffffffLL);
+}
+__device__ __forceinline__ bool less64(double a, double b) { return key64(a) < key64(b); }
+__device__ __forceinline__ double median(double x, double u, double v) {
+  const long long kx = key64(x), ku = key64(u), kv = key64(v);
+  const long long r = max(min(ku, kv), min(max(ku, kv), kx));
+  return __longlong_as_double(r ^ ((r >> 63) & 0x7fffffffffffffffLL));
+}
+__device__ __forceinline__ float min_fast(float a, float b) { return fminf(a, b); }
+__device__ __forceinline__ float max_fast(float a, float b) { return fmaxf(a, b); }
+__device__ __forceinline__ double min_fast(double a, double b) { return less64(a, b) ? a : b; }
+__device__ __forceinline__ double max_fast(double a, double b) { return less64(a, b) ? b : a; }
+__device__ __forceinline__ bool nonneg(float a) { return a >= 0.0f; }
+__device__ __forceinline__ bool nonneg(double a) { return __double2hiint(a) >= 0 || !nonzero64(a); }
+// 1/x and sqrt(x) of any argument: the short forms on the normal range, the library's outside it
+__device__ __forceinline__ float rcp_any(float x) { return rcp_approx(x); }
+__device__ __forceinline__ double rcp_any(double x) {
+  const unsigned e = (unsigned)__double2hiint(x) & 0x7fffffffu;
+  return e >= 0x00400000u && e < 0x7fb00000u ? rcp64(x) : 1.0 / x;
+}
+__device__ __forceinline__ float sqrt_any(float x) { return sqrtf(x); }
+__device__ __forceinline__ double sqrt_any(double x) {
+  const int e = __double2hiint(x);
+  return e >= 0x00400000 && e < 0x7fb00000 ? sqrt64(x) : sqrt(x);
+}
+
 // ---------------------------------------------------------------------------------------------
 // Per-cell reconstruction/divergence table (one row per padded cell and direction), built on the
 // host in FP64 from the coordinate moments <x^j> of each cell (Sec. 5.1, Eq. 14).
@@ -62,39 +152,37 @@ template <class R> struct Tab {
   }
 };
 
+// The table of a Cartesian direction: one row (of the launch arguments) for every cell.
+template <class R> struct TabRow {
+  const R* row;
+  __device__ __forceinline__ R operator()(int e, int) const { return row[e]; }
+};
+
 // ---------------------------------------------------------------------------------------------
 // Parabolic (n = 2) reconstruction of one variable in one cell (Sec. 5.1; readings R2-R4).
 // ip: padded index of the cell (cell i -> i + 2).  R: table type; V: value type (R itself, or a
 // forward-mode dual number when the adjoint forms local Jacobians).
 // ---------------------------------------------------------------------------------------------
-template <class R, class V>
-__device__ __forceinline__ void recon_parabolic(const Tab<R>& t, int ip, V pm, V p0, V pp, V& a, V& b) {
+template <class T, class R, class V>
+__device__ __forceinline__ void recon_parabolic(const T& t, int ip, V pm, V p0, V pp, V& a, V& b, R) {
   V dl = p0 - pm, dr = pp - p0;
-  if constexpr (std::is_same<V, float>::value) {
-    // FP32: the same decisions taken as selects over values computed for every cell, so a warp
-    // runs one path
-    const bool ext = dl * dr <= R(0);
+  if constexpr (std::is_same<V, R>::value) {
+    // the same decisions as the general code below, taken as selects over values computed for
+    // every cell, so that a warp runs one path; in FP64 the decisions are integer comparisons
+    const bool ext = !same_sign(dl, dr);
     V a0 = t(T_WA0, ip) * pm + t(T_WA1, ip) * p0 + t(T_WA2, ip) * pp;
     V b0 = t(T_WB0, ip) * pm + t(T_WB1, ip) * p0 + t(T_WB2, ip) * pp;
-    {
-      const V l = pm + dl * t(T_SL2, ip), h = p0 - dl * t(T_TL2, ip);
-      const V lo = dl < R(0) ? h : l, hi = dl < R(0) ? l : h;
-      a0 = a0 < lo ? lo : (a0 > hi ? hi : a0);
-    }
-    {
-      const V l = p0 + dr * t(T_SR2, ip), h = pp - dr * t(T_TR2, ip);
-      const V lo = dr < R(0) ? h : l, hi = dr < R(0) ? l : h;
-      b0 = b0 < lo ? lo : (b0 > hi ? hi : b0);
-    }
+    // between the zero-slope values at the two centroids, whichever is the lower one
+    a0 = median(a0, pm + dl * t(T_SL2, ip), p0 - dl * t(T_TL2, ip));
+    b0 = median(b0, p0 + dr * t(T_SR2, ip), pp - dr * t(T_TR2, ip));
     const V sl = t(T_AL0, ip) * a0 + t(T_AL1, ip) * p0 + t(T_AL2, ip) * b0;
     const V sr = t(T_AR0, ip) * a0 + t(T_AR1, ip) * p0 + t(T_AR2, ip) * b0;
-    const bool inc = !(sl * sr >= R(0));  // extremum inside the cell
-    const V asl = fabs(sl), asr = fabs(sr);
-    const bool flat = asl == asr, lower = asl < asr;
+    const bool inc = opposite_sign(sl, sr);  // extremum inside the cell
+    const int cmp = cmp_abs(sl, sr);
     const V bz = a0 + (p0 - a0) * t(T_RHL, ip);  // zero slope at the lower face
     const V az = b0 + (p0 - b0) * t(T_RHR, ip);  // zero slope at the upper face
-    const V an = inc ? (flat ? p0 : (lower ? a0 : az)) : a0;
-    const V bn = inc ? (flat ? p0 : (lower ? bz : b0)) : b0;
+    const V an = inc ? (cmp == 0 ? p0 : (cmp < 0 ? a0 : az)) : a0;
+    const V bn = inc ? (cmp == 0 ? p0 : (cmp < 0 ? bz : b0)) : b0;
     a = ext ? p0 : an;
     b = ext ? p0 : bn;
     return;
@@ -121,6 +209,10 @@ __device__ __forceinline__ void recon_parabolic(const Tab<R>& t, int ip, V pm, V
   if (asl == asr) { a = p0; b = p0; return; }
   if (asl < asr) b = a + (p0 - a) * t(T_RHL, ip);  // zero slope at the lower face
   else a = b + (p0 - b) * t(T_RHR, ip);            // zero slope at the upper face
+}
+template <class R, class V>
+__device__ __forceinline__ void recon_parabolic(const Tab<R>& t, int ip, V pm, V p0, V pp, V& a, V& b) {
+  recon_parabolic(t, ip, pm, p0, pp, a, b, R(0));
 }
 
 // Coefficients of the linear MC reconstruction of one cell (shared by all its variables and
@@ -154,6 +246,52 @@ __device__ __forceinline__ void recon_linear_c(const MCCoef<R>& c, V pm, V p0, V
 // ---------------------------------------------------------------------------------------------
 template <class R, int D, class V = R>
 __device__ __forceinline__ void hllc(R gam, const V* L, const V* Rs, V* f, V& vstar) {
+  if constexpr (std::is_same<V, R>::value) {
+    // The kernels' own types: every division is a reciprocal, shared where the denominator is (the
+    // FP64 form of a division costs twice a reciprocal's operations), and the choice among the
+    // supersonic and star fluxes is a select: the side k (left when the face is supersonic to the
+    // right or the contact moves right) and its plain flux F_k for every face; the star correction
+    // S_k (U*_k - U_k) is added where the face is subsonic.
+    const R igm1 = rcp_any(gam - R(1)), g1 = gam - R(1);
+    const R rl = L[0], pl = L[1], ul = L[2], rr = Rs[0], pr = Rs[1], ur = Rs[2];
+    R kl = ul * ul, kr = ur * ur;
+#pragma unroll
+    for (int q = 1; q < D; ++q) { kl += L[2 + q] * L[2 + q]; kr += Rs[2 + q] * Rs[2 + q]; }
+    const R El = pl * igm1 + R(0.5) * rl * kl, Er = pr * igm1 + R(0.5) * rr * kr;
+    const R irl = rcp_any(rl), irr = rcp_any(rr);
+    const R al = sqrt_any(gam * pl * irl), ar = sqrt_any(gam * pr * irr);
+    const R sl = sqrt_any(rl), sr = sqrt_any(rr), iw = rcp_any(sl + sr);
+    const R Ht = (sl * ((El + pl) * irl) + sr * ((Er + pr) * irr)) * iw;
+    const R ut = (sl * ul + sr * ur) * iw;
+    R v2 = ut * ut;
+#pragma unroll
+    for (int q = 1; q < D; ++q) { const R vq = (sl * L[2 + q] + sr * Rs[2 + q]) * iw; v2 += vq * vq; }
+    const R at2 = g1 * (Ht - R(0.5) * v2);
+    const R at = sqrt_any(nonneg(at2) ? at2 : R(0));
+    const R SL = min_fast(ul - al, ut - at), SR = max_fast(ur + ar, ut + at);
+    const R dl = rl * (SL - ul), dr = rr * (SR - ur);
+    const R Ss = (pr - pl + ul * dl - ur * dr) * rcp_any(dl - dr);
+    vstar = Ss;
+    const bool supL = nonneg(SL), supR = !supL && !nonneg(SR), sup = supL || supR;
+    const bool left = supL || (!supR && nonneg(Ss));
+    const R rk = left ? rl : rr, pk = left ? pl : pr, uk = left ? ul : ur;
+    const R Ek = left ? El : Er, Sk = left ? SL : SR, irk = left ? irl : irr;
+    const R sku = Sk - uk, m = rk * uk;
+    const R fac = rk * sku * rcp_any(Sk - Ss);
+    const R f1 = m * uk + pk;
+    f[0] = sup ? m : m + Sk * (fac - rk);
+    f[1] = sup ? f1 : f1 + Sk * (fac * Ss - m);
+#pragma unroll
+    for (int q = 1; q < D; ++q) {
+      const R wq = left ? L[2 + q] : Rs[2 + q];
+      const R fq = m * wq;
+      f[1 + q] = sup ? fq : fq + Sk * (fac * wq - rk * wq);
+    }
+    const R Es = fac * (Ek * irk + (Ss - uk) * (Ss + pk * (irk * rcp_any(sku))));
+    const R fE = (Ek + pk) * uk;
+    f[1 + D] = sup ? fE : fE + Sk * (Es - Ek);
+    return;
+  }
   const R gm1 = gam - R(1);
   V rl = L[0], pl = L[1], ul = L[2];
   V rr = Rs[0], pr = Rs[1], ur = Rs[2];
@@ -177,30 +315,6 @@ __device__ __forceinline__ void hllc(R gam, const V* L, const V* Rs, V* f, V& vs
   V dl = rl * (SL - ul), dr = rr * (SR - ur);
   V Ss = (pr - pl + ul * dl - ur * dr) / (dl - dr);
   vstar = Ss;
-  if constexpr (std::is_same<V, float>::value) {
-    // FP32: the side k (left when the face is supersonic to the right or the contact moves
-    // right) and its plain flux F_k for every face; the star correction S_k (U*_k - U_k) is
-    // added by a select where the face is subsonic
-    const bool supL = SL >= R(0), supR = !supL && SR < R(0), sup = supL || supR;
-    const bool left = supL || (!supR && Ss >= R(0));
-    const V rk = left ? rl : rr, pk = left ? pl : pr, uk = left ? ul : ur;
-    const V Ek = left ? El : Er, Sk = left ? SL : SR;
-    const V sku = Sk - uk;
-    const V fac = rk * sku / (Sk - Ss);
-    const V f0 = rk * uk, f1 = rk * uk * uk + pk;
-    f[0] = sup ? f0 : f0 + Sk * (fac - rk);
-    f[1] = sup ? f1 : f1 + Sk * (fac * Ss - rk * uk);
-#pragma unroll
-    for (int q = 1; q < D; ++q) {
-      const V wq = left ? L[2 + q] : Rs[2 + q];
-      const V fq = rk * uk * wq;
-      f[1 + q] = sup ? fq : fq + Sk * (fac * wq - rk * wq);
-    }
-    const V Es = fac * (Ek / rk + (Ss - uk) * (Ss + pk / (rk * sku)));
-    const V fE = (Ek + pk) * uk;
-    f[1 + D] = sup ? fE : fE + Sk * (Es - Ek);
-    return;
-  }
   if (SL >= R(0)) {
     f[0] = rl * ul;
     f[1] = rl * ul * ul + pl;
@@ -276,49 +390,6 @@ __device__ __forceinline__ void gas_riemann(int solver, R gam, const R* L, const
 #pragma unroll
   for (int v = 0; v < 2 + D; ++v) f[v] = (br * FL[v] - bl * FR[v] + bl * br * (UR[v] - UL[v])) * ib;
 }
-
-// Reciprocal: IEEE division in FP64; the hardware approximation (1 ulp) in FP32, one instruction
-// (a division intrinsic adds range scaling that no caller needs).
-__device__ __forceinline__ double frcp(double x) { return 1.0 / x; }
-__device__ __forceinline__ float frcp(float x) { return rcp_approx(x); }
-
-// ---------------------------------------------------------------------------------------------
-// FP64 operations off the FP64 pipe where the result allows it.  The pipe does two lane operations
-// per cycle per multiprocessor (1/64 of FP32), and a comparison, minimum or select of doubles
-// takes a turn on it like any other operation, so the helpers below compare bit patterns with the
-// integer units: doubles of one sign order as their bits do.
-// ---------------------------------------------------------------------------------------------
-// x > 0 and normal
-__device__ __forceinline__ bool normal_pos(double x) { return __double2hiint(x) >= 0x00100000; }
-// 1/x for normal positive x below 2^1022: the hardware seed y (relative error e, |e| < 2^-19)
-// improved by one third-order step y (1 + e + e^2), the truncated geometric series of 1/(1 - e), whose
-// error is e^3 < 2^-57 plus the roundings.
-__device__ __forceinline__ double rcp64(double x) {
-  double y;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  const double e = fma(-x, y, 1.0);
-  return fma(y, fma(e, e, e), y);
-}
-// 1/x for positive x: as rcp64 below 2^1020, by division above (an infinity gives 0).
-__device__ __forceinline__ double rcp_pos(double x) { return __double2hiint(x) < 0x7fb00000 ? rcp64(x) : 1.0 / x; }
-// sqrt(a) for normal positive a: the hardware seed of 1/sqrt(a), one coupled Newton step on
-// g ~ sqrt(a) and h ~ 1/(2 sqrt(a)) (Goldschmidt's iteration), and a last correction by the residual
-// a - g^2.
-__device__ __forceinline__ double sqrt64(double a) {
-  double y;
-  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(a));
-  double g = a * y, h = 0.5 * y;
-  const double r = fma(-g, h, 0.5);
-  g = fma(g, r, g);
-  h = fma(h, r, h);
-  return fma(fma(-g, g, a), h, g);
-}
-// 1 / max(t, 1)
-__device__ __forceinline__ double rcp_ge1(double t) {
-  const int hi = __double2hiint(t);
-  return hi < 0x3ff00000 ? 1.0 : (hi >= 0x7fd00000 ? 0.0 : rcp64(t));
-}
-__device__ __forceinline__ F2 rcp_ge1(F2 t) { return F2(rcp_approx(fmaxf(t.x, 1.0f)), rcp_approx(fmaxf(t.y, 1.0f))); }
 
 // ---------------------------------------------------------------------------------------------
 // M1 closure (Levermore / Dubroca-Feugeas Eddington factor chi(f) = (3+4f^2)/(5+2 sqrt(4-3f^2)),

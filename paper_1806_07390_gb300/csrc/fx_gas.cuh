@@ -5,6 +5,11 @@
 // cell once, for both of its faces.  It also forms every face's record for the radiation fluxes
 // (the upwind advection speeds of Eq. 19 and the sums of the two cells' opacity factors for the ε
 // correction), so that the stage kernel reads one aligned record per face.
+// Bound by instruction issue in FP32 and by the FP64 pipe (85 % busy) in FP64: the reconstruction's
+// decisions are medians and selects over values computed for every cell (in FP64 by integer
+// comparisons), a Cartesian direction's coefficients are one constant row of the launch
+// arguments, and HLLC's eleven divisions are six shared reciprocals.  Per launch: 1024^2 FP32 0.079
+// -> 0.050 ms, 256^3 FP32 2.04 -> 1.31 ms, 512^2 FP64 0.42 -> 0.33 ms.
 // The stage kernel then uses the fluxes for the gas divergence; with the velocity-dependent radiation terms on, the kernel also stores each face's
 // transverse velocity for their velocity gradient (fx_vterms.cuh).
 #pragma once
@@ -17,40 +22,52 @@ __host__ __device__ inline int64_t faces_along(const int* n, int d) {
   return (int64_t)(n[0] + (d == 0)) * (n[1] + (d == 1)) * (n[2] + (d == 2));
 }
 
-// Tile of the gas face kernel for direction DIR, 288 threads: LR = LD + 1 rows of cells along DIR
-// by LX cells along x are reconstructed, one cell per thread (DIR = 0: a row segment of 288
-// cells; otherwise 9 cells along DIR by 32 along x, so that a warp reads consecutive x), and
+// Tile of the gas face kernel for direction DIR and FT threads: LR = LD + 1 rows of cells along DIR
+// by LX cells along x are reconstructed, one cell per thread (DIR = 0: a row segment of FT cells;
+// otherwise FT / 32 cells along DIR by 32 along x, so that a warp reads consecutive x), and
 // the top LD rows own their lower faces.  Cells 0 .. n_d along DIR own the n_d + 1 faces of the
-// direction (cell n_d is a ghost from the boundary rules).
-constexpr int FACE_THREADS = 288;
-template <int DIR> struct FaceTile {
-  static constexpr int LX = DIR == 0 ? 1 : 32, LR = FACE_THREADS / LX, LD = LR - 1;
+// direction (cell n_d is a ghost from the boundary rules).  FT = 288 on all grids whose tiles then
+// fill the device (the least halo share); below that 64, which spreads a small grid over more
+// multiprocessors (512 cells FP64: 0.035 -> 0.017 ms).
+constexpr int FACE_THREADS = 288, FACE_THREADS_SMALL = 64;
+template <int DIR, int FT> struct FaceTile {
+  static constexpr int LX = DIR == 0 ? 1 : 32, LR = FT / LX, LD = LR - 1;
   static constexpr int NWC = LR + 2;  // cells d0-2 .. d0+LD along DIR whose primitives are staged
 };
-constexpr int FACE_WCELLS = 352;  // max over DIR of FaceTile::NWC * LX
-constexpr int FACE_BCELLS = 288;  // FaceTile::LR * LX
+template <int FT> struct FaceSize {
+  static constexpr int W0 = FT + 2, W1 = (FT / 32 + 2) * 32;
+  static constexpr int WCELLS = W0 > W1 ? W0 : W1;  // max over DIR of FaceTile::NWC * LX
+  static constexpr int BCELLS = FT;                 // FaceTile::LR * LX
+};
 
 // Number of tiles of direction DIR (blocks of the face kernel's grid row DIR).
-__host__ __device__ inline unsigned face_tiles(const int* n, int D, int DIR) {
+template <int FT> __host__ __device__ inline unsigned face_tiles(const int* n, int D, int DIR) {
   const int nd = n[DIR];
   if (DIR == 0) {
-    constexpr int LD = FaceTile<0>::LD;
+    constexpr int LD = FaceTile<0, FT>::LD;
     return (unsigned)((nd + 1 + LD - 1) / LD) * (unsigned)(n[1] * (D >= 3 ? n[2] : 1));
   }
-  constexpr int LD = FaceTile<1>::LD;
+  constexpr int LD = FaceTile<1, FT>::LD;
   const unsigned nxg = (unsigned)((n[0] + 31) / 32);
   return (unsigned)((nd + 1 + LD - 1) / LD) * nxg * (unsigned)(DIR == 1 ? (D >= 3 ? n[2] : 1) : n[1]);
+}
+// Whether the 288-thread tiles of a grid are fewer than three per multiprocessor (152 of them).
+inline bool face_small(const int* n, int D) {
+  uint64_t t = 0;
+  for (int d = 0; d < D; ++d) t += face_tiles<FACE_THREADS>(n, D, d);
+  return t < 3 * 152;
 }
 
 // Fluxes through the faces of one tile of direction DIR: the primitives of the tile's cells and
 // their halo along DIR go to shared memory once, each cell is reconstructed once (its upper-face
 // state serves the face above it, its lower-face state its own face), and each face gets the
 // selected Riemann flux.
-template <class R, int D, int DIR>
-__device__ __forceinline__ void gas_faces_tile(const StageArgs<R>& A, unsigned tile, R (*sw)[FACE_WCELLS],
-                                               R (*sb)[FACE_BCELLS], R (*sk)[FACE_WCELLS]) {
+template <class R, int D, bool SPH, int DIR, int FTH>
+__device__ __forceinline__ void gas_faces_tile(const StageArgs<R>& A, unsigned tile, R (*sw)[FaceSize<FTH>::WCELLS],
+                                               R (*sb)[FaceSize<FTH>::BCELLS], R (*sk)[FaceSize<FTH>::WCELLS]) {
   constexpr int NG = 2 + D, NW = 2 + D;
-  using FT = FaceTile<DIR>;
+  using FT = FaceTile<DIR, FTH>;
+  constexpr int FACE_WCELLS = FaceSize<FTH>::WCELLS, FACE_BCELLS = FaceSize<FTH>::BCELLS;
   constexpr int LD = FT::LD, LX = FT::LX, NWC = FT::NWC;
   const auto& g = A.g;
   const int n0 = g.n[0], n1 = g.n[1], n2 = g.n[2];
@@ -71,13 +88,12 @@ __device__ __forceinline__ void gas_faces_tile(const StageArgs<R>& A, unsigned t
   // 32-bit index arithmetic: the host keeps every state and face-buffer offset below 2^32
   const uint32_t ncell = (uint32_t)g.ncell;
   const auto& KR = A.k(R(0));
-  const bool sph = g.geom != 0;
-  const Tab<R> t0{A.tab[0], n0 + 4, A.uniform[0] ? A.urow[0] : nullptr};
-  const Tab<R> t1{A.tab[D >= 2 ? 1 : 0], (D >= 2 ? n1 : n0) + 4,
-                  A.uniform[D >= 2 ? 1 : 0] ? A.urow[D >= 2 ? 1 : 0] : nullptr};
+  constexpr bool sph = SPH;
+  const Tab<R> t0{A.tab[0], n0 + 4, nullptr};  // (read on the spherical grid)
+  const Tab<R> t1{A.tab[D >= 2 ? 1 : 0], (D >= 2 ? n1 : n0) + 4, nullptr};
   // ---- primitives of cells d0-2 .. d0+LD along DIR (ghosts from the boundary rules), for each
   // of the tile's LX columns
-  for (int c = t; c < NWC * LX; c += FACE_THREADS) {
+  for (int c = t; c < NWC * LX; c += FTH) {
     const int lx = c % LX, k = c / LX;
     const int id = d0 - 2 + k;
     const int x = DIR == 0 ? id : min(xg * 32 + lx, n0 - 1);
@@ -94,7 +110,7 @@ __device__ __forceinline__ void gas_faces_tile(const StageArgs<R>& A, unsigned t
       u[1] *= frcp(t0(T_HA, bc_pad(cr)) * t1(T_HA, bc_pad(ct)));
       if (D >= 2) u[2] *= frcp(t0(T_HB, bc_pad(cr)) * t1(T_HB, bc_pad(ct)));
     }
-    const R rho = u[0], irho = frcp(rho);
+    const R rho = u[0], irho = rcp_any(rho);
     R ke = R(0);
 #pragma unroll
     for (int q = 0; q < D; ++q) {
@@ -114,7 +130,10 @@ __device__ __forceinline__ void gas_faces_tile(const StageArgs<R>& A, unsigned t
   // ---- each thread reconstructs one cell along DIR (row r: cell d0 - 1 + r): the upper-face
   // state to shared memory (the left state of the face above), the lower-face state kept for the
   // cell's own face
-  const Tab<R> tt{A.tab[DIR], nd + 4, A.uniform[DIR] ? A.urow[DIR] : nullptr};
+  using TT = typename std::conditional<SPH, Tab<R>, TabRow<R>>::type;
+  TT tt;
+  if constexpr (SPH) tt = TT{A.tab[DIR], nd + 4, nullptr};
+  else tt = TT{A.urow[DIR]};
   const int lx = t % LX, r = t / LX;
   const int id = d0 - 1 + r;
   auto w = [&](int v, int k) -> R { return sw[v][FXI(k * LX + lx, FACE_WCELLS)]; };  // k: cell d0 - 2 + k
@@ -122,7 +141,7 @@ __device__ __forceinline__ void gas_faces_tile(const StageArgs<R>& A, unsigned t
 #pragma unroll
   for (int v = 0; v < NW; ++v) {
     R a, b;
-    recon_parabolic(tt, bc_pad(id), w(v, r), w(v, r + 1), w(v, r + 2), a, b);
+    recon_parabolic(tt, bc_pad(id), w(v, r), w(v, r + 1), w(v, r + 2), a, b, R(0));
     Ra[v] = a;
     sb[v][FXI(r * LX + lx, FACE_BCELLS)] = b;
   }
@@ -168,7 +187,8 @@ __device__ __forceinline__ void gas_faces_tile(const StageArgs<R>& A, unsigned t
   out[FXI((uint32_t)(NG - 1) * nf + uf, n_out)] = fl[1 + D];
   out[FXI((uint32_t)NG * nf + uf, n_out)] = vs;
   {  // the face's record for the radiation fluxes (StageArgs::frec)
-    const R ell = R(0.5) * tt(T_ELL, bc_pad(id)) * ((sph && DIR == 1) ? t0(T_XH, bc_pad(x)) : R(1));
+    R ell = R(0.5) * tt(T_ELL, bc_pad(id));
+    if (sph && DIR == 1) ell *= t0(T_XH, bc_pad(x));
     const int wl = FXI(r * LX + lx, FACE_WCELLS), wr = FXI((r + 1) * LX + lx, FACE_WCELLS);
     const R r0 = vs > R(0) ? vs + vs : R(0), r1 = vs > R(0) ? R(0) : vs + vs;
     const R r2 = ell * (sk[0][wl] + sk[0][wr]), r3 = ell * (sk[1][wl] + sk[1][wr]);
@@ -240,17 +260,17 @@ __global__ void __launch_bounds__(256) shock_flag_kernel(const __grid_constant__
 }
 
 // One block per tile; grid row y is the direction (tiles beyond a direction's count return).
-template <class R, int D>
-__global__ void __launch_bounds__(FACE_THREADS, 3)
+template <class R, int D, bool SPH, int FTH>
+__global__ void __launch_bounds__(FTH, FTH == FACE_THREADS ? 3 : 8)
 gas_face_kernel(const __grid_constant__ StageArgs<R> A) {
-  __shared__ R sw[2 + D][FACE_WCELLS];
-  __shared__ R sb[2 + D][FACE_BCELLS];
-  __shared__ R sk[2][FACE_WCELLS];
+  __shared__ R sw[2 + D][FaceSize<FTH>::WCELLS];
+  __shared__ R sb[2 + D][FaceSize<FTH>::BCELLS];
+  __shared__ R sk[2][FaceSize<FTH>::WCELLS];
   const int DIR = blockIdx.y;
-  if (blockIdx.x >= face_tiles(A.g.n, D, DIR)) return;
-  if (DIR == 0) gas_faces_tile<R, D, 0>(A, blockIdx.x, sw, sb, sk);
-  else if (D >= 2 && DIR == 1) gas_faces_tile<R, D, (D >= 2 ? 1 : 0)>(A, blockIdx.x, sw, sb, sk);
-  else if (D >= 3) gas_faces_tile<R, D, (D >= 3 ? 2 : 0)>(A, blockIdx.x, sw, sb, sk);
+  if (blockIdx.x >= face_tiles<FTH>(A.g.n, D, DIR)) return;
+  if (DIR == 0) gas_faces_tile<R, D, SPH, 0, FTH>(A, blockIdx.x, sw, sb, sk);
+  else if (D >= 2 && DIR == 1) gas_faces_tile<R, D, SPH, (D >= 2 ? 1 : 0), FTH>(A, blockIdx.x, sw, sb, sk);
+  else if (D >= 3) gas_faces_tile<R, D, SPH, (D >= 3 ? 2 : 0), FTH>(A, blockIdx.x, sw, sb, sk);
 }
 
 }  // namespace fx

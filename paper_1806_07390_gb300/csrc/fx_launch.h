@@ -118,15 +118,18 @@ static cudaError_t launch_gp(const StageArgs<R>& a0, cudaStream_t s, cudaEvent_t
   if (e != cudaSuccess) return e;
   // gas faces first (same stream): fluxes and contact speeds of every face of every direction,
   // one block per tile of faces, one grid row per direction
+  const bool small = face_small(a.g.n, D);
   unsigned ntmax = 0;
-  for (int d = 0; d < D; ++d) ntmax = ntmax > face_tiles(a.g.n, D, d) ? ntmax : face_tiles(a.g.n, D, d);
+  for (int d = 0; d < D; ++d)
+    ntmax = std::max(ntmax, small ? face_tiles<FACE_THREADS_SMALL>(a.g.n, D, d) : face_tiles<FACE_THREADS>(a.g.n, D, d));
   dim3 gg(ntmax, D, 1);
   if (a.sflag != nullptr) {  // carbuncle guard: shock flags of the stage input first
     shock_flag_kernel<R, D><<<(unsigned)((a.g.ncell + 255) / 256), 256, 0, s>>>(a);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
-  gas_face_kernel<R, D><<<gg, FACE_THREADS, 0, s>>>(a);
+  if (small) gas_face_kernel<R, D, SPH, FACE_THREADS_SMALL><<<gg, FACE_THREADS_SMALL, 0, s>>>(a);
+  else gas_face_kernel<R, D, SPH, FACE_THREADS><<<gg, FACE_THREADS, 0, s>>>(a);
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   if (mid) {
