@@ -167,11 +167,17 @@ static cudaError_t launch_gp(const StageArgs<R>& a0, cudaStream_t s, cudaEvent_t
     comp_kernel<R, D><<<(unsigned)((a.g.ncell + 255) / 256), 256, 0, s>>>(a);
     e = cudaGetLastError();
     if (e != cudaSuccess || !a.g.couple) return e;
-    auto ck = couple_ye_kernel<R, D>;
-    const size_t cs = couple_ye_smem_bytes(a.g.G);
-    e = cudaFuncSetAttribute(ck, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cs);
-    if (e != cudaSuccess) return e;
-    ck<<<(unsigned)((a.g.ncell + CPLYE_THREADS - 1) / CPLYE_THREADS), CPLYE_THREADS, cs, s>>>(a);
+    const bool f32 = std::is_same<R, float>::value;
+    const size_t cs = f32 ? couple_ye32_smem_bytes<D>(a.g.G) : couple_ye_smem_bytes(a.g.G);
+    if constexpr (f32) {
+      e = cudaFuncSetAttribute(couple_ye32_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cs);
+      if (e != cudaSuccess) return e;
+      couple_ye32_kernel<D><<<(unsigned)((a.g.ncell + CPL_THREADS - 1) / CPL_THREADS), CPL_THREADS, cs, s>>>(a);
+    } else {
+      e = cudaFuncSetAttribute(couple_ye_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cs);
+      if (e != cudaSuccess) return e;
+      couple_ye_kernel<D><<<(unsigned)((a.g.ncell + CPLYE_THREADS - 1) / CPLYE_THREADS), CPLYE_THREADS, cs, s>>>(a);
+    }
     return cudaGetLastError();
   }
   // the interaction, one thread per cell (FP32 state: couple_kernel; FP64 state: couple64_kernel)

@@ -6,11 +6,10 @@
 // a block after the radiation block.
 //   comp_kernel: its finite-volume update and RK combination (the gas mass flux times the
 //     reconstructed Y_e on the v* upwind side of each face, the HLLC passive-scalar flux);
-//   couple_ye_kernel: the interaction, one thread per cell, the iterate in FP64 for the FP64
-//     and the FP32 state alike (the FP32 forms store the result in FP32); with the FP32 state
-//     the band energies B_g(T) come from the FP32 Planck band table (as in the one-species FP32
-//     interaction), the channel arithmetic is FP32 and the iteration stops at FP32 resolution.
-//     Inner backward-Euler update of
+//   couple_ye_kernel (FP64 state) and couple_ye32_kernel (FP32 state): the interaction, one thread
+//     per cell, the iterate in FP64 in both; with the FP32 state the band energies B_g(T) come
+//     from the FP32 Planck band table (as in the one-species FP32 interaction), the channel
+//     arithmetic is FP32 and the iteration stops at FP32 resolution.  Inner backward-Euler update of
 //     every channel at (T, Y_e), with the equilibrium energy w_s(Y_e) B_g(T), w = 2 Y_e,
 //     2 (1 - Y_e), 1, and the lepton number per unit energy xi = -xi0/eps_g, +xi0/eps_g, 0;
 //     outer residuals r_E = u(T) - u^- + sum dE and r_X = rho (Y_e - Y_e^-) - sum xi dE, solved
@@ -97,17 +96,16 @@ inline size_t couple_ye_smem_bytes(int G) { return (size_t)2 * CPLYE_THREADS * (
 __device__ __forceinline__ double ye_w(int s, double Y) { return s == 0 ? 2.0 * Y : (s == 1 ? 2.0 * (1.0 - Y) : 1.0); }
 __device__ __forceinline__ double ye_dw(int s) { return s == 0 ? 2.0 : (s == 1 ? -2.0 : 0.0); }
 
-template <class R, int D>
-__global__ void __launch_bounds__(CPLYE_THREADS) couple_ye_kernel(const __grid_constant__ StageArgs<R> A) {
+template <int D>
+__global__ void __launch_bounds__(CPLYE_THREADS) couple_ye_kernel(const __grid_constant__ StageArgs<double> A) {
+  using R = double;
   constexpr int NG = 2 + D, NRV = 1 + D;
   extern __shared__ __align__(16) unsigned char ye_raw[];
   const DevGrid& g = A.g;
   const int G = g.G, Gs = g.Gs, RS = G + 1;
-  // E^- of the cell's channels and the last evaluation's E: FP32 rows in the FP32 forms (their
-  // values are FP32 state values), FP64 rows in the FP64 form
-  using RT = typename std::conditional<std::is_same<R, float>::value, float, double>::type;
-  RT* Em = reinterpret_cast<RT*>(ye_raw) + threadIdx.x * RS;
-  RT* En = Em + CPLYE_THREADS * RS;
+  // E^- of the cell's channels and the last evaluation's E
+  double* Em = reinterpret_cast<double*>(ye_raw) + threadIdx.x * RS;
+  double* En = Em + CPLYE_THREADS * RS;
   const uint32_t ncell = (uint32_t)g.ncell;
   const uint32_t c = blockIdx.x * CPLYE_THREADS + threadIdx.x;
   const GroupConst& gc = *A.gc;
@@ -146,8 +144,7 @@ __global__ void __launch_bounds__(CPLYE_THREADS) couple_ye_kernel(const __grid_c
   for (int k = 0; k < G; ++k) {
     double E = U[FXI(rad + c * (uint32_t)G + k, A.n_state)];
     if (E < g.E_floor) { fadd += g.E_floor - E; E = g.E_floor; }
-    Em[k] = (RT)E;
-    E = Em[k];  // (the FP32 forms: the floor as the FP32 state stores it)
+    Em[k] = E;
     Esum += E;
     const int s = k / Gs;
     if (s < 2) Lsum += fabs(xi0 * s_icen[FXI(k % Gs, MAXG)]) * E;
@@ -162,73 +159,35 @@ __global__ void __launch_bounds__(CPLYE_THREADS) couple_ye_kernel(const __grid_c
   // residuals and Jacobian at (T, Y); with keep, the channel energies into En.  A band edge is
   // evaluated once (the upper edge of group g is the lower edge of g + 1), and the backward-Euler
   // factor 1/(1 + tau) and xi once per group (the three species share the group's opacity)
-  constexpr bool F32 = std::is_same<R, float>::value;
-  // FP32 forms: the opacity, tau and xi of each group in FP32 from the FP32 constants
-  const float kpref = (float)kpre, cdtf = (float)(cl * dt), xi0f = (float)xi0;
   auto eval = [&](double T, double Y, double& rE, double& rX, double J[2][2], bool keep) {
     double dE = 0.0, dX = 0.0, eT = 0.0, eY = 0.0, xT = 0.0, xY = 0.0;
-    if constexpr (F32) {
-      // the three species' channel arithmetic in FP32 on the FP32 band table; each group's
-      // partial sums are added to the FP64 sums once
-      const float Tf = (float)T, Yf = (float)Y;
-      const PlanckAt pa = planck_at(A.ptab, A.kf.aN, Tf);
-      const float kTf = kpref * hpow(Tf, g.kap_T_h), hTf = 0.5f * (float)g.kap_T_h * pa.invT;
-      for (int gg = 0; gg < Gs; ++gg) {
-        float Bf, dBf;
-        planck_group(A.ptab, pa, gg, gc.edge32, Bf, dBf);
-        const float tf = cdtf * (kTf * gc.efac32[gg]), dtf = tf * hTf, invf = frcp(1.0f + tf);
-        const float xf = xi0f * (float)s_icen[FXI(gg, MAXG)];
-        float sE = 0.0f, sX = 0.0f, sT = 0.0f, sY = 0.0f, qT = 0.0f, qY = 0.0f;
-#pragma unroll
-        for (int s = 0; s < 3; ++s) {
-          const int k = s * Gs + gg;
-          const float w = s == 0 ? 2.0f * Yf : (s == 1 ? 2.0f * (1.0f - Yf) : 1.0f);
-          const float dw = s == 0 ? 2.0f : (s == 1 ? -2.0f : 0.0f);
-          const float xi = s == 0 ? -xf : (s == 1 ? xf : 0.0f);
-          const float Emk = (float)Em[k], Eq = w * Bf;
-          const float Ek = (Emk + tf * Eq) * invf;
-          const float dT_ = (tf * w * dBf + dtf * (Eq - Ek)) * invf;
-          const float dY_ = tf * dw * Bf * invf;
-          const float d = Ek - Emk;
-          sE += d;
-          sX += xi * d;
-          sT += dT_;
-          sY += dY_;
-          qT += xi * dT_;
-          qY += xi * dY_;
-          if (keep) En[k] = (RT)Ek;
-        }
-        dE += sE; dX += sX; eT += sT; eY += sY; xT += qT; xY += qY;
-      }
-    } else {
-      const double invT = 1.0 / T, T3 = T * T * T;
-      const double kT = kpre * hpow(T, g.kap_T_h);
-      PlanckEdge<double> lo = planck_edge_tab(gc.edge[0] * invT * 16.0, A.pk.petab, A.pk.c64);
-      for (int gg = 0; gg < Gs; ++gg) {
-        const PlanckEdge<double> hi = planck_edge_tab(gc.edge[gg + 1] * invT * 16.0, A.pk.petab, A.pk.c64);
-        const double I = planck_band(lo, hi);
-        const double B = norm * T3 * T * I;
-        const double dB = norm * (4.0 * T3 * I + T3 * (lo.w - hi.w));
-        lo = hi;
-        const double kap = kT * gc.efac[gg];
-        const double tau = cl * dt * kap, dtau = tau * (0.5 * g.kap_T_h * invT);
-        const double xg = xi0 * s_icen[FXI(gg, MAXG)];
-        const double inv = 1.0 / (1.0 + tau);
-        for (int s = 0; s < 3; ++s) {
-          const int k = s * Gs + gg;
-          const double w = ye_w(s, Y), dw = ye_dw(s), xi = s == 0 ? -xg : (s == 1 ? xg : 0.0);
-          const double Eq = w * B;
-          const double Ek = (Em[k] + tau * Eq) * inv;
-          const double dT_ = (tau * w * dB + dtau * (Eq - Ek)) * inv;
-          const double dY_ = tau * dw * B * inv;
-          dE += Ek - Em[k];
-          dX += xi * (Ek - Em[k]);
-          eT += dT_;
-          eY += dY_;
-          xT += xi * dT_;
-          xY += xi * dY_;
-          if (keep) En[k] = Ek;
-        }
+    const double invT = 1.0 / T, T3 = T * T * T;
+    const double kT = kpre * hpow(T, g.kap_T_h);
+    PlanckEdge<double> lo = planck_edge_tab(gc.edge[0] * invT * 16.0, A.pk.petab, A.pk.c64);
+    for (int gg = 0; gg < Gs; ++gg) {
+      const PlanckEdge<double> hi = planck_edge_tab(gc.edge[gg + 1] * invT * 16.0, A.pk.petab, A.pk.c64);
+      const double I = planck_band(lo, hi);
+      const double B = norm * T3 * T * I;
+      const double dB = norm * (4.0 * T3 * I + T3 * (lo.w - hi.w));
+      lo = hi;
+      const double kap = kT * gc.efac[gg];
+      const double tau = cl * dt * kap, dtau = tau * (0.5 * g.kap_T_h * invT);
+      const double xg = xi0 * s_icen[FXI(gg, MAXG)];
+      const double inv = rcp_pos(1.0 + tau);
+      for (int s = 0; s < 3; ++s) {
+        const int k = s * Gs + gg;
+        const double w = ye_w(s, Y), dw = ye_dw(s), xi = s == 0 ? -xg : (s == 1 ? xg : 0.0);
+        const double Eq = w * B;
+        const double Ek = (Em[k] + tau * Eq) * inv;
+        const double dT_ = (tau * w * dB + dtau * (Eq - Ek)) * inv;
+        const double dY_ = tau * dw * B * inv;
+        dE += Ek - Em[k];
+        dX += xi * (Ek - Em[k]);
+        eT += dT_;
+        eY += dY_;
+        xT += xi * dT_;
+        xY += xi * dY_;
+        if (keep) En[k] = Ek;
       }
     }
     rE = rho * cv * T - u_m + dE;
@@ -238,10 +197,7 @@ __global__ void __launch_bounds__(CPLYE_THREADS) couple_ye_kernel(const __grid_c
     J[1][0] = -xT;
     J[1][1] = rho - xY;
   };
-  // stopping tests: FP64 resolution for the FP64 state; with the FP32 band table, the FP32
-  // forms' tolerances (relative step 2e-7 at least, residual 1e-7)
-  const double rtol = F32 ? A.kd.rtol : g.newton_rtol;
-  const double n2ok = F32 ? A.kd.atol * A.kd.atol : 1e-28, n2fb = F32 ? n2ok : 1e-24;
+  const double rtol = g.newton_rtol, n2ok = 1e-28, n2fb = 1e-24;
   const double sE = u_m + Esum, sX = fabs(X_m) + Lsum + 1e-300;
   auto norm2 = [&](double rE, double rX) { const double a = rE / sE, b = rX / sX; return a * a + b * b; };
   double T = u_m / (rho * cv), Y = Y_m, rE, rX, J[2][2];
@@ -307,7 +263,7 @@ __global__ void __launch_bounds__(CPLYE_THREADS) couple_ye_kernel(const __grid_c
   eval(T, Y, rE, rX, J, true);
   double dEsum = 0.0, dXsum = 0.0;
   for (int k = 0; k < G; ++k) {
-    const double dk = (double)En[k] - (double)Em[k];  // exact for the FP32 rows
+    const double dk = En[k] - Em[k];
     dEsum += dk;
     dXsum += xi_of(k) * dk;
     U[FXI(rad + c * (uint32_t)G + k, A.n_state)] = (R)En[k];
@@ -322,7 +278,7 @@ __global__ void __launch_bounds__(CPLYE_THREADS) couple_ye_kernel(const __grid_c
   const double sig = g.sigma0 * rho;
   const double kT = kpre * hpow(T, g.kap_T_h);
   for (int k = 0; k < G; ++k) {
-    const double fac = 1.0 / (1.0 + cl * dt * (kT * gc.efac[k % Gs] + sig));
+    const double fac = rcp_pos(1.0 + cl * dt * (kT * gc.efac[k % Gs] + sig));
 #pragma unroll
     for (int q = 0; q < D; ++q) {
       R* Fp = FXP(U, rad + (uint32_t)(1 + q) * ncell * (uint32_t)G + c * (uint32_t)G + k, A.n_state);
@@ -349,6 +305,309 @@ __global__ void __launch_bounds__(CPLYE_THREADS) couple_ye_kernel(const __grid_c
     if (dwork != 0.0) atomicAdd(row + 6, dwork * ic2 * wv);
     if (fadd != 0.0) atomicAdd(row + 7, fadd * wv);
   }
+}
+
+// ---------------------------------------------------------------------------------------------
+// The same interaction for the FP32 state.  It was bound by the FP64 pipe (85 % busy): per-channel
+// sums, the flux absorption and the conserved updates in FP64 made ~1500 FP64 lane operations per
+// cell of 24 channels, and its rows were read and written one thread per cell, uncoalesced.  Here
+//   - the rows are staged through shared memory in coalesced copies (stage_rows);
+//   - what was summed in FP64 over channels is summed in pairs of floats that keep every rounding
+//     error (TwoSum), and the differences E - E^- and F_new - F are formed exactly as such pairs, so
+//     FP64 is left to the iterate, the residuals, the Jacobian's solve and the gas and composition
+//     updates;
+//   - the absorption factor 1/(1 + tau) of a group is one FP64 argument split into a float pair, its
+//     reciprocal corrected to a pair, so that F_new carries one FP32 rounding as before;
+//   - dr_E/dY_e vanishes identically (the weights w of nu_e and anti-nu_e have opposite derivatives
+//     and one opacity), so the 2 x 2 solve is two divisions;
+//   - every evaluation keeps its channel energies, so a run that ends on the residual test needs no
+//     evaluation more.
+// 512^2 cells x 24 channels: 0.72 -> 0.24 ms per launch (with the composition kernel).
+// ---------------------------------------------------------------------------------------------
+struct FPair { float h, l; };  // the sum h + l
+__device__ __forceinline__ void acc(FPair& a, float x) {
+  float s, e;
+  two_sum(a.h, x, s, e);
+  a.h = s;
+  a.l += e;
+}
+__device__ __forceinline__ void two_diff(float a, float b, float& s, float& e) {
+  s = a - b;
+  const float bv = s - a;
+  e = (a - (s - bv)) - (b + bv);
+}
+// a += x - y, the difference exact
+__device__ __forceinline__ void acc_diff(FPair& a, float x, float y) {
+  float d, f, s, e;
+  two_diff(x, y, d, f);
+  two_sum(a.h, d, s, e);
+  a.h = s;
+  a.l += e + f;
+}
+__device__ __forceinline__ double val(FPair a) { return (double)a.h + (double)a.l; }
+
+constexpr int couple_ye32_rows(int D) { return D > 2 ? D : 2; }
+template <int D> inline size_t couple_ye32_smem_bytes(int G) {
+  return (size_t)couple_ye32_rows(D) * CPL_THREADS * (size_t)(G + 1) * sizeof(float);
+}
+
+template <int D>
+__global__ void __launch_bounds__(CPL_THREADS, 5) couple_ye32_kernel(const __grid_constant__ StageArgs<float> A) {
+  constexpr int NG = 2 + D;
+  extern __shared__ __align__(16) unsigned char ye_raw[];
+  float* const srow = reinterpret_cast<float*>(ye_raw);  // E^- and E, then the F_q
+  __shared__ float s_ef[MAXG], s_ed[MAXG + 1], s_xi[MAXG];
+  __shared__ double s_efd[MAXG], s_xid[MAXG];
+  const DevGrid& g = A.g;
+  const int G = g.G, Gs = g.Gs, RS = G + 1, t = (int)threadIdx.x;
+  const uint32_t ncell = (uint32_t)g.ncell;
+  const uint32_t c0 = blockIdx.x * (uint32_t)CPL_THREADS, c = c0 + (uint32_t)t;
+  const int nc = (int)min((uint32_t)CPL_THREADS, ncell - c0);
+  const bool act = t < nc;
+  for (int j = t; j <= Gs; j += CPL_THREADS) {
+    s_ed[j] = A.gc->edge32[j];
+    if (j < Gs) {
+      s_ef[j] = A.gc->efac32[j];
+      s_efd[j] = A.gc->efac[j];
+      const double xi = g.xi0 * (1.0 / sqrt(A.gc->edge[j] * A.gc->edge[j + 1]));
+      s_xid[j] = xi;
+      s_xi[j] = (float)xi;
+    }
+  }
+  stage_rows<true>(FXPR(A.out, (size_t)NG * ncell + (size_t)c0 * G, nc * G, A.n_state), srow, nc, G, RS);
+  __syncthreads();
+  float* const Em = srow + t * RS;
+  float* const En = srow + (CPL_THREADS + t) * RS;
+  float* const U = A.out;
+  const uint32_t XO = (uint32_t)(NG + (1 + D) * G) * ncell;
+  unsigned st = 0;
+  double rho = 1.0, m[D], hq[D], ke = 0.0, ue = 0.0, T = 1.0, Xn = 0.0, kpre = 0.0, fadd = 0.0;
+#pragma unroll
+  for (int q = 0; q < D; ++q) { m[q] = 0.0; hq[q] = 1.0; }
+  const double cdt = A.kd.cdts;
+  if (act) {
+    rho = U[FXI(c, A.n_state)];
+    if (rho < g.rho_floor) { rho = g.rho_floor; st |= ST_FLOOR; }
+    // scale factors h_0, h_1 of the cell (1 on Cartesian grids): momentum and flux are covariant
+    if (g.geom != 0) {
+      const int i3[3] = {(int)(c % (uint32_t)g.n[0]), (int)((c / (uint32_t)g.n[0]) % (uint32_t)g.n[1]), 0};
+#pragma unroll
+      for (int d = 0; d < D; ++d) {
+        const Tab<float> td{A.tab[d], g.n[d] + 4, A.uniform[d] ? A.urow[d] : nullptr};
+        hq[0] *= (double)td(T_HA, bc_pad(i3[d]));
+        if (D > 1) hq[D > 1 ? 1 : 0] *= (double)td(T_HB, bc_pad(i3[d]));
+      }
+    }
+    const double irho = rcp_any(rho);
+#pragma unroll
+    for (int q = 0; q < D; ++q) {
+      m[q] = U[FXI((1 + q) * ncell + c, A.n_state)];
+      const double vh = g.geom != 0 ? m[q] * irho / hq[q] : m[q] * irho;
+      ke = fma(0.5 * rho * vh, vh, ke);
+    }
+    double u_m = (double)U[FXI((NG - 1) * ncell + c, A.n_state)] - ke;
+    const double u_floor = A.kd.u_floor;
+    if (u_m < u_floor) { u_m = u_floor; st |= ST_FLOOR; }
+    const double X_m = U[FXI(XO + c, A.n_state)], Y_m = X_m * irho;
+    // E^- with its silent floor, sum E^- and the tolerance's scale sum |xi| E^-
+    FPair Es = {0.0f, 0.0f};
+    float Ls = 0.0f;
+    const float flo = (float)g.E_floor;
+    for (int gg = 0; gg < Gs; ++gg) {
+      float ab = 0.0f;
+#pragma unroll
+      for (int s = 0; s < 3; ++s) {
+        float e = Em[s * Gs + gg];
+        if (e < flo) {
+          fadd += g.E_floor - (double)e;
+          e = flo;
+          Em[s * Gs + gg] = e;
+        }
+        acc(Es, e);
+        if (s < 2) ab += e;
+      }
+      Ls = fmaf(s_xi[gg], ab, Ls);
+    }
+    kpre = A.kd.kappa0 * hpow(rho, g.kap_rho_h);
+    const float kpref = (float)kpre, cdtf = A.kf.cdts;
+    const double rcv = rho * A.kd.cv;
+    // residuals r_E, r_X and dr_E/dT, dr_X/dT, dr_X/dY at (T, Y); the channel energies into En
+    auto eval = [&](double Tq, double Yq, double& rE, double& rX, double& JT, double& JX, double& JY) {
+      const float Tf = (float)Tq, Yf = (float)Yq;
+      const PlanckAt pa = planck_at(A.ptab, A.kf.aN, Tf);
+      const float kTf = cdtf * (kpref * hpow(Tf, g.kap_T_h)), hTf = 0.5f * (float)g.kap_T_h * pa.invT;
+      const float w0 = 2.0f * Yf, w1 = 2.0f * (1.0f - Yf);
+      FPair dE = {0.0f, 0.0f}, dX = dE, eT = dE, xT = dE, xY = dE;
+      for (int gg = 0; gg < Gs; ++gg) {
+        float Bf, dBf;
+        planck_group(A.ptab, pa, gg, s_ed, Bf, dBf);
+        const float tf = kTf * s_ef[gg], invf = frcp(1.0f + tf), xf = s_xi[gg];
+        float d[3], dt_[3];
+#pragma unroll
+        for (int s = 0; s < 3; ++s) {
+          const int k = s * Gs + gg;
+          const float w = s == 0 ? w0 : (s == 1 ? w1 : 1.0f);
+          const float Emk = Em[k], Eq = w * Bf;
+          const float Ek = fmaf(tf, Eq, Emk) * invf;
+          dt_[s] = tf * fmaf(hTf, Eq - Ek, w * dBf) * invf;
+          d[s] = Ek - Emk;
+          En[k] = Ek;
+        }
+        acc(dE, d[0] + d[1] + d[2]);
+        acc(dX, xf * (d[1] - d[0]));
+        acc(eT, dt_[0] + dt_[1] + dt_[2]);
+        acc(xT, xf * (dt_[1] - dt_[0]));
+        acc(xY, -4.0f * xf * (tf * Bf * invf));
+      }
+      rE = fma(rcv, Tq, -u_m) + val(dE);
+      rX = fma(rho, Yq - Y_m, -val(dX));
+      JT = rcv + val(eT);
+      JX = -val(xT);
+      JY = rho - val(xY);
+    };
+    // stopping tests at FP32 resolution (relative step 2e-7 at least, residual 1e-7)
+    const double rtol = A.kd.rtol, n2ok = A.kd.atol * A.kd.atol;
+    const double isE = rcp_any(u_m + val(Es)), isX = rcp_any(fabs(X_m) + (double)Ls + 1e-300);
+    auto norm2 = [&](double rE, double rX) { const double a = rE * isE, b = rX * isX; return fma(a, a, b * b); };
+    double Y = Y_m, rE, rX, JT, JX, JY;
+    T = u_m * rcp_any(rcv);
+    eval(T, Y, rE, rX, JT, JX, JY);
+    bool ok = false, fresh = true;  // fresh: En holds the energies at (T, Y)
+    double n0 = norm2(rE, rX);
+    for (int it = 0; it < g.newton_maxit; ++it) {
+      if (n0 <= n2ok) { ok = true; break; }
+      const double dT = -rE * rcp_any(JT), dY = -fma(JX, dT, rX) * rcp_any(JY);
+      if (fabs(dT) <= rtol * T && fabs(dY) <= rtol * fmax(Y, 1e-3)) {
+        T = T + dT;
+        Y = Y + dY;
+        ok = true;
+        fresh = false;
+        break;
+      }
+      double lam = 1.0;
+      bool got = false;
+      for (int ls = 0; ls < 40; ++ls) {
+        const double Tt = fma(lam, dT, T), Yt = fma(lam, dY, Y);
+        if (Tt > 0.0 && Yt >= 0.0 && Yt <= 1.0) {
+          double rEt, rXt, JTt, JXt, JYt;
+          eval(Tt, Yt, rEt, rXt, JTt, JXt, JYt);
+          const double nt = norm2(rEt, rXt);
+          fresh = false;
+          if (nt < n0) {
+            T = Tt; Y = Yt; rE = rEt; rX = rXt; JT = JTt; JX = JXt; JY = JYt; n0 = nt;
+            got = fresh = true;
+            break;
+          }
+        }
+        lam *= 0.5;
+      }
+      if (!got) break;
+    }
+    if (!ok) {
+      // alternating bisections (reading R33)
+      for (int round = 0; round < 20 && !ok; ++round) {
+        double r1, r2, rh, rm, j0, j1, j2;
+        double lo = 0.5 * T, hi = 2.0 * T;
+        eval(lo, Y, r1, r2, j0, j1, j2);
+        for (int k = 0; k < 200 && r1 > 0.0; ++k) { lo = 0.5 * lo; eval(lo, Y, r1, r2, j0, j1, j2); }
+        eval(hi, Y, rh, r2, j0, j1, j2);
+        for (int k = 0; k < 200 && rh < 0.0; ++k) { hi = 2.0 * hi; eval(hi, Y, rh, r2, j0, j1, j2); }
+        for (int k = 0; k < g.bisect_maxit && hi - lo > rtol * hi; ++k) {
+          const double mid = 0.5 * (lo + hi);
+          eval(mid, Y, rm, r2, j0, j1, j2);
+          if (rm > 0.0) hi = mid; else lo = mid;
+        }
+        T = 0.5 * (lo + hi);
+        double ylo = 0.0, yhi = 1.0;
+        for (int k = 0; k < g.bisect_maxit && yhi - ylo > rtol; ++k) {
+          const double mid = 0.5 * (ylo + yhi);
+          eval(T, mid, r1, rm, j0, j1, j2);
+          if (rm > 0.0) yhi = mid; else ylo = mid;
+        }
+        Y = 0.5 * (ylo + yhi);
+        eval(T, Y, rE, rX, j0, j1, j2);
+        if (norm2(rE, rX) <= n2ok) ok = true;
+      }
+      fresh = true;
+      if (!ok) st |= ST_NEWTON;
+    }
+    if (!fresh) eval(T, Y, rE, rX, JT, JX, JY);
+    // u and rho Y_e by conservation from the accepted channel energies
+    FPair dE = {0.0f, 0.0f};
+    Xn = X_m;
+    for (int gg = 0; gg < Gs; ++gg) {
+      FPair d = {0.0f, 0.0f};  // the group's anti-nu_e less nu_e changes
+#pragma unroll
+      for (int s = 0; s < 3; ++s) {
+        const float e1 = En[s * Gs + gg], e0 = Em[s * Gs + gg];
+        acc_diff(dE, e1, e0);
+        if (s == 0) acc_diff(d, e0, e1);
+        if (s == 1) acc_diff(d, e1, e0);
+      }
+      Xn = fma(s_xid[gg], val(d), Xn);
+    }
+    ue = ke + (u_m - val(dE));
+  }
+  __syncthreads();
+  // the new E back, then the F rows into the same shared rows
+  stage_rows<false>(FXPR(A.out, (size_t)NG * ncell + (size_t)c0 * G, nc * G, A.n_state), srow + CPL_THREADS * RS, nc, G, RS);
+  __syncthreads();
+#pragma unroll
+  for (int q = 0; q < D; ++q)
+    stage_rows<true>(FXPR(A.out, (size_t)NG * ncell + ((size_t)(1 + q) * ncell + c0) * G, nc * G, A.n_state), srow + q * CPL_THREADS * RS, nc, G, RS);
+  __syncthreads();
+  double dwork = 0.0;
+  if (act) {
+    // flux absorption (Eq. 28) with its momentum and energy feedback (Eqs. 31-32)
+    FPair dm[D];
+#pragma unroll
+    for (int q = 0; q < D; ++q) dm[q] = {0.0f, 0.0f};
+    const double sig = g.sigma0 * rho, kT = kpre * hpow(T, g.kap_T_h);
+    for (int gg = 0; gg < Gs; ++gg) {
+      const double x = fma(cdt, fma(kT, s_efd[gg], sig), 1.0);
+      const float xh = (float)x, xl = (float)(x - (double)xh);
+      const float fh = frcp(xh), fl = fh * (fmaf(-xh, fh, 1.0f) - xl * fh);  // 1/x = fh + fl
+#pragma unroll
+      for (int s = 0; s < 3; ++s) {
+#pragma unroll
+        for (int q = 0; q < D; ++q) {
+          float* const r = srow + (q * CPL_THREADS + t) * RS + s * Gs + gg;
+          const float F = *r, Fn = fmaf(F, fh, F * fl);
+          acc_diff(dm[q], Fn, F);
+          *r = Fn;
+        }
+      }
+    }
+    const double ic2 = A.kd.ic2, irho = rcp_any(rho);
+    double mn[D];
+    bool bad = false;
+#pragma unroll
+    for (int q = 0; q < D; ++q) {
+      const double d = val(dm[q]), v = g.geom != 0 ? m[q] * irho / (hq[q] * hq[q]) : m[q] * irho;
+      dwork = fma(v, d, dwork);
+      mn[q] = fma(-d, ic2, m[q]);
+      bad |= !isfinite(mn[q]);
+    }
+    ue -= dwork * ic2;
+    A.out[FXI(c, A.n_state)] = (float)rho;
+#pragma unroll
+    for (int q = 0; q < D; ++q) A.out[FXI((1 + q) * ncell + c, A.n_state)] = (float)mn[q];
+    A.out[FXI((NG - 1) * ncell + c, A.n_state)] = (float)ue;
+    A.out[FXI(XO + c, A.n_state)] = (float)Xn;
+    bad |= !isfinite(ue) || !isfinite(Xn);
+    if (bad) st |= ST_NONFINITE;
+    if (st) atomicOr(A.status, st);
+    if (A.budget != nullptr) {
+      const double wv = cell_volume(A, c) * A.bw_cpl;
+      double* row = A.budget + (size_t)(blockIdx.x % BUDGET_SLOTS) * NBUDGET;
+      if (dwork != 0.0) atomicAdd(row + 6, dwork * ic2 * wv);
+      if (fadd != 0.0) atomicAdd(row + 7, fadd * wv);
+    }
+  }
+  __syncthreads();
+#pragma unroll
+  for (int q = 0; q < D; ++q)
+    stage_rows<false>(FXPR(A.out, (size_t)NG * ncell + ((size_t)(1 + q) * ncell + c0) * G, nc * G, A.n_state), srow + q * CPL_THREADS * RS, nc, G, RS);
 }
 
 }  // namespace fx
