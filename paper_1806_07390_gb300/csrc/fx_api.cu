@@ -452,11 +452,44 @@ void build_planck_table(const fx_params& P, const GroupConst& gc, const PlanckPa
     }
 }
 
+// Coefficients of one interval (see PlanckTable) from its two nodes (L - floor(L), h dL/du, floor(L),
+// 2^floor(L)).
+void planck_interval_entry(const float4& p, const float4& q, float c[4]) {
+  const double d = ((double)q.z - (double)p.z) + ((double)q.x - (double)p.x);  // L at the right node less L at the left
+  const double m0 = p.y, m1 = q.y;
+  c[0] = p.x;
+  c[1] = p.y;
+  c[2] = (float)(3.0 * d - 2.0 * m0 - m1);
+  c[3] = (float)(m0 + m1 - 2.0 * d);
+  unsigned sc, b;
+  std::memcpy(&sc, &p.w, 4);
+  std::memcpy(&b, &c[3], 4);
+  b = (b & ~0xffu) | (sc >> 23);
+  std::memcpy(&c[3], &b, 4);
+}
+// The device table: (groups + 1)/2 pairs (an odd count's last pair repeats its group).
+std::vector<float4> planck_device_table(const std::vector<float4>& tab, int G, int nu, bool node_major) {
+  const int NP = (G + 1) / 2;
+  std::vector<float4> out((size_t)2 * NP * nu);
+  for (int p = 0; p < NP; ++p)
+    for (int i = 0; i < nu; ++i) {
+      float c[2][4];
+      for (int s = 0; s < 2; ++s) {
+        const float4* const t = tab.data() + (size_t)std::min(2 * p + s, G - 1) * nu;
+        planck_interval_entry(t[i], t[std::min(i + 1, nu - 1)], c[s]);
+      }
+      float4* const e = out.data() + 2 * (node_major ? (size_t)i * NP + p : (size_t)p * nu + i);
+      e[0] = make_float4(c[0][0], c[1][0], c[0][1], c[1][1]);
+      e[1] = make_float4(c[0][2], c[1][2], c[0][3], c[1][3]);
+    }
+  return out;
+}
+
 // Layout of the device Planck table, a measured choice (interaction kernel per launch, node-major
-// against group-major): kh2d (2-d, 16 groups) 0.142 against 0.156 ms; lognormal3d (3-d, 12
-// groups) 3.77 against 3.47 ms; blobs2d (2-d, 8 groups) 0.033 against 0.029 ms.  A warp's cells
-// read nodes i and i+1 of every group: group-major keeps the lanes' nodes of one group on one
-// cache line when their temperatures differ, node-major keeps a lane's groups together.
+// against group-major): 1024^2 x 16 0.118 against 0.121 ms, 256^3 x 12 2.89 against 2.75 ms, 515 x 389
+// x 7 0.026 against 0.025 ms.  A warp's cells read the intervals of their temperatures of every pair
+// of groups: group-major keeps the lanes' intervals of one pair on one cache line when their
+// temperatures differ, node-major keeps a lane's pairs together.
 bool ptab_node_major(const fx_grid* h) { return h->D <= 2 && h->P.ngroups >= 16; }
 
 // The FP64 scale-factor rows T_HA, T_HB of every direction, as k_init_equilibrium reads them.
@@ -726,13 +759,13 @@ StageArgs<R> stage_args(fx_grid* h) {
   a.ptab.tab = reinterpret_cast<const float4*>(h->ws + h->off_ptab);
   a.ptab.nu = h->ptab_nu;
   a.ptab.u0 = h->ptab_u0;
-  a.ptab.si = ptab_node_major(h) ? h->P.ngroups : 1;
+  a.ptab.si = ptab_node_major(h) ? (h->P.ngroups + 1) / 2 : 1;
   a.ptab.sg = ptab_node_major(h) ? 1 : h->ptab_nu;
   a.pk = h->pk;
   a.pk.petab = h->elem == 8 ? reinterpret_cast<const double*>(h->ws + h->off_petab) : nullptr;
   a.status = reinterpret_cast<unsigned*>(h->ws + h->off_status);
 #ifdef FX_BOUNDS_CHECK
-  a.ptab.n = (int)h->ptab.size();
+  a.ptab.n = 2 * h->ptab_nu * ((h->P.ngroups + 1) / 2);
   a.ptab.status = a.status;
   a.n_state = h->ncell * h->NV;
   a.n_faces = h->faces_elems;
@@ -1286,7 +1319,7 @@ fx_status fx_grid_create(const fx_params* params, fx_grid** out, size_t* workspa
     h->off_hrow = off; off = align_up(off + nh * sizeof(double));
   }
   h->off_vtc = off; off = align_up(off + sizeof(VtConst));
-  h->off_ptab = off; off = align_up(off + h->ptab.size() * sizeof(float4));
+  h->off_ptab = off; off = align_up(off + (size_t)2 * h->ptab_nu * ((P.ngroups + 1) / 2) * sizeof(float4));
   h->off_petab = off;
   if (h->elem == 8) off = align_up(off + planck_edge_table().size() * sizeof(double));
   {
@@ -1626,10 +1659,7 @@ fx_status fx_bind_workspace(fx_grid* h, void* dev_ptr, size_t bytes, void* cuda_
   {  // the device copy in the layout ptab_node_major picks; the host keeps the group-major table
     // (one table per group, ngroups of them: with three species the channels share them)
     const int G = h->P.ngroups, nu = h->ptab_nu;
-    const bool nmaj = ptab_node_major(h);
-    std::vector<float4> nm((size_t)G * nu);
-    for (int g = 0; g < G; ++g)
-      for (int i = 0; i < nu; ++i) nm[nmaj ? (size_t)i * G + g : (size_t)g * nu + i] = h->ptab[(size_t)g * nu + i];
+    const std::vector<float4> nm = planck_device_table(h->ptab, G, nu, ptab_node_major(h));
     e = cudaMemcpyAsync(h->ws + h->off_ptab, nm.data(), nm.size() * sizeof(float4),
                         cudaMemcpyHostToDevice, h->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);

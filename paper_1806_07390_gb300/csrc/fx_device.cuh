@@ -439,20 +439,28 @@ __device__ __forceinline__ void m1_row(R ic2, V E, const V* F, int n, V* P) {
 }
 
 // ---------------------------------------------------------------------------------------------
-// Powers with half-integer exponents, evaluated with correctly rounded operations only.
+// Powers with half-integer exponents: x^(h/2) = x^k sqrt(x)^(h mod 2), k = floor(h/2), by binary
+// powers and one reciprocal for k < 0.  The exponent is the launch's: every branch is uniform, and
+// the common |k| < 8 take no loop (with a loop and signed divisions the powers were a fifth of the
+// interaction kernel's instructions).
 // ---------------------------------------------------------------------------------------------
-template <class R> __device__ __forceinline__ R ipow(R x, int n) {
-  R r = R(1), b = x;
-  int m = n < 0 ? -n : n;
-  while (m) { if (m & 1) r *= b; b *= b; m >>= 1; }
-  return n < 0 ? R(1) / r : r;
-}
-// x^(h/2) for integer h (exponent in halves)
 template <class R> __device__ __forceinline__ R hpow(R x, int h) {
-  if (h % 2 == 0) return ipow(x, h / 2);
-  int k = (h - 1) / 2;  // h = 2k + 1 -> x^k sqrt(x)
-  R s = sqrt(x);
-  return k >= 0 ? ipow(x, k) * s : s / ipow(x, -k);
+  const int k = h >> 1, n = k < 0 ? -k : k;
+  R r = n & 1 ? x : R(1);
+  if (n > 1) {
+    R b = x * x;
+    if (n & 2) r = r * b;
+    if (n > 3) {
+      b = b * b;
+      if (n & 4) r = r * b;
+      for (int m = n >> 3; m; m >>= 1) {
+        b = b * b;
+        if (m & 1) r = r * b;
+      }
+    }
+  }
+  if (k < 0) r = rcp_any(r);
+  return h & 1 ? r * sqrt_any(x) : r;
 }
 
 // ---------------------------------------------------------------------------------------------

@@ -43,19 +43,24 @@ struct PlanckParams {
   float wd32[NPLANCK_LO32];
 };
 
-// FP32 Planck band tables: for group g and u = log2 T on nodes u0 + i/PTAB_PER_OCT, the pair
-// (L, h dL/du) with L = log2 Int_{eps_g-1/2/T}^{eps_g+1/2/T} t^3/(e^t-1) dt, built on the host in
-// FP64 and interpolated with cubic Hermite polynomials.
+// FP32 Planck band tables on nodes u0 + i/PTAB_PER_OCT of u = log2 T: per group and interval [i, i+1]
+// the cubic Hermite polynomial of L(u) = log2 Int_{eps_g-1/2/T}^{eps_g+1/2/T} s^3/(e^s-1) ds through
+// the nodes' values and slopes (built on the host in FP64), as
+//   L - k = c0 + c1 t + c2 t^2 + c3 t^3,  k = floor(L) at the left node, t in [0, 1].
+// The low eight bits of c3, whose term is below 3e-4, hold the exponent field of 2^k (0: 2^k below
+// 2^-126, the band flushes to zero), so that small numbers are interpolated and the scale is exact.
+// Two groups' coefficients are interleaved, (c0 c0' c1 c1'), (c2 c2' c3 c3'), so that an evaluation
+// for both reads two 16-byte words straight into packed FP32 pairs (the nodes' values and slopes were
+// four words for two groups).
 struct PlanckTable {
-  // entry (node i, group g) at tab[i * si + g * sg]: (L - floor(L), h dL/du, floor(L), 2^floor(L)
-  // or 0 below 2^-126).  An evaluation reads nodes i and i+1 of every group; the host picks the
-  // layout (node-major si = G, sg = 1, or group-major si = 1, sg = nu)
+  // interval i, pair p of groups at tab[2 (i * si + p * sg)]; the host picks the layout (node-major
+  // si = pairs, sg = 1, or group-major si = 1, sg = nu)
   const float4* tab;
-  int nu;
+  int nu;            // nodes
   float u0;
   int si, sg;
 #ifdef FX_BOUNDS_CHECK
-  int n;             // entries (nu x groups), for the index checks of the debug build
+  int n;             // words (2 x nu x pairs), for the index checks of the debug build
   unsigned* status;  // status word those checks report to
 #endif
 };
@@ -138,6 +143,14 @@ template <class R> struct StageArgs {
   __device__ __forceinline__ const Consts<double>& k(double) const { return kd; }
   __device__ __forceinline__ const Consts<float>& k(float) const { return kf; }
 };
+
+__device__ __forceinline__ float ex2_approx(float x) {  // 2^x, relative error about 2^-22
+  float y;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+// 2^k from the low bits of c3
+__device__ __forceinline__ float planck_scale(float c3) { return __uint_as_float((__float_as_uint(c3) << 23) & 0x7f800000u); }
 
 __device__ __forceinline__ int bc_pad(int i) { return i + 2; }  // padded table row of cell i
 
@@ -279,16 +292,10 @@ struct LanePlanck {
     } else {
       const int i = (int)s;
       const float t = s - (float)i;
-      const float4 p0 = __ldg(FXP_AT(ptab.status, ptab.tab, i * ptab.si + lane * ptab.sg, ptab.n));
-      const float4 p1 = __ldg(FXP_AT(ptab.status, ptab.tab, (i + 1) * ptab.si + lane * ptab.sg, ptab.n));
-      const float t2 = t * t, t3 = t2 * t;
-      // node values relative to floor(L) of the left node: small numbers, full FP32 precision
-      const float d1 = (p1.z - p0.z) + p1.x;
-      const float Lr = (2.0f * t3 - 3.0f * t2 + 1.0f) * p0.x + (t3 - 2.0f * t2 + t) * p0.y +
-                       (3.0f * t2 - 2.0f * t3) * d1 + (t3 - t2) * p1.y;
-      const float dLdt = (6.0f * t2 - 6.0f * t) * (p0.x - d1) + (3.0f * t2 - 4.0f * t + 1.0f) * p0.y +
-                         (3.0f * t2 - 2.0f * t) * p1.y;
-      I = exp2f(Lr) * p0.w;
+      const float* const c = reinterpret_cast<const float*>(FXP_AT(ptab.status, ptab.tab, 2 * (i * ptab.si + (lane >> 1) * ptab.sg), ptab.n - 1)) + (lane & 1);
+      const float c0 = __ldg(c), c1 = __ldg(c + 2), c2 = __ldg(c + 4), c3 = __ldg(c + 6);
+      const float dLdt = fmaf(fmaf(3.0f * c3, t, 2.0f * c2), t, c1);
+      I = ex2_approx(fmaf(fmaf(fmaf(c3, t, c2), t, c1), t, c0)) * planck_scale(c3);
       dLdu = dLdt * float(PTAB_PER_OCT);
     }
     const float T2 = T * T, T3 = T2 * T;

@@ -311,7 +311,7 @@ __global__ void __launch_bounds__(CPLYE_THREADS) couple_ye_kernel(const __grid_c
 // The same interaction for the FP32 state.  It was bound by the FP64 pipe (85 % busy): per-channel
 // sums, the flux absorption and the conserved updates in FP64 made ~1500 FP64 lane operations per
 // cell of 24 channels, and its rows were read and written one thread per cell, uncoalesced.  Here
-//   - the rows are staged through shared memory in coalesced copies (stage_rows);
+//   - the rows are staged through shared memory in coalesced copies (RowCopy);
 //   - what was summed in FP64 over channels is summed in pairs of floats that keep every rounding
 //     error (TwoSum), and the differences E - E^- and F_new - F are formed exactly as such pairs, so
 //     FP64 is left to the iterate, the residuals, the Jacobian's solve and the gas and composition
@@ -374,7 +374,8 @@ __global__ void __launch_bounds__(CPL_THREADS, 5) couple_ye32_kernel(const __gri
       s_xi[j] = (float)xi;
     }
   }
-  stage_rows<true>(FXPR(A.out, (size_t)NG * ncell + (size_t)c0 * G, nc * G, A.n_state), srow, nc, G, RS);
+  const RowCopy rc(A.out + ((size_t)NG * ncell + (size_t)c0 * G), nc, G, RS);
+  rc.run<true, false>(FXPR(A.out, (size_t)NG * ncell + (size_t)c0 * G, nc * G, A.n_state), srow);
   __syncthreads();
   float* const Em = srow + t * RS;
   float* const En = srow + (CPL_THREADS + t) * RS;
@@ -438,9 +439,10 @@ __global__ void __launch_bounds__(CPL_THREADS, 5) couple_ye32_kernel(const __gri
       const float kTf = cdtf * (kpref * hpow(Tf, g.kap_T_h)), hTf = 0.5f * (float)g.kap_T_h * pa.invT;
       const float w0 = 2.0f * Yf, w1 = 2.0f * (1.0f - Yf);
       FPair dE = {0.0f, 0.0f}, dX = dE, eT = dE, xT = dE, xY = dE;
+      F2 B2(0.0f), dB2(0.0f);
       for (int gg = 0; gg < Gs; ++gg) {
-        float Bf, dBf;
-        planck_group(A.ptab, pa, gg, s_ed, Bf, dBf);
+        if ((gg & 1) == 0) planck_pair(A.ptab, pa, gg >> 1, Gs, s_ed, B2, dB2);
+        const float Bf = gg & 1 ? B2.y : B2.x, dBf = gg & 1 ? dB2.y : dB2.x;
         const float tf = kTf * s_ef[gg], invf = frcp(1.0f + tf), xf = s_xi[gg];
         float d[3], dt_[3];
 #pragma unroll
@@ -550,11 +552,11 @@ __global__ void __launch_bounds__(CPL_THREADS, 5) couple_ye32_kernel(const __gri
   }
   __syncthreads();
   // the new E back, then the F rows into the same shared rows
-  stage_rows<false>(FXPR(A.out, (size_t)NG * ncell + (size_t)c0 * G, nc * G, A.n_state), srow + CPL_THREADS * RS, nc, G, RS);
+  rc.run<false, false>(FXPR(A.out, (size_t)NG * ncell + (size_t)c0 * G, nc * G, A.n_state), srow + CPL_THREADS * RS);
   __syncthreads();
 #pragma unroll
   for (int q = 0; q < D; ++q)
-    stage_rows<true>(FXPR(A.out, (size_t)NG * ncell + ((size_t)(1 + q) * ncell + c0) * G, nc * G, A.n_state), srow + q * CPL_THREADS * RS, nc, G, RS);
+    rc.run<true, false>(FXPR(A.out, (size_t)NG * ncell + ((size_t)(1 + q) * ncell + c0) * G, nc * G, A.n_state), srow + q * CPL_THREADS * RS);
   __syncthreads();
   double dwork = 0.0;
   if (act) {
@@ -607,7 +609,7 @@ __global__ void __launch_bounds__(CPL_THREADS, 5) couple_ye32_kernel(const __gri
   __syncthreads();
 #pragma unroll
   for (int q = 0; q < D; ++q)
-    stage_rows<false>(FXPR(A.out, (size_t)NG * ncell + ((size_t)(1 + q) * ncell + c0) * G, nc * G, A.n_state), srow + q * CPL_THREADS * RS, nc, G, RS);
+    rc.run<false, false>(FXPR(A.out, (size_t)NG * ncell + ((size_t)(1 + q) * ncell + c0) * G, nc * G, A.n_state), srow + q * CPL_THREADS * RS);
 }
 
 }  // namespace fx
