@@ -50,6 +50,14 @@ __device__ __forceinline__ double sqrt64(double a) {
   h = fma(h, r, h);
   return fma(fma(-g, g, a), h, g);
 }
+// 1/sqrt(a) for normal positive a: the hardware seed y with e = 1 - a y^2, and the series of
+// (1 - e)^(-1/2) to its second power, y (1 + e/2 + 3 e^2/8).
+__device__ __forceinline__ double rsqrt64(double a) {
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(a));
+  const double e = fma(-(a * y), y, 1.0);
+  return fma(y * e, fma(e, 0.375, 0.5), y);
+}
 // 1 / max(t, 1)
 __device__ __forceinline__ double rcp_ge1(double t) {
   const int hi = __double2hiint(t);

@@ -147,18 +147,12 @@ static cudaError_t launch_gp(const StageArgs<R>& a0, cudaStream_t s, cudaEvent_t
     if (e != cudaSuccess) return e;
   }
   // the velocity-dependent radiation terms of the stage input, added to the explicit update
-  // before the interaction (one lane per group)
+  // before the interaction
   if (a.g.vterms) {
-    if constexpr (std::is_same<R, float>::value && GP >= 16) {
-      // FP32 forms from 9 groups: two groups per lane, GP/2 lanes per cell
-      constexpr int CPB = VT_THREADS / (GP / 2);
-      const dim3 vg((unsigned)(a.g.n[1] * a.g.n[2]), (unsigned)((a.g.n[0] + CPB - 1) / CPB), 1);
-      vterm_kernel2<D, GP / 2, SPH><<<vg, VT_THREADS, 0, s>>>(a);
-    } else {
-      constexpr int CPB = VT_THREADS / GP;  // cells of one x row per block, GP lanes each
-      const dim3 vg((unsigned)(a.g.n[1] * a.g.n[2]), (unsigned)((a.g.n[0] + CPB - 1) / CPB), 1);
-      vterm_kernel<R, D, GP, SPH><<<vg, VT_THREADS, 0, s>>>(a);
-    }
+    constexpr int W = LaneOf<R>::W;
+    const int cells = VT_THREADS / 32 * (32 / ((a.g.G + W - 1) / W));  // cells of one x row per block
+    const dim3 vg((unsigned)((a.g.n[1] * a.g.n[2] + VT_ROWS - 1) / VT_ROWS), (unsigned)((a.g.n[0] + cells - 1) / cells), 1);
+    vterm_kernel<R, D, SPH><<<vg, VT_THREADS, 0, s>>>(a);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }

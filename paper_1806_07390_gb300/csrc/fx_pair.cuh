@@ -150,6 +150,16 @@ __device__ __forceinline__ void st_lane(float* p, F2 v, bool h0, bool h1) {
   else if (h0) *p = v.x;
 }
 
+// Global load of a lane's groups: one 8-byte load where the pair is aligned (vec), else one by one
+// (an absent second group is zero).
+__device__ __forceinline__ double ld_global_lane(const double* p, bool, bool, double) { return *p; }
+__device__ __forceinline__ F2 ld_global_lane(const float* p, bool vec, bool h1, F2) {
+  if (vec) {
+    const float2 v = *reinterpret_cast<const float2*>(p);
+    return F2(v.x, v.y);
+  }
+  return F2(p[0], h1 ? p[1] : 0.0f);
+}
 // Global store of a lane's groups: one 8-byte store where the pair is aligned (vec: both exist).
 __device__ __forceinline__ void st_global_lane(double* p, double v, bool, bool) { *p = v; }
 __device__ __forceinline__ void st_global_lane(float* p, F2 v, bool vec, bool h1) {

@@ -18,6 +18,8 @@
 // transverse components of the reconstructed state on the v* upwind side (the spherical form is
 // described at the kernel).
 #pragma once
+#include <utility>
+
 #include "fx_stage.cuh"
 
 namespace fx {
@@ -43,54 +45,64 @@ __host__ __device__ constexpr int vt_sym3(int i, int j, int k, int D) {
   return idx + vt_sym2(b - a, c - a, D - a);
 }
 
-template <class R> __device__ __forceinline__ R vt_mc(R sL, R sR, R sC) {
-  if (sL * sR <= R(0)) return R(0);
-  const R m = fmin(fmin(R(2) * fabs(sL), R(2) * fabs(sR)), fabs(sC));
-  return sC > R(0) ? m : -m;
+// f(integral constant) for every index of the sequence
+template <int... I, class F> __device__ __forceinline__ void vt_each(std::integer_sequence<int, I...>, F f) {
+  (f(std::integral_constant<int, I>{}), ...);
 }
 
-// Components of P (units of E) and Q (units of F) of one group, the distinct ones in the order
-// of vt_sym2 / vt_sym3: x[0 .. NP) = P, x[NP .. NC) = Q.
-// 1/sqrt and 1/x: FP64 exact division and square root; FP32 the hardware approximations (a few
-// ulp), far inside the FP32 forms' tolerance.
-__device__ __forceinline__ double vt_rsqrt(double x) { return 1.0 / sqrt(x); }
-__device__ __forceinline__ float vt_rsqrt(float x) { return rsqrtf(x); }
-__device__ __forceinline__ double vt_rcp(double x) { return 1.0 / x; }
-__device__ __forceinline__ float vt_rcp(float x) { return __fdividef(1.0f, x); }
+// Reciprocals and roots of the closure for a lane's groups, 0 where the group has no flux or no
+// energy (then f = 0: P = E/3 isotropic, Q = 0).
+__device__ __forceinline__ void vt_roots(F2 FF, F2 cE, F2& iF, F2& iE) {
+  const bool a = FF.x > 0.0f && cE.x > 0.0f, b = FF.y > 0.0f && cE.y > 0.0f;
+  iF = F2(a ? rsqrtf(FF.x) : 0.0f, b ? rsqrtf(FF.y) : 0.0f);
+  iE = F2(a ? rcp_approx(cE.x) : 0.0f, b ? rcp_approx(cE.y) : 0.0f);
+}
+__device__ __forceinline__ void vt_roots(double FF, double cE, double& iF, double& iE) {
+  const bool ok = FF > 0.0 && cE > 0.0;
+  const int e = __double2hiint(FF);
+  iF = !ok ? 0.0 : (e >= 0x00400000 && e < 0x7fb00000 ? rsqrt64(FF) : 1.0 / sqrt(FF));
+  iE = ok ? rcp_any(cE) : 0.0;
+}
 
-template <class R, int D>
-__device__ __forceinline__ void vt_moments(R c, R E, const R* F, R* x) {
+// Components of P (units of E) and Q (units of F) of the lane's groups, in the order of vt_sym2 /
+// vt_sym3: x[0 .. NP) = P, x[NP .. NC) = Q.  With s = sqrt(4 - 3 f^2) the closure is polynomial in s:
+// (1 - chi)/2 = (s - 1)/3, (3 chi - 1)/2 = 2 - s, and with q = f (2 + 3 chi)/5 = f (7 - 2 s)/5,
+// (f - q)/2 = f (s - 1)/5, (5 q - 3 f)/2 = f (2 - s): one reciprocal of cE, one inverse root of F^2,
+// one square root.
+template <int D, class V>
+__device__ __forceinline__ void vt_moments(V c, V one, V p4, V m3, V E, const V* F, V* x) {
   using VC = VtComp<D>;
-  R F2 = R(0);
+  V FF = F[0] * F[0];
 #pragma unroll
-  for (int q = 0; q < D; ++q) F2 += F[q] * F[q];
+  for (int q = 1; q < D; ++q) FF = vfma(F[q], F[q], FF);
+  const V cE = E * c;
+  V iF, iE;
+  vt_roots(FF, cE, iF, iE);
+  const V f = vmin((FF * iF) * iE, one);
+  const V s = vsqrt(vfma(m3, f * f, p4)), s1 = s - one, b = (one + one) - s;
+  using T = decltype(vget(E, 0));
+  const V g = f * cE, a3 = E * s1 * T(1.0 / 3.0), bE = E * b, qa = g * s1 * T(0.2), qb = g * b;
+  V n[D];
 #pragma unroll
-  for (int m = 0; m < VC::NC; ++m) x[m] = R(0);
-  if (!(F2 > R(0)) || !(E > R(0))) {
-#pragma unroll
-    for (int i = 0; i < D; ++i) x[vt_sym2(i, i, D)] = E * R(1.0 / 3.0);
-    return;
-  }
-  const R iFm = vt_rsqrt(F2), cE = c * E;
-  const R f = fmin(F2 * iFm * vt_rcp(cE), R(1)), f2 = f * f;
-  const R chi = (R(3) + R(4) * f2) * vt_rcp(R(5) + R(2) * sqrt(R(4) - R(3) * f2));
-  const R q = f * (R(2) + R(3) * chi) * R(0.2);
-  const R a = R(0.5) * (R(1) - chi), b = R(0.5) * (R(3) * chi - R(1));
-  const R qa = R(0.5) * (f - q) * cE, qb = R(0.5) * (R(5) * q - R(3) * f) * cE;
-  R n[D];
-#pragma unroll
-  for (int i = 0; i < D; ++i) n[i] = F[i] * iFm;
-#pragma unroll
-  for (int i = 0; i < D; ++i)
-#pragma unroll
-    for (int j = i; j < D; ++j) {
-      x[vt_sym2(i, j, D)] = E * ((i == j ? a : R(0)) + b * n[i] * n[j]);
-#pragma unroll
-      for (int k = j; k < D; ++k)
-        x[VC::NP + vt_sym3(i, j, k, D)] =
-            qa * ((j == k ? n[i] : R(0)) + (i == k ? n[j] : R(0)) + (i == j ? n[k] : R(0))) +
-            qb * n[i] * n[j] * n[k];
+  for (int i = 0; i < D; ++i) n[i] = F[i] * iF;
+  vt_each(std::make_integer_sequence<int, D * D>{}, [&](auto t) {
+    constexpr int i = decltype(t)::value / D, j = decltype(t)::value % D;
+    if constexpr (i <= j) {
+      const V nn = n[i] * n[j];
+      x[vt_sym2(i, j, D)] = i == j ? vfma(bE, nn, a3) : bE * nn;
+      vt_each(std::make_integer_sequence<int, D>{}, [&](auto u) {
+        constexpr int k = decltype(u)::value;
+        if constexpr (k >= j) {
+          constexpr int m = VC::NP + vt_sym3(i, j, k, D);
+          V r = qb * nn * n[k];
+          if constexpr (j == k) r = vfma(qa, n[i], r);
+          if constexpr (i == k) r = vfma(qa, n[j], r);
+          if constexpr (i == j) r = vfma(qa, n[k], r);
+          x[m] = r;
+        }
+      });
     }
+  });
 }
 
 // Per-group frequency constants of the limited reconstruction (host-computed): the reciprocal
@@ -124,10 +136,19 @@ inline void vt_constants(const double* edge, int G, VtConst& v) {
     for (int j = 0; j < MAXG; ++j) v.c32[k][j] = (float)v.c[k][j];
 }
 
-// One lane per group, GP lanes (a power of two >= G) per cell, 256 threads per block over
-// 256/GP consecutive cells of one x row (grid: rows y, z by x tiles): each lane forms its
-// group's P and Q components and spectral densities, takes its neighbours' through warp
-// shuffles for the limited slopes, and the flux through its upper edge from the lane above.
+// One lane per W groups (a packed pair in FP32, one group in FP64), GL = ceil(G / W) lanes per cell and
+// 32 / GL cells of one x row per warp; a block's warps take VT_ROWS rows in turn, so that the
+// per-group constants are read once for them.  Each lane forms its groups' P and Q components and
+// spectral densities, takes its neighbours' (the lane below's last group, the lane above's first)
+// through warp shuffles for the limited slopes, and the flux through its upper edge from the lane
+// above; the edge between a lane's two groups needs no shuffle.
+//
+// The upwind choice of component pair (i, j) depends on the sign of V_ij, the cell's: a lane splits
+// V_ij into max(V_ij, 0) and min(V_ij, 0), adds the pairs that share a symmetric component, and
+// contracts them with the lower-edge values and with the values below the edge, without selects.
+//
+// Bound by instruction issue (63 % of cycles).  768^2 x 16 groups 0.135 -> 0.104 ms per launch, against one kernel with the
+// closure's reciprocals in chi, a select per component pair and lanes padded to a power of two.
 //
 // SPH: the 2-d spherical (r, theta) grid.  The tensors are those of 3 dimensions (DT = 3, with
 // F_phi = 0 and the V_phiphi entry), in physical components: the state's covariant flux
@@ -137,7 +158,7 @@ inline void vt_constants(const double* edge, int G, VtConst& v) {
 // theta faces: the cell's h), differences them over the cell, adds the volume-averaged
 // connection coefficients times the coordinate velocity at the centroid (linear profile between
 // the two faces), and turns V^a_b into physical components V^a_b h_a / h_b.
-constexpr int VT_THREADS = 256;
+constexpr int VT_THREADS = 256, VT_ROWS = 4;
 
 // The cell's velocity gradient V (physical components, DT x DT) and the scale factors h of the
 // flux components (1 on Cartesian grids), from the face velocities: component i of a face of
@@ -218,359 +239,170 @@ __device__ __forceinline__ double vt_volume(const StageArgs<R>& A, int ix, int i
   }
 }
 
-template <class R, int D, int GP, bool SPH>
-__global__ void __launch_bounds__(VT_THREADS) vterm_kernel(const __grid_constant__ StageArgs<R> A) {
+// x shuffled from the lane below (its last group) or above (its first group): the neighbouring
+// groups of the lane's first and last group, as lane values of the groups below and above each
+__device__ __forceinline__ F2 vt_below(F2 x) { return F2(__shfl_up_sync(0xffffffffu, x.y, 1), x.x); }
+__device__ __forceinline__ F2 vt_above(F2 x) { return F2(x.y, __shfl_down_sync(0xffffffffu, x.x, 1)); }
+__device__ __forceinline__ double vt_below(double x) { return __shfl_up_sync(0xffffffffu, x, 1); }
+__device__ __forceinline__ double vt_above(double x) { return __shfl_down_sync(0xffffffffu, x, 1); }
+// the same with zero where the lane's first (last) group has no neighbour below (above)
+__device__ __forceinline__ F2 vt_keep(F2 x, bool k0, bool k1) { return F2(k0 ? x.x : 0.0f, k1 ? x.y : 0.0f); }
+__device__ __forceinline__ double vt_keep(double x, bool k0, bool) { return k0 ? x : 0.0; }
+
+// Whether component (a <= b <= c) of Q enters the flux equation q (with the pair of its other two
+// indices; the pairs (0, 2) and (1, 2) of the gradient vanish on the spherical grid), or any of D.
+__host__ __device__ constexpr bool vt_enters(int a, int b, int c, int q, bool sph) {
+  return (q == a || q == b || q == c) && (!sph || (q == a ? b : a) == (q == c ? b : c) || (q == c ? b : c) < 2);
+}
+__host__ __device__ constexpr bool vt_needed(int a, int b, int c, int D, bool sph) {
+  for (int q = 0; q < D; ++q)
+    if (vt_enters(a, b, c, q, sph)) return true;
+  return false;
+}
+template <class R, int D, bool SPH>
+__global__ void __launch_bounds__(VT_THREADS, sizeof(R) == 4 ? (D == 3 || SPH ? 2 : 3) : 1) vterm_kernel(const __grid_constant__ StageArgs<R> A) {
   static_assert(!SPH || D == 2, "the spherical grid is 2-d");
+  using V = typename LaneOf<R>::V;
+  constexpr int W = LaneOf<R>::W;
   constexpr int DT = SPH ? 3 : D;  // dimension of the tensors
   using VC = VtComp<DT>;
-  constexpr int NG = 2 + D, NP = VC::NP, NC = VC::NC, CPB = VT_THREADS / GP;
+  constexpr int NG = 2 + D, NP = VC::NP, NC = VC::NC;
   const DevGrid& g = A.g;
-  const int G = g.G;
+  const int G = g.G, GL = (G + W - 1) / W;
   const uint32_t ncell = (uint32_t)g.ncell;
-  const int lane = (int)(threadIdx.x % GP);
-  const int kg = lane % g.Gs;  // group of the lane's channel (species-major channels)
-  const int x0 = (int)(blockIdx.y * CPB + threadIdx.x / GP);
-  const bool cok = x0 < g.n[0], act = cok && lane < G;
+  const int cpw = 32 / GL, wl = (int)threadIdx.x & 31, cw = wl / GL, lane = wl - cw * GL;
+  const int x0 = (int)(blockIdx.y * (VT_THREADS / 32) + threadIdx.x / 32) * cpw + cw;
+  const bool cok = cw < cpw && x0 < g.n[0];
+  const int ga = lane * W, gb = ga + W - 1;
+  const int ka = ga % g.Gs, kb = gb < G ? gb % g.Gs : 0;  // groups of the channels (species-major)
+  const bool acta = cok && ga < G, actb = W == 2 && cok && gb < G;
   const int ix = cok ? x0 : g.n[0] - 1;  // every lane takes part in the shuffles
-  const int iy = (int)(blockIdx.x % (unsigned)g.n[1]), iz = (int)(blockIdx.x / (unsigned)g.n[1]);
-  // 32-bit offsets: the host keeps every state offset below 2^32
-  const uint32_t cc = ((uint32_t)iz * g.n[1] + (uint32_t)iy) * g.n[0] + (uint32_t)ix;
-  R V[DT][DT], h[DT];
-  vt_gradient<R, D, SPH, DT>(A, ix, iy, iz, V, h);
-  // this lane's group of the stage input (physical flux components)
-  const uint32_t rad = (uint32_t)NG * ncell, gid = cc * (uint32_t)G + (uint32_t)lane,
-                 vstr = ncell * (uint32_t)G;
-  R E = R(0), F[DT], oE = R(0), oF[D];
-#pragma unroll
-  for (int q = 0; q < DT; ++q) F[q] = R(0);
-#pragma unroll
-  for (int q = 0; q < D; ++q) oF[q] = R(0);
-  if (act) {
-    // the stage output this lane updates, read here so that its latency overlaps the work
-    oE = A.out[FXI(rad + gid, A.n_state)];
-#pragma unroll
-    for (int q = 0; q < D; ++q) oF[q] = A.out[FXI(rad + (uint32_t)(1 + q) * vstr + gid, A.n_state)];
-    E = A.in[FXI(rad + gid, A.n_state)];
-#pragma unroll
-    for (int q = 0; q < D; ++q) F[q] = A.in[FXI(rad + (uint32_t)(1 + q) * vstr + gid, A.n_state)];
-    if constexpr (SPH) {
-#pragma unroll
-      for (int q = 0; q < D; ++q) F[q] = F[q] / h[q];
-    }
-  }
-  R x[NC];
-  vt_moments<R, DT>(A.k(R(0)).c, E, F, x);
-  // work terms V_ij P^ij and sum_i V_ij F^i
-  R wE = R(0), wF[D];
-#pragma unroll
-  for (int i = 0; i < DT; ++i)
-#pragma unroll
-    for (int j = 0; j < DT; ++j) wE += V[i][j] * x[vt_sym2(i, j, DT)];
-#pragma unroll
-  for (int j = 0; j < D; ++j) {
-    R s2 = R(0);
-#pragma unroll
-    for (int i = 0; i < D; ++i) s2 += V[i][j] * F[i];
-    wF[j] = s2;
-  }
-  const int k = act ? kg : 0;
+  // per-group frequency constants (the first and last groups and absent ones have zero midpoint
+  // constants: zero slope), and the lower edges (no flux through the lower end of a species' range)
   const VtConst& vc = *A.vtc;
-  const R inu = act ? vc.of(VT_INU, k, R(0)) : R(0);
-  const R lm = vc.of(VT_LMID, k, R(0)), hm = vc.of(VT_HMID, k, R(0)), cm = vc.of(VT_CMID, k, R(0));
-  const R mlo = vc.of(VT_MLO, k, R(0)), mhi = vc.of(VT_MHI, k, R(0));
-  const bool inner = act && kg > 0 && kg + 1 < g.Gs;
-  // spectral densities, limited slopes, values at the group's lower (x[m] after) and upper edge
-  R hi[NC];
+  auto cpair = [&](int e) { return vpair(acta ? vc.of(e, ka, R(0)) : R(0), actb ? vc.of(e, kb, R(0)) : R(0), V()); };
+  const V inu = cpair(VT_INU), lm = cpair(VT_LMID), hm = cpair(VT_HMID), cm = cpair(VT_CMID);
+  const V mlo = cpair(VT_MLO), mhi = cpair(VT_MHI);
+  const bool lo_a = acta && ka > 0, lo_b = actb && kb > 0;
+  const V el = vpair(lo_a ? A.gc->edge_of(ka, R(0)) : R(0), lo_b ? A.gc->edge_of(kb, R(0)) : R(0), V());
+  // whether the channel above each group is its upper neighbour in frequency
+  const bool up_a = W == 2 ? true : !(ga + 1 >= G || ka + 1 >= g.Gs);
+  const bool up_b = W == 2 && !(gb + 1 >= G || kb + 1 >= g.Gs);
+  const V one(R(1)), p4(R(4)), m3(R(-3)), cc_(A.k(R(0)).c);
+  const R wdt = A.k(R(0)).dt * A.k(R(0)).beta;  // w = 1 (stage 1) or 1/2 (stage 2)
+  const uint32_t rad = (uint32_t)NG * ncell, vstr = ncell * (uint32_t)G;
+  const bool vec = A.rt.vec != 0;
+  const int nrow = g.n[1] * g.n[2];
+  double esum = 0.0;
+  for (int row = (int)blockIdx.x * VT_ROWS; row < min((int)(blockIdx.x + 1) * VT_ROWS, nrow); ++row) {
+    const int iy = D == 3 ? row % g.n[1] : row, iz = D == 3 ? row / g.n[1] : 0;
+    // 32-bit offsets: the host keeps every state offset below 2^32
+    const uint32_t gid = ((uint32_t)row * g.n[0] + (uint32_t)ix) * (uint32_t)G + (uint32_t)ga;
+    // the stage output this lane updates, read first so that its latency overlaps the work, and
+    // the groups of the stage input
+    V o[1 + D], Q[1 + D];
 #pragma unroll
-  for (int m = 0; m < NC; ++m) {
-    const R xc = x[m] * inu;
-    const R xm = __shfl_up_sync(0xffffffffu, xc, 1, GP), xp = __shfl_down_sync(0xffffffffu, xc, 1, GP);
-    const R sl = inner ? vt_mc((xc - xm) * lm, (xp - xc) * hm, (xp - xm) * cm) : R(0);
-    x[m] = xc - sl * mlo;
-    hi[m] = xc + sl * mhi;
-  }
-  // flux through the lower edge nu_k: per component pair, the upper-edge value of group k-1 when
-  // V_ij < 0, else this group's lower-edge value
-  R fE = R(0), fF[D];
+    for (int v = 0; v < 1 + D; ++v) o[v] = Q[v] = V(R(0));
+    if (acta) {
 #pragma unroll
-  for (int j = 0; j < D; ++j) fF[j] = R(0);
-  R hp[NC];
+      for (int v = 0; v < 1 + D; ++v) {
+        o[v] = ld_global_lane(FXP(A.out, rad + v * vstr + gid, A.n_state), vec, actb, V());
+        Q[v] = ld_global_lane(FXP(A.in, rad + v * vstr + gid, A.n_state), vec, actb, V());
+      }
+    }
+    R Vg[DT][DT], h[DT];
+    vt_gradient<R, D, SPH, DT>(A, ix, iy, iz, Vg, h);
+    V F[DT], x[NC];
 #pragma unroll
-  for (int m = 0; m < NC; ++m) hp[m] = __shfl_up_sync(0xffffffffu, hi[m], 1, GP);
-  if (act && kg > 0) {  // no flux through the lower end of a species' group range
-    const R el = A.gc->edge_of(kg, R(0));
+    for (int q = 0; q < DT; ++q) F[q] = V(R(0));
+#pragma unroll
+    for (int q = 0; q < D; ++q) F[q] = SPH ? Q[1 + q] * rcp_any(h[q]) : Q[1 + q];  // physical components
+    vt_moments<DT>(cc_, one, p4, m3, Q[0], F, x);
+    // the split gradient per symmetric pair p = (i <= j): cp, cn the sums of the positive and
+    // negative parts, and their total (the pairs (0, 2) and (1, 2) vanish on the spherical grid)
+    R cp[NP], cn[NP];
 #pragma unroll
     for (int i = 0; i < DT; ++i)
 #pragma unroll
-      for (int j = 0; j < DT; ++j) {
-        const int m = vt_sym2(i, j, DT);
-        fE += V[i][j] * (V[i][j] < R(0) ? hp[m] : x[m]);
-      }
-    fE *= el;
-#pragma unroll
-    for (int j = 0; j < D; ++j) {
-      R sF = R(0);
-#pragma unroll
-      for (int i = 0; i < DT; ++i)
-#pragma unroll
-        for (int kk = 0; kk < DT; ++kk) {
-          const int m = NP + vt_sym3(kk, j, i, DT);
-          sF += V[i][kk] * (V[i][kk] < R(0) ? hp[m] : x[m]);
+      for (int j = i; j < DT; ++j) {
+        const int p = vt_sym2(i, j, DT);
+        cp[p] = max_fast(Vg[i][j], R(0));
+        cn[p] = min_fast(Vg[i][j], R(0));
+        if (i != j) {
+          cp[p] += max_fast(Vg[j][i], R(0));
+          cn[p] += min_fast(Vg[j][i], R(0));
         }
-      fF[j] = sF * el;
-    }
-  }
-  // flux through the upper edge: the lane above's lower-edge flux (none through the top edge)
-  const bool top = lane + 1 >= G || kg + 1 >= g.Gs;  // the upper end of the range
-  R uE = __shfl_down_sync(0xffffffffu, fE, 1, GP);
-  if (top) uE = R(0);
-  const R dE = uE - fE - wE;
-  const R wdt = A.k(R(0)).dt * A.k(R(0)).beta;  // w = 1 (stage 1) or 1/2 (stage 2)
-  bool bad = false;
-  R uF[D];
-#pragma unroll
-  for (int j = 0; j < D; ++j) {
-    uF[j] = __shfl_down_sync(0xffffffffu, fF[j], 1, GP);
-    if (top) uF[j] = R(0);
-  }
-  if (act) {
-    const R e = oE + wdt * dE;
-    bad |= !isfinite(e);
-    A.out[FXI(rad + gid, A.n_state)] = e;
-#pragma unroll
-    for (int j = 0; j < D; ++j) {
-      R dF = uF[j] - fF[j] - wF[j];
-      if constexpr (SPH) dF *= h[j];  // covariant component
-      const R f = oF[j] + wdt * dF;
-      bad |= !isfinite(f);
-      A.out[FXI(rad + (uint32_t)(1 + j) * vstr + gid, A.n_state)] = f;
-    }
-  }
-  if (bad) atomicOr(A.status, ST_NONFINITE);
-  if (A.budget != nullptr) {
-    // radiation energy the terms add, weighted as the RK combination weighs this stage; each
-    // lane weighs its own cell's volume (a warp spans 32/GP cells, of different volumes on the
-    // spherical grid)
-    double e = act ? (double)dE * vt_volume<R, D, SPH>(A, ix, iy) : 0.0;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) e += __shfl_xor_sync(0xffffffffu, e, o);
-    if ((threadIdx.x & 31) == 0)
-      atomicAdd(A.budget + (blockIdx.x % BUDGET_SLOTS) * NBUDGET + 8, e * A.bw_flux);
-  }
-}
-
-// Two groups per lane (the FP32 forms from 9 groups): lane l of a cell owns groups 2l and 2l + 1
-// as one packed FP32 pair (fx_pair.cuh), GQ lanes per cell (a power of two >= G/2), 256/GQ cells
-// of one x row per block, four blocks per SM (64 registers).  The closure runs per group; the spectral densities, limited slopes,
-// upwind edge values, work terms and the update run on the pair.  A group's neighbour across the
-// lane boundary comes by one shuffle each way (group 2l - 1 is the lane below's second, 2l + 2
-// the lane above's first); the flux through the edge between a lane's two groups needs none.
-// vt_moments for the pair: the closure per group (a group without flux or energy takes f = 0:
-// chi = 1/3, q = 0, the isotropic P = E/3 and Q = 0 of the one-group form), the components on
-// the pair.
-template <int D>
-__device__ __forceinline__ void vt_moments2(float c, F2 E, const F2* F, F2* x) {
-  using VC = VtComp<D>;
-  F2 F2s(0.0f);
-#pragma unroll
-  for (int q = 0; q < D; ++q) F2s = vfma(F[q], F[q], F2s);
-  float iF[2], av[2], bv[2], qav[2], qbv[2];
-#pragma unroll
-  for (int s = 0; s < 2; ++s) {
-    const float Fs = s ? F2s.y : F2s.x, Es = s ? E.y : E.x;
-    const bool ok = Fs > 0.0f && Es > 0.0f;
-    const float i1 = ok ? rsqrtf(Fs) : 0.0f, cE = c * Es;
-    const float f = ok ? fminf(Fs * i1 * __fdividef(1.0f, cE), 1.0f) : 0.0f, f2 = f * f;
-    const float chi = (3.0f + 4.0f * f2) * __fdividef(1.0f, 5.0f + 2.0f * sqrtf(4.0f - 3.0f * f2));
-    const float q = f * (2.0f + 3.0f * chi) * 0.2f;
-    iF[s] = i1;
-    av[s] = 0.5f * (1.0f - chi);
-    bv[s] = 0.5f * (3.0f * chi - 1.0f);
-    qav[s] = 0.5f * (f - q) * cE;
-    qbv[s] = 0.5f * (5.0f * q - 3.0f * f) * cE;
-  }
-  const F2 a(av[0], av[1]), b(bv[0], bv[1]), qa(qav[0], qav[1]), qb(qbv[0], qbv[1]);
-  F2 n[D];
-#pragma unroll
-  for (int i = 0; i < D; ++i) n[i] = F[i] * F2(iF[0], iF[1]);
-#pragma unroll
-  for (int i = 0; i < D; ++i)
-#pragma unroll
-    for (int j = i; j < D; ++j) {
-      const F2 nn = n[i] * n[j];
-      x[vt_sym2(i, j, D)] = E * (i == j ? vfma(b, nn, a) : b * nn);
-#pragma unroll
-      for (int k = j; k < D; ++k) {
-        F2 t(0.0f);
-        if (j == k) t = t + n[i];
-        if (i == k) t = t + n[j];
-        if (i == j) t = t + n[k];
-        x[VC::NP + vt_sym3(i, j, k, D)] = vfma(qb, nn * n[k], qa * t);
       }
-    }
-}
-
-template <int D, int GQ, bool SPH>
-__global__ void __launch_bounds__(VT_THREADS, 4) vterm_kernel2(const __grid_constant__ StageArgs<float> A) {
-  static_assert(!SPH || D == 2, "the spherical grid is 2-d");
-  using R = float;
-  constexpr int DT = SPH ? 3 : D;
-  using VC = VtComp<DT>;
-  constexpr int NG = 2 + D, NP = VC::NP, NC = VC::NC, CPB = VT_THREADS / GQ;
-  constexpr unsigned FULL = 0xffffffffu;
-  const DevGrid& g = A.g;
-  const int G = g.G;
-  const uint32_t ncell = (uint32_t)g.ncell;
-  const int lane = (int)(threadIdx.x % GQ);
-  const int x0 = (int)(blockIdx.y * CPB + threadIdx.x / GQ);
-  const bool cok = x0 < g.n[0];
-  const int ga = 2 * lane, gb = ga + 1;
-  const int kga = ga % g.Gs, kgb = gb % g.Gs;  // groups of the two channels (species-major)
-  const bool acta = cok && ga < G, actb = cok && gb < G;
-  const int ix = cok ? x0 : g.n[0] - 1;  // every lane takes part in the shuffles
-  const int iy = (int)(blockIdx.x % (unsigned)g.n[1]), iz = (int)(blockIdx.x / (unsigned)g.n[1]);
-  const uint32_t cc = ((uint32_t)iz * g.n[1] + (uint32_t)iy) * g.n[0] + (uint32_t)ix;
-  R V[DT][DT], h[DT];
-  vt_gradient<R, D, SPH, DT>(A, ix, iy, iz, V, h);
-  // the two groups of the stage input (physical flux components)
-  const uint32_t rad = (uint32_t)NG * ncell, gia = cc * (uint32_t)G + (uint32_t)ga,
-                 vstr = ncell * (uint32_t)G;
-  R Ea = 0.0f, Eb = 0.0f, Fa[DT], Fb[DT], oE[2] = {0.0f, 0.0f}, oF[2][D];
+    // work terms V_ij P^ij and sum_i V_ij F^i
+    V d[1 + D];
 #pragma unroll
-  for (int q = 0; q < DT; ++q) { Fa[q] = 0.0f; Fb[q] = 0.0f; }
-#pragma unroll
-  for (int q = 0; q < D; ++q) { oF[0][q] = 0.0f; oF[1][q] = 0.0f; }
-  // the stage output the lane updates, read first so that its latency overlaps the work
-#pragma unroll
-  for (int t = 0; t < 2; ++t)
-    if (t ? actb : acta) {
-      oE[t] = A.out[FXI(rad + gia + t, A.n_state)];
-#pragma unroll
-      for (int q = 0; q < D; ++q) oF[t][q] = A.out[FXI(rad + (uint32_t)(1 + q) * vstr + gia + t, A.n_state)];
-    }
-  if (acta) {
-    Ea = A.in[FXI(rad + gia, A.n_state)];
-#pragma unroll
-    for (int q = 0; q < D; ++q) Fa[q] = A.in[FXI(rad + (uint32_t)(1 + q) * vstr + gia, A.n_state)];
-  }
-  if (actb) {
-    Eb = A.in[FXI(rad + gia + 1, A.n_state)];
-#pragma unroll
-    for (int q = 0; q < D; ++q) Fb[q] = A.in[FXI(rad + (uint32_t)(1 + q) * vstr + gia + 1, A.n_state)];
-  }
-  if constexpr (SPH) {
-#pragma unroll
-    for (int q = 0; q < D; ++q) { Fa[q] = Fa[q] / h[q]; Fb[q] = Fb[q] / h[q]; }
-  }
-  F2 x[NC];
-  {
-    F2 Fp[DT];
-#pragma unroll
-    for (int q = 0; q < DT; ++q) Fp[q] = F2(Fa[q], Fb[q]);
-    vt_moments2<DT>(A.k(R(0)).c, F2(Ea, Eb), Fp, x);
-  }
-  // work terms V_ij P^ij and sum_i V_ij F^i
-  F2 wE(0.0f), wF[D];
-#pragma unroll
-  for (int i = 0; i < DT; ++i)
-#pragma unroll
-    for (int j = 0; j < DT; ++j)
-      if (!SPH || i == j || (i < 2 && j < 2)) wE = vfma(F2(V[i][j]), x[vt_sym2(i, j, DT)], wE);
-#pragma unroll
-  for (int j = 0; j < D; ++j) {
-    F2 s2(0.0f);
-#pragma unroll
-    for (int i = 0; i < D; ++i) s2 = vfma(F2(V[i][j]), F2(Fa[i], Fb[i]), s2);
-    wF[j] = s2;
-  }
-  // per-group frequency constants
-  const VtConst& vc = *A.vtc;
-  const int ka = acta ? kga : 0, kb = actb ? kgb : 0;
-  auto cpair = [&](int e) { return F2(acta ? vc.c32[e][ka] : 0.0f, actb ? vc.c32[e][kb] : 0.0f); };
-  const F2 inu = cpair(VT_INU), lm = cpair(VT_LMID), hm = cpair(VT_HMID), cm = cpair(VT_CMID);
-  const F2 mlo = cpair(VT_MLO), mhi = cpair(VT_MHI);
-  // spectral densities, limited slopes, values at each group's lower (x[m] after) and upper edge
-  F2 hi[NC];
-#pragma unroll
-  for (int m = 0; m < NC; ++m) {
-    const F2 xc = x[m] * inu;
-    const float below = __shfl_up_sync(FULL, xc.y, 1, GQ);   // group 2l - 1
-    const float above = __shfl_down_sync(FULL, xc.x, 1, GQ); // group 2l + 2
-    const F2 xm(below, xc.x), xp(xc.y, above);
-    // (the first and last groups and absent ones have zero midpoint constants: zero slope)
-    const F2 sl = mc_slope((xc - xm) * lm, (xp - xc) * hm, (xp - xm) * cm);
-    x[m] = vfma(-sl, mlo, xc);
-    hi[m] = vfma(sl, mhi, xc);
-  }
-  // fluxes through the lower edges of the two groups: edge 2l takes, per component pair, the
-  // upper-edge value of group 2l - 1 (the lane below's second) when V_ij < 0, else group 2l's
-  // lower-edge value; edge 2l + 1 takes group 2l's upper-edge value or group 2l + 1's lower-edge
-  // value
-  float hb[NC];
-#pragma unroll
-  for (int m = 0; m < NC; ++m) hb[m] = __shfl_up_sync(FULL, hi[m].y, 1, GQ);
-  // (no flux through the lower end of a species' group range)
-  const F2 el((acta && kga > 0) ? A.gc->edge_of(kga, R(0)) : 0.0f, (actb && kgb > 0) ? A.gc->edge_of(kgb, R(0)) : 0.0f);
-  F2 fE(0.0f), fF[D];
-#pragma unroll
-  for (int j = 0; j < D; ++j) fF[j] = F2(0.0f);
-#pragma unroll
-  for (int i = 0; i < DT; ++i)
-#pragma unroll
-    for (int j = 0; j < DT; ++j) {
-      if (SPH && i != j && (i >= 2 || j >= 2)) continue;  // V_ij = 0 there
-      const int m = vt_sym2(i, j, DT);
-      fE = vfma(F2(V[i][j]), V[i][j] < 0.0f ? F2(hb[m], hi[m].x) : x[m], fE);
-    }
-  fE = fE * el;
-#pragma unroll
-  for (int j = 0; j < D; ++j) {
-    F2 sF(0.0f);
+    for (int v = 0; v < 1 + D; ++v) d[v] = V(R(0));
 #pragma unroll
     for (int i = 0; i < DT; ++i)
 #pragma unroll
-      for (int kk = 0; kk < DT; ++kk) {
-        if (SPH && i != kk && (i >= 2 || kk >= 2)) continue;
-        const int m = NP + vt_sym3(kk, j, i, DT);
-        sF = vfma(F2(V[i][kk]), V[i][kk] < 0.0f ? F2(hb[m], hi[m].x) : x[m], sF);
+      for (int j = i; j < DT; ++j)
+        if (!SPH || i == j || j < 2) d[0] = vfma(V(-(cp[vt_sym2(i, j, DT)] + cn[vt_sym2(i, j, DT)])), x[vt_sym2(i, j, DT)], d[0]);
+#pragma unroll
+    for (int j = 0; j < D; ++j)
+#pragma unroll
+      for (int i = 0; i < D; ++i) d[1 + j] = vfma(V(-Vg[i][j]), F[i], d[1 + j]);
+    // fluxes through the groups' lower edges, component by component of P and Q: the spectral
+    // density's limited slope, its value at the lower edge and the value of the group below at it
+    V fl[1 + D];
+#pragma unroll
+    for (int v = 0; v < 1 + D; ++v) fl[v] = V(R(0));
+    auto edge = [&](V xm, V& low, V& below) {
+      const V xc = xm * inu;
+      const V xb = vt_below(xc), xa = vt_above(xc);
+      const V sl = mc_min((xc - xb) * lm, (xa - xc) * hm, (xa - xb) * cm, R(2));
+      low = vfma(sl * R(-1), mlo, xc);
+      below = vt_below(vfma(sl, mhi, xc));
+    };
+#pragma unroll
+    for (int i = 0; i < DT; ++i)
+#pragma unroll
+      for (int j = i; j < DT; ++j) {
+        if (SPH && i != j && j >= 2) continue;  // V_ij = 0 there
+        const int p = vt_sym2(i, j, DT);
+        V low, below;
+        edge(x[p], low, below);
+        fl[0] = vfma(V(cp[p]), low, vfma(V(cn[p]), below, fl[0]));
       }
-    fF[j] = sF * el;
-  }
-  // fluxes through the upper edges: group 2l's is group 2l + 1's lower-edge flux; group
-  // 2l + 1's the lane above's first (none through the top edge of the range)
-  const bool topb = gb + 1 >= G || kgb + 1 >= g.Gs;
-  float up = __shfl_down_sync(FULL, fE.x, 1, GQ);
-  const F2 uE(fE.y, topb ? 0.0f : up);
-  const F2 dE = uE - fE - wE;
-  const R wdt = A.k(R(0)).dt * A.k(R(0)).beta;  // w = 1 (stage 1) or 1/2 (stage 2)
-  F2 dF[D];
+    // Q^kji: the component (a <= b <= c) enters flux q for every split of it into q and a pair u <= w
+    // (constant indices: an index computed in an unrolled loop left the components in local memory)
+    vt_each(std::make_integer_sequence<int, DT * DT * DT>{}, [&](auto t) {
+      constexpr int a = decltype(t)::value / (DT * DT), b = decltype(t)::value / DT % DT, c = decltype(t)::value % DT;
+      if constexpr (a <= b && b <= c && vt_needed(a, b, c, D, SPH)) {
+        constexpr int m = NP + vt_sym3(a, b, c, DT);
+        V low, below;
+        edge(x[m], low, below);
+        vt_each(std::make_integer_sequence<int, D>{}, [&](auto qt) {
+          constexpr int q = decltype(qt)::value, u = q == a ? b : a, w = q == c ? b : c, p = vt_sym2(u, w, DT);
+          if constexpr (vt_enters(a, b, c, q, SPH)) fl[1 + q] = vfma(V(cp[p]), low, vfma(V(cn[p]), below, fl[1 + q]));
+        });
+      }
+    });
+    bool bad = false;
 #pragma unroll
-  for (int j = 0; j < D; ++j) {
-    up = __shfl_down_sync(FULL, fF[j].x, 1, GQ);
-    dF[j] = F2(fF[j].y, topb ? 0.0f : up) - fF[j] - wF[j];
-    if constexpr (SPH) dF[j] = dF[j] * h[j];  // covariant component
-  }
-  bool bad = false;
-#pragma unroll
-  for (int t = 0; t < 2; ++t)
-    if (t ? actb : acta) {
-      const R e = fmaf(wdt, vget(dE, t), oE[t]);
-      bad |= !isfinite(e);
-      A.out[FXI(rad + gia + t, A.n_state)] = e;
-#pragma unroll
-      for (int j = 0; j < D; ++j) {
-        const R f = fmaf(wdt, vget(dF[j], t), oF[t][j]);
-        bad |= !isfinite(f);
-        A.out[FXI(rad + (uint32_t)(1 + j) * vstr + gia + t, A.n_state)] = f;
+    for (int v = 0; v < 1 + D; ++v) {
+      const V f = vt_keep(fl[v] * el, lo_a, lo_b);
+      d[v] = d[v] + (vt_keep(vt_above(f), up_a, up_b) - f);  // upper-edge flux less lower-edge flux
+      if (SPH && v >= 1) d[v] = d[v] * h[v - 1];             // covariant component
+      const V r = vfma(V(wdt), d[v], o[v]);
+      if (acta) {
+        st_global_lane(FXP(A.out, rad + v * vstr + gid, A.n_state), r, vec, actb);
+        bad |= !isfinite(vget(r, 0)) || (actb && !isfinite(vget(r, W - 1)));
       }
     }
-  if (bad) atomicOr(A.status, ST_NONFINITE);
+    if (bad) atomicOr(A.status, ST_NONFINITE);
+    if (A.budget != nullptr && acta)
+      esum += ((double)vget(d[0], 0) + (actb ? (double)vget(d[0], W - 1) : 0.0)) * vt_volume<R, D, SPH>(A, ix, iy);
+  }
   if (A.budget != nullptr) {
-    double e = ((acta ? (double)dE.x : 0.0) + (actb ? (double)dE.y : 0.0)) * vt_volume<R, D, SPH>(A, ix, iy);
+    // radiation energy the terms add, weighted as the RK combination weighs this stage
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) e += __shfl_xor_sync(FULL, e, o);
-    if ((threadIdx.x & 31) == 0)
-      atomicAdd(A.budget + (blockIdx.x % BUDGET_SLOTS) * NBUDGET + 8, e * A.bw_flux);
+    for (int s = 16; s > 0; s >>= 1) esum += __shfl_xor_sync(0xffffffffu, esum, s);
+    if (wl == 0) atomicAdd(A.budget + (blockIdx.x % BUDGET_SLOTS) * NBUDGET + 8, esum * A.bw_flux);
   }
 }
 
