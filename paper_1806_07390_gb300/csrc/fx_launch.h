@@ -26,8 +26,9 @@ namespace fx {
 // tiles against each other.  So small grids get small tiles and short chunks that spread over the
 // device, and large ones the tiles with the least halo share and the fewest idle lanes.  Measured
 // against a sweep of tiles and chunks (stage kernel, microseconds, chosen / best of the sweep):
-// 1024^2 x 16 FP32 253 / 245, 256^3 x 12 FP32 7140 / 7140, 640 x 128 x 20 spherical FP32 70 / 70,
-// 75 x 61 x 50 x 20 FP32 250 / 243, 96 x 80 x 8 FP32 10.9 / 10.5, 512^2 x 16 FP64 1862 / 1862.
+// 1024^2 x 16 FP32 253 / 245, 640 x 128 x 20 spherical FP32 70 / 70, 96 x 80 x 8 FP32 10.9 / 10.5,
+// 512^2 x 16 FP64 1862 / 1862; with blocks of up to 192 threads in 3-d 256^3 x 12 FP32 7140 / 7140,
+// 75 x 61 x 50 x 20 FP32 250 / 243 (blocks of 256: 6235 and 166, see StageCap).
 template <class R, int D>
 inline void fit_tile(const int* n, int G, int nsm, int regs, RadTile& best, int& chunk) {
   using C = StageCap<R, D>;
@@ -50,7 +51,7 @@ inline void fit_tile(const int* n, int G, int nsm, int regs, RadTile& best, int&
       // upper faces: at most one per thread; in 1-d and 2-d also one halo reconstruction, one halo
       // copy and two records
       const int nt = (ty + (D == 3 ? tx : 0)) * gl;
-      if (nt > t.nth || (D < 3 && (4 * gl > t.nth || tile_recs<D>(t) > 2 * t.nth))) continue;
+      if (nt > t.nth || (D < 3 && (4 * gl > t.nth || 8 * gl > C::NT || tile_recs<D>(t) > 2 * t.nth))) continue;
       // copies past the ones whose offsets a thread keeps
       const int late = std::max(0, tile_halo<D>(t) * gl - (D == 3 ? 2 : 1) * t.nth) + std::max(0, tile_recs<D>(t) - 2 * t.nth);
       const size_t smem = stage_smem_bytes<R, D>(t);

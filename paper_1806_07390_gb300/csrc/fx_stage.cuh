@@ -437,24 +437,30 @@ __device__ __forceinline__ void cp_async16(void* s, const void* g) {
 // blocks of the grid do it, one thread per cell, in the slots that the radiation blocks leave free
 // and as they finish (no launch of its own, and no gas variables in the radiation blocks).
 //
-// Bound by instruction issue and by the latency between the plane barriers (1024^2 x 16: 669 instructions
-// per warp and plane, issued in about 56 % of cycles at 20 warps per multiprocessor; DRAM 1.0x the
-// algorithmic bytes).  Measured
-// (FP32 state unless noted, one launch): 1024^2 x 16 groups 0.455 -> 0.250 ms, 256^3 x 12 16.4 ->
-// 7.3 ms, 640 x 128 x 20 spherical 0.124 -> 0.064 ms, 512^2 x 24 channels 0.23 -> 0.099 ms, 512^2 x
-// 16 FP64 2.99 -> 1.84 ms, against one kernel with lanes padded to a power of two, geometry tables
-// on every grid, and the gas update in its lanes.
+// Bound by instruction issue and by the latency between the plane barriers (1024^2 x 16: about 700
+// instructions per warp and plane, issued in 66 % of cycles at 20 warps per multiprocessor; 256^3 x
+// 12: 1355 in 58 % at 16 warps; DRAM 1.0x the algorithmic bytes), the FP64 state by the FP64 pipe (86
+// % busy, 239 operations per cell and group).  Measured (FP32 state unless noted, one launch):
+// 1024^2 x 16 groups 0.455 -> 0.234 ms, 256^3 x 12 16.4 -> 6.2 ms, 640 x 128 x 20 spherical 0.124 ->
+// 0.067 ms, 512^2 x 24 channels 0.23 -> 0.094 ms, 512^2 x 16 FP64 2.99 -> 1.86 ms, against one kernel
+// with lanes padded to a power of two, geometry tables on every grid, and the gas update in its lanes.
+//
+// Block sizes (StageCap).  A thread holds about 90 values at order 1, so 20 warps of 96 registers in
+// 2-d (4 blocks of 160: 2 of 256 0.244 ms, 3 of 160 0.229 ms but the 24-channel and 400 x 300 grids
+// 6 to 8 % slower, 5 of 160 0.264 ms) and, with the second in-plane direction, 16 warps of 128 in 3-d
+// (256^3 x 12, 2 blocks of 256: 6.2 ms; 4 of 128 6.4, 3 of 192 spill 7.3, 1 of 512 6.5: larger tiles
+// have less halo).
 //
 // SPH selects the spherical (r, theta) geometry, RO the radiation reconstruction (1: linear with
 // the MC limiter, the paper's; 2: the gas's parabola), BUD the boundary-outflow budgets (R13).
 // ---------------------------------------------------------------------------------------------
 template <class R, int D> struct StageCap {
-  static constexpr int NT = sizeof(R) == 8 ? 256 : (D == 3 ? 192 : 160);  // most threads per block
+  static constexpr int NT = sizeof(R) == 8 ? 256 : (D == 3 ? 256 : 160);  // most threads per block
   static constexpr int XP = sizeof(R) == 8 ? 128 : 64;  // room for the upper face of every row
   // ... and for the threads past the tile (at most 31), which run along on entries of their own
   static constexpr int XC = NT + XP + 32 + (D == 3 ? XP : 32);
   static constexpr int PB = D == 3 ? 1 : 2;             // planes of xb (and yb) in use at once
-  static constexpr int MINB = sizeof(R) == 8 ? 2 : (D == 3 ? 3 : 4);  // resident blocks aimed at
+  static constexpr int MINB = sizeof(R) == 8 ? 2 : (D == 3 ? 2 : 4);  // resident blocks aimed at
 };
 
 // Halo cells per plane and face records per plane of a tile.
@@ -476,7 +482,7 @@ template <class R, int D> struct StageLayout {
     xr = yb + (D == 3 ? C::PB * NRV * C::XC : 0);
     yr = xr + NRV * t.ty * t.gl;
     halo = yr + (D == 3 ? NRV * t.tx * t.gl : 0);
-    rec = (halo + 2 * NRV * tile_halo<D>(t) * t.gl + 1) & ~1;        // 16-byte aligned
+    rec = (halo + (D == 3 ? 2 * NRV * tile_halo<D>(t) * t.gl : NRV * C::NT) + 1) & ~1;  // 16-byte aligned
     end = rec + 2 * tile_recs<D>(t) * (4 * (int)sizeof(R) / 8);
   }
 };
@@ -723,7 +729,10 @@ stage_kernel(const __grid_constant__ StageArgs<R> A) {
   V* const halo = sm + L.halo;
   R* const rec = reinterpret_cast<R*>(sm + L.rec);
   const int n_ring = (D == 1 ? 1 : 4) * NRV * NT, n_base = NRV * NT, n_xb = PB * NRV * XC;
-  const int n_xr = NRV * TY * GL, n_yr = NRV * TX * GL, n_halo = 2 * NRV * HS, n_rec = 8 * NREC;
+  const int n_xr = NRV * TY * GL, n_yr = NRV * TX * GL, n_halo = D == 3 ? 2 * NRV * HS : NRV * NT, n_rec = 8 * NREC;
+  // halo planes: variable stride and offset of the second plane (below 3-d the ring's stride, so that
+  // both are read with the same immediate offsets; two planes fit in it, fit_tile)
+  const int HV = D == 3 ? HS : NT, HPAR = D == 3 ? NRV * HS : HS;
   (void)n_ring; (void)n_base; (void)n_xb; (void)n_xr; (void)n_yr; (void)n_halo; (void)n_rec;
 
   const Tab<R> tx{A.tab[0], nx + 4, A.uniform[0] ? A.urow[0] : nullptr};
@@ -811,23 +820,27 @@ stage_kernel(const __grid_constant__ StageArgs<R> A) {
   // ---- copies.  A plane's address is block-uniform (the state's base, the variable, the plane)
   // plus the thread's fixed offset.
   auto plane_at = [&](const R* S, int v, uint32_t row) -> const R* { return S + ((size_t)NG * ncell + (size_t)v * vstride + row); };
-  auto ring_slot = [&](int P) -> int { return D == 1 ? 0 : (P & 3) * NRV * NT; };
-  auto issue_own = [&](int P) {
+  // ring slot of plane P (counted from the chunk's first plane, as are the parities of halo and
+  // record planes)
+  auto ring_slot = [&](int P) -> int { return D == 1 ? 0 : ((P - kbeg + 1) & 3) * NRV * NT; };
+  auto row_of = [&](int P) -> uint32_t {  // first element of plane P in a variable (P >= 0: upper ghosts mapped)
     bool f = false;
-    const uint32_t row = (uint32_t)map_m(P, f) * pstride;
-    const int s = ring_slot(P) + tid;
+    return (uint32_t)(P < nmarch && P >= 0 ? P : map_m(P, f)) * pstride;
+  };
+  auto issue_own = [&](int P, int slot) {
+    const uint32_t row = row_of(P);
+    const int s = slot + tid;
 #pragma unroll
     for (int v = 0; v < NRV; ++v)
       cp_async_lane(&ring[FXI(s + v * NT, n_ring)], FXP(plane_at(A.in, v, row), toff, vstride - row), vec, h1);
   };
-  auto issue_halo = [&](int P) {
-    bool f = false;
-    const uint32_t row = (uint32_t)map_m(P, f) * pstride;
+  auto issue_halo = [&](int P, int par) {
+    const uint32_t row = row_of(P);
     auto one = [&](int t, uint32_t off, bool two) {
-      const int s = (P & 1) * NRV * HS + t;
+      const int s = par * HPAR + t;
 #pragma unroll
       for (int v = 0; v < NRV; ++v)
-        cp_async_lane(&halo[FXI(s + v * HS, n_halo)], FXP(plane_at(A.in, v, row), off, vstride - row), vec, two);
+        cp_async_lane(&halo[FXI(s + v * HV, n_halo)], FXP(plane_at(A.in, v, row), off, vstride - row), vec, two);
     };
 #pragma unroll
     for (int p = 0; p < HP; ++p)
@@ -841,9 +854,9 @@ stage_kernel(const __grid_constant__ StageArgs<R> A) {
       }
     }
   };
-  auto issue_rec = [&](int P) {
+  auto issue_rec = [&](int P, int par) {
     auto one = [&](int t, uint32_t f) {
-      R* const d = rec + FXI(((P & 1) * NREC + t) * 4, n_rec);
+      R* const d = rec + FXI((par * NREC + t) * 4, n_rec);
       const R* const s = A.frec + (size_t)4 * FXI(f, A.n_recs);
       cp_async16(d, s);
       if (sizeof(R) == 8) cp_async16(d + 2, s + 2);
@@ -886,13 +899,13 @@ stage_kernel(const __grid_constant__ StageArgs<R> A) {
       p[(1 + q) * vs] = x;
     }
   };
-  auto finish_own = [&](int P) {
+  auto finish_own = [&](int P, int slot) {
     bool fm = false;
     map_m(P, fm);
     if (SPH || fx_own || fy_own || fm)
-      finish_one(&ring[FXI(ring_slot(P) + tid, n_ring)], NT, fx_own, fy_own, fm, gx, P);
+      finish_one(&ring[FXI(slot + tid, n_ring)], NT, fx_own, fy_own, fm, gx, P);
   };
-  auto finish_halo = [&](int P) {
+  auto finish_halo = [&](int P, int par) {
     bool fm = false;
     map_m(P, fm);
     for (int t = ht0; t < HS; t += NTH) {
@@ -900,22 +913,21 @@ stage_kernel(const __grid_constant__ StageArgs<R> A) {
       bool f0 = false, f1 = false;
       halo_pos(div_gl(t), sx, sy);
       inplane(sx, sy, f0, f1);
-      if (SPH || f0 || f1 || fm) finish_one(&halo[FXI((P & 1) * NRV * HS + t, n_halo)], HS, f0, f1, fm, x0 + sx, P);
+      if (SPH || f0 || f1 || fm) finish_one(&halo[FXI(par * HPAR + t, n_halo)], HV, f0, f1, fm, x0 + sx, P);
     }
   };
 
   // ---- reads.  The in-plane neighbours of the own cell: in the ring, or for an edge cell in the
   // halo (other base and variable stride, both fixed along the march up to the plane's slot).
-  auto own_ld = [&](int P, V* Q) {
-    const int s = ring_slot(P) + tid;
+  auto own_ld = [&](int slot, V* Q) {
+    const int s = slot + tid;
 #pragma unroll
     for (int v = 0; v < NRV; ++v) Q[v] = ring[FXI(s + v * NT, n_ring)];
   };
-  // p, st: first entry and variable stride of a neighbour, o: its offset in the plane of the ring
-  // or the halo
-  auto nb_ld = [&](int P, bool in_halo, int o, V* Q) {
-    const V* const p = in_halo ? halo + FXI((P & 1) * NRV * HS + o, n_halo) : ring + FXI(ring_slot(P) + o, n_ring);
-    const int st = in_halo ? HS : NT;
+  // o: a neighbour's offset in the plane of the ring (slot) or of the halo (par)
+  auto nb_ld = [&](int slot, int par, bool in_halo, int o, V* Q) {
+    const V* const p = in_halo ? halo + FXI(par * HPAR + o, n_halo) : ring + FXI(slot + o, n_ring);
+    const int st = D == 3 && in_halo ? HV : NT;  // (below 3-d the same)
 #pragma unroll
     for (int v = 0; v < NRV; ++v) Q[v] = p[v * st];
   };
@@ -966,8 +978,8 @@ stage_kernel(const __grid_constant__ StageArgs<R> A) {
 #pragma unroll
     for (int q = 0; q < D; ++q) out[1 + q] = vfma(kR, QR[1 + q], vfma(kL, QL[1 + q], PL[q] + PR[q]));
   };
-  auto rec_ld = [&](int P, int i, R* r) {
-    const R* const p = rec + FXI(((P & 1) * NREC + i) * 4, n_rec);
+  auto rec_ld = [&](int par, int i, R* r) {
+    const R* const p = rec + FXI((par * NREC + i) * 4, n_rec);
     if constexpr (sizeof(R) == 4) {
       const float4 x = *reinterpret_cast<const float4*>(p);
       r[0] = x.x; r[1] = x.y; r[2] = x.z; r[3] = x.w;
@@ -990,18 +1002,18 @@ stage_kernel(const __grid_constant__ StageArgs<R> A) {
 #pragma unroll
   for (int v = 0; v < NRV; ++v) bm0[v] = rfm_old[v] = V(R(0));
   if constexpr (D == 1) {
-    issue_own(0);
-    issue_halo(0);
-    issue_rec(0);
+    issue_own(0, 0);
+    issue_halo(0, 0);
+    issue_rec(0, 0);
     cp_async_commit();
     cp_async_wait_all();
-    finish_own(0);
-    finish_halo(0);
+    finish_own(0, 0);
+    finish_halo(0, 0);
     __syncthreads();
   } else {
-    for (int P = kbeg - 1; P <= kbeg + 2; ++P) issue_own(P);
-    issue_halo(kbeg);
-    issue_rec(kbeg);
+    for (int P = kbeg - 1; P <= kbeg + 2; ++P) issue_own(P, ring_slot(P));
+    issue_halo(kbeg, 0);
+    issue_rec(kbeg, 0);
     cp_async_commit();
     V Qa[NRV];  // own column of plane kbeg-2, straight from global memory
     {
@@ -1027,14 +1039,14 @@ stage_kernel(const __grid_constant__ StageArgs<R> A) {
       for (int c = 0; c < 4; ++c) r[c] = s[c];
     }
     cp_async_wait_all();
-    for (int P = kbeg - 1; P <= kbeg + 2; ++P) finish_own(P);
-    finish_halo(kbeg);
+    for (int P = kbeg - 1; P <= kbeg + 2; ++P) finish_own(P, ring_slot(P));
+    finish_halo(kbeg, 0);
     __syncthreads();
     // march reconstruction of planes kbeg-1 (upper face) and kbeg, and the flux at kbeg-1/2
     V Qb[NRV], Qc[NRV], Qd[NRV], ta[NRV], tb[NRV], am[NRV];
-    own_ld(kbeg - 1, Qb);
-    own_ld(kbeg, Qc);
-    own_ld(kbeg + 1, Qd);
+    own_ld(ring_slot(kbeg - 1), Qb);
+    own_ld(ring_slot(kbeg), Qc);
+    own_ld(ring_slot(kbeg + 1), Qd);
     recon(tm, bc_pad(kbeg - 1), Qa, Qb, Qc, ta, tb);
     recon(tm, bc_pad(kbeg), Qb, Qc, Qd, am, bm0);
     face_flux(MD, tb, am, r, efv, rfm_old);
@@ -1067,11 +1079,11 @@ stage_kernel(const __grid_constant__ StageArgs<R> A) {
     }
     return b;
   };
-  auto run_task = [&](int k, int px, const Task& b_) {
+  auto run_task = [&](int slot, int par, int px, const Task& b_) {
     V Qi[NRV], Q0[NRV], Qo[NRV], a[NRV], b[NRV];
-    nb_ld(k, false, b_.in, Qi);
-    nb_ld(k, true, b_.h, Q0);
-    nb_ld(k, true, b_.h + b_.hs, Qo);
+    nb_ld(slot, par, false, b_.in, Qi);
+    nb_ld(slot, par, true, b_.h, Q0);
+    nb_ld(slot, par, true, b_.h + b_.hs, Qo);
     if constexpr (TABLES) {
       const Tab<R>& tt = b_.x ? tx : ty;
       const int ip = b_.x ? bc_pad(b_.up ? x0 + TX : x0 - 1) : bc_pad(b_.up ? y0 + TY : y0 - 1);
@@ -1096,42 +1108,46 @@ stage_kernel(const __grid_constant__ StageArgs<R> A) {
   const bool stage2 = A.base != nullptr;
 
   // ---------------------------------------------------------------- march
+  // (unrolled by four planes, with every slot a constant, the kernel lost 8 to 25 % to instruction
+  // fetch)
   for (int k = kbeg; k < kend; ++k) {
+    const int u = k - kbeg, par = u & 1, SL = D == 1 ? 0 : NRV * NT;
+    const int s0 = ((u + 1) & 3) * SL, s1 = ((u + 2) & 3) * SL, s2 = ((u + 3) & 3) * SL, s3 = (u & 3) * SL;
     const bool more = D >= 2 && k + 1 < kend;
     if (more) {
-      issue_own(k + 3);
-      issue_halo(k + 1);
-      issue_rec(k + 1);
+      issue_own(k + 3, s3);
+      issue_halo(k + 1, par ^ 1);
+      issue_rec(k + 1, par ^ 1);
     }
     issue_base(k);
     cp_async_commit();
-    const int px = PB == 2 ? (k & 1) * NRV * XC : 0;  // this plane's half of xb and yb
+    const int px = PB == 2 ? par * NRV * XC : 0;  // this plane's half of xb and yb
     // ---- B
     V ax[NRV], ay[NRV], am1[NRV], bm1[NRV];
     {
       V Q0[NRV], Qm[NRV], Qp[NRV], b[NRV];
-      own_ld(k, Q0);
-      nb_ld(k, xm_h, xm_o, Qm);
-      nb_ld(k, xp_h, xp_o, Qp);
+      own_ld(s0, Q0);
+      nb_ld(s0, par, xm_h, xm_o, Qm);
+      nb_ld(s0, par, xp_h, xp_o, Qp);
       recon(tx, ipx, Qm, Q0, Qp, ax, b);
 #pragma unroll
       for (int v = 0; v < NRV; ++v) xb[FXI(px + v * XC + xo + GL, n_xb)] = b[v];
       if constexpr (D == 3) {
-        nb_ld(k, ym_h, ym_o, Qm);
-        nb_ld(k, yp_h, yp_o, Qp);
+        nb_ld(s0, par, ym_h, ym_o, Qm);
+        nb_ld(s0, par, yp_h, yp_o, Qp);
         recon(ty, ipy, Qm, Q0, Qp, ay, b);
 #pragma unroll
         for (int v = 0; v < NRV; ++v) yb[FXI(px + v * XC + yo + TX * GL, n_xb)] = b[v];
       }
       if constexpr (D >= 2) {
-        own_ld(k + 1, Qm);
-        own_ld(k + 2, Qp);
+        own_ld(s1, Qm);
+        own_ld(s2, Qp);
         recon(tm, bc_pad(k + 1), Q0, Qm, Qp, am1, bm1);
       }
     }
-    if (tid < ntask) run_task(k, px, my);
+    if (tid < ntask) run_task(s0, par, px, my);
     if (D == 3 && ntask > NTH)
-      for (int t = tid + NTH; t < ntask; t += NTH) run_task(k, px, task_of(t));
+      for (int t = tid + NTH; t < ntask; t += NTH) run_task(s0, par, px, task_of(t));
     __syncthreads();
     // ---- C
     V rfm_new[NRV];
@@ -1142,20 +1158,20 @@ stage_kernel(const __grid_constant__ StageArgs<R> A) {
       R r[4];
 #pragma unroll
       for (int v = 0; v < NRV; ++v) QL[v] = xb[FXI(px + v * XC + xo, n_xb)];
-      rec_ld(k, ly * (TX + 1) + lx, r);
+      rec_ld(par, ly * (TX + 1) + lx, r);
       face_flux(0, QL, ax, r, efv, out);
 #pragma unroll
       for (int v = 0; v < NRV; ++v) xb[FXI(px + v * XC + xo, n_xb)] = out[v];
       if constexpr (D == 3) {
 #pragma unroll
         for (int v = 0; v < NRV; ++v) QL[v] = yb[FXI(px + v * XC + yo, n_xb)];
-        rec_ld(k, NXF + ly * TX + lx, r);
+        rec_ld(par, NXF + ly * TX + lx, r);
         face_flux(1, QL, ay, r, efv, out);
 #pragma unroll
         for (int v = 0; v < NRV; ++v) yb[FXI(px + v * XC + yo, n_xb)] = out[v];
       }
       if constexpr (D >= 2) {
-        rec_ld(k, NXF + NYF + tc, r);
+        rec_ld(par, NXF + NYF + tc, r);
         face_flux(MD, bm0, am1, r, efv, rfm_new);
       }
     }
@@ -1171,7 +1187,7 @@ stage_kernel(const __grid_constant__ StageArgs<R> A) {
       R r[4];
 #pragma unroll
       for (int v = 0; v < NRV; ++v) { QL[v] = p[v * XC]; QR[v] = pr[v * sr]; }
-      rec_ld(k, isx ? c * (TX + 1) + TX : NXF + TY * TX + c, r);
+      rec_ld(par, isx ? c * (TX + 1) + TX : NXF + TY * TX + c, r);
       if (D < 3 || isx) face_flux(0, QL, QR, r, ef_of(ln), out);
       else face_flux(D == 3 ? 1 : 0, QL, QR, r, ef_of(ln), out);
 #pragma unroll
@@ -1179,14 +1195,14 @@ stage_kernel(const __grid_constant__ StageArgs<R> A) {
     }
     cp_async_wait_all();
     if (more && (fin_xy || k + 3 >= nmarch)) {
-      finish_own(k + 3);
-      finish_halo(k + 1);
+      finish_own(k + 3, s3);
+      finish_halo(k + 1, par ^ 1);
     }
     __syncthreads();
     // ---- D
     if (cell_in) {
       V Q0[NRV], U[NRV];
-      own_ld(k, Q0);
+      own_ld(s0, Q0);
       const uint32_t cidx = cxy + (uint32_t)k * pcells;
       V xm[NRV], xp[NRV], ym[NRV], yp[NRV];
 #pragma unroll
