@@ -366,7 +366,7 @@ __device__ __forceinline__ void adj_face_dir(const AdjArgs<R>& A, int64_t f) {
     Sc[s] = KR.sigma0 * rho;
   }
   const R ell = t(T_ELL, bc_pad(id));
-  const MCCoef<R> mcL = mc_coef(t, bc_pad(id - 1)), mcR = mc_coef(t, bc_pad(id));
+  const MCCoef<R> mcL = mc_coef<R>(t, bc_pad(id - 1)), mcR = mc_coef<R>(t, bc_pad(id));
   for (int gg = 0; gg < G; ++gg) {
     R lout[NRV];
     bool any = objective;

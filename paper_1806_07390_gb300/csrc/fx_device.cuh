@@ -166,6 +166,15 @@ template <class R> struct TabRow {
   __device__ __forceinline__ R operator()(int e, int) const { return row[e]; }
 };
 
+// One row of a direction's table, found once: a kernel that reads several entries of a row pays
+// for the test, the clamp and the address of Tab's reads once per row instead of once per entry.
+template <class R> struct TabAt {
+  const R* p;  // entry 0 of the row
+  int np;
+  __device__ __forceinline__ TabAt(const R* tab, int n, int ip) : p(tab + min(max(ip, 0), n + 3)), np(n + 4) {}
+  __device__ __forceinline__ R operator()(int e, int) const { return __ldg(p + e * np); }
+};
+
 // ---------------------------------------------------------------------------------------------
 // Parabolic (n = 2) reconstruction of one variable in one cell (Sec. 5.1; readings R2-R4).
 // ip: padded index of the cell (cell i -> i + 2).  R: table type; V: value type (R itself, or a
@@ -226,7 +235,7 @@ __device__ __forceinline__ void recon_parabolic(const Tab<R>& t, int ip, V pm, V
 // Coefficients of the linear MC reconstruction of one cell (shared by all its variables and
 // groups): inverse centroid gaps and the face offsets from the centroid.
 template <class R> struct MCCoef { R il, ir, ic, dl, dr; };
-template <class R> __device__ __forceinline__ MCCoef<R> mc_coef(const Tab<R>& t, int ip) {
+template <class R, class T> __device__ __forceinline__ MCCoef<R> mc_coef(const T& t, int ip) {
   return {t(T_IL, ip), t(T_IR, ip), t(T_IC, ip), t(T_DL, ip), t(T_DR, ip)};
 }
 template <class R, class V>

@@ -442,7 +442,7 @@ __device__ __forceinline__ void cp_async16(void* s, const void* g) {
 // 12: 1355 in 58 % at 16 warps; DRAM 1.0x the algorithmic bytes), the FP64 state by the FP64 pipe (86
 // % busy, 239 operations per cell and group).  Measured (FP32 state unless noted, one launch):
 // 1024^2 x 16 groups 0.455 -> 0.234 ms, 256^3 x 12 16.4 -> 6.2 ms, 640 x 128 x 20 spherical 0.124 ->
-// 0.067 ms, 512^2 x 24 channels 0.23 -> 0.094 ms, 512^2 x 16 FP64 2.99 -> 1.86 ms, against one kernel
+// 0.050 ms, 512^2 x 24 channels 0.23 -> 0.094 ms, 512^2 x 16 FP64 2.99 -> 1.86 ms, against one kernel
 // with lanes padded to a power of two, geometry tables on every grid, and the gas update in its lanes.
 //
 // Block sizes (StageCap).  A thread holds about 90 values at order 1, so 20 warps of 96 registers in
@@ -735,10 +735,15 @@ stage_kernel(const __grid_constant__ StageArgs<R> A) {
   const int HV = D == 3 ? HS : NT, HPAR = D == 3 ? NRV * HS : HS;
   (void)n_ring; (void)n_base; (void)n_xb; (void)n_xr; (void)n_yr; (void)n_halo; (void)n_rec;
 
-  const Tab<R> tx{A.tab[0], nx + 4, A.uniform[0] ? A.urow[0] : nullptr};
-  const Tab<R> ty{A.tab[D >= 2 ? 1 : 0], (D >= 2 ? ny : nx) + 4, A.uniform[D >= 2 ? 1 : 0] ? A.urow[D >= 2 ? 1 : 0] : nullptr};
-  const Tab<R> tz{A.tab[D >= 3 ? 2 : 0], (D >= 3 ? nz : nx) + 4, A.uniform[D >= 3 ? 2 : 0] ? A.urow[D >= 3 ? 2 : 0] : nullptr};
-  const Tab<R>& tm = D == 3 ? tz : ty;
+  // The geometry tables, a row at a time: a Cartesian direction has one row for every cell (of the
+  // launch arguments).  On the spherical grid a thread keeps the address of its own cell's row and
+  // takes the other rows (halo cells, planes) once for all their entries; every entry fetched
+  // through the general reader (Tab) made 640 x 128 x 20 67 us instead of 50.
+  using TT = typename std::conditional<SPH, TabAt<R>, TabRow<R>>::type;
+  auto row_of_dir = [&](int d, int i) -> TT {
+    if constexpr (SPH) return TT(A.tab[d], g.n[d], bc_pad(i));
+    else return TT{A.urow[d]};
+  };
 
   // ---- positions.  Ghost cells are index maps (Sec. 7.5); tiles may overhang the grid, their
   // cells past the first two ghosts are never used and clamped into the array.
@@ -763,6 +768,7 @@ stage_kernel(const __grid_constant__ StageArgs<R> A) {
   bool fx_own = false, fy_own = false;
   const uint32_t cxy = inplane(lx, ly, fx_own, fy_own);
   const int gx = x0 + lx, gy = y0 + ly;
+  const TT tx = row_of_dir(0, gx), ty = row_of_dir(D == 3 ? 1 : 0, gy);  // rows of the own cell
   const bool cell_in = act && gx < nx && (D < 3 || gy < ny);
   const uint32_t toff = cxy * (uint32_t)G + g0;  // the thread's elements in a plane of a radiation variable
   const uint32_t vstride = ncell * (uint32_t)G, pstride = pcells * (uint32_t)G;
@@ -880,21 +886,21 @@ stage_kernel(const __grid_constant__ StageArgs<R> A) {
       cp_async_lane(&sbase[FXI(v * NT + tid, n_base)], FXP(plane_at(A.base, v, row), toff, vstride - row), vec, h1);
   };
   // scale factor of component q of the cell with x index ix on plane k
-  auto hfac = [&](int q, int ix, int k) -> R {
+  auto hfac = [&](int q, const TT& rx, const TT& rm) -> R {
     if (!SPH) return R(1);
     const int e = q == 0 ? T_HA : T_HB;
-    return tx(e, bc_pad(ix)) * tm(e, bc_pad(k));
+    return rx(e, 0) * rm(e, 0);
   };
   // after the wait, each thread finishes what it copied: the mirrored components of ghost cells
   // change sign, and on the spherical grid covariant flux components become physical.  Planes
   // inside the grid of blocks without mirrored in-plane ghosts need neither.
   const bool fin_xy = SPH || g.bc_lo[0] >= 2 || g.bc_hi[0] >= 2 || (D == 3 && (g.bc_lo[1] >= 2 || g.bc_hi[1] >= 2));
-  auto finish_one = [&](V* p, int vs, bool fx, bool fy, bool fm, int ix, int P) {
+  auto finish_one = [&](V* p, int vs, bool fx, bool fy, bool fm, const TT& rx, const TT& rm) {
 #pragma unroll
     for (int q = 0; q < D; ++q) {
       const bool fl = q == MD && D > 1 ? fm : (q == 0 ? fx : fy);
       V x = p[(1 + q) * vs];
-      if (SPH) x = x * frcp(hfac(q, ix, P));
+      if (SPH) x = x * frcp(hfac(q, rx, rm));
       if (fl) x = -x;
       p[(1 + q) * vs] = x;
     }
@@ -903,17 +909,18 @@ stage_kernel(const __grid_constant__ StageArgs<R> A) {
     bool fm = false;
     map_m(P, fm);
     if (SPH || fx_own || fy_own || fm)
-      finish_one(&ring[FXI(slot + tid, n_ring)], NT, fx_own, fy_own, fm, gx, P);
+      finish_one(&ring[FXI(slot + tid, n_ring)], NT, fx_own, fy_own, fm, tx, row_of_dir(MD, P));
   };
   auto finish_halo = [&](int P, int par) {
     bool fm = false;
     map_m(P, fm);
+    const TT rm = row_of_dir(MD, P);
     for (int t = ht0; t < HS; t += NTH) {
       int sx, sy;
       bool f0 = false, f1 = false;
       halo_pos(div_gl(t), sx, sy);
       inplane(sx, sy, f0, f1);
-      if (SPH || f0 || f1 || fm) finish_one(&halo[FXI(par * HPAR + t, n_halo)], HV, f0, f1, fm, x0 + sx, P);
+      if (SPH || f0 || f1 || fm) finish_one(&halo[FXI(par * HPAR + t, n_halo)], HV, f0, f1, fm, row_of_dir(0, x0 + sx), rm);
     }
   };
 
@@ -937,18 +944,18 @@ stage_kernel(const __grid_constant__ StageArgs<R> A) {
   const int ym_o = ym_h ? (4 * TY + TX + lx) * GL + lane : otid - TX * GL;
   const int yp_o = yp_h ? (4 * TY + 2 * TX + lx) * GL + lane : otid + TX * GL;
   // face states of one cell along a direction: a at its lower face, b at its upper face
-  auto recon = [&](const Tab<R>& t, int ip, const V* Qm, const V* Q0, const V* Qp, V* a, V* b) {
+  auto recon = [&](const TT& t, const V* Qm, const V* Q0, const V* Qp, V* a, V* b) {
     if constexpr (RO == 2) {
 #pragma unroll
       for (int v = 0; v < NRV; ++v) {
         R a0, b0, a1 = R(0), b1 = R(0);
-        recon_parabolic(t, ip, vget(Qm[v], 0), vget(Q0[v], 0), vget(Qp[v], 0), a0, b0);
-        if (W == 2) recon_parabolic(t, ip, vget(Qm[v], 1), vget(Q0[v], 1), vget(Qp[v], 1), a1, b1);
+        recon_parabolic(t, 0, vget(Qm[v], 0), vget(Q0[v], 0), vget(Qp[v], 0), a0, b0, R(0));
+        if (W == 2) recon_parabolic(t, 0, vget(Qm[v], 1), vget(Q0[v], 1), vget(Qp[v], 1), a1, b1, R(0));
         a[v] = vpair(a0, a1, V());
         b[v] = vpair(b0, b1, V());
       }
     } else if constexpr (SPH) {
-      const MCCoef<R> c = mc_coef(t, ip);
+      const MCCoef<R> c = mc_coef<R>(t, 0);
 #pragma unroll
       for (int v = 0; v < NRV; ++v) {
         const V s = mc_min((Q0[v] - Qm[v]) * c.il, (Qp[v] - Q0[v]) * c.ir, (Qp[v] - Qm[v]) * c.ic, R(2));
@@ -1018,6 +1025,7 @@ stage_kernel(const __grid_constant__ StageArgs<R> A) {
     V Qa[NRV];  // own column of plane kbeg-2, straight from global memory
     {
       bool fm = false;
+      const TT rm = row_of_dir(MD, kbeg - 2);
       const uint32_t o = NG * ncell + toff + (uint32_t)map_m(kbeg - 2, fm) * pstride;
 #pragma unroll
       for (int v = 0; v < NRV; ++v) {
@@ -1027,7 +1035,7 @@ stage_kernel(const __grid_constant__ StageArgs<R> A) {
 #pragma unroll
       for (int q = 0; q < D; ++q) {
         const bool fl = q == MD ? fm : (q == 0 ? fx_own : fy_own);
-        if (SPH) Qa[1 + q] = Qa[1 + q] * frcp(hfac(q, gx, kbeg - 2));
+        if (SPH) Qa[1 + q] = Qa[1 + q] * frcp(hfac(q, tx, rm));
         if (fl) Qa[1 + q] = -Qa[1 + q];
       }
     }
@@ -1047,11 +1055,10 @@ stage_kernel(const __grid_constant__ StageArgs<R> A) {
     own_ld(ring_slot(kbeg - 1), Qb);
     own_ld(ring_slot(kbeg), Qc);
     own_ld(ring_slot(kbeg + 1), Qd);
-    recon(tm, bc_pad(kbeg - 1), Qa, Qb, Qc, ta, tb);
-    recon(tm, bc_pad(kbeg), Qb, Qc, Qd, am, bm0);
+    recon(row_of_dir(MD, kbeg - 1), Qa, Qb, Qc, ta, tb);
+    recon(row_of_dir(MD, kbeg), Qb, Qc, Qd, am, bm0);
     face_flux(MD, tb, am, r, efv, rfm_old);
   }
-  const int ipx = bc_pad(gx), ipy = bc_pad(gy);
 
   // the halo reconstructions as tasks, one per (row or column end, lane): the upper-face state of
   // cells -1 (left state of the tile's first face) and the lower-face state of cells TX, TY (right
@@ -1085,13 +1092,12 @@ stage_kernel(const __grid_constant__ StageArgs<R> A) {
     nb_ld(slot, par, true, b_.h, Q0);
     nb_ld(slot, par, true, b_.h + b_.hs, Qo);
     if constexpr (TABLES) {
-      const Tab<R>& tt = b_.x ? tx : ty;
-      const int ip = b_.x ? bc_pad(b_.up ? x0 + TX : x0 - 1) : bc_pad(b_.up ? y0 + TY : y0 - 1);
-      if (b_.up) recon(tt, ip, Qi, Q0, Qo, a, b);
-      else recon(tt, ip, Qo, Q0, Qi, b, a);
+      const TT tt = b_.x ? row_of_dir(0, b_.up ? x0 + TX : x0 - 1) : ty;
+      if (b_.up) recon(tt, Qi, Q0, Qo, a, b);
+      else recon(tt, Qo, Q0, Qi, b, a);
     } else {
       // (uniform spacing: the other way round gives the mirrored states)
-      recon(tx, 0, Qi, Q0, Qo, a, b);
+      recon(tx, Qi, Q0, Qo, a, b);
     }
     V* const d = b_.up ? (b_.x ? xr + FXI(b_.dst, n_xr) : yr + FXI(b_.dst, n_yr))
                        : (b_.x ? xb : yb) + FXI(px + b_.dst, n_xb);
@@ -1129,20 +1135,20 @@ stage_kernel(const __grid_constant__ StageArgs<R> A) {
       own_ld(s0, Q0);
       nb_ld(s0, par, xm_h, xm_o, Qm);
       nb_ld(s0, par, xp_h, xp_o, Qp);
-      recon(tx, ipx, Qm, Q0, Qp, ax, b);
+      recon(tx, Qm, Q0, Qp, ax, b);
 #pragma unroll
       for (int v = 0; v < NRV; ++v) xb[FXI(px + v * XC + xo + GL, n_xb)] = b[v];
       if constexpr (D == 3) {
         nb_ld(s0, par, ym_h, ym_o, Qm);
         nb_ld(s0, par, yp_h, yp_o, Qp);
-        recon(ty, ipy, Qm, Q0, Qp, ay, b);
+        recon(ty, Qm, Q0, Qp, ay, b);
 #pragma unroll
         for (int v = 0; v < NRV; ++v) yb[FXI(px + v * XC + yo + TX * GL, n_xb)] = b[v];
       }
       if constexpr (D >= 2) {
         own_ld(s1, Qm);
         own_ld(s2, Qp);
-        recon(tm, bc_pad(k + 1), Q0, Qm, Qp, am1, bm1);
+        recon(row_of_dir(MD, k + 1), Q0, Qm, Qp, am1, bm1);
       }
     }
     if (tid < ntask) run_task(s0, par, px, my);
@@ -1218,10 +1224,10 @@ stage_kernel(const __grid_constant__ StageArgs<R> A) {
         // area/volume factors of the two face pairs per flux class (half: twice the flux is
         // carried), and the geometric sources <Gamma^l_jk> T^k_l of the stage's input state (Eq. 9;
         // Appendix D)
-        const int ipm = bc_pad(k);
-        const R hq[2] = {hfac(0, gx, k), hfac(1, gx, k)};
-        const R g111 = tx(T_GA, ipx), g221 = tx(T_GB, ipx), g122 = tx(T_GC, ipx);
-        const R g222 = tm(T_GA, ipm), g332 = tm(T_GB, ipm);
+        const TT tm = row_of_dir(MD, k);
+        const R hq[2] = {hfac(0, tx, tm), hfac(1, tx, tm)};
+        const R g111 = tx(T_GA, 0), g221 = tx(T_GB, 0), g122 = tx(T_GC, 0);
+        const R g222 = tm(T_GA, 0), g332 = tm(T_GB, 0);
         const R rho = A.in[FXI(cidx, A.n_state)], irho = frcp(rho);
         const R v1 = A.in[FXI(ncell + cidx, A.n_state)] * irho * frcp(hq[0]), v2 = A.in[FXI(2 * ncell + cidx, A.n_state)] * irho * frcp(hq[1]);
         const R r12 = hq[0] * frcp(hq[1]), r21 = hq[1] * frcp(hq[0]);
@@ -1238,9 +1244,9 @@ stage_kernel(const __grid_constant__ StageArgs<R> A) {
 #pragma unroll
         for (int v = 0; v < NRV; ++v) {
           const V Fp[2] = {xp[v], rfm_new[v]}, Fm[2] = {xm[v], rfm_old[v]};
-          const R xs = R(0.5) * tm(eX[v], ipm), ms = R(0.5) * tx(eX[v], ipx);
-          const R Ap[2] = {tx(eR[v], ipx) * xs, tm(eR[v], ipm) * ms};
-          const R Am[2] = {tx(eL[v], ipx) * xs, tm(eL[v], ipm) * ms};
+          const R xs = R(0.5) * tm(eX[v], 0), ms = R(0.5) * tx(eX[v], 0);
+          const R Ap[2] = {tx(eR[v], 0) * xs, tm(eR[v], 0) * ms};
+          const R Am[2] = {tx(eL[v], 0) * xs, tm(eL[v], 0) * ms};
           const V cov = v >= 1 ? Q0[v] * hq[v - 1] : Q0[v];  // covariant F
           U[v] = fv_update(Fp, Ap, Fm, Am, cov, src[v], KR.dt, stage2, stage2 ? sbase[FXI(v * NT + tid, n_base)] : V(R(0)),
                            KR.alpha, KR.beta);
@@ -1261,27 +1267,27 @@ stage_kernel(const __grid_constant__ StageArgs<R> A) {
         const bool yl = D == 3 && gy == 0 && g.bc_lo[1] != 1, yh = D == 3 && gy == ny - 1 && g.bc_hi[1] != 1;
         const bool ml = D >= 2 && k == 0 && g.bc_lo[MD] != 1, mh = D >= 2 && k == nmarch - 1 && g.bc_hi[MD] != 1;
         if (xl || xh || yl || yh || ml || mh) {
-          const int ipm = bc_pad(k);
-          double vol = (double)tx(T_VOL, ipx);
-          if (D == 3) vol *= (double)ty(T_VOL, ipy);
-          if (D >= 2) vol *= (double)tm(T_VOL, ipm);
+          const TT tm = row_of_dir(MD, k);
+          double vol = (double)tx(T_VOL, 0);
+          if (D == 3) vol *= (double)ty(T_VOL, 0);
+          if (D >= 2) vol *= (double)tm(T_VOL, 0);
           const double bs = 0.5 * vol * A.bw_flux;  // (twice the flux is carried)
           double* const bud = A.budget + (size_t)(blockIdx.x % BUDGET_SLOTS) * NBUDGET;
           const int eL[3] = {T_FL, T_FL1, T_FL2}, eR[3] = {T_FR, T_FR1, T_FR2}, eX[3] = {T_XS, T_X1, T_X2};
 #pragma unroll
           for (int v = 0; v < NRV; ++v) {
             const int c = SPH ? v : 0;
-            const R sx = SPH ? tm(eX[c], ipm) : R(1), sm_ = SPH ? tx(eX[c], ipx) : R(1);
+            const R sx = SPH ? tm(eX[c], 0) : R(1), sm_ = SPH ? tx(eX[c], 0) : R(1);
             double o = 0.0;
 #pragma unroll
             for (int j = 0; j < W; ++j) {
               if (j == 1 && !h1) continue;
-              if (xh) o += (double)(vget(xp[v], j) * (tx(eR[c], ipx) * sx));
-              if (xl) o -= (double)(vget(xm[v], j) * (tx(eL[c], ipx) * sx));
-              if (D == 3 && yh) o += (double)(vget(yp[v], j) * ty(T_FR, ipy));
-              if (D == 3 && yl) o -= (double)(vget(ym[v], j) * ty(T_FL, ipy));
-              if (D >= 2 && mh) o += (double)(vget(rfm_new[v], j) * (tm(eR[c], ipm) * sm_));
-              if (D >= 2 && ml) o -= (double)(vget(rfm_old[v], j) * (tm(eL[c], ipm) * sm_));
+              if (xh) o += (double)(vget(xp[v], j) * (tx(eR[c], 0) * sx));
+              if (xl) o -= (double)(vget(xm[v], j) * (tx(eL[c], 0) * sx));
+              if (D == 3 && yh) o += (double)(vget(yp[v], j) * ty(T_FR, 0));
+              if (D == 3 && yl) o -= (double)(vget(ym[v], j) * ty(T_FL, 0));
+              if (D >= 2 && mh) o += (double)(vget(rfm_new[v], j) * (tm(eR[c], 0) * sm_));
+              if (D >= 2 && ml) o -= (double)(vget(rfm_old[v], j) * (tm(eL[c], 0) * sm_));
             }
             if (o != 0.0) {
               if (v == 0) {
