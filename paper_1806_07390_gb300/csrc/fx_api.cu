@@ -817,12 +817,12 @@ fx_status launch_one_stage(fx_grid* h, const StageArgs<R>& a, const char* what) 
     if (e != cudaSuccess) return cuda_fail(h, e, "timing event");
   }
   switch (h->D) {
-    case 1: e = launch_stage<R, 1, NT, false>(a, h->GP, h->stream, e4[1], e4[2]); break;
+    case 1: e = launch_stage<R, 1, NT, false>(a, h->stream, e4[1], e4[2]); break;
     case 2:
-      e = h->P.geom == FX_SPH ? launch_stage<R, 2, NT, true>(a, h->GP, h->stream, e4[1], e4[2])
-                              : launch_stage<R, 2, NT, false>(a, h->GP, h->stream, e4[1], e4[2]);
+      e = h->P.geom == FX_SPH ? launch_stage<R, 2, NT, true>(a, h->stream, e4[1], e4[2])
+                              : launch_stage<R, 2, NT, false>(a, h->stream, e4[1], e4[2]);
       break;
-    default: e = launch_stage<R, 3, NT, false>(a, h->GP, h->stream, e4[1], e4[2]); break;
+    default: e = launch_stage<R, 3, NT, false>(a, h->stream, e4[1], e4[2]); break;
   }
   if (e == cudaSuccess && e4[3]) e = cudaEventRecord(e4[3], h->stream);
   if (e == cudaSuccess && a.phi_out) {
@@ -868,11 +868,11 @@ cudaGraphExec_t capture_step(fx_grid* h, const StageArgs<R>& a1, const StageArgs
   }
   auto launch = [&](const StageArgs<R>& a) -> cudaError_t {
     switch (h->D) {
-      case 1: return launch_stage<R, 1, NT, false>(a, h->GP, h->cap_stream, nullptr, nullptr);
+      case 1: return launch_stage<R, 1, NT, false>(a, h->cap_stream, nullptr, nullptr);
       case 2:
-        return h->P.geom == FX_SPH ? launch_stage<R, 2, NT, true>(a, h->GP, h->cap_stream, nullptr, nullptr)
-                                   : launch_stage<R, 2, NT, false>(a, h->GP, h->cap_stream, nullptr, nullptr);
-      default: return launch_stage<R, 3, NT, false>(a, h->GP, h->cap_stream, nullptr, nullptr);
+        return h->P.geom == FX_SPH ? launch_stage<R, 2, NT, true>(a, h->cap_stream, nullptr, nullptr)
+                                   : launch_stage<R, 2, NT, false>(a, h->cap_stream, nullptr, nullptr);
+      default: return launch_stage<R, 3, NT, false>(a, h->cap_stream, nullptr, nullptr);
     }
   };
   // the step waits for the bound stream's earlier work through the graph launch itself
@@ -1104,8 +1104,11 @@ fx_status adjoint_impl(fx_grid* h, double dt, int nsteps, int k, unsigned char* 
 #ifdef FX_BOUNDS_CHECK
   b.status = a.status;
   b.n_state = a.n_state;
+  b.n_lvs = a.n_recs;
 #endif
   b.lam_w = LW;
+  b.lvs = a.frec;
+  for (int d = 0; d < 3; ++d) b.lvs_off[d] = a.rec_off[d];
   b.kpart = kpart;
   b.phi_area = (R)h->phi_area;
   b.dt = dt;
@@ -1115,6 +1118,7 @@ fx_status adjoint_impl(fx_grid* h, double dt, int nsteps, int k, unsigned char* 
   b2.alpha = 0.5; b2.kd = a2.kd; b2.kf = a2.kf;
   e = cudaMemsetAsync(LA, 0, h->state_bytes, st);
   if (e == cudaSuccess) e = cudaMemsetAsync(obj + 1, 0, sizeof(double), st);
+  if (e == cudaSuccess) e = cudaMemsetAsync(kpart, 0, (size_t)L.nblk * sizeof(double), st);
   if (e != cudaSuccess) { h->timing = tim; return cuda_fail(h, e, "adjoint setup"); }
   auto run = [&](AdjArgs<R>& bb) -> cudaError_t {
     cudaError_t x;
@@ -1124,7 +1128,6 @@ fx_status adjoint_impl(fx_grid* h, double dt, int nsteps, int k, unsigned char* 
       default: x = adj_launch_couple<R, 3>(bb, h->GP, st); break;
     }
     if (x != cudaSuccess) return x;
-    k_sum_into<double><<<1, 1024, 0, st>>>(kpart, L.nblk, 1.0, obj + 1);
     x = cudaMemsetAsync(LW, 0, L.LWn, st);
     if (x != cudaSuccess) return x;
     switch (h->D) {
@@ -1138,9 +1141,7 @@ fx_status adjoint_impl(fx_grid* h, double dt, int nsteps, int k, unsigned char* 
       case 2: x = adj_launch_cell<R, 2>(bb, h->GP, st); break;
       default: x = adj_launch_cell<R, 3>(bb, h->GP, st); break;
     }
-    if (x != cudaSuccess) return x;
-    k_sum_into<double><<<1, 1024, 0, st>>>(kpart, L.nblk, 1.0, obj + 1);
-    return cudaGetLastError();
+    return x;
   };
   const bool recorded = h->adj_rec_ws == ws && h->adj_rec_nsteps == nsteps && h->adj_rec_k == k &&
                         h->adj_rec_dt == dt;
@@ -1172,6 +1173,10 @@ fx_status adjoint_impl(fx_grid* h, double dt, int nsteps, int k, unsigned char* 
       if (e != cudaSuccess) { h->timing = tim; return cuda_fail(h, e, "adjoint stage 1"); }
     }
   }
+  // the kappa0 partials that every stage's kernels added to, block by block
+  k_sum_into<double><<<1, 1024, 0, st>>>(kpart, L.nblk, 1.0, obj + 1);
+  e = cudaGetLastError();
+  if (e != cudaSuccess) { h->timing = tim; return cuda_fail(h, e, "adjoint sum"); }
   h->timing = tim;
   if (grad_state) {
     e = cudaMemcpyAsync(grad_state, LA, h->state_bytes, cudaMemcpyDeviceToDevice, st);

@@ -72,6 +72,10 @@ __device__ __forceinline__ bool opposite_sign(float a, float b) { return a * b <
 __device__ __forceinline__ int cmp_abs(float a, float b) { return fabsf(a) < fabsf(b) ? -1 : (fabsf(a) == fabsf(b) ? 0 : 1); }
 __device__ __forceinline__ float median(float x, float u, float v) { return fmaxf(fminf(u, v), fminf(fmaxf(u, v), x)); }
 __device__ __forceinline__ bool nonzero64(double a) { return (__double_as_longlong(a) << 1) != 0; }
+__device__ __forceinline__ bool nonzero(float a) { return a != 0.0f; }
+__device__ __forceinline__ bool nonzero(double a) { return nonzero64(a); }
+__device__ __forceinline__ bool differ(float a, float b) { return __float_as_int(a) != __float_as_int(b); }
+__device__ __forceinline__ bool differ(double a, double b) { return __double_as_longlong(a) != __double_as_longlong(b); }
 __device__ __forceinline__ bool same_sign(double a, double b) {
   return (__double2hiint(a) ^ __double2hiint(b)) >= 0 && nonzero64(a) && nonzero64(b);
 }
@@ -177,59 +181,29 @@ template <class R> struct TabAt {
 
 // ---------------------------------------------------------------------------------------------
 // Parabolic (n = 2) reconstruction of one variable in one cell (Sec. 5.1; readings R2-R4).
-// ip: padded index of the cell (cell i -> i + 2).  R: table type; V: value type (R itself, or a
-// forward-mode dual number when the adjoint forms local Jacobians).
+// ip: padded index of the cell (cell i -> i + 2).
 // ---------------------------------------------------------------------------------------------
-template <class T, class R, class V>
-__device__ __forceinline__ void recon_parabolic(const T& t, int ip, V pm, V p0, V pp, V& a, V& b, R) {
-  V dl = p0 - pm, dr = pp - p0;
-  if constexpr (std::is_same<V, R>::value) {
-    // the same decisions as the general code below, taken as selects over values computed for
-    // every cell, so that a warp runs one path; in FP64 the decisions are integer comparisons
-    const bool ext = !same_sign(dl, dr);
-    V a0 = t(T_WA0, ip) * pm + t(T_WA1, ip) * p0 + t(T_WA2, ip) * pp;
-    V b0 = t(T_WB0, ip) * pm + t(T_WB1, ip) * p0 + t(T_WB2, ip) * pp;
-    // between the zero-slope values at the two centroids, whichever is the lower one
-    a0 = median(a0, pm + dl * t(T_SL2, ip), p0 - dl * t(T_TL2, ip));
-    b0 = median(b0, p0 + dr * t(T_SR2, ip), pp - dr * t(T_TR2, ip));
-    const V sl = t(T_AL0, ip) * a0 + t(T_AL1, ip) * p0 + t(T_AL2, ip) * b0;
-    const V sr = t(T_AR0, ip) * a0 + t(T_AR1, ip) * p0 + t(T_AR2, ip) * b0;
-    const bool inc = opposite_sign(sl, sr);  // extremum inside the cell
-    const int cmp = cmp_abs(sl, sr);
-    const V bz = a0 + (p0 - a0) * t(T_RHL, ip);  // zero slope at the lower face
-    const V az = b0 + (p0 - b0) * t(T_RHR, ip);  // zero slope at the upper face
-    const V an = inc ? (cmp == 0 ? p0 : (cmp < 0 ? a0 : az)) : a0;
-    const V bn = inc ? (cmp == 0 ? p0 : (cmp < 0 ? bz : b0)) : b0;
-    a = ext ? p0 : an;
-    b = ext ? p0 : bn;
-    return;
-  }
-  if (dl * dr <= R(0)) { a = p0; b = p0; return; }  // extremum of the data (R4)
-  a = t(T_WA0, ip) * pm + t(T_WA1, ip) * p0 + t(T_WA2, ip) * pp;
-  b = t(T_WB0, ip) * pm + t(T_WB1, ip) * p0 + t(T_WB2, ip) * pp;
-  // face-interval monotonicity (R2): clamp between the zero-slope values at the two centroids
-  {
-    V lo = pm + dl * t(T_SL2, ip), hi = p0 - dl * t(T_TL2, ip);
-    if (dl < R(0)) { V s = lo; lo = hi; hi = s; }
-    a = a < lo ? lo : (a > hi ? hi : a);
-  }
-  {
-    V lo = p0 + dr * t(T_SR2, ip), hi = pp - dr * t(T_TR2, ip);
-    if (dr < R(0)) { V s = lo; lo = hi; hi = s; }
-    b = b < lo ? lo : (b > hi ? hi : b);
-  }
-  // system 2 end slopes; opposite signs mean an extremum inside the cell (R3)
-  V sl = t(T_AL0, ip) * a + t(T_AL1, ip) * p0 + t(T_AL2, ip) * b;
-  V sr = t(T_AR0, ip) * a + t(T_AR1, ip) * p0 + t(T_AR2, ip) * b;
-  if (sl * sr >= R(0)) return;
-  V asl = fabs(sl), asr = fabs(sr);
-  if (asl == asr) { a = p0; b = p0; return; }
-  if (asl < asr) b = a + (p0 - a) * t(T_RHL, ip);  // zero slope at the lower face
-  else a = b + (p0 - b) * t(T_RHR, ip);            // zero slope at the upper face
-}
-template <class R, class V>
-__device__ __forceinline__ void recon_parabolic(const Tab<R>& t, int ip, V pm, V p0, V pp, V& a, V& b) {
-  recon_parabolic(t, ip, pm, p0, pp, a, b, R(0));
+template <class T, class V>
+__device__ __forceinline__ void recon_parabolic(const T& t, int ip, V pm, V p0, V pp, V& a, V& b) {
+  const V dl = p0 - pm, dr = pp - p0;
+  // decisions are selects over values computed for every cell, so that a warp runs one path; in FP64
+  // they are integer comparisons
+  const bool ext = !same_sign(dl, dr);
+  V a0 = t(T_WA0, ip) * pm + t(T_WA1, ip) * p0 + t(T_WA2, ip) * pp;
+  V b0 = t(T_WB0, ip) * pm + t(T_WB1, ip) * p0 + t(T_WB2, ip) * pp;
+  // between the zero-slope values at the two centroids, whichever is the lower one
+  a0 = median(a0, pm + dl * t(T_SL2, ip), p0 - dl * t(T_TL2, ip));
+  b0 = median(b0, p0 + dr * t(T_SR2, ip), pp - dr * t(T_TR2, ip));
+  const V sl = t(T_AL0, ip) * a0 + t(T_AL1, ip) * p0 + t(T_AL2, ip) * b0;
+  const V sr = t(T_AR0, ip) * a0 + t(T_AR1, ip) * p0 + t(T_AR2, ip) * b0;
+  const bool inc = opposite_sign(sl, sr);  // extremum inside the cell
+  const int cmp = cmp_abs(sl, sr);
+  const V bz = a0 + (p0 - a0) * t(T_RHL, ip);  // zero slope at the lower face
+  const V az = b0 + (p0 - b0) * t(T_RHR, ip);  // zero slope at the upper face
+  const V an = inc ? (cmp == 0 ? p0 : (cmp < 0 ? a0 : az)) : a0;
+  const V bn = inc ? (cmp == 0 ? p0 : (cmp < 0 ? bz : b0)) : b0;
+  a = ext ? p0 : an;
+  b = ext ? p0 : bn;
 }
 
 // Coefficients of the linear MC reconstruction of one cell (shared by all its variables and
@@ -238,22 +212,6 @@ template <class R> struct MCCoef { R il, ir, ic, dl, dr; };
 template <class R, class T> __device__ __forceinline__ MCCoef<R> mc_coef(const T& t, int ip) {
   return {t(T_IL, ip), t(T_IR, ip), t(T_IC, ip), t(T_DL, ip), t(T_DR, ip)};
 }
-template <class R, class V>
-__device__ __forceinline__ void recon_linear_c(const MCCoef<R>& c, V pm, V p0, V pp, V& a, V& b) {
-  V sL = (p0 - pm) * c.il;
-  V sR = (pp - p0) * c.ir;
-  V s = V(R(0));
-  if constexpr (std::is_same<V, float>::value) {
-    // FP32: the limited slope computed unconditionally and selected (no divergent branch)
-    s = mc_slope(sL, sR, (pp - pm) * c.ic);
-  } else if (sL * sR > R(0)) {
-    V sC = (pp - pm) * c.ic;
-    V m = fmin(fmin(R(2) * fabs(sL), R(2) * fabs(sR)), fabs(sC));
-    s = sC > R(0) ? m : -m;
-  }
-  a = p0 + s * c.dl;
-  b = p0 + s * c.dr;
-}
 
 // ---------------------------------------------------------------------------------------------
 // HLLC (Sec. 5.2; Toro, Spruce & Speares 1994 with Batten et al. 1997 / Einfeldt speed bounds,
@@ -261,105 +219,51 @@ __device__ __forceinline__ void recon_linear_c(const MCCoef<R>& c, V pm, V p0, V
 // Output: fluxes of (rho, rho u_n, rho u_t1, rho u_t2, rho e) per unit physical area and the
 // contact speed (the particle velocity used to upwind radiation advection, Eq. 19).
 // ---------------------------------------------------------------------------------------------
-template <class R, int D, class V = R>
-__device__ __forceinline__ void hllc(R gam, const V* L, const V* Rs, V* f, V& vstar) {
-  if constexpr (std::is_same<V, R>::value) {
-    // The kernels' own types: every division is a reciprocal, shared where the denominator is (the
-    // FP64 form of a division costs twice a reciprocal's operations), and the choice among the
-    // supersonic and star fluxes is a select: the side k (left when the face is supersonic to the
-    // right or the contact moves right) and its plain flux F_k for every face; the star correction
-    // S_k (U*_k - U_k) is added where the face is subsonic.
-    const R igm1 = rcp_any(gam - R(1)), g1 = gam - R(1);
-    const R rl = L[0], pl = L[1], ul = L[2], rr = Rs[0], pr = Rs[1], ur = Rs[2];
-    R kl = ul * ul, kr = ur * ur;
-#pragma unroll
-    for (int q = 1; q < D; ++q) { kl += L[2 + q] * L[2 + q]; kr += Rs[2 + q] * Rs[2 + q]; }
-    const R El = pl * igm1 + R(0.5) * rl * kl, Er = pr * igm1 + R(0.5) * rr * kr;
-    const R irl = rcp_any(rl), irr = rcp_any(rr);
-    const R al = sqrt_any(gam * pl * irl), ar = sqrt_any(gam * pr * irr);
-    const R sl = sqrt_any(rl), sr = sqrt_any(rr), iw = rcp_any(sl + sr);
-    const R Ht = (sl * ((El + pl) * irl) + sr * ((Er + pr) * irr)) * iw;
-    const R ut = (sl * ul + sr * ur) * iw;
-    R v2 = ut * ut;
-#pragma unroll
-    for (int q = 1; q < D; ++q) { const R vq = (sl * L[2 + q] + sr * Rs[2 + q]) * iw; v2 += vq * vq; }
-    const R at2 = g1 * (Ht - R(0.5) * v2);
-    const R at = sqrt_any(nonneg(at2) ? at2 : R(0));
-    const R SL = min_fast(ul - al, ut - at), SR = max_fast(ur + ar, ut + at);
-    const R dl = rl * (SL - ul), dr = rr * (SR - ur);
-    const R Ss = (pr - pl + ul * dl - ur * dr) * rcp_any(dl - dr);
-    vstar = Ss;
-    const bool supL = nonneg(SL), supR = !supL && !nonneg(SR), sup = supL || supR;
-    const bool left = supL || (!supR && nonneg(Ss));
-    const R rk = left ? rl : rr, pk = left ? pl : pr, uk = left ? ul : ur;
-    const R Ek = left ? El : Er, Sk = left ? SL : SR, irk = left ? irl : irr;
-    const R sku = Sk - uk, m = rk * uk;
-    const R fac = rk * sku * rcp_any(Sk - Ss);
-    const R f1 = m * uk + pk;
-    f[0] = sup ? m : m + Sk * (fac - rk);
-    f[1] = sup ? f1 : f1 + Sk * (fac * Ss - m);
-#pragma unroll
-    for (int q = 1; q < D; ++q) {
-      const R wq = left ? L[2 + q] : Rs[2 + q];
-      const R fq = m * wq;
-      f[1 + q] = sup ? fq : fq + Sk * (fac * wq - rk * wq);
-    }
-    const R Es = fac * (Ek * irk + (Ss - uk) * (Ss + pk * (irk * rcp_any(sku))));
-    const R fE = (Ek + pk) * uk;
-    f[1 + D] = sup ? fE : fE + Sk * (Es - Ek);
-    return;
-  }
-  const R gm1 = gam - R(1);
-  V rl = L[0], pl = L[1], ul = L[2];
-  V rr = Rs[0], pr = Rs[1], ur = Rs[2];
-  V kl = ul * ul, kr = ur * ur;
+template <class R, int D>
+__device__ __forceinline__ void hllc(R gam, const R* L, const R* Rs, R* f, R& vstar) {
+  // Every division is a reciprocal, shared where the denominator is (the
+  // FP64 form of a division costs twice a reciprocal's operations), and the choice among the
+  // supersonic and star fluxes is a select: the side k (left when the face is supersonic to the
+  // right or the contact moves right) and its plain flux F_k for every face; the star correction
+  // S_k (U*_k - U_k) is added where the face is subsonic.
+  const R igm1 = rcp_any(gam - R(1)), g1 = gam - R(1);
+  const R rl = L[0], pl = L[1], ul = L[2], rr = Rs[0], pr = Rs[1], ur = Rs[2];
+  R kl = ul * ul, kr = ur * ur;
 #pragma unroll
   for (int q = 1; q < D; ++q) { kl += L[2 + q] * L[2 + q]; kr += Rs[2 + q] * Rs[2 + q]; }
-  V El = pl / gm1 + R(0.5) * rl * kl;
-  V Er = pr / gm1 + R(0.5) * rr * kr;
-  V al = sqrt(gam * pl / rl), ar = sqrt(gam * pr / rr);
-  V sl = sqrt(rl), sr = sqrt(rr);
-  V iw = R(1) / (sl + sr);
-  V Ht = (sl * ((El + pl) / rl) + sr * ((Er + pr) / rr)) * iw;
-  V ut = (sl * ul + sr * ur) * iw;
-  V v2 = ut * ut;
+  const R El = pl * igm1 + R(0.5) * rl * kl, Er = pr * igm1 + R(0.5) * rr * kr;
+  const R irl = rcp_any(rl), irr = rcp_any(rr);
+  const R al = sqrt_any(gam * pl * irl), ar = sqrt_any(gam * pr * irr);
+  const R sl = sqrt_any(rl), sr = sqrt_any(rr), iw = rcp_any(sl + sr);
+  const R Ht = (sl * ((El + pl) * irl) + sr * ((Er + pr) * irr)) * iw;
+  const R ut = (sl * ul + sr * ur) * iw;
+  R v2 = ut * ut;
 #pragma unroll
-  for (int q = 1; q < D; ++q) { V vq = (sl * L[2 + q] + sr * Rs[2 + q]) * iw; v2 += vq * vq; }
-  V at2 = gm1 * (Ht - R(0.5) * v2);
-  V at = sqrt(at2 > R(0) ? at2 : V(R(0)));
-  V SL = fmin(ul - al, ut - at);
-  V SR = fmax(ur + ar, ut + at);
-  V dl = rl * (SL - ul), dr = rr * (SR - ur);
-  V Ss = (pr - pl + ul * dl - ur * dr) / (dl - dr);
+  for (int q = 1; q < D; ++q) { const R vq = (sl * L[2 + q] + sr * Rs[2 + q]) * iw; v2 += vq * vq; }
+  const R at2 = g1 * (Ht - R(0.5) * v2);
+  const R at = sqrt_any(nonneg(at2) ? at2 : R(0));
+  const R SL = min_fast(ul - al, ut - at), SR = max_fast(ur + ar, ut + at);
+  const R dl = rl * (SL - ul), dr = rr * (SR - ur);
+  const R Ss = (pr - pl + ul * dl - ur * dr) * rcp_any(dl - dr);
   vstar = Ss;
-  if (SL >= R(0)) {
-    f[0] = rl * ul;
-    f[1] = rl * ul * ul + pl;
+  const bool supL = nonneg(SL), supR = !supL && !nonneg(SR), sup = supL || supR;
+  const bool left = supL || (!supR && nonneg(Ss));
+  const R rk = left ? rl : rr, pk = left ? pl : pr, uk = left ? ul : ur;
+  const R Ek = left ? El : Er, Sk = left ? SL : SR, irk = left ? irl : irr;
+  const R sku = Sk - uk, m = rk * uk;
+  const R fac = rk * sku * rcp_any(Sk - Ss);
+  const R f1 = m * uk + pk;
+  f[0] = sup ? m : m + Sk * (fac - rk);
+  f[1] = sup ? f1 : f1 + Sk * (fac * Ss - m);
 #pragma unroll
-    for (int q = 1; q < D; ++q) f[1 + q] = rl * ul * L[2 + q];
-    f[1 + D] = (El + pl) * ul;
-    return;
+  for (int q = 1; q < D; ++q) {
+    const R wq = left ? L[2 + q] : Rs[2 + q];
+    const R fq = m * wq;
+    f[1 + q] = sup ? fq : fq + Sk * (fac * wq - rk * wq);
   }
-  if (SR < R(0)) {
-    f[0] = rr * ur;
-    f[1] = rr * ur * ur + pr;
-#pragma unroll
-    for (int q = 1; q < D; ++q) f[1 + q] = rr * ur * Rs[2 + q];
-    f[1 + D] = (Er + pr) * ur;
-    return;
-  }
-  const bool left = Ss >= R(0);
-  const V* W = left ? L : Rs;
-  V rk = W[0], pk = W[1], uk = W[2], Ek = left ? El : Er, Sk = left ? SL : SR;
-  V sku = Sk - uk;
-  V fac = rk * sku / (Sk - Ss);
-  // F* = F_k + S_k (U*_k - U_k)
-  f[0] = rk * uk + Sk * (fac - rk);
-  f[1] = rk * uk * uk + pk + Sk * (fac * Ss - rk * uk);
-#pragma unroll
-  for (int q = 1; q < D; ++q) f[1 + q] = rk * uk * W[2 + q] + Sk * (fac * W[2 + q] - rk * W[2 + q]);
-  V Es = fac * (Ek / rk + (Ss - uk) * (Ss + pk / (rk * sku)));
-  f[1 + D] = (Ek + pk) * uk + Sk * (Es - Ek);
+  const R Es = fac * (Ek * irk + (Ss - uk) * (Ss + pk * (irk * rcp_any(sku))));
+  const R fE = (Ek + pk) * uk;
+  f[1 + D] = sup ? fE : fE + Sk * (Es - Ek);
 }
 
 // Gas flux of one face by the selected solver (Sec. 5.2 names local Lax-Friedrichs, HLLE and
@@ -406,53 +310,6 @@ __device__ __forceinline__ void gas_riemann(int solver, R gam, const R* L, const
   const R ib = R(1) / (br - bl);
 #pragma unroll
   for (int v = 0; v < 2 + D; ++v) f[v] = (br * FL[v] - bl * FR[v] + bl * br * (UR[v] - UL[v])) * ib;
-}
-
-// ---------------------------------------------------------------------------------------------
-// M1 closure (Levermore / Dubroca-Feugeas Eddington factor chi(f) = (3+4f^2)/(5+2 sqrt(4-3f^2)),
-// reading R7): the row n of the radiation pressure tensor P_{nq} for a state (E, physical F).
-// With s = sqrt(4 - 3f^2) the closure's two coefficients reduce exactly to
-//   (1 - chi)/2 = 1/3 - f^2/(2+s),   (3 chi - 1)/2 = 3 f^2/(2+s),
-// so P_{nq} = E [1/3 - f^2/(2+s)] delta_{nq} + 3 F_n F_q / ((2+s) c^2 E): one reciprocal of E, one
-// square root and one reciprocal per state, and F = 0 needs no special case.  In FP32 the two
-// special cases (E <= 0: isotropic E/3; f > 1: the direction kept, f clamped to 1) are selects
-// instead of branches: 1/E is taken as 0 for E <= 0, which leaves exactly E/3 on the diagonal, and
-// the clamp factor min(1, 1/f^2) is computed for every state.
-// ---------------------------------------------------------------------------------------------
-template <class R, int D, class V = R>
-__device__ __forceinline__ void m1_row(R ic2, V E, const V* F, int n, V* P) {
-  if constexpr (std::is_same<V, float>::value) {
-    V F2 = F[0] * F[0];
-#pragma unroll
-    for (int q = 1; q < D; ++q) F2 += F[q] * F[q];
-    const V iE = E > R(0) ? frcp(E) : V(R(0));
-    V f2 = F2 * iE * iE * ic2;
-    const V scale = fminf(1.0f, frcp(fmaxf(f2, 1e-30f)));
-    f2 = fminf(f2, 1.0f);
-    const V qd = frcp(R(2) + sqrt(R(4) - R(3) * f2));
-    const V diag = E * (R(1.0 / 3.0) - f2 * qd);
-    const V w = R(3) * qd * iE * ic2 * scale * F[n];
-#pragma unroll
-    for (int q = 0; q < D; ++q) P[q] = w * F[q] + (q == n ? diag : V(R(0)));
-    return;
-  }
-  if (!(E > R(0))) {
-#pragma unroll
-    for (int q = 0; q < D; ++q) P[q] = q == n ? E * R(1.0 / 3.0) : V(R(0));
-    return;
-  }
-  V F2 = F[0] * F[0];
-#pragma unroll
-  for (int q = 1; q < D; ++q) F2 += F[q] * F[q];
-  const V iE = frcp(E);
-  V f2 = F2 * iE * iE * ic2;
-  V scale = V(R(1));
-  if (f2 > R(1)) { scale = frcp(f2); f2 = V(R(1)); }  // |F| > cE: keep the direction, clamp f to 1
-  const V qd = frcp(R(2) + sqrt(R(4) - R(3) * f2));
-  const V diag = E * (R(1.0 / 3.0) - f2 * qd);
-  const V w = R(3) * qd * iE * ic2 * scale * F[n];
-#pragma unroll
-  for (int q = 0; q < D; ++q) P[q] = w * F[q] + (q == n ? diag : V(R(0)));
 }
 
 // ---------------------------------------------------------------------------------------------

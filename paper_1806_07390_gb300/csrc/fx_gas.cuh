@@ -68,6 +68,7 @@ __device__ __forceinline__ void gas_faces_tile(const StageArgs<R>& A, unsigned t
   constexpr int NG = 2 + D, NW = 2 + D;
   using FT = FaceTile<DIR, FTH>;
   constexpr int FACE_WCELLS = FaceSize<FTH>::WCELLS, FACE_BCELLS = FaceSize<FTH>::BCELLS;
+  (void)FACE_WCELLS; (void)FACE_BCELLS;
   constexpr int LD = FT::LD, LX = FT::LX, NWC = FT::NWC;
   const auto& g = A.g;
   const int n0 = g.n[0], n1 = g.n[1], n2 = g.n[2];
@@ -141,7 +142,7 @@ __device__ __forceinline__ void gas_faces_tile(const StageArgs<R>& A, unsigned t
 #pragma unroll
   for (int v = 0; v < NW; ++v) {
     R a, b;
-    recon_parabolic(tt, bc_pad(id), w(v, r), w(v, r + 1), w(v, r + 2), a, b, R(0));
+    recon_parabolic(tt, bc_pad(id), w(v, r), w(v, r + 1), w(v, r + 2), a, b);
     Ra[v] = a;
     sb[v][FXI(r * LX + lx, FACE_BCELLS)] = b;
   }

@@ -90,7 +90,7 @@ inline void fit_tile(const int* n, int G, int nsm, int regs, RadTile& best, int&
 // face kernel and `mid2` after the radiation/update kernel (per-kernel timing).  Returns the CUDA
 // error of the launches.
 template <class R, int D, class NT, bool SPH>
-cudaError_t launch_stage(const StageArgs<R>& a, int GP, cudaStream_t s, cudaEvent_t mid,
+cudaError_t launch_stage(const StageArgs<R>& a, cudaStream_t s, cudaEvent_t mid,
                          cudaEvent_t mid2);
 
 // Registers per thread of the stage kernel (radiation reconstruction order ro), for fit_tile.
@@ -100,8 +100,8 @@ cudaError_t stage_regs(int ro, int* regs);
 #ifdef FX_LAUNCH_DEFINE
 // Definition, included only by the per-instantiation translation units.  The group arithmetic
 // type of the stage kernel is the state type R.
-template <class R, int D, int GP, class NT, bool SPH>
-static cudaError_t launch_gp(const StageArgs<R>& a0, cudaStream_t s, cudaEvent_t mid, cudaEvent_t mid2) {
+template <class R, int D, class NT, bool SPH>
+cudaError_t launch_stage(const StageArgs<R>& a0, cudaStream_t s, cudaEvent_t mid, cudaEvent_t mid2) {
   if ((a0.g.geom != 0) != SPH) return cudaErrorInvalidValue;  // the grid's geometry decides SPH
   StageArgs<R> a = a0;
   // lanes copy and store pairs with 8-byte accesses where every pair is complete and aligned
@@ -207,16 +207,6 @@ cudaError_t stage_regs(int ro, int* regs) {
   return e;
 }
 
-template <class R, int D, class NT, bool SPH>
-cudaError_t launch_stage(const StageArgs<R>& a, int GP, cudaStream_t s, cudaEvent_t mid,
-                         cudaEvent_t mid2) {
-  switch (GP) {
-    case 8: return launch_gp<R, D, 8, NT, SPH>(a, s, mid, mid2);
-    case 16: return launch_gp<R, D, 16, NT, SPH>(a, s, mid, mid2);
-    case 32: return launch_gp<R, D, 32, NT, SPH>(a, s, mid, mid2);
-    default: return cudaErrorInvalidValue;
-  }
-}
 #endif
 
 }  // namespace fx

@@ -85,22 +85,6 @@ __device__ __forceinline__ F2 vabs(F2 a) { return F2(fabsf(a.x), fabsf(a.y)); }
 __device__ __forceinline__ double vmin(double a, double b) { return fmin(a, b); }
 __device__ __forceinline__ double vmax(double a, double b) { return fmax(a, b); }
 __device__ __forceinline__ double vabs(double a) { return fabs(a); }
-// Slope of the MC limiter from the one-sided slopes sL, sR and the centred slope sC: the least of
-// 2|sL|, 2|sR| and |sC|, with the common sign of sL and sR, and zero where their signs differ or
-// one is zero.  Where sL and sR share a sign, sC has it too (the centred difference is the sum
-// of the two one-sided ones, each scaled by a positive reciprocal distance), so the sign factor
-// (-1, 0 or 1, exact) replaces the product test and the selects.  FP32 and the pair.
-__device__ __forceinline__ float mc_slope(float sL, float sR, float sC) {
-  const float m = fminf(2.0f * fminf(fabsf(sL), fabsf(sR)), fabsf(sC));
-  return m * (copysignf(0.5f, sL) + copysignf(0.5f, sR));
-}
-__device__ __forceinline__ F2 mc_slope(F2 sL, F2 sR, F2 sC) {
-  const F2 m2 = F2(fminf(fabsf(sL.x), fabsf(sR.x)), fminf(fabsf(sL.y), fabsf(sR.y))) * 2.0f;
-  const F2 m(fminf(m2.x, fabsf(sC.x)), fminf(m2.y, fabsf(sC.y)));
-  return m * (F2(copysignf(0.5f, sL.x), copysignf(0.5f, sL.y)) +
-              F2(copysignf(0.5f, sR.x), copysignf(0.5f, sR.y)));
-}
-
 // The limited difference of the MC limiter from the one-sided differences dl, dr and the centred
 // one q: the least of m|dl|, m|dr| and |q| with their common sign, zero where the signs of dl and dr
 // differ or one is zero (q has their sign where they agree).  In FP32 three instructions per value:

@@ -379,14 +379,6 @@ template <class R> __device__ __forceinline__ void cp_async(R* smem, const R* gm
     asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(sa), "l"(gmem) : "memory");
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-// Named barrier `id` (1..15) of `n` threads: arrive without waiting, or arrive and wait.  The
-// shared-memory writes a thread made before arriving are visible to the threads that waited.
-__device__ __forceinline__ void bar_arrive(int id, int n) {
-  asm volatile("bar.arrive %0, %1;\n" ::"r"(id), "r"(n) : "memory");
-}
-__device__ __forceinline__ void bar_wait(int id, int n) {
-  asm volatile("bar.sync %0, %1;\n" ::"r"(id), "r"(n) : "memory");
-}
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
 
 // cp.async of one lane value (the lane's groups: both values of a pair where they are 8-byte
@@ -949,8 +941,8 @@ stage_kernel(const __grid_constant__ StageArgs<R> A) {
 #pragma unroll
       for (int v = 0; v < NRV; ++v) {
         R a0, b0, a1 = R(0), b1 = R(0);
-        recon_parabolic(t, 0, vget(Qm[v], 0), vget(Q0[v], 0), vget(Qp[v], 0), a0, b0, R(0));
-        if (W == 2) recon_parabolic(t, 0, vget(Qm[v], 1), vget(Q0[v], 1), vget(Qp[v], 1), a1, b1, R(0));
+        recon_parabolic(t, 0, vget(Qm[v], 0), vget(Q0[v], 0), vget(Qp[v], 0), a0, b0);
+        if (W == 2) recon_parabolic(t, 0, vget(Qm[v], 1), vget(Q0[v], 1), vget(Qp[v], 1), a1, b1);
         a[v] = vpair(a0, a1, V());
         b[v] = vpair(b0, b1, V());
       }

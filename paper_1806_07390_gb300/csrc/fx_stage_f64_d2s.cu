@@ -4,7 +4,7 @@
 #include "fx_launch.h"
 
 namespace fx {
-template cudaError_t launch_stage<double, 2, double, true>(const StageArgs<double>&, int, cudaStream_t, cudaEvent_t,
+template cudaError_t launch_stage<double, 2, double, true>(const StageArgs<double>&, cudaStream_t, cudaEvent_t,
                                                   cudaEvent_t);
 template cudaError_t stage_regs<double, 2, double, true>(int, int*);
 }  // namespace fx
