@@ -31,15 +31,20 @@
 
 namespace fx {
 
-constexpr int CPL64_THREADS = 128;  // threads per block of couple64_kernel
+constexpr int CPL64_THREADS = 32;  // threads per block of couple64_kernel
 
 // Lanes per cell of couple64_kernel.  One lane per cell does the least FP64 work: every operation
-// serves 32 cells, and neighbouring groups share their edge.  A grid whose cells at one lane each
-// would leave a multiprocessor with fewer than four warps is bound by the latency of a cell's group
-// loop instead: eight lanes share it (512 cells x 12 groups: 0.117 -> 0.031 ms
-// per launch, with the edge table).
-constexpr int64_t CPL64_SPLIT_CELLS = 152 * 128;
-constexpr int CPL64_SPLIT_LANES = 8;
+// serves 32 cells, and neighbouring groups share their edge.  A grid that leaves a multiprocessor with
+// few warps is bound by the latency of a cell's group loop instead, so lanes share it, twice as many
+// at a time (no more than the groups need) while the threads stay within seven warps per
+// multiprocessor, where the FP64 pipe is about full.  Measured (us per launch, 16 groups, 1 / 2 / 4 / 8 / 16 lanes): 512 cells
+// 105 / 80 / 49 / 35 / 27, 3072 cells 104 / 78 / 50 / 39 / 46, 6144 cells 103 / 78 / 55 / 61 / 88, 12288
+// cells 104 / 88 / 92 / 111 / 138, 20480 cells 117 / 129 / 152 / 173 / 217.
+inline int couple64_lanes(int64_t ncell, int G) {
+  int L = 1;
+  while (L < 16 && L < G && ncell * (2 * L) <= 152 * 7 * 32) L *= 2;
+  return L;
+}
 
 // Rows of couple64_kernel's shared memory per cell: E^- (then the new E), the last evaluation's
 // E_g and dE_g/dT (then the F_q).
@@ -92,7 +97,7 @@ template <int L> __device__ __forceinline__ double cell_sum(double v) {
 }
 
 template <int D, int L>
-__global__ void __launch_bounds__(CPL64_THREADS, 4) couple64_kernel(const __grid_constant__ StageArgs<double> A) {
+__global__ void __launch_bounds__(CPL64_THREADS, 512 / CPL64_THREADS) couple64_kernel(const __grid_constant__ StageArgs<double> A) {
   constexpr int NG = 2 + D, NRV = 1 + D;
   const DevGrid& g = A.g;
   const int G = g.G;

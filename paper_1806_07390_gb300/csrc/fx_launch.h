@@ -185,13 +185,16 @@ cudaError_t launch_stage(const StageArgs<R>& a0, cudaStream_t s, cudaEvent_t mid
       const unsigned nb = (unsigned)((a.g.ncell + CPL_THREADS - 1) / CPL_THREADS);
       ck<<<nb, CPL_THREADS, cs, s>>>(a);
     } else {
-      const bool split = a.g.ncell <= CPL64_SPLIT_CELLS;
-      const int lanes = split ? CPL64_SPLIT_LANES : 1, threads = split ? 32 : CPL64_THREADS, cells = threads / lanes;
-      auto ck = split ? couple64_kernel<D, CPL64_SPLIT_LANES> : couple64_kernel<D, 1>;
+      const int lanes = couple64_lanes(a.g.ncell, a.g.G), cells = CPL64_THREADS / lanes;
+      auto ck = lanes == 1   ? couple64_kernel<D, 1>
+                : lanes == 2 ? couple64_kernel<D, 2>
+                : lanes == 4 ? couple64_kernel<D, 4>
+                : lanes == 8 ? couple64_kernel<D, 8>
+                             : couple64_kernel<D, 16>;
       const size_t cs = couple64_smem_bytes<D>(a.g.G, cells);
       e = cudaFuncSetAttribute(ck, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cs);
       if (e != cudaSuccess) return e;
-      ck<<<(unsigned)((a.g.ncell + cells - 1) / cells), threads, cs, s>>>(a);
+      ck<<<(unsigned)((a.g.ncell + cells - 1) / cells), CPL64_THREADS, cs, s>>>(a);
     }
     e = cudaGetLastError();
   }
