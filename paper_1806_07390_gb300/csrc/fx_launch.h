@@ -109,8 +109,10 @@ cudaError_t launch_stage(const StageArgs<R>& a0, cudaStream_t s, cudaEvent_t mid
   a.rt.vec = a.g.G % 2 == 0 && ((2 + D) * a.g.ncell) % 2 == 0 && al8(a.in) && al8(a.base) && al8(a.out);
   // (the boundary budgets are compiled into the kernel for grids with a non-periodic boundary;
   // the second-order radiation reconstruction always carries them)
-  auto kern = a.g.rad_order == 2 ? stage_kernel<R, D, SPH, 2, true>
-              : (a.budget_bnd ? stage_kernel<R, D, SPH, 1, true> : stage_kernel<R, D, SPH, 1, false>);
+  constexpr bool PV = sizeof(R) == 4 && D < 3;  // an instance for whole pairs
+  auto kern = a.g.rad_order == 2 ? (a.rt.vec ? stage_kernel<R, D, SPH, 2, true, PV> : stage_kernel<R, D, SPH, 2, true, false>)
+              : a.budget_bnd     ? (a.rt.vec ? stage_kernel<R, D, SPH, 1, true, PV> : stage_kernel<R, D, SPH, 1, true, false>)
+                                 : (a.rt.vec ? stage_kernel<R, D, SPH, 1, false, PV> : stage_kernel<R, D, SPH, 1, false, false>);
   const size_t smem = stage_smem_bytes<R, D>(a.rt);
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
@@ -204,8 +206,8 @@ cudaError_t launch_stage(const StageArgs<R>& a0, cudaStream_t s, cudaEvent_t mid
 template <class R, int D, class NT, bool SPH>
 cudaError_t stage_regs(int ro, int* regs) {
   cudaFuncAttributes fa;
-  const cudaError_t e = ro == 2 ? cudaFuncGetAttributes(&fa, stage_kernel<R, D, SPH, 2, true>)
-                                : cudaFuncGetAttributes(&fa, stage_kernel<R, D, SPH, 1, false>);
+  const cudaError_t e = ro == 2 ? cudaFuncGetAttributes(&fa, stage_kernel<R, D, SPH, 2, true, false>)
+                                : cudaFuncGetAttributes(&fa, stage_kernel<R, D, SPH, 1, false, false>);
   if (e == cudaSuccess) *regs = fa.numRegs;
   return e;
 }

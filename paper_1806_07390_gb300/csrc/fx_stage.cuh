@@ -443,6 +443,10 @@ __device__ __forceinline__ void cp_async16(void* s, const void* g) {
 // (256^3 x 12, 2 blocks of 256: 6.2 ms; 4 of 128 6.4, 3 of 192 spill 7.3, 1 of 512 6.5: larger tiles
 // have less halo).
 //
+// VEC (FP32 below 3-d): an even group count on aligned buffers, so every lane's pair is complete and
+// is copied and stored as one 8-byte word without a test (1024^2 x 16 234 -> 229 us with the slots
+// rotated, 515 x 389 x 7 34.4 -> 32.4, 96 x 80 x 8 10.4 -> 8.8; in 3-d 0.6 % slower, so tested there).
+//
 // SPH selects the spherical (r, theta) geometry, RO the radiation reconstruction (1: linear with
 // the MC limiter, the paper's; 2: the gas's parabola), BUD the boundary-outflow budgets (R13).
 // ---------------------------------------------------------------------------------------------
@@ -667,7 +671,7 @@ __device__ __forceinline__ void gas_update(const StageArgs<R>& A, uint32_t cid) 
   (void)MD;
 }
 
-template <class R, int D, bool SPH, int RO, bool BUD>
+template <class R, int D, bool SPH, int RO, bool BUD, bool VEC>
 __global__ void __launch_bounds__((StageCap<R, D>::NT), (StageCap<R, D>::MINB))
 stage_kernel(const __grid_constant__ StageArgs<R> A) {
   static_assert(!SPH || D == 2, "the spherical geometry is 2-d (r, theta)");
@@ -705,8 +709,8 @@ stage_kernel(const __grid_constant__ StageArgs<R> A) {
   const int tc = act ? tcell : 0;
   const int lx = D == 3 ? tc % TX : tc, ly = D == 3 ? tc / TX : 0;
   const int g0 = lane * W;
-  const bool h1 = W == 2 && g0 + 1 < G;
-  const bool vec = RT.vec != 0;
+  const bool h1 = W == 2 && (VEC || g0 + 1 < G);
+  const bool vec = VEC || (D == 3 && RT.vec != 0);  // pairs copied and stored whole (all complete and aligned)
 
   extern __shared__ __align__(16) unsigned char smem_raw[];
   V* const sm = reinterpret_cast<V*>(smem_raw);
@@ -776,7 +780,7 @@ stage_kernel(const __grid_constant__ StageArgs<R> A) {
     bool f0 = false, f1 = false;
     halo_pos(h, sx, sy);
     off = inplane(sx, sy, f0, f1) * (uint32_t)G + ln * W;
-    two = W == 2 && ln * W + 1 < G;
+    two = W == 2 && (VEC || ln * W + 1 < G);
   };
   uint32_t hoff[HP];
   bool hh1[HP];
@@ -810,7 +814,7 @@ stage_kernel(const __grid_constant__ StageArgs<R> A) {
     roff[p] = rstr[p] = 0;
     if (tid + p * NTH < NREC) rec_entry(tid + p * NTH, roff[p], rstr[p]);
   }
-  if (W == 2 && (G & 1)) {  // the pad component of an odd group count's last pair stays zero
+  if (W == 2 && !VEC && (G & 1)) {  // the pad component of an odd group count's last pair stays zero
     for (int i = tid; i < L.rec; i += NTH) sm[i] = V(R(0));
     __syncthreads();
   }
@@ -1108,9 +1112,14 @@ stage_kernel(const __grid_constant__ StageArgs<R> A) {
   // ---------------------------------------------------------------- march
   // (unrolled by four planes, with every slot a constant, the kernel lost 8 to 25 % to instruction
   // fetch)
+  constexpr int SL = D == 1 ? 0 : NRV * NT;
+  int par = 0, s0 = SL, s1 = 2 * SL, s2 = 3 * SL, s3 = 0;  // slots of planes k, k+1, k+2 and the one to fill
   for (int k = kbeg; k < kend; ++k) {
-    const int u = k - kbeg, par = u & 1, SL = D == 1 ? 0 : NRV * NT;
-    const int s0 = ((u + 1) & 3) * SL, s1 = ((u + 2) & 3) * SL, s2 = ((u + 3) & 3) * SL, s3 = (u & 3) * SL;
+    if (D == 3) {  // (rotated below: 256^3 x 12 slower by 0.7 %, 2-d faster by 1 to 2 %)
+      const int u = k - kbeg;
+      par = u & 1;
+      s0 = ((u + 1) & 3) * SL; s1 = ((u + 2) & 3) * SL; s2 = ((u + 3) & 3) * SL; s3 = (u & 3) * SL;
+    }
     const bool more = D >= 2 && k + 1 < kend;
     if (more) {
       issue_own(k + 3, s3);
@@ -1325,6 +1334,11 @@ stage_kernel(const __grid_constant__ StageArgs<R> A) {
     for (int v = 0; v < NRV; ++v) {
       if (D >= 2) bm0[v] = bm1[v];
       rfm_old[v] = rfm_new[v];
+    }
+    if (D < 3) {
+      const int s4 = s0;
+      s0 = s1; s1 = s2; s2 = s3; s3 = s4;
+      par ^= 1;
     }
   }
 }
