@@ -240,7 +240,7 @@ __global__ void __launch_bounds__(CPL_THREADS, 7) couple_kernel(const __grid_con
     if (um < kn.u_floor) { um = kn.u_floor; st |= ST_FLOOR; }
     const LT rcv_f = rr * kl.cv;
     const NT rcv = (NT)rcv_f;
-    const LT Tm = (LT)um * ir * kl.gm1;  // c_v = 1/(gamma - 1)
+    const LT Tm = to_f32(um) * ir * kl.gm1;  // c_v = 1/(gamma - 1)
     // opacity factors (they only enter the FP32 group arithmetic)
     Kc = kl.kappa0 * hpow(rr, g.kap_rho_h);
     Sc = kl.sigma0 * rr;
@@ -257,7 +257,7 @@ __global__ void __launch_bounds__(CPL_THREADS, 7) couple_kernel(const __grid_con
     }
     const LT Esum = Es2.x + Es2.y;
     if (A.budget != nullptr) s_floor[t] = fadd.x + fadd.y;
-    const NT ats = (NT)(kl.atol * ((LT)um + Esum));
+    const NT ats = (NT)(kl.atol * (to_f32(um) + Esum));
     const LT hh = LT(0.5) * (LT)g.kap_T_h;
     // one evaluation at T: the group sums of E_g(T) - E_g^- (Eq. 25) and of dE_g/dT; the first
     // one also keeps each group's E_g and dE_g/dT (most cells converge from it)
@@ -285,9 +285,9 @@ __global__ void __launch_bounds__(CPL_THREADS, 7) couple_kernel(const __grid_con
     // ---- Newton with backtracking (Eqs. 26-27; reading R11).  The iterate dl = T - T^- and the
     // residual r are NT; the direction -r/(dr/dT) only needs FP32 (a Newton step is as good as
     // its residual), so dr/dT, the step and the step test are FP32.
-    // Below 3-d the residuals are compared by the integer units (cmp_abs; an FP64 comparison holds the
-    // pipe for 16 cycles): 1024^2 x 16 118 -> 113 us.  In 3-d the registers that this takes cost more
-    // (256^3 x 12 2.52 -> 2.72 ms).
+    // An FP64 comparison or conversion holds the FP64 pipe for 16 cycles, so the residuals are compared by the
+    // integer units (cmp_abs) and values go to FP32 without the compiler's flush test (to_f32): 1024^2 x 16 118 ->
+    // 111 us, 256^3 x 12 2.54 -> 2.45 ms.
     NT dl = NT(0), dacc = NT(0), r;
     LT drf, dTf = LT(0), lam = LT(1);
     LT Tacc = Tm;      // T at the accepted point, in FP32
@@ -304,9 +304,9 @@ __global__ void __launch_bounds__(CPL_THREADS, 7) couple_kernel(const __grid_con
     for (int kk = 0; kk < guard; ++kk) {
       if (need_dir) {
         if (it >= g.newton_maxit) { done = true; }
-        else if (D == 3 ? fabs(r) <= ats : cmp_abs(r, ats) <= 0) { done = true; ok = true; }
+        else if (cmp_abs(r, ats) <= 0) { done = true; ok = true; }
         else {
-          dTf = -(LT)r * frcp(drf);
+          dTf = -to_f32(r) * frcp(drf);
           ++it;
           if (fabsf(dTf) <= kl.rtol * Tacc) {
             // converged: the group energies at T + dT follow from the linearisation
@@ -319,13 +319,13 @@ __global__ void __launch_bounds__(CPL_THREADS, 7) couple_kernel(const __grid_con
       }
       if (done) break;
       const NT dtt = dl + (NT)(lam * dTf);
-      const LT Ttr = Tm + (LT)dtt;
+      const LT Ttr = Tm + to_f32(dtt);
       const bool valid = Ttr > LT(0);
       const LT Tl = valid ? Ttr : Tacc;
       LT a, b;
       eval(Tl, a, b, false);
       const NT rt = rcv * dtt + (NT)a;
-      if (valid && (D == 3 ? fabs(rt) < fabs(r) : cmp_abs(rt, r) < 0)) {
+      if (valid && cmp_abs(rt, r) < 0) {
         dl = dtt;
         dacc = dtt;
         Tacc = Tl;
@@ -349,7 +349,7 @@ __global__ void __launch_bounds__(CPL_THREADS, 7) couple_kernel(const __grid_con
       NT Te = lo;
       for (int kk = 0; kk < 400 + g.bisect_maxit + 4 && phase < 3; ++kk) {
         LT a, b;
-        eval((LT)(Tmn + Te), a, b, false);
+        eval(to_f32(Tmn + Te), a, b, false);
         const NT rq = rcv * Te + (NT)a;
         if (phase == 0) {
           if (rq > NT(0) && cnt < 200) { lo = NT(0.5) * (lo + Tmn) - Tmn; ++cnt; }  // T_lo /= 2
@@ -371,7 +371,7 @@ __global__ void __launch_bounds__(CPL_THREADS, 7) couple_kernel(const __grid_con
       first = false;
     }
     if (!ok) st |= ST_NEWTON;
-    Tst = Tm + (LT)dl;
+    Tst = Tm + to_f32(dl);
     if (A.tstar_out != nullptr) A.tstar_out[FXI(cid, ncell)] = Tst;
 
     // ---- the accepted group energies (from the kept first evaluation when it is the accepted
@@ -390,7 +390,7 @@ __global__ void __launch_bounds__(CPL_THREADS, 7) couple_kernel(const __grid_con
 #pragma unroll 2
       for (int j = 0; j < NPR; ++j) accept(j, lin != LT(0) ? vfma(rD0[j], F2(lin), rE0[j]) : rE0[j]);
     } else {
-      const LT Ta = Tm + (LT)dacc;
+      const LT Ta = Tm + to_f32(dacc);
       const PlanckAt p = planck_at(A.ptab, kl.aN, Ta);
       const LT ck = kl.cdts * (Kc * hpow(Ta, g.kap_T_h));
       const LT hi = hh * p.invT;

@@ -25,6 +25,14 @@ __device__ __forceinline__ float frcp(float x) { return rcp_approx(x); }
 // takes a turn on it like any other operation, so the helpers below compare bit patterns with the
 // integer units: doubles of one sign order as their bits do.
 // ---------------------------------------------------------------------------------------------
+// FP32 value of a double without the flush of denormal results, which the compiler adds as a
+// comparison and a multiplication under flush-to-zero (every FP32 operation that takes the value flushes it)
+__device__ __forceinline__ float to_f32(double x) {
+  float y;
+  asm("cvt.rn.f32.f64 %0, %1;" : "=f"(y) : "d"(x));
+  return y;
+}
+__device__ __forceinline__ float to_f32(float x) { return x; }
 // x > 0 and normal
 __device__ __forceinline__ bool normal_pos(double x) { return __double2hiint(x) >= 0x00100000; }
 // 1/x for normal positive x below 2^1022: the hardware seed y (relative error e, |e| < 2^-19)
