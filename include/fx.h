@@ -267,8 +267,8 @@ fx_status fx_state_download(fx_grid* h, void* dst, int dst_precision, int dst_is
 int fx_launches_per_step(const fx_grid* h);
 
 /* Planes of the slowest axis that one block of the radiation/update kernel marches over: 32 (or
- * the axis length) until the workspace is bound, then fitted to the bound device by
- * fx_bind_workspace (fewest waves of blocks times planes per block).  0 for 1-d grids, -1 for a
+ * the axis length) until the workspace is bound, then fitted with the tile to the bound device by
+ * fx_bind_workspace (a model of the kernel's time over tiles and chunks).  0 for 1-d grids, -1 for a
  * null handle. */
 int fx_march_chunk(const fx_grid* h);
 

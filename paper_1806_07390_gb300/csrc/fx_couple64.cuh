@@ -16,7 +16,7 @@
 // Bound by the FP64 pipe (87 % busy), so the band edges come from a table of polynomials instead of
 // the power and exponential series (planck_edge_tab: 20 operations an edge), reciprocals are a
 // hardware seed with one third-order step instead of divisions, and a group takes 36 operations an
-// evaluation: 512^2 x 16 groups 1.90 -> 0.97 ms per launch, 217 -> 120 FP64 operations per group.
+// evaluation: 512^2 x 16 groups 1.90 -> 0.93 ms per launch, 217 -> 110 FP64 operations per group.
 //
 // The stage kernel leaves the state after the explicit update and RK combination in its output;
 // this kernel updates that state in place.  The decisions (Newton step and its tests, the

@@ -432,7 +432,7 @@ __device__ __forceinline__ void cp_async16(void* s, const void* g) {
 // Bound by instruction issue and by the latency between the plane barriers (1024^2 x 16: about 700
 // instructions per warp and plane, issued in 66 % of cycles at 20 warps per multiprocessor; 256^3 x
 // 12: 1355 in 58 % at 16 warps; DRAM 1.0x the algorithmic bytes), the FP64 state by the FP64 pipe (86
-// % busy, 239 operations per cell and group).  Measured (FP32 state unless noted, one launch):
+// % busy, 224 operations per cell and group).  Measured (FP32 state unless noted, one launch):
 // 1024^2 x 16 groups 0.455 -> 0.234 ms, 256^3 x 12 16.4 -> 6.2 ms, 640 x 128 x 20 spherical 0.124 ->
 // 0.050 ms, 512^2 x 24 channels 0.23 -> 0.094 ms, 512^2 x 16 FP64 2.99 -> 1.86 ms, against one kernel
 // with lanes padded to a power of two, geometry tables on every grid, and the gas update in its lanes.
