@@ -35,14 +35,15 @@ constexpr int CPL64_THREADS = 32;  // threads per block of couple64_kernel
 
 // Lanes per cell of couple64_kernel.  One lane per cell does the least FP64 work: every operation
 // serves 32 cells, and neighbouring groups share their edge.  A grid that leaves a multiprocessor with
-// few warps is bound by the latency of a cell's group loop instead, so lanes share it, twice as many
-// at a time (no more than the groups need) while the threads stay within seven warps per
-// multiprocessor, where the FP64 pipe is about full.  Measured (us per launch, 16 groups, 1 / 2 / 4 / 8 / 16 lanes): 512 cells
-// 105 / 80 / 49 / 35 / 27, 3072 cells 104 / 78 / 50 / 39 / 46, 6144 cells 103 / 78 / 55 / 61 / 88, 12288
-// cells 104 / 88 / 92 / 111 / 138, 20480 cells 117 / 129 / 152 / 173 / 217.
+// few warps is bound by the latency of a cell's group loop instead, so lanes share it, each a run of neighbouring
+// groups: two lanes, which repeat little, while the threads stay within fourteen warps per
+// multiprocessor, and up to sixteen (no more than the groups need) within eight.  Measured with 16 groups, us per
+// launch: 512 cells 16 lanes 21; 3072 cells 8 lanes 35, 16 lanes 46; 5120 cells 4 lanes 46, 8 lanes 46; 6144
+// cells 4 lanes 47, 8 lanes 57; 12288 cells 2 lanes 70, 4 lanes 77; 20480 cells 1 lane 118, 2 lanes
+// 99; 30720 cells 1 lane 152, 2 lanes 139.
 inline int couple64_lanes(int64_t ncell, int G) {
-  int L = 1;
-  while (L < 16 && L < G && ncell * (2 * L) <= 152 * 7 * 32) L *= 2;
+  int L = G > 1 && 2 * ncell <= 152 * 14 * 32 ? 2 : 1;
+  while (L >= 2 && L < 16 && L < G && ncell * (2 * L) <= 152 * 8 * 32) L *= 2;
   return L;
 }
 
@@ -113,6 +114,8 @@ __global__ void __launch_bounds__(CPL64_THREADS, 512 / CPL64_THREADS) couple64_k
   const int nc = (int)min((uint32_t)CPB, ncell - c0);
   const bool act = t < nc;
   const uint32_t cid = c0 + (uint32_t)t;
+  // the lane's run of groups (neighbours share their edge; lanes past the last group have none)
+  const int gpl = (G + L - 1) / L, j0 = min(ln * gpl, G), j1 = min(j0 + gpl, G);
 
   for (int j = threadIdx.x; j <= G; j += (int)blockDim.x) {
     if (j < G) s_ef[j] = A.gc->efac[j];
@@ -161,7 +164,7 @@ __global__ void __launch_bounds__(CPL64_THREADS, 512 / CPL64_THREADS) couple64_k
     double um = rhoe - ke;
     if (um < kn.u_floor) { um = kn.u_floor; rhoe = ke + um; st |= ST_FLOOR; }
     double Esum = 0.0, fadd = 0.0;
-    for (int j = ln; j < G; j += L) {
+    for (int j = j0; j < j1; ++j) {
       double e = rE[j];
       if (e < kn.E_floor) {  // silent positivity floor (Wien tails)
         fadd += kn.E_floor - e;
@@ -187,11 +190,9 @@ __global__ void __launch_bounds__(CPL64_THREADS, 512 / CPL64_THREADS) couple64_k
       const double kT = K * hpow(T, g.kap_T_h);
       const double aT3 = aN * T3, aT4 = aT3 * T, ck = cdts * kT, hT = hh * invT;
       double s1 = 0.0, s2 = 0.0;
-      PlanckEdge<double> lo;
-      if (L == 1) lo = planck_edge_tab(s_ed[0] * invT, A.pk.petab, A.pk.c64);
+      PlanckEdge<double> lo = planck_edge_tab(s_ed[j0] * invT, A.pk.petab, A.pk.c64);
 #pragma unroll 2
-      for (int j = ln; j < G; j += L) {
-        if (L > 1) lo = planck_edge_tab(s_ed[j] * invT, A.pk.petab, A.pk.c64);
+      for (int j = j0; j < j1; ++j) {
         const PlanckEdge<double> hi = planck_edge_tab(s_ed[j + 1] * invT, A.pk.petab, A.pk.c64);
         const double I = planck_band(lo, hi);
         const double B = aT4 * I;
@@ -280,7 +281,7 @@ __global__ void __launch_bounds__(CPL64_THREADS, 512 / CPL64_THREADS) couple64_k
     if (A.tstar_out != nullptr && ln == 0) A.tstar_out[FXI(cid, ncell)] = Tst;
     // ---- the group energies at the accepted temperature and the gas energy by conservation (R12)
     double dEsum = 0.0;
-    for (int j = ln; j < G; j += L) {
+    for (int j = j0; j < j1; ++j) {
       const double En = rEt[j] + rDt[j] * lin;
       dEsum += En - rE[j];
       rE[j] = En;
@@ -298,7 +299,7 @@ __global__ void __launch_bounds__(CPL64_THREADS, 512 / CPL64_THREADS) couple64_k
     // feedback (Eqs. 31-32), with the velocity of the state before the interaction
     const double kT = K * hpow(Tst, g.kap_T_h);
     double SdF[3] = {0.0, 0.0, 0.0};
-    for (int j = ln; j < G; j += L) {
+    for (int j = j0; j < j1; ++j) {
       const double fac = rcp_pos(1.0 + kn.cdts * (kT * s_ef[j] + Sg));
 #pragma unroll
       for (int q = 0; q < D; ++q) {
@@ -333,7 +334,7 @@ __global__ void __launch_bounds__(CPL64_THREADS, 512 / CPL64_THREADS) couple64_k
     if (!work) {
       for (int v = 0; v < NRV; ++v) {
         const double* rv = srow + (v * CPB + t) * RS;
-        for (int j = ln; j < G; j += L) chk += rv[j] * 0.0;
+        for (int j = j0; j < j1; ++j) chk += rv[j] * 0.0;
       }
     }
     if (!isfinite(chk)) st |= ST_NONFINITE;
