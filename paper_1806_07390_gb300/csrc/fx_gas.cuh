@@ -27,9 +27,11 @@ __host__ __device__ inline int64_t faces_along(const int* n, int d) {
 // otherwise FT / 32 cells along DIR by 32 along x, so that a warp reads consecutive x), and
 // the top LD rows own their lower faces.  Cells 0 .. n_d along DIR own the n_d + 1 faces of the
 // direction (cell n_d is a ghost from the boundary rules).  FT = 288 on all grids whose tiles then
-// fill the device (the least halo share); below that 64, which spreads a small grid over more
-// multiprocessors (512 cells FP64: 0.035 -> 0.017 ms).
-constexpr int FACE_THREADS = 288, FACE_THREADS_SMALL = 64;
+// fill the device (the least halo share); in 3-d 160, whose rows along x leave fewer threads idle on the narrower grids
+// and cost nothing on wide ones (us per launch at 288 / 160 threads: 75 x 61 x 50 38 / 31, 128 x 96 x 100 126 / 102,
+// 256^3 1266 / 1262, 75 x 61 x 50 FP64 792 / 683; in 2-d 1024^2 47.8 / 49.2, 520 x 160 15.3 / 15.4); below
+// that 64, which spreads a small grid over more multiprocessors (512 cells FP64: 0.035 -> 0.017 ms).
+constexpr int FACE_THREADS = 288, FACE_THREADS_3D = 160, FACE_THREADS_SMALL = 64;
 template <int DIR, int FT> struct FaceTile {
   static constexpr int LX = DIR == 0 ? 1 : 32, LR = FT / LX, LD = LR - 1;
   static constexpr int NWC = LR + 2;  // cells d0-2 .. d0+LD along DIR whose primitives are staged
@@ -262,7 +264,7 @@ __global__ void __launch_bounds__(256) shock_flag_kernel(const __grid_constant__
 
 // One block per tile; grid row y is the direction (tiles beyond a direction's count return).
 template <class R, int D, bool SPH, int FTH>
-__global__ void __launch_bounds__(FTH, FTH == FACE_THREADS ? 3 : 8)
+__global__ void __launch_bounds__(FTH, FTH == FACE_THREADS ? 3 : (FTH == FACE_THREADS_3D ? 5 : 8))
 gas_face_kernel(const __grid_constant__ StageArgs<R> A) {
   __shared__ R sw[2 + D][FaceSize<FTH>::WCELLS];
   __shared__ R sb[2 + D][FaceSize<FTH>::BCELLS];

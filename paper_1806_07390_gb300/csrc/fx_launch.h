@@ -121,10 +121,11 @@ cudaError_t launch_stage(const StageArgs<R>& a0, cudaStream_t s, cudaEvent_t mid
   if (e != cudaSuccess) return e;
   // gas faces first (same stream): fluxes and contact speeds of every face of every direction,
   // one block per tile of faces, one grid row per direction
+  constexpr int FT = D == 3 ? FACE_THREADS_3D : FACE_THREADS;
   const bool small = face_small(a.g.n, D);
   unsigned ntmax = 0;
   for (int d = 0; d < D; ++d)
-    ntmax = std::max(ntmax, small ? face_tiles<FACE_THREADS_SMALL>(a.g.n, D, d) : face_tiles<FACE_THREADS>(a.g.n, D, d));
+    ntmax = std::max(ntmax, small ? face_tiles<FACE_THREADS_SMALL>(a.g.n, D, d) : face_tiles<FT>(a.g.n, D, d));
   dim3 gg(ntmax, D, 1);
   if (a.sflag != nullptr) {  // carbuncle guard: shock flags of the stage input first
     shock_flag_kernel<R, D><<<(unsigned)((a.g.ncell + 255) / 256), 256, 0, s>>>(a);
@@ -132,7 +133,7 @@ cudaError_t launch_stage(const StageArgs<R>& a0, cudaStream_t s, cudaEvent_t mid
     if (e != cudaSuccess) return e;
   }
   if (small) gas_face_kernel<R, D, SPH, FACE_THREADS_SMALL><<<gg, FACE_THREADS_SMALL, 0, s>>>(a);
-  else gas_face_kernel<R, D, SPH, FACE_THREADS><<<gg, FACE_THREADS, 0, s>>>(a);
+  else gas_face_kernel<R, D, SPH, FT><<<gg, FT, 0, s>>>(a);
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   if (mid) {

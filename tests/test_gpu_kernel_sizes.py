@@ -32,13 +32,14 @@ def random_case(shape, G, precision, steps=2, vterms=0):
 
 # smallest grid; one group and the most; tile and chunk edges (20 x 8-lane and 256-thread tiles),
 # more groups than a block's tasks hold once in 3-d; 1 to 16 lanes per cell of the FP64 interaction and
-# both sides of its last step (152 x 224 cells); small and large gas-face tiles (520 x 160)
+# both sides of its last step (152 x 224 cells); small and large gas-face tiles (520 x 160,
+# 33 x 20 x 21, 161 x 18 x 19)
 @pytest.mark.parametrize("shape,G,precision", [
     ((4,), 1, "fp64"), ((33,), 32, "fp64"), ((34049,), 2, "fp64"), ((161,), 17, "fp32"),
     ((4, 4), 32, "fp64"), ((129, 7), 3, "fp64"), ((45, 9), 7, "fp64"), ((152, 224), 2, "fp64"), ((152, 225), 3, "fp64"),
     ((4, 5), 1, "fp32"), ((21, 33), 15, "fp32"), ((41, 19), 16, "fp32n64"), ((520, 160), 1, "fp32"),
     ((19, 23), 32, "fp32"), ((4, 4, 4), 1, "fp32"), ((17, 9, 5), 13, "fp32"), ((7, 18, 6), 20, "fp32n64"),
-    ((9, 5, 8), 32, "fp32"), ((6, 5, 7), 32, "fp64"),
+    ((9, 5, 8), 32, "fp32"), ((6, 5, 7), 32, "fp64"), ((33, 20, 21), 2, "fp32"), ((161, 18, 19), 1, "fp64"),
 ])
 def test_step_at_the_edges_of_tiles_and_rules(fxmod, shape, G, precision):  # noqa: F811
     pb, s = random_case(shape, G, precision)
