@@ -1,7 +1,7 @@
 // Cell-local implicit matter-radiation interaction of the FP64 state as a kernel of its own, one
-// thread per cell on all but the smallest grids (Sec. 5.3: the backward-Euler group update of Eq. 25 inside the Newton iteration
-// on T of Eqs. 26-27, the gas energy by conservation, then the flux absorption of Eq. 28 and its
-// momentum and energy feedback, Eqs. 31-32; readings R10-R12).
+// thread per cell on all but small grids (Sec. 5.3: the backward-Euler group update of Eq. 25 inside
+// the Newton iteration on T of Eqs. 26-27, the gas energy by conservation, then the flux absorption
+// of Eq. 28 and its momentum and energy feedback, Eqs. 31-32; readings R10-R12).
 //
 // GB300 executes two FP64 lane-operations per cycle per multiprocessor, and an FP64 warp
 // instruction occupies the FP64 pipe for the same time whether one lane or all 32 are active.

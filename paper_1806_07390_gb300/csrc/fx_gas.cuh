@@ -10,8 +10,9 @@
 // comparisons), a Cartesian direction's coefficients are one constant row of the launch
 // arguments, and HLLC's eleven divisions are six shared reciprocals.  Per launch: 1024^2 FP32 0.079
 // -> 0.050 ms, 256^3 FP32 2.04 -> 1.31 ms, 512^2 FP64 0.42 -> 0.33 ms.
-// The stage kernel then uses the fluxes for the gas divergence; with the velocity-dependent radiation terms on, the kernel also stores each face's
-// transverse velocity for their velocity gradient (fx_vterms.cuh).
+// The stage kernel then uses the fluxes for the gas divergence; with the velocity-dependent radiation
+// terms on, the kernel also stores each face's transverse velocity for their velocity gradient
+// (fx_vterms.cuh).
 #pragma once
 #include "fx_device.cuh"
 
@@ -27,10 +28,11 @@ __host__ __device__ inline int64_t faces_along(const int* n, int d) {
 // otherwise FT / 32 cells along DIR by 32 along x, so that a warp reads consecutive x), and
 // the top LD rows own their lower faces.  Cells 0 .. n_d along DIR own the n_d + 1 faces of the
 // direction (cell n_d is a ghost from the boundary rules).  FT = 288 on all grids whose tiles then
-// fill the device (the least halo share); in 3-d 160, whose rows along x leave fewer threads idle on the narrower grids
-// and cost nothing on wide ones (us per launch at 288 / 160 threads: 75 x 61 x 50 38 / 31, 128 x 96 x 100 126 / 102,
-// 256^3 1266 / 1262, 75 x 61 x 50 FP64 792 / 683; in 2-d 1024^2 47.8 / 49.2, 520 x 160 15.3 / 15.4); below
-// that 64, which spreads a small grid over more multiprocessors (512 cells FP64: 0.035 -> 0.017 ms).
+// fill the device (the least halo share); in 3-d 160, whose rows along x leave fewer threads idle on
+// the narrower grids and cost nothing on wide ones (us per launch at 288 / 160 threads: 75 x 61 x 50
+// 38 / 31, 128 x 96 x 100 126 / 102, 256^3 1266 / 1262, 75 x 61 x 50 FP64 792 / 683; in 2-d 1024^2
+// 47.8 / 49.2, 520 x 160 15.3 / 15.4); below that 64, which spreads a small grid over more
+// multiprocessors (512 cells FP64: 0.035 -> 0.017 ms).
 constexpr int FACE_THREADS = 288, FACE_THREADS_3D = 160, FACE_THREADS_SMALL = 64;
 template <int DIR, int FT> struct FaceTile {
   static constexpr int LX = DIR == 0 ? 1 : 32, LR = FT / LX, LD = LR - 1;

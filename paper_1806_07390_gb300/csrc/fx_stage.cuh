@@ -404,7 +404,7 @@ __device__ __forceinline__ void cp_async16(void* s, const void* g) {
 // exactly as many lanes as its groups need: GL = ceil(G / W) lanes of W groups, W = 2 as one packed
 // FP32 pair (F2), W = 1 in FP64.  A block owns a tile of TX x TY cells (TY = 1 below 3-d),
 // tid = cell * GL + lane, and marches along the slowest axis over a chunk of planes.  The tile is
-// chosen at run time (stage_tile): all shared arrays are addressed by tid and compile-time
+// chosen at run time (fit_tile): all shared arrays are addressed by tid and compile-time
 // capacities, so no group or tile count is a template parameter and no lane is padding.
 //   ring   four planes of the tile's own cells [slot][v][NT]: a thread copies its own cell with
 //          cp.async three planes ahead and reads its own march column from it;
