@@ -507,14 +507,17 @@ __device__ __forceinline__ void m1_state(const LaneConst<double>& K, double cE, 
 __device__ __forceinline__ F2 max1(F2 f2) { return vmax(f2, F2(1.0f)); }
 __device__ __forceinline__ double max1(double f2) { return __double2hiint(f2) >= 0x3ff00000 ? f2 : 1.0; }  // f2 >= 0
 __device__ __forceinline__ F2 rcp_fast(F2 x) { return F2(rcp_approx(x.x), rcp_approx(x.y)); }
-__device__ __forceinline__ double rcp_fast(double x) { return rcp64(x); }
+// (x > 0; 0 for an infinite x: f^2 overflows where a flux meets a cell whose energy lies at its floor, and
+// rcp64 has no value there)
+__device__ __forceinline__ double rcp_fast(double x) { return __double2hiint(x) == 0x7ff00000 ? 0.0 : rcp64(x); }
 
 // c^2 times row n of the M1 pressure tensor (reading R7) for the lane's groups.  With f = |F|/(cE)
 // and s = sqrt(4 - 3 f^2), f^2 = (4 - s^2)/3 turns the closure's two coefficients into
 //   (1 - chi)/2 = (s - 1)/3,   (3 chi - 1)/2 = 3 f^2/(2 + s),
 // so c^2 P_nq = cE (c/3)(s - 1) delta_nq + F_n F_q / ((2 + s) cE/(3c)): one reciprocal of cE, one square
 // root, one reciprocal.  f > 1 keeps the direction with f clamped to 1 (the factor max(f^2, 1) in
-// the second reciprocal's argument); E <= 0 is isotropic (1/(cE) taken as 0).
+// the second reciprocal's argument, which is 0 where f^2 overflows); E <= 0 is isotropic (1/(cE) taken
+// as 0).
 template <int D, class V>
 __device__ __forceinline__ void m1_c2row(const LaneConst<V>& K, V E, const V* F, int n, V* P) {
   const V cE = E * K.c;

@@ -1,0 +1,47 @@
+"""The M1 closure where |F| exceeds cE by so much that |F|^2 / (cE)^2 overflows: cold cells lie at the
+energy floor (1e-300 by default) or in the Wien tail, and a flux can reach them a step before its
+energy does.  The closure keeps its clamped value there.  Bars of the parity tests (FP64: 1e-10 in
+L1, 1e-8 at most)."""
+import numpy as np
+import pytest
+
+from paper_1806_07390_gb300 import workloads as W
+from tests import helpers as H
+from tests.test_gpu_kernel_sizes import random_case
+from tests.test_gpu_parity import FP64_L1, FP64_MAX, fxmod, run_gpu, run_oracle  # noqa: F401
+
+pytestmark = pytest.mark.gpu
+
+
+# f^2 = (|F| / cE)^2 just below and above 2^1022 and far past the largest double
+@pytest.mark.parametrize("energy", [1e-152, 1e-156, 1e-250, 1e-300])
+@pytest.mark.parametrize("shape", [(24,), (13, 12), (9, 8, 7)])
+def test_flux_far_above_the_free_streaming_limit(fxmod, shape, energy):  # noqa: F811
+    pb, s = random_case(shape, 3, "fp64")
+    N, G, NG = pb.ncell, pb.ngroups, 2 + pb.dims
+    E = s[NG * N:(NG + G) * N].reshape(pb.shape + (G,))
+    # a block of cells wide enough that the reconstruction leaves face states of its value
+    E[tuple(slice(1, 7) for _ in pb.shape) + (1,)] = energy
+    got, st, _ = run_gpu(fxmod, pb, state=s)
+    ref, rst = run_oracle(pb, state=s)
+    assert np.all(np.isfinite(ref))
+    assert st == 0 and rst == 0
+    H.assert_parity(pb, got, ref, FP64_L1, FP64_MAX)
+
+
+def test_fronts_that_meet_in_cold_gas(fxmod):  # noqa: F811
+    # radiation at T = 1 runs from both sides into 31 cells of gas and radiation at T = 0.004, whose
+    # upper group holds 1e-197
+    pb, _ = W.sod_1d(n=64, ngroups=4, precision="fp64")
+    pb.bc_lo = pb.bc_hi = ("periodic",) * 3
+    pb.kappa0, pb.kap_rho_exp, pb.kap_T_exp, pb.kap_eps_exp, pb.sigma0 = 1.0, 0, 0, 0, 0.0
+    pb.c_light, pb.nsteps = 20.0, 45
+    pb.dt = 0.4 / 64 / pb.c_light
+    prim = np.zeros((4, 64))
+    prim[0], prim[1], prim[3] = 1.0, 0.004, 1.0
+    prim[3, 16:47] = 0.004
+    got, st, _ = run_gpu(fxmod, pb, prim)
+    ref, rst = run_oracle(pb, prim)
+    assert np.all(np.isfinite(ref))
+    assert st == 0 and rst == 0
+    H.assert_parity(pb, got, ref, FP64_L1, FP64_MAX)
