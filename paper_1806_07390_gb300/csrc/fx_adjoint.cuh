@@ -103,6 +103,7 @@ __global__ void __launch_bounds__(256) adj_couple_kernel(const __grid_constant__
       any = any || nonzero(lFo[q]);
     }
   }
+  double lk = 0.0;  // the cell's dJ/dkappa0
   if (!g.couple) {  // no interaction: U_out = U_pre
     if (active) {
       if (lane < NG) A.lam_pre[FXI(lane * ncell + c, A.n_state)] = A.lam_out[FXI(lane * ncell + c, A.n_state)];
@@ -112,11 +113,8 @@ __global__ void __launch_bounds__(256) adj_couple_kernel(const __grid_constant__
         for (int q = 0; q < D; ++q) A.lam_pre[FXI(NG * ncell + ((1 + q) * ncell + c) * G + gl, A.n_state)] = lFo[q];
       }
     }
-    block_partial(0.0, A.kpart);
-    return;
-  }
-  // where nothing depends on the outputs of the warp's cells, nothing does on their inputs
-  if (!__any_sync(0xffffffffu, any)) {
+  } else if (!__any_sync(0xffffffffu, any)) {
+    // where nothing depends on the outputs of the warp's cells, nothing does on their inputs
     if (active) {
       if (lane < NG) A.lam_pre[FXI(lane * ncell + c, A.n_state)] = R(0);
       if (has) {
@@ -124,114 +122,114 @@ __global__ void __launch_bounds__(256) adj_couple_kernel(const __grid_constant__
         for (int v = 0; v < 1 + D; ++v) A.lam_pre[FXI(NG * ncell + (v * ncell + c) * G + gl, A.n_state)] = R(0);
       }
     }
-    block_partial(0.0, A.kpart);
-    return;
-  }
-  const R ugas = A.pre[FXI(gv * ncell + c, A.n_state)];
+  } else {
+    const R ugas = A.pre[FXI(gv * ncell + c, A.n_state)];
 #pragma unroll
-  for (int v = 0; v < NG; ++v) {
-    u[v] = __shfl_sync(0xffffffffu, ugas, v, GP);
-    lo[v] = __shfl_sync(0xffffffffu, lgas, v, GP);
-  }
-  R E = R(0), F[3] = {R(0), R(0), R(0)};
-  if (has) {
-    E = A.pre[FXI(NG * ncell + c * G + gl, A.n_state)];
-#pragma unroll
-    for (int q = 0; q < D; ++q) F[q] = A.pre[FXI(NG * ncell + ((1 + q) * ncell + c) * G + gl, A.n_state)];
-  }
-  // the interaction's silent positivity floor on E_g^-: a floored group's energy does not depend
-  // on its input
-  const bool floored = has && E < KR.E_floor;
-  if (floored) E = KR.E_floor;
-  const R T = A.tstar[FXI(c, ncell)], iT = rcp_any(T);
-  const R rho = u[0], irho = rcp_any(rho), rhoe = u[NG - 1];
-  R m[3] = {R(0), R(0), R(0)}, ke = R(0);
-#pragma unroll
-  for (int q = 0; q < D; ++q) { m[q] = u[1 + q]; ke += R(0.5) * m[q] * m[q] * irho; }
-  const R ra = R(0.5) * R(g.kap_rho_h), tb = R(0.5) * R(g.kap_T_h);
-  const R K0 = hpow(rho, g.kap_rho_h) * hpow(T, g.kap_T_h);  // kappa / (kappa0 eps^d)
-  const GroupConst& gc = *A.gc;
-  const R ef = has ? R(gc.efac_of(gl, R(0))) : R(0);
-  const R kap = KR.kappa0 * K0 * ef;
-  const R cdts = KR.cdts;
-  const R tau = cdts * kap;
-  const R i1 = rcp_any(R(1) + tau);
-  // Planck group energy and its T derivative at the converged temperature
-  R B, dB;
-  {
-    LanePlanck<GP, R> cp{A.pk, A.ptab, lane, has, (G == GP) && (lane == G - 1), KR.aN,
-                         R(gc.edge_of(lane <= G ? lane : G, R(0))), R(gc.edge_of(lane < G ? lane + 1 : G, R(0)))};
-    cp.planck(T, iT, B, dB);
-    if (!has) { B = R(0); dB = R(0); }
-  }
-  const R Ep = (E + tau * B) * i1;
-  const R fac = rcp_any(R(1) + cdts * (kap + KR.sigma0 * rho));
-  R SdF[3] = {R(0), R(0), R(0)};
-#pragma unroll
-  for (int q = 0; q < D; ++q) SdF[q] = seg_sum<GP>(has ? F[q] * (fac - R(1)) : R(0));
-
-  const R ic2 = KR.ic2;
-  const R lre_o = lo[NG - 1];
-  // rho e' = rho e - sum_g (E'_g - E_g) - ic2 sum_q (m_q / rho) sum_g dF_gq;  m'_q = m_q - ic2 sum_g dF_gq
-  R lrho = lo[0], lm[3] = {R(0), R(0), R(0)}, ldF[3] = {R(0), R(0), R(0)};
-#pragma unroll
-  for (int q = 0; q < D; ++q) {
-    ldF[q] = -ic2 * (lo[1 + q] + m[q] * irho * lre_o);
-    lm[q] = lo[1 + q] - ic2 * SdF[q] * irho * lre_o;
-    lrho += ic2 * m[q] * SdF[q] * irho * irho * lre_o;
-  }
-  // F' = F fac, dF = F (fac - 1)
-  R lF[3] = {R(0), R(0), R(0)}, lfac = R(0);
-#pragma unroll
-  for (int q = 0; q < D; ++q) {
-    lF[q] = lFo[q] * fac + ldF[q] * (fac - R(1));
-    lfac += F[q] * (lFo[q] + ldF[q]);
-  }
-  // fac = 1 / (1 + cdts (kappa + sigma0 rho))
-  R lkap = -fac * fac * cdts * lfac;
-  lrho += KR.sigma0 * seg_sum<GP>(has ? lkap : R(0));
-  // energy: E'_g = (E_g + tau B)/(1 + tau) at T*
-  R lrhoe = lre_o;
-  const R lEp = lEo - lre_o;
-  R lE = lre_o + lEp * i1;
-  const R ltau = lEp * (B - Ep) * i1;
-  R lT = seg_sum<GP>(has ? lEp * tau * i1 * dB : R(0));
-  lkap += ltau * cdts;
-  // kappa = kappa0 K0(rho, T) eps^d
-  const R Slk = seg_sum<GP>(has ? lkap * kap : R(0));
-  lrho += ra * Slk * irho;
-  lT += tb * Slk * iT;
-  R lk0 = seg_sum<GP>(has ? lkap * K0 * ef : R(0));
-  // T* from r(T*; rho, u^-, E^-, kappa0) = 0
-  const R dtau = tau * tb * iT;
-  const R drdT = rho * KR.cv + seg_sum<GP>(has ? (tau * dB + dtau * (B - Ep)) * i1 : R(0));
-  const R lr = -lT * rcp_any(drdT);
-  const R Sb = seg_sum<GP>(has ? (B - Ep) * i1 * tau : R(0));
-  lrho += lr * (KR.cv * T + ra * Sb * irho);
-  const R lum = -lr;
-  lE += lr * (-tau * i1);
-  lk0 += lr * seg_sum<GP>(has ? (B - Ep) * i1 * cdts * K0 * ef : R(0));
-  // u^- = rho e - |m|^2 / (2 rho)
-  lrhoe += lum;
-#pragma unroll
-  for (int q = 0; q < D; ++q) lm[q] -= lum * m[q] * irho;
-  lrho += lum * ke * irho;
-
-  if (active) {
-    if (lane < NG) {
-      R val = lrho;
-#pragma unroll
-      for (int q = 0; q < D; ++q) if (lane == 1 + q) val = lm[q];
-      if (lane == NG - 1) val = lrhoe;
-      A.lam_pre[FXI(lane * ncell + c, A.n_state)] = val;
+    for (int v = 0; v < NG; ++v) {
+      u[v] = __shfl_sync(0xffffffffu, ugas, v, GP);
+      lo[v] = __shfl_sync(0xffffffffu, lgas, v, GP);
     }
+    R E = R(0), F[3] = {R(0), R(0), R(0)};
     if (has) {
-      A.lam_pre[FXI(NG * ncell + c * G + gl, A.n_state)] = floored ? R(0) : lE;
+      E = A.pre[FXI(NG * ncell + c * G + gl, A.n_state)];
 #pragma unroll
-      for (int q = 0; q < D; ++q) A.lam_pre[FXI(NG * ncell + ((1 + q) * ncell + c) * G + gl, A.n_state)] = lF[q];
+      for (int q = 0; q < D; ++q) F[q] = A.pre[FXI(NG * ncell + ((1 + q) * ncell + c) * G + gl, A.n_state)];
     }
+    // the interaction's silent positivity floor on E_g^-: a floored group's energy does not depend
+    // on its input
+    const bool floored = has && E < KR.E_floor;
+    if (floored) E = KR.E_floor;
+    const R T = A.tstar[FXI(c, ncell)], iT = rcp_any(T);
+    const R rho = u[0], irho = rcp_any(rho), rhoe = u[NG - 1];
+    R m[3] = {R(0), R(0), R(0)}, ke = R(0);
+#pragma unroll
+    for (int q = 0; q < D; ++q) { m[q] = u[1 + q]; ke += R(0.5) * m[q] * m[q] * irho; }
+    const R ra = R(0.5) * R(g.kap_rho_h), tb = R(0.5) * R(g.kap_T_h);
+    const R K0 = hpow(rho, g.kap_rho_h) * hpow(T, g.kap_T_h);  // kappa / (kappa0 eps^d)
+    const GroupConst& gc = *A.gc;
+    const R ef = has ? R(gc.efac_of(gl, R(0))) : R(0);
+    const R kap = KR.kappa0 * K0 * ef;
+    const R cdts = KR.cdts;
+    const R tau = cdts * kap;
+    const R i1 = rcp_any(R(1) + tau);
+    // Planck group energy and its T derivative at the converged temperature
+    R B, dB;
+    {
+      LanePlanck<GP, R> cp{A.pk, A.ptab, lane, has, (G == GP) && (lane == G - 1), KR.aN,
+                           R(gc.edge_of(lane <= G ? lane : G, R(0))), R(gc.edge_of(lane < G ? lane + 1 : G, R(0)))};
+      cp.planck(T, iT, B, dB);
+      if (!has) { B = R(0); dB = R(0); }
+    }
+    const R Ep = (E + tau * B) * i1;
+    const R fac = rcp_any(R(1) + cdts * (kap + KR.sigma0 * rho));
+    R SdF[3] = {R(0), R(0), R(0)};
+#pragma unroll
+    for (int q = 0; q < D; ++q) SdF[q] = seg_sum<GP>(has ? F[q] * (fac - R(1)) : R(0));
+
+    const R ic2 = KR.ic2;
+    const R lre_o = lo[NG - 1];
+    // rho e' = rho e - sum_g (E'_g - E_g) - ic2 sum_q (m_q / rho) sum_g dF_gq;  m'_q = m_q - ic2 sum_g dF_gq
+    R lrho = lo[0], lm[3] = {R(0), R(0), R(0)}, ldF[3] = {R(0), R(0), R(0)};
+#pragma unroll
+    for (int q = 0; q < D; ++q) {
+      ldF[q] = -ic2 * (lo[1 + q] + m[q] * irho * lre_o);
+      lm[q] = lo[1 + q] - ic2 * SdF[q] * irho * lre_o;
+      lrho += ic2 * m[q] * SdF[q] * irho * irho * lre_o;
+    }
+    // F' = F fac, dF = F (fac - 1)
+    R lF[3] = {R(0), R(0), R(0)}, lfac = R(0);
+#pragma unroll
+    for (int q = 0; q < D; ++q) {
+      lF[q] = lFo[q] * fac + ldF[q] * (fac - R(1));
+      lfac += F[q] * (lFo[q] + ldF[q]);
+    }
+    // fac = 1 / (1 + cdts (kappa + sigma0 rho))
+    R lkap = -fac * fac * cdts * lfac;
+    lrho += KR.sigma0 * seg_sum<GP>(has ? lkap : R(0));
+    // energy: E'_g = (E_g + tau B)/(1 + tau) at T*
+    R lrhoe = lre_o;
+    const R lEp = lEo - lre_o;
+    R lE = lre_o + lEp * i1;
+    const R ltau = lEp * (B - Ep) * i1;
+    R lT = seg_sum<GP>(has ? lEp * tau * i1 * dB : R(0));
+    lkap += ltau * cdts;
+    // kappa = kappa0 K0(rho, T) eps^d
+    const R Slk = seg_sum<GP>(has ? lkap * kap : R(0));
+    lrho += ra * Slk * irho;
+    lT += tb * Slk * iT;
+    R lk0 = seg_sum<GP>(has ? lkap * K0 * ef : R(0));
+    // T* from r(T*; rho, u^-, E^-, kappa0) = 0
+    const R dtau = tau * tb * iT;
+    const R drdT = rho * KR.cv + seg_sum<GP>(has ? (tau * dB + dtau * (B - Ep)) * i1 : R(0));
+    const R lr = -lT * rcp_any(drdT);
+    const R Sb = seg_sum<GP>(has ? (B - Ep) * i1 * tau : R(0));
+    lrho += lr * (KR.cv * T + ra * Sb * irho);
+    const R lum = -lr;
+    lE += lr * (-tau * i1);
+    lk0 += lr * seg_sum<GP>(has ? (B - Ep) * i1 * cdts * K0 * ef : R(0));
+    // u^- = rho e - |m|^2 / (2 rho)
+    lrhoe += lum;
+#pragma unroll
+    for (int q = 0; q < D; ++q) lm[q] -= lum * m[q] * irho;
+    lrho += lum * ke * irho;
+
+    if (active) {
+      if (lane < NG) {
+        R val = lrho;
+#pragma unroll
+        for (int q = 0; q < D; ++q) if (lane == 1 + q) val = lm[q];
+        if (lane == NG - 1) val = lrhoe;
+        A.lam_pre[FXI(lane * ncell + c, A.n_state)] = val;
+      }
+      if (has) {
+        A.lam_pre[FXI(NG * ncell + c * G + gl, A.n_state)] = floored ? R(0) : lE;
+#pragma unroll
+        for (int q = 0; q < D; ++q) A.lam_pre[FXI(NG * ncell + ((1 + q) * ncell + c) * G + gl, A.n_state)] = lF[q];
+      }
+    }
+    if (active && lane == 0) lk = (double)lk0;
   }
-  block_partial((active && lane == 0) ? (double)lk0 : 0.0, A.kpart);
+  block_partial(lk, A.kpart);
 }
 
 // Adjoint of the M1 pressure row n at the state Q = (E, F): adds sum_q lam_q dP_nq/dQ to lQ (lam in

@@ -89,3 +89,23 @@ def test_adjoint_at_the_edges_of_blocks(fxmod, shape, G):  # noqa: F811
     assert abs(J - Jr) <= 1e-12 * abs(Jr)
     got = float(gs @ t) + dk * dkap
     assert abs(got - dJ) <= 1e-6 * abs(dJ), (got, dJ)
+
+
+# after two steps only cells near the upper x boundary have adjoints: of the warps of one block (32 cells
+# of rows of 40, 4 per warp) some have cells to work on and some have none, and kappa0's partial is
+# the block's sum over both
+@pytest.mark.parametrize("shape,G,couple", [((40, 9), 2, 1), ((40, 9), 2, 0), ((67,), 20, 1)])
+def test_adjoint_where_warps_of_a_block_are_idle(fxmod, shape, G, couple):  # noqa: F811
+    pb, s = random_case(shape, G, "fp64")
+    pb.couple = couple
+    J, gs, gr, dk, _ = gpu_adjoint(fxmod, pb, s, 2, 1)
+    g = gs[:pb.ncell].reshape(pb.shape)
+    assert np.all(g[..., :20] == 0.0) and np.all(g[..., -1] != 0.0)
+    t = _random_tangent(pb, s, 1)
+    dkap = 0.3 * pb.kappa0
+    _, Jr, dJ, _, _ = oracle.run_objective(pb, s, pb.dt, 2, tangent=t, dkappa0=dkap)
+    assert abs(J - Jr) <= 1e-12 * abs(Jr)
+    got = float(gs @ t) + dk * dkap
+    assert abs(got - dJ) <= 1e-6 * abs(dJ), (got, dJ)
+    _, _, dJk, _, _ = oracle.run_objective(pb, s, pb.dt, 2, tangent=np.zeros_like(t), dkappa0=dkap)
+    assert abs(dk * dkap - dJk) <= 1e-6 * abs(dJk), (dk * dkap, dJk)
