@@ -730,7 +730,10 @@ LaneConst<V> make_lane_consts(const fx_grid* h, double dt, double alpha) {
   k.m3 = v(-3.0);
   k.p4 = v(4.0);
   k.q25 = v(0.25);
-  for (int d = 0; d < 3; ++d) k.hdt[d] = v(0.5 * dt * h->dg.inv_dx[d]);
+  for (int d = 0; d < 3; ++d) {
+    k.hdt[d] = v(0.5 * dt * h->dg.inv_dx[d]);
+    k.mhdt[d] = v(-0.5 * dt * h->dg.inv_dx[d]);
+  }
   k.alpha = v(alpha);
   k.beta = v(1.0 - alpha);
   return k;
