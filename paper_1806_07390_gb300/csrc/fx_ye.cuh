@@ -582,7 +582,8 @@ __global__ void __launch_bounds__(CPL_THREADS, 5) couple_ye32_kernel(const __gri
     for (int gg = 0; gg < Gs; ++gg) {
       const double x = fma(cdt, fma(kT, s_efd[gg], sig), 1.0);
       const float xh = to_f32(x), xl = to_f32(x - (double)xh);
-      const float fh = frcp(xh), fl = fh * (fmaf(-xh, fh, 1.0f) - xl * fh);  // 1/x = fh + fl
+      // 1/x = fh + fl (0 where x is past FP32's range: its float is infinite there)
+      const float fh = frcp(xh), fl = fh > 0.0f ? fh * (fmaf(-xh, fh, 1.0f) - xl * fh) : 0.0f;
 #pragma unroll
       for (int s = 0; s < 3; ++s) {
 #pragma unroll

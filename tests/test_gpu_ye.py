@@ -234,3 +234,22 @@ def test_three_species_totals_after_upload(fxmod, precision):
     ref = oracle.totals(pb, s0)
     np.testing.assert_allclose(t, ref, rtol=1e-13 if precision == "fp64" else 1e-6,
                                atol=1e-12 * np.abs(ref).max())
+
+
+@pytest.mark.parametrize("precision,tol", [("fp64", 1e-10), ("fp32", 1e-5), ("fp32n64", 1e-5)])
+def test_three_species_scattering_past_the_range_of_floats(fxmod, precision, tol):
+    # c dt sigma0 rho = 1e39: the flux absorption's factor 1/(1 + c dt chi) is 0 in FP32
+    pb, prim = case("box2d")
+    pb.precision, pb.sigma0, pb.x_hi = precision, 3e38, (1000.0,) * 3
+    pb.dt *= 1000.0
+    s0 = oracle.init_equilibrium(pb, prim)
+    ref, rst = oracle.run(pb, s0, pb.dt, pb.nsteps, nthreads=8)
+    assert rst == 0 and np.all(np.isfinite(ref))
+    g = fxmod.Grid(pb)
+    g.init_equilibrium(prim)
+    g.step(pb.dt, pb.nsteps)
+    st = g.status()
+    got = g.download()
+    g.close()
+    assert st == 0
+    H.assert_parity(pb, got, ref, tol, natural=True)
