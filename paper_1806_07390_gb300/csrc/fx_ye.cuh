@@ -351,6 +351,12 @@ __device__ __forceinline__ void acc_diff(FPair& a, float x, float y) {
   a.h = s;
   a.l += e + f;
 }
+// a += (x + xl) y, the product with its rounding errors
+__device__ __forceinline__ void acc_mul(FPair& a, float x, float xl, float y) {
+  const float p = __fmul_rn(x, y);
+  acc(a, p);
+  a.l += fmaf(xl, y, fmaf(x, y, -p));
+}
 __device__ __forceinline__ double val(FPair a) { return (double)a.h + (double)a.l; }
 
 constexpr int couple_ye32_rows(int D) { return D > 2 ? D : 2; }
@@ -363,7 +369,7 @@ __global__ void __launch_bounds__(CPL_THREADS, 5) couple_ye32_kernel(const __gri
   constexpr int NG = 2 + D;
   extern __shared__ __align__(16) unsigned char ye_raw[];
   float* const srow = reinterpret_cast<float*>(ye_raw);  // E^- and E, then the F_q
-  __shared__ float s_ef[MAXG], s_ed[MAXG + 1], s_xi[MAXG];
+  __shared__ float s_ef[MAXG], s_ed[MAXG + 1], s_xi[MAXG], s_xil[MAXG];  // (xi0/eps_g: s_xi + s_xil)
   __shared__ double s_efd[MAXG], s_xid[MAXG];
   const DevGrid& g = A.g;
   const int G = g.G, Gs = g.Gs, RS = G + 1, t = (int)threadIdx.x;
@@ -379,6 +385,7 @@ __global__ void __launch_bounds__(CPL_THREADS, 5) couple_ye32_kernel(const __gri
       const double xi = g.xi0 * (1.0 / sqrt(A.gc->edge[j] * A.gc->edge[j + 1]));
       s_xid[j] = xi;
       s_xi[j] = (float)xi;
+      s_xil[j] = (float)(xi - (double)s_xi[j]);
     }
   }
   const RowCopy rc(A.out + ((size_t)NG * ncell + (size_t)c0 * G), nc, G, RS);
@@ -418,8 +425,7 @@ __global__ void __launch_bounds__(CPL_THREADS, 5) couple_ye32_kernel(const __gri
     if (u_m < u_floor) { u_m = u_floor; st |= ST_FLOOR; }
     const double X_m = U[FXI(XO + c, A.n_state)], Y_m = X_m * irho;
     // E^- with its silent floor, sum E^- and the tolerance's scale sum |xi| E^-
-    FPair Es = {0.0f, 0.0f};
-    float Ls = 0.0f;
+    FPair Es = {0.0f, 0.0f}, Ls = Es;
     const float flo = (float)g.E_floor;
     // (floored channels are rare: found by a minimum, and the energy the floor adds summed in FP64 apart
     // from the loop, where its conversions and sums would run for every channel)
@@ -434,14 +440,12 @@ __global__ void __launch_bounds__(CPL_THREADS, 5) couple_ye32_kernel(const __gri
         }
     }
     for (int gg = 0; gg < Gs; ++gg) {
-      float ab = 0.0f;
 #pragma unroll
       for (int s = 0; s < 3; ++s) {
         const float e = Em[s * Gs + gg];
         acc(Es, e);
-        if (s < 2) ab += e;
+        if (s < 2) acc_mul(Ls, s_xi[gg], s_xil[gg], e);
       }
-      Ls = fmaf(s_xi[gg], ab, Ls);
     }
     kpre = A.kd.kappa0 * hpow(rho, g.kap_rho_h);
     const float kpref = to_f32(kpre), cdtf = A.kf.cdts;
@@ -483,7 +487,7 @@ __global__ void __launch_bounds__(CPL_THREADS, 5) couple_ye32_kernel(const __gri
     };
     // stopping tests at FP32 resolution (relative step 2e-7 at least, residual 1e-7)
     const double rtol = A.kd.rtol, n2ok = A.kd.atol * A.kd.atol;
-    const double isE = rcp_any(u_m + val(Es)), isX = rcp_any(fabs(X_m) + (double)Ls + 1e-300);
+    const double isE = rcp_any(u_m + val(Es)), isX = rcp_any(fabs(X_m) + val(Ls) + 1e-300);
     auto norm2 = [&](double rE, double rX) { const double a = rE * isE, b = rX * isX; return fma(a, a, b * b); };
     double Y = Y_m, rE, rX, JT, JX, JY;
     T = u_m * rcp_any(rcv);

@@ -3,6 +3,7 @@
 #include <cuda_runtime.h>
 
 #include "fx_stage.cuh"
+#include "fx_ye.cuh"
 
 namespace {
 
@@ -27,7 +28,30 @@ template <int D> __global__ void net_kernel(const float* in, float* out, int n) 
   out[n + i] = r.y;
 }
 
+// sums of n terms by one thread each: of x, of x - y, of x y with x = (float)x + (float)(x - (float)x)
+__global__ void pair_kernel(const double* x, const float* y, double* out, int n, int m) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= m) return;
+  fx::FPair a = {0.0f, 0.0f}, d = a, p = a;
+  for (int k = 0; k < n; ++k) {
+    const double xk = x[k * m + i];
+    const float xh = (float)xk, xl = (float)(xk - (double)xh), yk = y[k * m + i];
+    fx::acc(a, xh);
+    fx::acc_diff(d, xh, yk);
+    fx::acc_mul(p, xh, xl, yk);
+  }
+  out[i] = fx::val(a);
+  out[m + i] = fx::val(d);
+  out[2 * m + i] = fx::val(p);
+}
+
 }  // namespace
+
+// m sums of n terms each (device arrays [n][m]; out [3][m])
+extern "C" int arith_pairs(const double* x, const float* y, double* out, int n, int m) {
+  pair_kernel<<<(m + 127) / 128, 128>>>(x, y, out, n, m);
+  return (int)cudaDeviceSynchronize();
+}
 
 // in: (3 D) x n floats, out: 2 x n floats (device).  Returns the CUDA error.
 extern "C" int arith_net(int D, const float* in, float* out, int n) {

@@ -67,3 +67,25 @@ def test_net_update_is_compensated(probe, D, kind):
     bound = 2.0 ** -24 * np.abs(ref) + 16 * 2.0 ** -47 * m + 2.0 ** -126
     assert np.array_equal(got[1], -got[0])
     assert np.all(np.abs(got[0] - ref) <= bound), np.max(np.abs(got[0] - ref) / bound)
+
+
+# The channel sums of the FP32 two-equation interaction, pairs of floats: every term enters with its
+# rounding error, so a sum's error is that of the low parts, each below 2^-24 of the running sum or of a
+# term and rounded again twice: 2^-47 of the sum of magnitudes a term.  (A plain FP32 sum is off by 2^-25
+# of the sum a term.)
+def test_pair_sums_hold_twice_the_bits_of_a_float(probe):
+    import torch
+    rng = np.random.default_rng(5)
+    n, m = 24, 4000
+    x = rng.uniform(0.1, 1.0, (n, m)) * 10.0 ** rng.uniform(-3.0, 0.0, (n, m))
+    y = (x * (1.0 + 1e-3 * rng.normal(size=(n, m)))).astype(np.float32)
+    out = torch.zeros(3 * m, dtype=torch.float64, device="cuda")
+    assert probe.arith_pairs(ptr(on_gpu(x)), ptr(on_gpu(y)), ptr(out), n, m) == 0
+    got = out.cpu().numpy().reshape(3, m)
+    xf, yf = x.astype(np.float32).astype(np.float64), y.astype(np.float64)
+    L = np.longdouble
+    for k, (terms, what) in enumerate([(xf.astype(L), "sum"), (xf.astype(L) - yf.astype(L), "difference"),
+                                       (x.astype(L) * yf.astype(L), "product")]):
+        size = np.sum(np.abs(xf), axis=0) if k < 2 else np.sum(np.abs(x * yf), axis=0)
+        err = np.abs(got[k] - np.sum(terms, axis=0)).astype(np.float64)
+        assert np.all(err <= n * 2.0 ** -47 * size), (what, np.max(err / size))
