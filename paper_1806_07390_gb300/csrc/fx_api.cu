@@ -452,39 +452,6 @@ void build_planck_table(const fx_params& P, const GroupConst& gc, const PlanckPa
     }
 }
 
-// Coefficients of one interval (see PlanckTable) from its two nodes (L - floor(L), h dL/du, floor(L),
-// 2^floor(L)).
-void planck_interval_entry(const float4& p, const float4& q, float c[4]) {
-  const double d = ((double)q.z - (double)p.z) + ((double)q.x - (double)p.x);  // L at the right node less L at the left
-  const double m0 = p.y, m1 = q.y;
-  c[0] = p.x;
-  c[1] = p.y;
-  c[2] = (float)(3.0 * d - 2.0 * m0 - m1);
-  c[3] = (float)(m0 + m1 - 2.0 * d);
-  unsigned sc, b;
-  std::memcpy(&sc, &p.w, 4);
-  std::memcpy(&b, &c[3], 4);
-  b = (b & ~0xffu) | (sc >> 23);
-  std::memcpy(&c[3], &b, 4);
-}
-// The device table: (groups + 1)/2 pairs (an odd count's last pair repeats its group).
-std::vector<float4> planck_device_table(const std::vector<float4>& tab, int G, int nu, bool node_major) {
-  const int NP = (G + 1) / 2;
-  std::vector<float4> out((size_t)2 * NP * nu);
-  for (int p = 0; p < NP; ++p)
-    for (int i = 0; i < nu; ++i) {
-      float c[2][4];
-      for (int s = 0; s < 2; ++s) {
-        const float4* const t = tab.data() + (size_t)std::min(2 * p + s, G - 1) * nu;
-        planck_interval_entry(t[i], t[std::min(i + 1, nu - 1)], c[s]);
-      }
-      float4* const e = out.data() + 2 * (node_major ? (size_t)i * NP + p : (size_t)p * nu + i);
-      e[0] = make_float4(c[0][0], c[1][0], c[0][1], c[1][1]);
-      e[1] = make_float4(c[0][2], c[1][2], c[0][3], c[1][3]);
-    }
-  return out;
-}
-
 // Layout of the device Planck table, a measured choice (interaction kernel per launch, node-major
 // against group-major): 1024^2 x 16 0.118 against 0.121 ms, 256^3 x 12 2.89 against 2.75 ms, 515 x 389
 // x 7 0.026 against 0.025 ms.  A warp's cells read the intervals of their temperatures of every pair

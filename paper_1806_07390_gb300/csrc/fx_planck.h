@@ -1,5 +1,7 @@
-// Host construction of the FP64 Planck edge table (PETAB_ROWS rows of 8 coefficients; see
-// planck_edge_tab in fx_device.cuh).  Row n holds the polynomial in t = 16 x - n, |t| <= 1/2, that
+// Host construction of the Planck tables as the kernels read them: the FP64 edge table, and the FP32 band
+// table's coefficients from its nodes (at the end).
+//
+// FP64 edge table (PETAB_ROWS rows of 8 coefficients; see planck_edge_tab in fx_device.cuh).  Row n holds the polynomial in t = 16 x - n, |t| <= 1/2, that
 // interpolates at the 8 Chebyshev nodes
 //   n < PETAB_SPLIT:   R(x) = x^-3 Int_0^x s^3/(e^s - 1) ds   (Q = x^3 R)
 //   n >= PETAB_SPLIT:  Q(x) = Int_x^inf s^3/(e^s - 1) ds.
@@ -7,7 +9,11 @@
 // below it, so the coefficients are formed in double-double arithmetic (two doubles with error-free
 // sums and products; Dekker 1971, Knuth) and rounded once.
 #pragma once
+#include <cuda_runtime.h>
+
+#include <algorithm>
 #include <cmath>
+#include <cstring>
 #include <vector>
 
 #include "fx_types.h"
@@ -156,6 +162,39 @@ inline const std::vector<double>& planck_edge_table() {
     return t;
   }();
   return table;
+}
+
+// Coefficients of one interval (see PlanckTable) from its two nodes (L - floor(L), h dL/du, floor(L),
+// 2^floor(L)).
+inline void planck_interval_entry(const float4& p, const float4& q, float c[4]) {
+  const double d = ((double)q.z - (double)p.z) + ((double)q.x - (double)p.x);  // L at the right node less L at the left
+  const double m0 = p.y, m1 = q.y;
+  c[0] = p.x;
+  c[1] = p.y;
+  c[2] = (float)(3.0 * d - 2.0 * m0 - m1);
+  c[3] = (float)(m0 + m1 - 2.0 * d);
+  unsigned sc, b;
+  std::memcpy(&sc, &p.w, 4);
+  std::memcpy(&b, &c[3], 4);
+  b = (b & ~0xffu) | (sc >> 23);
+  std::memcpy(&c[3], &b, 4);
+}
+// The device table: (groups + 1)/2 pairs (an odd count's last pair repeats its group).
+inline std::vector<float4> planck_device_table(const std::vector<float4>& tab, int G, int nu, bool node_major) {
+  const int NP = (G + 1) / 2;
+  std::vector<float4> out((size_t)2 * NP * nu);
+  for (int p = 0; p < NP; ++p)
+    for (int i = 0; i < nu; ++i) {
+      float c[2][4];
+      for (int s = 0; s < 2; ++s) {
+        const float4* const t = tab.data() + (size_t)std::min(2 * p + s, G - 1) * nu;
+        planck_interval_entry(t[i], t[std::min(i + 1, nu - 1)], c[s]);
+      }
+      float4* const e = out.data() + 2 * (node_major ? (size_t)i * NP + p : (size_t)p * nu + i);
+      e[0] = make_float4(c[0][0], c[1][0], c[0][1], c[1][1]);
+      e[1] = make_float4(c[0][2], c[1][2], c[0][3], c[1][3]);
+    }
+  return out;
 }
 
 }  // namespace fx

@@ -2,6 +2,10 @@
 // of n operand sets.  The net update of a cell is built with the FP32 units' flags (see build.py).
 #include <cuda_runtime.h>
 
+#include <cstring>
+#include <vector>
+
+#include "fx_planck.h"
 #include "fx_stage.cuh"
 #include "fx_ye.cuh"
 
@@ -45,7 +49,100 @@ __global__ void pair_kernel(const double* x, const float* y, double* out, int n,
   out[2 * m + i] = fx::val(p);
 }
 
+// out = f(x) by the FP64 function of the given number (in the order of the test's list)
+__global__ void fp64_kernel(int f, const double* x, double* out, int n) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  const double v = x[i];
+  out[i] = f == 0   ? fx::rcp64(v)
+           : f == 1 ? fx::rcp_pos(v)
+           : f == 2 ? fx::rcp_any(v)
+           : f == 3 ? fx::rcp_fast(v)
+           : f == 4 ? fx::rcp_ge1(v)
+           : f == 5 ? fx::sqrt64(v)
+           : f == 6 ? fx::sqrt_any(v)
+                    : fx::rsqrt64(v);
+}
+__global__ void hpow_kernel(const double* x, const int* h, double* out, int n) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < n) out[i] = fx::hpow(x[i], h[i]);
+}
+// Q, w and whether Q is the upper integral, at x = x16 / 16
+__global__ void edge_kernel(const double* x16, const double* tab, const fx::PlanckCoef pc, double* out, int n) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  const fx::PlanckEdge<double> e = fx::planck_edge_tab(x16[i], tab, pc);
+  out[i] = e.Q;
+  out[n + i] = e.w;
+  out[2 * n + i] = e.upper ? 1.0 : 0.0;
+}
+// B_g(T) and dB_g/dT of every group, by pairs, with a_N = 1: out [2][G][n]
+__global__ void band_kernel(const fx::PlanckTable tab, const float* edge, const float* T, float* out, int G, int n) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  const fx::PlanckAt p = fx::planck_at(tab, 1.0f, T[i]);
+  for (int pr = 0; pr < (G + 1) / 2; ++pr) {
+    fx::F2 B, dB;
+    fx::planck_pair(tab, p, pr, G, edge, B, dB);
+    out[(2 * pr) * n + i] = B.x;
+    out[(G + 2 * pr) * n + i] = dB.x;
+    if (2 * pr + 1 < G) {
+      out[(2 * pr + 1) * n + i] = B.y;
+      out[(G + 2 * pr + 1) * n + i] = dB.y;
+    }
+  }
+}
+
 }  // namespace
+
+extern "C" int arith_fp64(int f, const double* x, double* out, int n) {
+  fp64_kernel<<<(n + 127) / 128, 128>>>(f, x, out, n);
+  return (int)cudaDeviceSynchronize();
+}
+extern "C" int arith_hpow(const double* x, const int* h, double* out, int n) {
+  hpow_kernel<<<(n + 127) / 128, 128>>>(x, h, out, n);
+  return (int)cudaDeviceSynchronize();
+}
+extern "C" int arith_planck_edge(const double* x16, double* out, int n) {
+  const std::vector<double>& t = fx::planck_edge_table();
+  fx::PlanckCoef pc{};  // (the table is left for the exponential series only)
+  for (int k = 1; k <= fx::NPLANCK_UP; ++k) pc.rn[k - 1] = 1.0 / k;
+  double* d = nullptr;
+  cudaError_t e = cudaMalloc(&d, t.size() * sizeof(double));
+  if (e == cudaSuccess) e = cudaMemcpy(d, t.data(), t.size() * sizeof(double), cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) {
+    edge_kernel<<<(n + 127) / 128, 128>>>(x16, d, pc, out, n);
+    e = cudaDeviceSynchronize();
+  }
+  cudaFree(d);
+  return (int)e;
+}
+// nodes: the host table [G][nu][4]; edge: G + 1 band edges (host); T, out on the device
+extern "C" int arith_planck_bands(const float* nodes, int G, int nu, float u0, int node_major, const float* edge, const float* T,
+                                  float* out, int n) {
+  std::vector<float4> host((size_t)G * nu);
+  std::memcpy(host.data(), nodes, host.size() * sizeof(float4));
+  const std::vector<float4> t = fx::planck_device_table(host, G, nu, node_major != 0);
+  float4* d = nullptr;
+  float* ed = nullptr;
+  cudaError_t e = cudaMalloc(&d, t.size() * sizeof(float4));
+  if (e == cudaSuccess) e = cudaMalloc(&ed, (G + 1) * sizeof(float));
+  if (e == cudaSuccess) e = cudaMemcpy(d, t.data(), t.size() * sizeof(float4), cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) e = cudaMemcpy(ed, edge, (G + 1) * sizeof(float), cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) {
+    fx::PlanckTable pt{};
+    pt.tab = d;
+    pt.nu = nu;
+    pt.u0 = u0;
+    pt.si = node_major ? (G + 1) / 2 : 1;
+    pt.sg = node_major ? 1 : nu;
+    band_kernel<<<(n + 127) / 128, 128>>>(pt, ed, T, out, G, n);
+    e = cudaDeviceSynchronize();
+  }
+  cudaFree(d);
+  cudaFree(ed);
+  return (int)e;
+}
 
 // m sums of n terms each (device arrays [n][m]; out [3][m])
 extern "C" int arith_pairs(const double* x, const float* y, double* out, int n, int m) {
