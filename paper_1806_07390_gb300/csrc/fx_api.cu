@@ -266,7 +266,9 @@ void build_table(const fx_params& P, int d, std::vector<double>& T) {
     double mu1[3], mu2[3];
     for (int k = -1; k <= 1; ++k) {
       const Moments& m = mo[ip + 1 + k];
-      double s = (xc[ip + 1 + k] - xc[ip + 1]) / h;
+      // (a Cartesian direction's cells lie one width apart: exact, so that every row is the same for any
+      // size and origin, and the kernels may read any one of them)
+      double s = P.geom == FX_CART || d >= 2 ? k : (xc[ip + 1 + k] - xc[ip + 1]) / h;
       double a1 = m.m1 / h, a2 = m.m2 / (h * h);
       mu1[k + 1] = s + a1;
       mu2[k + 1] = s * s + 2.0 * s * a1 + a2;

@@ -264,3 +264,27 @@ def test_spherical_tables_match_oracle_geometry(L, map1):
     np.testing.assert_allclose(T[0][e["RI"]], 1.0 / rf[:-1], rtol=1e-14)
     assert np.all(T[1][e["QI"]] == 1.0) and np.all(T[1][e["RI"]] == 1.0)
     L.fx_grid_destroy(h)
+
+
+@pytest.mark.parametrize("n,x_lo", [(64, 0.0), (75, 0.0), (96, -3.7), (515, 2.0 ** 20), (6, 1e6)])
+def test_cartesian_table_rows_are_one_row(L, n, x_lo):
+    # the kernels read one row of a Cartesian direction for every cell: all rows are bit-equal, whatever the
+    # size and the origin, and are those of a uniform grid
+    pb, _ = W.kh_2d(nx=n, ny=n + 1, ngroups=2)
+    pb.x_lo, pb.x_hi = (x_lo, x_lo, 0.0), (x_lo + 1.0, x_lo + 1.0, 1.0)
+    st, h, _ = create(pb)
+    assert st == 0
+    for d in range(2):
+        np_ = pb.n[d] + 4
+        T = np.zeros(L.fx_debug_ntab() * np_)
+        assert L.fx_debug_table(h, d, T.ctypes.data_as(ctypes.POINTER(ctypes.c_double)), T.size) == T.size
+        T = T.reshape(-1, np_)
+        assert np.all(T == T[:, :1])
+        w = 1.0 / pb.n[d]
+        # face weights of the parabola, end slopes, inverse gaps, face offsets, area/volume, gap, volume
+        want = {0: 1 / 3, 1: 5 / 6, 2: -1 / 6, 3: -1 / 6, 4: 5 / 6, 5: 1 / 3, 6: 0.25, 7: 0.25, 8: 0.25, 9: 0.25,
+                18: 1 / w, 19: 1 / w, 20: 0.5 / w, 21: -0.5 * w, 22: 0.5 * w, 23: 1 / w, 24: 1 / w, 25: w, 26: w}
+        h_d = (pb.x_hi[d] - pb.x_lo[d]) / pb.n[d]
+        for e, v in want.items():
+            assert abs(T[e, 0] - v) <= 4e-15 * abs(v) + abs(h_d - w) * abs(v) / w, (e, T[e, 0], v)
+    L.fx_grid_destroy(h)

@@ -109,3 +109,23 @@ def test_adjoint_where_warps_of_a_block_are_idle(fxmod, shape, G, couple):  # no
     assert abs(got - dJ) <= 1e-6 * abs(dJ), (got, dJ)
     _, _, dJk, _, _ = oracle.run_objective(pb, s, pb.dt, 2, tangent=np.zeros_like(t), dkappa0=dkap)
     assert abs(dk * dkap - dJk) <= 1e-6 * abs(dJk), (dk * dkap, dJk)
+
+
+# A Cartesian grid's coefficients depend on its cell width alone: moved by 2^20 widths of the domain, the same
+# state gives the same step and the same gradient, bit for bit.
+@pytest.mark.parametrize("shape,G,precision", [((75,), 3, "fp64"), ((45, 37), 2, "fp64"), ((9, 11, 7), 2, "fp64"),
+                                               ((45, 37), 3, "fp32n64")])
+def test_step_and_gradient_do_not_depend_on_the_origin(fxmod, shape, G, precision):  # noqa: F811
+    pb, s = random_case(shape, G, precision)
+    got, J = [], []
+    for x0 in (0.0, 2.0 ** 20):
+        pb.x_lo, pb.x_hi = (x0,) * 3, (x0 + 1.0,) * 3
+        state, st, _ = run_gpu(fxmod, pb, state=s)
+        assert st == 0
+        j, gs, _, dk, _ = gpu_adjoint(fxmod, pb, s, 2, 1)
+        got.append((state, gs))
+        J.append((j, dk))
+    np.testing.assert_array_equal(got[0][0], got[1][0])
+    # (the adjoint's atomic sums come in any order)
+    np.testing.assert_allclose(got[0][1], got[1][1], rtol=0.0, atol=(1e-13 if precision == "fp64" else 1e-5) * np.max(np.abs(got[0][1])))
+    np.testing.assert_allclose(J[0], J[1], rtol=1e-12 if precision == "fp64" else 1e-5)
