@@ -740,7 +740,6 @@ StageArgs<R> stage_args(fx_grid* h) {
   a.ptab.n = 2 * h->ptab_nu * ((h->P.ngroups + 1) / 2);
   a.ptab.status = a.status;
   a.n_state = h->ncell * h->NV;
-  a.n_faces = h->faces_elems;
   a.n_recs = h->n_recs;
 #endif
   a.chunk = h->chunk;
@@ -1222,7 +1221,8 @@ fx_status fx_grid_create(const fx_params* params, fx_grid** out, size_t* workspa
   h->ncell = 1;
   for (int d = 0; d < P.dims; ++d) h->ncell *= P.n[d];
   h->elem = P.precision == FX_FP64 ? 8 : 4;
-  // kernels index the state and the gas face buffer with 32-bit element offsets
+  // kernels index the state, and each direction's block of the gas face buffer (at most 2 D + 2 rows of
+  // faces, of which there are 5/4 per cell or fewer), with 32-bit element offsets
   if ((double)h->ncell * h->NV >= 4294967295.0 || (double)h->ncell * (3 + P.dims) * P.dims * 1.01 >= 4294967295.0) {
     delete h;
     return FX_ERR_UNSUPPORTED;

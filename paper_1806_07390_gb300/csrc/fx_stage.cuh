@@ -111,9 +111,8 @@ template <class R> struct StageArgs {
   PlanckParams pk;
   unsigned* status;
 #ifdef FX_BOUNDS_CHECK
-  int64_t n_state;     // elements of a state (in, base, out, pre_out) and of the gas face buffer,
-  int64_t n_faces;     // and faces in frec, for the index checks of the debug build
-  int64_t n_recs;
+  int64_t n_state;     // elements of a state (in, base, out, pre_out) and faces in frec, for the index
+  int64_t n_recs;      // checks of the debug build
 #endif
   double dt;           // stage step
   double dts;          // coupling step (dt after stage 1, dt/2 after stage 2; reading R10)
@@ -594,7 +593,8 @@ __device__ __forceinline__ void gas_update(const StageArgs<R>& A, uint32_t cid) 
   const uint32_t fl[3] = {((uint32_t)gz * ny + gy) * (nx + 1) + gx, ((uint32_t)gz * (ny + 1) + gy) * nx + gx, cid};
   const uint32_t fs[3] = {1u, (uint32_t)nx, (uint32_t)nx * ny};  // to the upper face
   auto face = [&](int d, int v, uint32_t f) -> R {
-    return __ldg(FXP(A.faces, (uint32_t)A.face_off[d] + v * nfd[d] + f, A.n_faces));
+    const R* const fr = A.faces + A.face_off[d];  // (64 bits: the blocks before this one may hold 2^32 elements)
+    return __ldg(FXP(fr, v * nfd[d] + f, (NG + 1 + (g.vterms ? D - 1 : 0)) * nfd[d]));
   };
   R u0[NG];
 #pragma unroll

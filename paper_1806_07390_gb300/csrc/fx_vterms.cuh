@@ -175,7 +175,7 @@ __device__ __forceinline__ void vt_gradient(const StageArgs<R>& A, int ix, int i
     const uint32_t nf = ex * ey * (uint32_t)(g.n[2] + (j == 2));
     const uint32_t lf = ((uint32_t)iz * ey + (uint32_t)iy) * ex + (uint32_t)ix;
     const uint32_t uf = lf + (j == 0 ? 1u : (j == 1 ? ex : ex * ey));
-    const R* fr = A.faces + (uint32_t)A.face_off[j];
+    const R* fr = A.faces + A.face_off[j];
     const uint32_t nfr = (uint32_t)(NG + D) * nf;  // this direction's block (fluxes, v*, D-1 velocities)
     (void)nfr;
 #pragma unroll

@@ -71,7 +71,7 @@ __global__ void __launch_bounds__(256) comp_kernel(const __grid_constant__ Stage
     const uint32_t nf = ex * ey * (uint32_t)(n2 + (d == 2));
     const uint32_t lf = ((uint32_t)iz * ey + (uint32_t)iy) * ex + (uint32_t)ix;
     const uint32_t uf = lf + (d == 0 ? 1u : (d == 1 ? ex : ex * ey));
-    const R* fr = A.faces + (uint32_t)A.face_off[d];
+    const R* fr = A.faces + A.face_off[d];
     const uint32_t nfr = (uint32_t)(NG + 1 + (g.vterms ? D - 1 : 0)) * nf;  // this direction's block
     (void)nfr;
     const R mlo = fr[FXI(lf, nfr)], mhi = fr[FXI(uf, nfr)];

@@ -129,3 +129,31 @@ def test_step_and_gradient_do_not_depend_on_the_origin(fxmod, shape, G, precisio
     # (the adjoint's atomic sums come in any order)
     np.testing.assert_allclose(got[0][1], got[1][1], rtol=0.0, atol=(1e-13 if precision == "fp64" else 1e-5) * np.max(np.abs(got[0][1])))
     np.testing.assert_allclose(J[0], J[1], rtol=1e-12 if precision == "fp64" else 1e-5)
+
+
+def test_face_buffer_past_32_bit_offsets(fxmod):  # noqa: F811
+    # 3-d with the velocity terms: the face buffer's third direction begins past 2^32 elements on the largest
+    # grids that are accepted (236e6 cells; 71 GB here).  A state of period 8 along z steps like the small
+    # grid of one period.
+    import torch
+    pb, s = random_case((4, 24, 8), 1, "fp32", steps=1, vterms=1)
+    pb.bc_lo, pb.bc_hi = ("reflect", "outflow", "periodic"), ("outflow", "reflect", "periodic")
+    pb.dt = 0.3 / 24 / pb.c_light
+    pb.x_lo, pb.x_hi = (0.0,) * 3, (1.0, 1.0, 1.0)
+    ref, st, _ = run_gpu(fxmod, pb, state=s)
+    assert st == 0
+    reps = 306875
+    pb.n, pb.x_hi = (4, 24, 8 * reps), (1.0, 1.0, float(reps))
+    assert 8 * (5 * 24 + 4 * 25) * 8 * reps >= 2 ** 32
+    fields = torch.from_numpy(s.astype(np.float32)).cuda().reshape(9, 1, -1)
+    g = fxmod.Grid(pb)
+    state = fields.expand(9, reps, fields.shape[2]).contiguous().reshape(-1)
+    g.upload(state)
+    g.step(pb.dt, 1)
+    assert g.status() == 0
+    g.download(state)
+    g.close()
+    out, want = state.reshape(9, reps, -1), torch.from_numpy(ref).cuda().to(torch.float32).reshape(9, -1)
+    for v in range(9):
+        scale = float(want[v].abs().max())
+        assert float((out[v] - want[v]).abs().max()) <= 1e-5 * scale, v
