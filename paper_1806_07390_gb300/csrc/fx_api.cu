@@ -387,10 +387,6 @@ void planck_coefficients(PlanckParams& pk) {
     pk.c64.wd[m - 1] = b[2 * m];
   }
   for (int n = 1; n <= NPLANCK_UP; ++n) pk.c64.rn[n - 1] = 1.0 / n;
-  for (int m = 1; m <= NPLANCK_LO32; ++m) {
-    pk.lo32[m - 1] = (float)pk.c64.lo[m - 1];
-    pk.wd32[m - 1] = (float)pk.c64.wd[m - 1];
-  }
 }
 
 // Host FP64 Planck integrals for the FP32 band tables: D(x) = Int_0^x (Bernoulli series in

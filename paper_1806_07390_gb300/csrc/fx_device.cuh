@@ -431,34 +431,6 @@ __device__ __forceinline__ PlanckEdge<double> planck_edge_tab(double x16, const 
   return e;
 }
 
-// FP32 edge evaluation (Newton iterations of the FP32 form).
-__device__ __forceinline__ PlanckEdge<float> planck_edge32(float x, const float* lo32, const float* wd32) {
-  PlanckEdge<float> e;
-  if (x < float(XSPLIT)) {
-    float x2 = x * x, x3 = x2 * x;
-    float sd = lo32[NPLANCK_LO32 - 1], sw = wd32[NPLANCK_LO32 - 1];
-#pragma unroll
-    for (int m = NPLANCK_LO32 - 2; m >= 0; --m) { sd = fmaf(sd, x2, lo32[m]); sw = fmaf(sw, x2, wd32[m]); }
-    e.Q = x3 * (1.0f / 3.0f - 0.125f * x + x2 * sd);
-    e.w = x3 * (1.0f - 0.5f * x + x2 * sw);
-    e.upper = false;
-  } else {
-    float y = __expf(-x), yn = y, x2 = x * x, x3 = x2 * x, s = 0.0f;
-    const float a2 = 3.0f * x2, a1 = 6.0f * x;
-    for (int n = 1; n <= 16; ++n) {
-      float rn = __frcp_rn((float)n);
-      float t = yn * rn * (x3 + rn * (a2 + rn * (a1 + 6.0f * rn)));
-      s += t;
-      if (t <= 3e-8f * s) break;
-      yn *= y;
-    }
-    e.Q = s;
-    e.w = __fdividef(x3 * x * y, 1.0f - y);
-    e.upper = true;
-  }
-  return e;
-}
-
 // Band integral Int_{x_lo}^{x_hi} t^3/(e^t-1) dt from the two edge evaluations.
 template <class R>
 __device__ __forceinline__ R planck_band(const PlanckEdge<R>& lo, const PlanckEdge<R>& hi) {

@@ -80,11 +80,8 @@ __device__ __forceinline__ float vmin(float a, float b) { return fminf(a, b); }
 __device__ __forceinline__ F2 vmin(F2 a, F2 b) { return F2(fminf(a.x, b.x), fminf(a.y, b.y)); }
 __device__ __forceinline__ float vmax(float a, float b) { return fmaxf(a, b); }
 __device__ __forceinline__ F2 vmax(F2 a, F2 b) { return F2(fmaxf(a.x, b.x), fmaxf(a.y, b.y)); }
-__device__ __forceinline__ float vabs(float a) { return fabsf(a); }
-__device__ __forceinline__ F2 vabs(F2 a) { return F2(fabsf(a.x), fabsf(a.y)); }
 __device__ __forceinline__ double vmin(double a, double b) { return fmin(a, b); }
 __device__ __forceinline__ double vmax(double a, double b) { return fmax(a, b); }
-__device__ __forceinline__ double vabs(double a) { return fabs(a); }
 // The limited difference of the MC limiter from the one-sided differences dl, dr and the centred
 // one q: the least of m|dl|, m|dr| and |q| with their common sign, zero where the signs of dl and dr
 // differ or one is zero (q has their sign where they agree).  In FP32 three instructions per value:
@@ -117,22 +114,6 @@ __device__ __forceinline__ F2 vpair(float a, float b, F2) { return F2(a, b); }
 __device__ __forceinline__ float vget(float x, int) { return x; }
 __device__ __forceinline__ double vget(double x, int) { return x; }
 __device__ __forceinline__ float vget(F2 x, int j) { return j ? x.y : x.x; }
-
-// Shared-memory access of the values of a lane's groups at p (the lane's first group): one
-// value, or (F2) the two values at p[0], p[1] with one 8-byte access (p 8-byte aligned).  The
-// store writes only the groups that exist (h0, h1).
-__device__ __forceinline__ float ld_lane(const float* p, float) { return *p; }
-__device__ __forceinline__ double ld_lane(const double* p, double) { return *p; }
-__device__ __forceinline__ F2 ld_lane(const float* p, F2) {
-  const float2 v = *reinterpret_cast<const float2*>(p);
-  return F2(v.x, v.y);
-}
-__device__ __forceinline__ void st_lane(float* p, float v, bool h0, bool) { if (h0) *p = v; }
-__device__ __forceinline__ void st_lane(double* p, double v, bool h0, bool) { if (h0) *p = v; }
-__device__ __forceinline__ void st_lane(float* p, F2 v, bool h0, bool h1) {
-  if (h1) *reinterpret_cast<float2*>(p) = make_float2(v.x, v.y);
-  else if (h0) *p = v.x;
-}
 
 // Global load of a lane's groups: one 8-byte load where the pair is aligned (vec), else one by one
 // (an absent second group is zero).

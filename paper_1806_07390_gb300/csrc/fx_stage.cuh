@@ -39,8 +39,6 @@ template <class T> struct Consts {
 struct PlanckParams {
   PlanckCoef c64;
   const double* petab;  // FP64 edge table (fx_planck.h) in device memory; null in the FP32 forms
-  float lo32[NPLANCK_LO32];
-  float wd32[NPLANCK_LO32];
 };
 
 // FP32 Planck band tables on nodes u0 + i/PTAB_PER_OCT of u = log2 T: per group and interval [i, i+1]
