@@ -36,11 +36,11 @@ UNIT = "zone-group-stages/s"
 # interaction kernel, from the committed ncu capture profiles/traffic_kh2d_1024x1024x16.txt; None
 # where not captured for the current kernels.
 TRAFFIC_PER_LAUNCH = {"kh2d": {"fp32n64": 602.1e6}}
-TRAFFIC_INTERACTION = {"kh2d": {"fp32n64": 371.5e6}}
+TRAFFIC_INTERACTION = {"kh2d": {"fp32n64": 371.4e6}}
 # FP64 lane operations (DFMA + DADD + DMUL thread instructions) per zone-group of the FP64 form's
 # radiation/update and interaction kernels, from the committed ncu capture
 # profiles/fp64_pipe_kh2d_512x512x16.txt (kh2d recipe at 512 x 512 cells x 16 groups).
-FP64_OPS_PER_ZG = {"kh2d": {"stage": 224.4, "interaction": 110.0}}
+FP64_OPS_PER_ZG = {"kh2d": {"stage": 224.4, "interaction": 110.2}}
 
 
 def load_peaks():
@@ -492,7 +492,7 @@ def main():
             # the interaction kernel reads and writes the state once per stage
             cb = 2.0 * b * nv * pbh.ncell
             out["interaction_kernel"] = {
-                "kernel": "couple_kernel / couple64_kernel (interaction, one thread per cell)",
+                "kernel": "couple_kernel / couple64_kernel (interaction)",
                 "bytes_per_launch": cb, "avg_launch_ms": cs * 1e3, "achieved": cb / cs / 1e9,
                 "frac": cb / cs / 1e9 / peak, "share_of_step": kt["couple_ms"] / total,
                 "traffic": TRAFFIC_INTERACTION.get(args.workload, {}).get(kind)}

@@ -378,8 +378,8 @@ __device__ __forceinline__ R parabola_form(const Tab<R>& t, int ip, bool up, R p
 //   adj_gas_kernel   one thread per face.
 // A block, or a face of the gas kernel, whose flux adjoints all vanish is done at once: the objective sits on
 // one boundary, so after n steps back only its neighbourhood has any.  Bound by the FP64 pipe where all
-// faces have adjoints and by the latency of a block's chains on small grids (128 x 96 x 8 FP64: 60 and
-// 43 us per launch).  One thread per face that looped over the groups and carried the tangents of
+// faces have adjoints and by the latency of a block's chains on small grids (128 x 96 x 8 FP64: 61 and
+// 42 us per launch).  One thread per face that looped over the groups and carried the tangents of
 // both sides in forward mode held 255 registers, kept the pipe half busy and took 287 us; the two kernels
 // without the early end and with HLLC in forward mode took 96 and 94 us.  Radiation blocks of 256
 // threads take 76 us (the few busy blocks crowd some multiprocessors), of 64 threads 61 (as long: the

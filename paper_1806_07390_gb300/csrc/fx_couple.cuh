@@ -156,9 +156,10 @@ struct RowCopy {
 // The groups run in pairs (packed FP32 arithmetic, fx_pair.cuh): an odd count's last pair carries a
 // group of zero energy and zero opacity, which changes nothing.  Bound by latency (the table words,
 // shared rows and FP64 steps of a cell's chain; FP64 pipe 40 %, DRAM 35 % busy), so seven resident
-// blocks at 72 registers: 1024^2 x 16 0.118 ms, against 0.123 with six and 0.116 with eight, where
-// 256^3 x 12 loses 6 %.  With two table words per group, scalar rows and divisions in the copies and
-// powers, 0.133 ms; 256^3 x 12 3.31 -> 2.52 ms, 75 x 61 x 50 x 20 0.129 -> 0.092 ms.
+// blocks at 72 registers (at 0.118 ms for 1024^2 x 16, six took 0.123 and eight 0.116, where 256^3 x 12
+// loses 6 %).  With two table words per group, scalar rows, divisions in the copies and powers and FP64
+// comparisons, 1024^2 x 16 took 0.133 ms, now 0.111; 256^3 x 12 3.31 -> 2.45 ms, 75 x 61 x 50 x 20 0.129 ->
+// 0.091 ms.
 template <int D, class NT>
 __global__ void __launch_bounds__(CPL_THREADS, 7) couple_kernel(const __grid_constant__ StageArgs<float> A) {
   using LT = float;

@@ -9,7 +9,7 @@
 // decisions are medians and selects over values computed for every cell (in FP64 by integer
 // comparisons), a Cartesian direction's coefficients are one constant row of the launch
 // arguments, and HLLC's eleven divisions are six shared reciprocals.  Per launch: 1024^2 FP32 0.079
-// -> 0.050 ms, 256^3 FP32 2.04 -> 1.31 ms, 512^2 FP64 0.42 -> 0.33 ms.
+// -> 0.049 ms, 256^3 FP32 2.04 -> 1.26 ms, 512^2 FP64 0.42 -> 0.32 ms.
 // The stage kernel then uses the fluxes for the gas divergence; with the velocity-dependent radiation
 // terms on, the kernel also stores each face's transverse velocity for their velocity gradient
 // (fx_vterms.cuh).

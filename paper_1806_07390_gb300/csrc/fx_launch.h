@@ -86,9 +86,8 @@ inline void fit_tile(const int* n, int G, int nsm, int regs, RadTile& best, int&
 // Enqueue one stage (state type R, D dimensions, Newton/bookkeeping type NT; SPH: the 2-d
 // spherical grid) on stream s: the gas face kernel, the radiation/update kernel, with the
 // velocity-dependent terms on the velocity-term kernel, and with the interaction on the
-// interaction kernel (one thread per cell).  When non-null, `mid` is recorded after the
-// face kernel and `mid2` after the radiation/update kernel (per-kernel timing).  Returns the CUDA
-// error of the launches.
+// interaction kernel.  When non-null, `mid` is recorded after the face kernel and `mid2` after the
+// radiation/update kernel (per-kernel timing).  Returns the CUDA error of the launches.
 template <class R, int D, class NT, bool SPH>
 cudaError_t launch_stage(const StageArgs<R>& a, cudaStream_t s, cudaEvent_t mid,
                          cudaEvent_t mid2);
@@ -178,7 +177,7 @@ cudaError_t launch_stage(const StageArgs<R>& a0, cudaStream_t s, cudaEvent_t mid
     }
     return cudaGetLastError();
   }
-  // the interaction, one thread per cell (FP32 state: couple_kernel; FP64 state: couple64_kernel)
+  // the interaction (FP32 state: couple_kernel, one thread per cell; FP64 state: couple64_kernel, 1 to 16)
   if (a.g.couple) {
     if constexpr (std::is_same<R, float>::value) {
       auto ck = couple_kernel<D, NT>;

@@ -1,9 +1,9 @@
 // SSP-RK2 stage kernel: explicit transport (reconstruction, M1/HLL radiation fluxes, flux divergence
 // of gas and radiation) + RK combine in one pass over HBM.  The gas faces run before it
 // (gas_face_kernel, fx_gas.cuh) and the cell-local implicit interaction after it, as kernels of
-// their own, one thread per cell (couple_kernel in fx_couple.cuh for the FP32 state,
-// couple64_kernel in fx_couple64.cuh for the FP64 state).  Ghost cells are index maps applied when
-// cells are loaded (Sec. 7.5): no separate ghost-fill pass touches HBM.
+// their own (couple_kernel in fx_couple.cuh for the FP32 state, one thread per cell; couple64_kernel in
+// fx_couple64.cuh for the FP64 state, 1 to 16).  Ghost cells are index maps applied when cells are
+// loaded (Sec. 7.5): no separate ghost-fill pass touches HBM.
 #pragma once
 #include <type_traits>
 
@@ -427,13 +427,14 @@ __device__ __forceinline__ void cp_async16(void* s, const void* g) {
 // blocks of the grid do it, one thread per cell, in the slots that the radiation blocks leave free
 // and as they finish (no launch of its own, and no gas variables in the radiation blocks).
 //
-// Bound by instruction issue and by the latency between the plane barriers (1024^2 x 16: about 700
-// instructions per warp and plane, issued in 66 % of cycles at 20 warps per multiprocessor; 256^3 x
-// 12: 1355 in 58 % at 16 warps; DRAM 1.0x the algorithmic bytes), the FP64 state by the FP64 pipe (86
+// Bound by instruction issue and by the latency between the plane barriers (1024^2 x 16: 351 thread
+// instructions per cell and group, issued in 66 % of cycles at 20 warps per multiprocessor; 128^3 x 12:
+// 690 in 57 % at 16 warps; DRAM 1.1x the algorithmic bytes), the FP64 state by the FP64 pipe (87
 // % busy, 224 operations per cell and group).  Measured (FP32 state unless noted, one launch):
-// 1024^2 x 16 groups 0.455 -> 0.234 ms, 256^3 x 12 16.4 -> 6.2 ms, 640 x 128 x 20 spherical 0.124 ->
-// 0.050 ms, 512^2 x 24 channels 0.23 -> 0.094 ms, 512^2 x 16 FP64 2.99 -> 1.86 ms, against one kernel
+// 1024^2 x 16 groups 0.455 -> 0.241 ms, 256^3 x 12 16.4 -> 6.6 ms, 640 x 128 x 20 spherical 0.124 ->
+// 0.047 ms, 512^2 x 24 channels 0.23 -> 0.098 ms, 512^2 x 16 FP64 2.99 -> 1.84 ms, against one kernel
 // with lanes padded to a power of two, geometry tables on every grid, and the gas update in its lanes.
+// (The variants below were measured while the divergence took the shorter sum that net_update names.)
 //
 // Block sizes (StageCap).  A thread holds about 90 values at order 1, so 20 warps of 96 registers in
 // 2-d (4 blocks of 160: 2 of 256 0.244 ms, 3 of 160 0.229 ms but the 24-channel and 400 x 300 grids
@@ -540,8 +541,8 @@ template <int D, class V> __device__ __forceinline__ V m1_c2perp(const LaneConst
 // FMA, the directions are added by TwoSum, and the errors of all three are summed beside (ml, the negated
 // sum of what the high part n has lost) and join it at the end, so that directions that cancel leave no
 // rounding of their parts.  Without the errors of the products and of the sum over directions, and with
-// Dekker's shorter difference, a step of 1024^2 x 16 groups took 0.82 ms instead of 0.86, of 256^3 x 12
-// 10.96 instead of 11.36, but left 1e-7 of the parts where the directions cancel, which this sum does not.
+// Dekker's shorter difference, the kernel took 229 us instead of 241 at 1024^2 x 16 groups and 6.24 ms
+// instead of 6.57 at 256^3 x 12, but left 1e-7 of the parts where the directions cancel.
 template <int D>
 __device__ __forceinline__ F2 net_update(F2 xp, F2 xm, F2 yp, F2 ym, F2 mp, F2 mm, const F2* h, const F2* mh) {
   F2 s, e;

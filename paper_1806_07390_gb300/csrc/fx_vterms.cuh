@@ -147,8 +147,9 @@ inline void vt_constants(const double* edge, int G, VtConst& v) {
 // V_ij into max(V_ij, 0) and min(V_ij, 0), adds the pairs that share a symmetric component, and
 // contracts them with the lower-edge values and with the values below the edge, without selects.
 //
-// Bound by instruction issue (63 % of cycles).  768^2 x 16 groups 0.135 -> 0.104 ms per launch, against one kernel with the
-// closure's reciprocals in chi, a select per component pair and lanes padded to a power of two.
+// Bound by instruction issue (63 % of cycles).  768^2 x 16 groups 0.125 -> 0.104 ms per launch, against a
+// kernel with the closure's reciprocals in chi, a select per component pair and lanes padded to a power of
+// two.
 //
 // SPH: the 2-d spherical (r, theta) grid.  The tensors are those of 3 dimensions (DT = 3, with
 // F_phi = 0 and the V_phiphi entry), in physical components: the state's covariant flux
