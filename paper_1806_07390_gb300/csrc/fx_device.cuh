@@ -108,10 +108,14 @@ __device__ __forceinline__ double median(double x, double u, double v) {
 }
 __device__ __forceinline__ float min_fast(float a, float b) { return fminf(a, b); }
 __device__ __forceinline__ float max_fast(float a, float b) { return fmaxf(a, b); }
-__device__ __forceinline__ double min_fast(double a, double b) { return less64(a, b) ? a : b; }
-__device__ __forceinline__ double max_fast(double a, double b) { return less64(a, b) ? b : a; }
+// (as fmin and fmax, the other operand where one is NaN: the sound speed of a state with negative pressure.
+// The result of an operation, whose NaN is a quiet one, is told by its high word.)
+__device__ __forceinline__ bool nan64(double a) { return ((unsigned)__double2hiint(a) << 1) > 0xffe00000u; }
+__device__ __forceinline__ double min_fast(double a, double b) { return nan64(b) || (less64(a, b) && !nan64(a)) ? a : b; }
+__device__ __forceinline__ double max_fast(double a, double b) { return nan64(a) || (less64(a, b) && !nan64(b)) ? b : a; }
+// a >= 0 (false for NaN)
 __device__ __forceinline__ bool nonneg(float a) { return a >= 0.0f; }
-__device__ __forceinline__ bool nonneg(double a) { return __double2hiint(a) >= 0 || !nonzero64(a); }
+__device__ __forceinline__ bool nonneg(double a) { return (unsigned)__double2hiint(a) <= 0x7ff00000u || !nonzero64(a); }
 // 1/x and sqrt(x) of any argument: the short forms on the normal range, the library's outside it
 __device__ __forceinline__ float rcp_any(float x) { return rcp_approx(x); }
 __device__ __forceinline__ double rcp_any(double x) {
