@@ -439,8 +439,8 @@ void build_planck_table(const fx_params& P, const GroupConst& gc, const PlanckPa
         L = std::log2(I);
         m = h * (host_w(a) - host_w(b)) / I;  // h dL/du, L = log2 I, u = log2 T
       } else {
-        L = -200.0;
-        m = -h * a;  // the band underflows in FP32 here; keep the table smooth and negative
+        L = -200.0;  // the band underflows in FP32 here (scale 0): a flat table, so that no interval
+        m = 0.0;     // between two such nodes rises to an infinite power, which times 0 is NaN
       }
       const double k = std::floor(L);
       // 2^floor(L), exact in FP32 down to the smallest normal number (0 below, where the band

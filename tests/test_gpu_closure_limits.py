@@ -73,3 +73,22 @@ def test_cells_with_negative_pressure(fxmod, shape, solver, precision, part):  #
         H.assert_parity(pb, got, ref, FP64_L1, FP64_MAX)
     else:
         H.assert_parity(pb, got, ref, 1e-4, natural=True)
+
+
+# Gas far colder than the upper groups' band edges (eps/T up to 1e6): their Planck energies are 0 in FP32.
+# The radiation heats it by several orders of magnitude within the step.
+@pytest.mark.parametrize("precision", ["fp64", "fp32", "fp32n64"])
+@pytest.mark.parametrize("G", [1, 15, 16])
+def test_gas_far_below_the_groups(fxmod, G, precision):  # noqa: F811
+    pb, prim = W.kh_2d(nx=24, ny=20, ngroups=G, nsteps=2, precision=precision)
+    prim = np.array(prim)
+    prim[1] = prim[0] * 10.0 ** np.random.default_rng(4).uniform(-5.0, -3.0, pb.ncell)
+    prim[-1] = 0.3
+    ref, rst = run_oracle(pb, prim)
+    assert np.all(np.isfinite(ref)) and rst == 0
+    got, st, _ = run_gpu(fxmod, pb, prim)
+    assert np.all(np.isfinite(got)) and st == 0
+    if precision == "fp64":
+        H.assert_parity(pb, got, ref, FP64_L1, FP64_MAX)
+    else:
+        H.assert_parity(pb, got, ref, 1e-4, natural=True)
