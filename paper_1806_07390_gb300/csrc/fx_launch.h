@@ -14,6 +14,8 @@
 
 namespace fx {
 
+constexpr int STAGE_SMEM_MAX = 200 * 1024;  // most dynamic shared memory of a stage kernel block
+
 // Tile and march chunk of the stage kernel for a grid, fitted to the device.  A model of its time
 // over every tile that the kernel's capacities allow and every chunk length picks the least:
 //   waves x ((chunk + 2) x (time of one plane) + start), two planes being the prologue's share,
@@ -55,7 +57,7 @@ inline void fit_tile(const int* n, int G, int nsm, int regs, RadTile& best, int&
       // copies past the ones whose offsets a thread keeps
       const int late = std::max(0, tile_halo<D>(t) * gl - (D == 3 ? 2 : 1) * t.nth) + std::max(0, tile_recs<D>(t) - 2 * t.nth);
       const size_t smem = stage_smem_bytes<R, D>(t);
-      if (smem > 200 * 1024) continue;
+      if (smem > STAGE_SMEM_MAX) continue;
       const int rmax = std::max(1, std::min({65536 / (regs * t.nth), (int)(227 * 1024 / (smem + 1024)), 2048 / t.nth, 32}));
       const double instr = t.nth / 32 * own + (2 * nt + 31) / 32 * (recon + 30.0) + (nt + 31) / 32 * (flux + 30.0) + (late + 31) / 32 * 60.0;
       const double tiles = (double)t.ntx * t.nty;
@@ -113,7 +115,9 @@ cudaError_t launch_stage(const StageArgs<R>& a0, cudaStream_t s, cudaEvent_t mid
               : a.budget_bnd     ? (a.rt.vec ? stage_kernel<R, D, SPH, 1, true, PV> : stage_kernel<R, D, SPH, 1, true, false>)
                                  : (a.rt.vec ? stage_kernel<R, D, SPH, 1, false, PV> : stage_kernel<R, D, SPH, 1, false, false>);
   const size_t smem = stage_smem_bytes<R, D>(a.rt);
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  // (a function's limit is the process's: it is set to the same value by every handle, the most that any
+  // needs, so that handles of other threads cannot lower it between this call and the launch)
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, STAGE_SMEM_MAX);
   if (e != cudaSuccess) return e;
   e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout,
                            cudaSharedmemCarveoutMaxShared);
@@ -167,11 +171,11 @@ cudaError_t launch_stage(const StageArgs<R>& a0, cudaStream_t s, cudaEvent_t mid
     const bool f32 = std::is_same<R, float>::value;
     const size_t cs = f32 ? couple_ye32_smem_bytes<D>(a.g.G) : couple_ye_smem_bytes(a.g.G);
     if constexpr (f32) {
-      e = cudaFuncSetAttribute(couple_ye32_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cs);
+      e = cudaFuncSetAttribute(couple_ye32_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)couple_ye32_smem_bytes<D>(MAXG));
       if (e != cudaSuccess) return e;
       couple_ye32_kernel<D><<<(unsigned)((a.g.ncell + CPL_THREADS - 1) / CPL_THREADS), CPL_THREADS, cs, s>>>(a);
     } else {
-      e = cudaFuncSetAttribute(couple_ye_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cs);
+      e = cudaFuncSetAttribute(couple_ye_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)couple_ye_smem_bytes(MAXG));
       if (e != cudaSuccess) return e;
       couple_ye_kernel<D><<<(unsigned)((a.g.ncell + CPLYE_THREADS - 1) / CPLYE_THREADS), CPLYE_THREADS, cs, s>>>(a);
     }
@@ -182,7 +186,7 @@ cudaError_t launch_stage(const StageArgs<R>& a0, cudaStream_t s, cudaEvent_t mid
     if constexpr (std::is_same<R, float>::value) {
       auto ck = couple_kernel<D, NT>;
       const size_t cs = couple_smem_bytes<D>(a.g.G);
-      e = cudaFuncSetAttribute(ck, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cs);
+      e = cudaFuncSetAttribute(ck, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)couple_smem_bytes<D>(MAXG));
       if (e != cudaSuccess) return e;
       const unsigned nb = (unsigned)((a.g.ncell + CPL_THREADS - 1) / CPL_THREADS);
       ck<<<nb, CPL_THREADS, cs, s>>>(a);
@@ -194,7 +198,7 @@ cudaError_t launch_stage(const StageArgs<R>& a0, cudaStream_t s, cudaEvent_t mid
                 : lanes == 8 ? couple64_kernel<D, 8>
                              : couple64_kernel<D, 16>;
       const size_t cs = couple64_smem_bytes<D>(a.g.G, cells);
-      e = cudaFuncSetAttribute(ck, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cs);
+      e = cudaFuncSetAttribute(ck, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)couple64_smem_bytes<D>(MAXG, CPL64_THREADS));
       if (e != cudaSuccess) return e;
       ck<<<(unsigned)((a.g.ncell + cells - 1) / cells), CPL64_THREADS, cs, s>>>(a);
     }

@@ -4,6 +4,8 @@ fx_step replays one captured CUDA graph per step unless per-kernel timing or the
 on; with timing on it launches the kernels one by one.  Both must give the same state bit for
 bit, on a grid with boundary layers (their time advances on the device), on the three-species
 form with the velocity terms and the budgets, and across a change of dt (a new capture).
+
+Handles of several threads, each on a stream of its own, step as they do alone.
 """
 import numpy as np
 import pytest
@@ -66,3 +68,45 @@ def test_graph_replay_three_species_with_budgets(fxmod, precision):
     assert sa == 0 and sb == 0
     assert np.array_equal(a, b)
     np.testing.assert_allclose(ba, bb, rtol=1e-12, atol=1e-300)  # (atomic sums: order may differ)
+
+
+@pytest.mark.parametrize("direct", [False, True])
+@pytest.mark.parametrize("precision", ["fp32n64", "fp64"])
+def test_handles_of_several_threads(fxmod, precision, direct):
+    # grids whose kernels are the same functions with other amounts of shared memory
+    import threading
+
+    import torch
+    jobs = [W.kh_2d(nx=nx, ny=ny, ngroups=G, precision=precision) for nx, ny, G in
+            [(64, 64, 16), (40, 36, 3), (96, 80, 31), (21, 90, 32)]]
+
+    def step(pb, prim, stream):
+        g = fxmod.Grid(pb, stream=stream)
+        g.init_equilibrium(prim)
+        g.kernel_timing(direct)
+        for _ in range(40):
+            g.step(pb.dt, 1)
+        st, out = g.status(), g.download()
+        g.close()
+        return st, out
+
+    alone = [step(pb, prim, None) for pb, prim in jobs]
+    assert all(st == 0 for st, _ in alone)
+    found = [None] * len(jobs)
+
+    def work(k):
+        try:
+            stream = torch.cuda.Stream()
+            with torch.cuda.stream(stream):
+                for _ in range(5):
+                    st, out = step(*jobs[k], stream)
+                    assert st == 0 and np.array_equal(out, alone[k][1]), st
+        except Exception as e:  # (reported by the main thread)
+            found[k] = repr(e)
+
+    threads = [threading.Thread(target=work, args=(k,)) for k in range(len(jobs))]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert found == [None] * len(jobs), found
