@@ -10,6 +10,8 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <exception>
+#include <memory>
 #include <mutex>
 #include <string>
 #include <vector>
@@ -1166,7 +1168,9 @@ fx_status adjoint_impl(fx_grid* h, double dt, int nsteps, int k, unsigned char* 
 
 extern "C" {
 
-fx_status fx_grid_create(const fx_params* params, fx_grid** out, size_t* workspace_bytes) {
+// (No exception leaves the entry points: those that take host memory by the grid's size report that there
+// is none.)
+fx_status fx_grid_create(const fx_params* params, fx_grid** out, size_t* workspace_bytes) try {
   if (out) *out = nullptr;
   if (!params || !out || !workspace_bytes) return FX_ERR_ARG;
   const fx_params& P = *params;
@@ -1208,7 +1212,8 @@ fx_status fx_grid_create(const fx_params* params, fx_grid** out, size_t* workspa
   if (!(P.eps_min > 0.0) || !(P.eps_max > P.eps_min)) return FX_ERR_ARG;
   if (P.newton_maxit < 1 || P.bisect_maxit < 0 || !(P.newton_rtol > 0.0)) return FX_ERR_ARG;
   if (!(P.rho_floor > 0.0) || !(P.p_floor > 0.0) || !(P.E_floor > 0.0)) return FX_ERR_ARG;
-  fx_grid* h = new fx_grid();
+  std::unique_ptr<fx_grid> own(new fx_grid());
+  fx_grid* const h = own.get();
   h->P = P;
   h->D = P.dims;
   h->G = NCH;
@@ -1219,10 +1224,8 @@ fx_status fx_grid_create(const fx_params* params, fx_grid** out, size_t* workspa
   h->elem = P.precision == FX_FP64 ? 8 : 4;
   // kernels index the state, and each direction's block of the gas face buffer (at most 2 D + 2 rows of
   // faces, of which there are 5/4 per cell or fewer), with 32-bit element offsets
-  if ((double)h->ncell * h->NV >= 4294967295.0 || (double)h->ncell * (3 + P.dims) * P.dims * 1.01 >= 4294967295.0) {
-    delete h;
+  if ((double)h->ncell * h->NV >= 4294967295.0 || (double)h->ncell * (3 + P.dims) * P.dims * 1.01 >= 4294967295.0)
     return FX_ERR_UNSUPPORTED;
-  }
 
   DevGrid& g = h->dg;
   g.D = P.dims;
@@ -1339,8 +1342,10 @@ fx_status fx_grid_create(const fx_params* params, fx_grid** out, size_t* workspa
   h->off_layers = off; off = align_up(off + sizeof(LayerSet));
   h->ws_bytes = off;
   *workspace_bytes = off;
-  *out = h;
+  *out = own.release();
   return FX_OK;
+} catch (const std::exception&) {
+  return FX_ERR_UNSUPPORTED;
 }
 
 size_t fx_state_elems(const fx_grid* h) { return h ? (size_t)h->ncell * h->NV : 0; }
@@ -1583,7 +1588,7 @@ fx_status choose_tile(fx_grid* h) {
   return e == cudaSuccess ? FX_OK : cuda_fail(h, e, "stage kernel attributes");
 }
 
-fx_status fx_bind_workspace(fx_grid* h, void* dev_ptr, size_t bytes, void* cuda_stream) {
+fx_status fx_bind_workspace(fx_grid* h, void* dev_ptr, size_t bytes, void* cuda_stream) try {
   if (!h) return FX_ERR_ARG;
   if (!dev_ptr || bytes < h->ws_bytes || (reinterpret_cast<uintptr_t>(dev_ptr) % kAlign) != 0)
     return fail(h, FX_ERR_WORKSPACE, "workspace missing, too small or not 256-byte aligned");
@@ -1664,9 +1669,11 @@ fx_status fx_bind_workspace(fx_grid* h, void* dev_ptr, size_t bytes, void* cuda_
     if (e != cudaSuccess) return cuda_fail(h, e, "boundary layer upload");
   }
   return FX_OK;
+} catch (const std::exception&) {
+  return fail(h, FX_ERR_UNSUPPORTED, "out of host memory");
 }
 
-fx_status fx_state_upload(fx_grid* h, const void* src, int src_precision, int src_is_device) {
+fx_status fx_state_upload(fx_grid* h, const void* src, int src_precision, int src_is_device) try {
   if (!h || !src) return FX_ERR_ARG;
   if (h->sticky != FX_OK) return h->sticky;
   if (!has_ws(h)) return fail(h, FX_ERR_WORKSPACE, "no workspace bound");
@@ -1695,6 +1702,8 @@ fx_status fx_state_upload(fx_grid* h, const void* src, int src_precision, int sr
   }
   if (e != cudaSuccess) return cuda_fail(h, e, "state upload");
   return FX_OK;
+} catch (const std::exception&) {
+  return fail(h, FX_ERR_UNSUPPORTED, "out of host memory");
 }
 
 fx_status fx_state_init_equilibrium(fx_grid* h, const double* prim, int prim_is_device) {
@@ -1784,7 +1793,7 @@ fx_status fx_conserved_totals(fx_grid* h, double out[FX_NTOTALS]) {
   return FX_OK;
 }
 
-fx_status fx_state_download(fx_grid* h, void* dst, int dst_precision, int dst_is_device) {
+fx_status fx_state_download(fx_grid* h, void* dst, int dst_precision, int dst_is_device) try {
   if (!h || !dst) return FX_ERR_ARG;
   if (!has_ws(h)) return fail(h, FX_ERR_WORKSPACE, "no workspace bound");
   const int64_t n = (int64_t)h->ncell * h->NV;
@@ -1816,6 +1825,8 @@ fx_status fx_state_download(fx_grid* h, void* dst, int dst_precision, int dst_is
   }
   if (e != cudaSuccess) return cuda_fail(h, e, "state download");
   return FX_OK;
+} catch (const std::exception&) {
+  return fail(h, FX_ERR_UNSUPPORTED, "out of host memory");
 }
 
 const char* fx_last_error(const fx_grid* h) { return h ? h->err.c_str() : "null handle"; }

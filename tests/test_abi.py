@@ -288,3 +288,25 @@ def test_cartesian_table_rows_are_one_row(L, n, x_lo):
         for e, v in want.items():
             assert abs(T[e, 0] - v) <= 4e-15 * abs(v) + abs(h_d - w) * abs(v) / w, (e, T[e, 0], v)
     L.fx_grid_destroy(h)
+
+
+def test_a_grid_beyond_the_host_memory_is_refused(L):
+    # 4e8 cells in 1-d are within the index range, but their reconstruction table takes 134 GB on the host: with
+    # 16 GB of address space the library reports it, and no exception ends the process
+    import subprocess
+    import sys
+    code = """
+import ctypes, resource
+from paper_1806_07390_gb300 import fx, workloads as W
+pb, _ = W.sod_1d(n=16, ngroups=1, precision="fp32")
+L = fx.lib()
+resource.setrlimit(resource.RLIMIT_AS, (1 << 34, 1 << 34))
+def create(n):
+    pb.n = (n, 1, 1)
+    P, h, ws = fx.params(pb), ctypes.c_void_p(), ctypes.c_size_t()
+    return L.fx_grid_create(ctypes.byref(P), ctypes.byref(h), ctypes.byref(ws)), h.value
+print(create(400_000_000), create(16)[0])
+"""
+    r = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True, cwd=ROOT, timeout=120)
+    assert r.returncode == 0, r.stderr[-400:]
+    assert r.stdout.split("\n")[0] == "(-7, None) 0"
