@@ -275,9 +275,9 @@ int fx_march_chunk(const fx_grid* h);
 
 /* Per-kernel device timing (instrumentation, not part of the method).  While enabled, every
  * stage that fx_step enqueues records four CUDA events on the bound stream: before the gas face
- * kernel, after it, after the radiation/update kernel, and after the interaction kernel (one
- * thread per cell, in every form; with the interaction off the last two events coincide; with
- * vterms the velocity-term kernel runs between the last two events).
+ * kernel, after it, after the radiation/update kernel, and after the interaction kernel (with
+ * the interaction off the last two events coincide; with vterms the velocity-term kernel runs
+ * between the last two events).
  * fx_kernel_timing_enable(h, on) switches this on or off and discards what was recorded.
  * fx_kernel_timing_read(h, out) waits for the last recorded event and writes
  * out[0] = total milliseconds of the radiation/update kernel, out[1] = its launches,
